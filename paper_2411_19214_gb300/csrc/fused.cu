@@ -454,9 +454,18 @@ constexpr int kSharedTopK = 14;
 constexpr int kEpiThreads = kEpiWarps * 32;
 constexpr int kTopKListBytes = kSharedTopK * kEpiThreads * 8;
 constexpr int kWideShiftBytes = 2 * kFusedOwnRows * 4;  // kModeSweepWide: the row hand-over's shifts
+// kModeMu: each epilogue warp turns its 32 rows x mu_width columns through
+// shared memory, so that its stores run along the rows of the output (rows of
+// mu_width + 1 floats: conflict-free columns). Half the width where a
+// four-block own tile leaves no room for more.
+constexpr int mu_width(int KB) { return KB == 4 ? 16 : 32; }
+constexpr int mu_stage_floats(int KB) { return 32 * (mu_width(KB) + 1); }
 // shared memory a mode needs after the tail area
-constexpr int mode_extra_bytes(int mode) {
-  return mode == kModeTopKShared ? kTopKListBytes : (mode == kModeSweepWide ? kWideShiftBytes : 0);
+constexpr int mode_extra_bytes(int mode, int KB) {
+  return mode == kModeTopKShared  ? kTopKListBytes
+         : mode == kModeSweepWide ? kWideShiftBytes
+         : mode == kModeMu        ? kEpiWarps * mu_stage_floats(KB) * 4
+                                  : 0;
 }
 
 __device__ __forceinline__ float lds_f32(uint32_t a) {
@@ -512,21 +521,57 @@ __device__ __forceinline__ void chunk_topk_shared(const uint32_t (&v)[32], const
   }
 }
 
-// mu block: mu = 2^(c * phi_hat + g + lo) * 2^hi, where hi + lo = (shift + ell_row) log2 e.
-template <bool RS>
+// mu block: mu = 2^(c * phi_hat + g + lo) * 2^hi, where hi + lo = (shift + ell_row) log2 e;
+// 2^hi as the two factors s1, s2 (hi clamped to +-252: beyond, the product is
+// 0 or infinite all the same). The warp's 32 rows x 32 columns go through
+// `st` in shared memory, W columns at a time, so that every store of the warp
+// writes 32 / W runs of W consecutive floats of the output; lane = row before,
+// (row % (32 / W), column) after. nrow: the warp's rows inside the block, orow:
+// its first row there.
+template <bool RS, int W>
 __device__ __forceinline__ void chunk_mu(const uint32_t (&v)[32], const float* g, const float* fs, float c,
-                                         int64_t colbase, float lo, int hi, bool row_ok, int64_t r,
-                                         const FusedParams& p) {
-  if (!row_ok) return;
-  float* orow = p.out + r * p.ld;
+                                         int64_t colbase, float lo, int hi, float s1, float s2, int lane, int nrow,
+                                         int64_t orow, float* st, const FusedParams& p) {
+  const float4* g4 = reinterpret_cast<const float4*>(g);
+  float t[32];
+  float far = 0.0f;
 #pragma unroll
-  for (int i = 0; i < 32; ++i) {
-    const int64_t col = colbase + i;
-    if (col >= p.y0 && col < p.y0 + p.ny) {
-      const float t = fmaf(scaled_phi<RS>(v[i], fs, i), c, g[i]) + lo;
-      // (wide markets: an exponent beyond the FP32 range is brought back by hi first)
-      orow[col - p.y0] = fabsf(t) <= 100.0f ? ldexpf(ex2_approx(t), hi) : ex2_approx(t + (float)hi);
+  for (int i = 0; i < 8; ++i) {
+    const float4 gg = g4[i];
+    t[4 * i + 0] = fmaf(scaled_phi<RS>(v[4 * i + 0], fs, 4 * i + 0), c, gg.x) + lo;
+    t[4 * i + 1] = fmaf(scaled_phi<RS>(v[4 * i + 1], fs, 4 * i + 1), c, gg.y) + lo;
+    t[4 * i + 2] = fmaf(scaled_phi<RS>(v[4 * i + 2], fs, 4 * i + 2), c, gg.z) + lo;
+    t[4 * i + 3] = fmaf(scaled_phi<RS>(v[4 * i + 3], fs, 4 * i + 3), c, gg.w) + lo;
+    far = fmaxf(far, fmaxf(fmaxf(fabsf(t[4 * i + 0]), fabsf(t[4 * i + 1])),
+                           fmaxf(fabsf(t[4 * i + 2]), fabsf(t[4 * i + 3]))));
+  }
+  const bool near = !__any_sync(0xffffffffu, far > 100.0f);
+#pragma unroll
+  for (int c0 = 0; c0 < 32; c0 += W) {
+    float* mine = st + lane * (W + 1);
+    if (near) {
+#pragma unroll
+      for (int i = 0; i < W; ++i) mine[i] = ex2_approx(t[c0 + i]) * s1 * s2;
+    } else {
+      // (an exponent beyond the FP32 range is brought back by hi first)
+#pragma unroll
+      for (int i = 0; i < W; ++i)
+        mine[i] = fabsf(t[c0 + i]) <= 100.0f ? ex2_approx(t[c0 + i]) * s1 * s2 : ex2_approx(t[c0 + i] + (float)hi);
     }
+    __syncwarp();
+    const int64_t col = colbase + c0 + lane % W;
+    if (col >= p.y0 && col < p.y0 + p.ny) {
+      float* o = p.out + (orow + lane / W) * p.ld + (col - p.y0);
+      const float* src = st + (lane / W) * (W + 1) + lane % W;
+      const int64_t step = (32 / W) * p.ld;
+      if (nrow == 32) {
+#pragma unroll 8
+        for (int i = 0; i < W; ++i) o[i * step] = src[i * (32 / W) * (W + 1)];
+      } else {
+        for (int i = 0; i * (32 / W) + lane / W < nrow; ++i) o[i * step] = src[i * (32 / W) * (W + 1)];
+      }
+    }
+    __syncwarp();
   }
 }
 
@@ -605,7 +650,8 @@ __global__ void __launch_bounds__(kThreads, 1)
     k_fused_halfsweep(const __grid_constant__ CUtensorMap tm_own, const __grid_constant__ CUtensorMap tm_partner,
                       const FusedParams p) {
   static_assert(!BATCH || MODE == kModeSweep, "batched launches run half-sweeps only");
-  static_assert(!SPLIT || (MODE == kModeSweep && !BATCH), "partner splits are single-market half-sweeps");
+  static_assert(!SPLIT || ((MODE == kModeSweep || MODE == kModeMu) && !BATCH),
+                "partner splits are single-market half-sweeps and mu blocks");
   constexpr bool kSweepLike = MODE == kModeSweep || MODE == kModeSweepWide;
   static_assert(!(BATCH && SMALL), "batched launches use 256-row own tiles");
   constexpr int kOwn = SMALL ? kFusedOwnRows / 2 : kFusedOwnRows;  // rows of an own tile
@@ -945,6 +991,10 @@ __global__ void __launch_bounds__(kThreads, 1)
       float sum = 0.0f, comp = 0.0f;
       float mu_lo = 0.0f;
       int mu_hi = 0;
+      float mu_s1 = 1.0f, mu_s2 = 1.0f;
+      // mu blocks: this warp's first row of the block, and how many it has there
+      const int64_t mu_row = (int64_t)t * kOwn + h * 128 + q * 32;
+      const int mu_nrow = MODE == kModeMu ? (int)(p.rows - mu_row < 32 ? p.rows - mu_row : 32) : 0;
       float wide_m = -INFINITY;  // wide markets: the row's running shift (an integer, log2 units)
       if constexpr (MODE == kModeMu) {
         if (row_ok) {
@@ -952,6 +1002,9 @@ __global__ void __launch_bounds__(kThreads, 1)
           const double fl = floor(off);
           mu_hi = (int)fl;
           mu_lo = (float)(off - fl);
+          const int e = mu_hi < -252 ? -252 : (mu_hi > 252 ? 252 : mu_hi);
+          mu_s1 = __int_as_float((127 + e / 2) << 23);
+          mu_s2 = __int_as_float((127 + e - e / 2) << 23);
         }
       }
       if constexpr (MODE == kModeTopK) {
@@ -995,7 +1048,9 @@ __global__ void __launch_bounds__(kThreads, 1)
           if constexpr (MODE == kModeTopK) chunk_topk<RS>(va, gsf, fsf, crow, colbase, p.k, tv, ti, &tcnt, thr);
           if constexpr (MODE == kModeTopKShared)
             chunk_topk_shared<RS>(va, gsf, fsf, crow, colbase, p.k, lv, li, thr);
-          if constexpr (MODE == kModeMu) chunk_mu<RS>(va, gsf, fsf, crow, colbase, mu_lo, mu_hi, row_ok, r, p);
+          if constexpr (MODE == kModeMu)
+            chunk_mu<RS, mu_width(KB)>(va, gsf, fsf, crow, colbase, mu_lo, mu_hi, mu_s1, mu_s2, lane, mu_nrow, mu_row,
+                         topk_list + ew * mu_stage_floats(KB), p);
           tmem_ld_wait(vb);
         }
         // this warp's part of the accumulator buffer has been read: hand it back to the MMA warp
@@ -1011,7 +1066,8 @@ __global__ void __launch_bounds__(kThreads, 1)
           if constexpr (MODE == kModeTopKShared)
             chunk_topk_shared<RS>(vb, gsf + 32, fsf + 32, crow, colbase + 32, p.k, lv, li, thr);
           if constexpr (MODE == kModeMu)
-            chunk_mu<RS>(vb, gsf + 32, fsf + 32, crow, colbase + 32, mu_lo, mu_hi, row_ok, r, p);
+            chunk_mu<RS, mu_width(KB)>(vb, gsf + 32, fsf + 32, crow, colbase + 32, mu_lo, mu_hi, mu_s1, mu_s2, lane, mu_nrow,
+                         mu_row, topk_list + ew * mu_stage_floats(KB), p);
         }
         // the g slot has been read by this warp
         __syncwarp();
@@ -1290,7 +1346,7 @@ constexpr int kSmemLimit = 232448;  // dynamic shared memory per CTA (227 KB)
 // most 6 whole tiles (one k block per row), 4 (two) or 5 single k blocks
 // (four: 1.25 partner tiles in flight).
 constexpr int stages_for(int KB, int MODE, int fmt, bool fold) {
-  const int fixed = smem_bytes(KB, fmt, 0, fold) + mode_extra_bytes(MODE);
+  const int fixed = smem_bytes(KB, fmt, 0, fold) + mode_extra_bytes(MODE, KB);
   const int fit = (kSmemLimit - fixed) / stage_bytes(KB, fold);
   const int cap = KB == 1 ? 6 : (KB == 2 ? 4 : 5);
   return fit < cap ? fit : cap;
@@ -1301,7 +1357,7 @@ constexpr int kStages = stages_for(KB, MODE, FMT, FOLD);
 
 template <int KB, int MODE, int FMT, bool FOLD>
 constexpr int kSmemTotal =
-    smem_bytes(KB, FMT, kStages<KB, MODE, FMT, FOLD>, FOLD) + mode_extra_bytes(MODE);
+    smem_bytes(KB, FMT, kStages<KB, MODE, FMT, FOLD>, FOLD) + mode_extra_bytes(MODE, KB);
 
 // Instantiations that exist: batched launches take one or two k blocks
 // (e4m3: one); the shared-memory ranked lists leave too little room for
@@ -1313,7 +1369,8 @@ constexpr int kSmemTotal =
 // entry point).
 template <int KB, int MODE, bool BATCH, int FMT, bool SPLIT = false, bool SMALL = false, bool NOFOLD = false>
 constexpr bool kBuilt = !(BATCH && (KB == 4 || (FMT != kFmtBF16 && KB != 1))) &&
-                        !(MODE == kModeTopKShared && KB == 4) && !(SPLIT && (MODE != kModeSweep || BATCH)) &&
+                        !(MODE == kModeTopKShared && KB == 4) && !(SPLIT && MODE != kModeSweep && MODE != kModeMu) &&
+                        !(SPLIT && BATCH) && !(MODE == kModeMu && (!SPLIT || SMALL)) &&
                         !(NOFOLD && (!fold_for(KB, MODE, BATCH, FMT, false) || SPLIT || SMALL));
 
 template <int KB, int MODE, bool BATCH, int FMT = kFmtBF16, bool SMALL = false, bool SPLIT = false,
@@ -1365,6 +1422,9 @@ template <int MODE, bool BATCH>
 cudaError_t set_attributes_mode() {
   cudaError_t e = set_attributes_variant<MODE, BATCH, false>();
   if (e == cudaSuccess && !BATCH) e = set_attributes_variant<MODE, false, true>();
+  if (MODE == kModeMu) {
+    if (e == cudaSuccess) e = set_attributes_variant<MODE, false, false, true>();
+  }
   if (MODE == kModeSweep && !BATCH) {
     if (e == cudaSuccess) e = set_attributes_variant<MODE, false, false, true>();
     if (e == cudaSuccess) e = set_attributes_variant<MODE, false, true, true>();
@@ -1473,6 +1533,24 @@ FusedParams base_params(int64_t rows, int64_t row0, int64_t col0, int64_t ncols,
   return p;
 }
 
+// Partner ranges of a launch of `tiles` own tiles by `ptiles` partner tiles on
+// `sms` persistent CTAs, at most `most`: the fewest that minimise the longest
+// CTA's work, in partner tiles, where an item costs `overhead` of them besides
+// its own (own-tile load, pipeline fill, row updates).
+int best_split(int64_t tiles, int64_t ptiles, int sms, int most, double overhead) {
+  int best = 1;
+  double best_cost = 0.0;
+  for (int s = 1; s <= most && s <= ptiles; ++s) {
+    const int64_t waves = (tiles * s + sms - 1) / sms;
+    const double cost = (double)waves * ((double)((ptiles + s - 1) / s) + overhead);
+    if (s == 1 || cost < 0.98 * best_cost) {
+      best = s;
+      best_cost = cost;
+    }
+  }
+  return best;
+}
+
 int grid_for_tiles(int tiles, int num_sms) {
   int grid = tiles < num_sms ? tiles : num_sms;
   if (grid > kMaxPartials) grid = kMaxPartials;
@@ -1572,8 +1650,12 @@ cudaError_t launch_fused_topk(tu_market* m, int side, int k, int64_t row0, int64
 // vector must have been prepared in log2 mode).
 cudaError_t launch_fused_mu(tu_market* m, int64_t x0, int64_t nx, int64_t y0, int64_t ny, float* out, int64_t ld) {
   const int64_t c0 = y0 & ~(int64_t)3;  // the g bulk copies start 16-byte aligned
-  const bool small = use_small_tiles(m, nx);
-  FusedParams p = base_params(nx, x0, c0, y0 + ny - c0, m->cmul, small);
+  FusedParams p = base_params(nx, x0, c0, y0 + ny - c0, m->cmul);
+  // A block is bounded by its stores (128 KB per 256 x 128 tile), so every SM
+  // takes part: the partner tiles of an own tile go to several CTAs.
+  // (7,150 x 9,336 at d = 50: 795 us on 56 CTAs with each thread storing along
+  // its own row, 109 us with the stores turned through shared memory on 140.)
+  p.split = best_split(p.num_own_tiles, p.num_partner_tiles, m->num_sms, 64, 1.0);
   p.g = m->Y.pvec;
   p.lmax = m->st + kStShift;
   p.ell = m->X.ell;
@@ -1585,8 +1667,8 @@ cudaError_t launch_fused_mu(tu_market* m, int64_t x0, int64_t nx, int64_t y0, in
   p.ny = ny;
   p.fs_own = m->X.fs;
   p.fs_par = m->Y.fs;
-  return launch_any<kModeMu>(m->kp, fmt_of(m->dtype), m->X.tm_own, m->Y.tm_partner, p,
-                             grid_for_tiles(p.num_own_tiles, m->num_sms), m->stream, small);
+  return launch_variant<kModeMu, false, false, true>(m->kp, fmt_of(m->dtype), m->X.tm_own, m->Y.tm_partner, p,
+                                                     grid_for_tiles(p.num_own_tiles * p.split, m->num_sms), m->stream);
 }
 
 // Same kernel on caller-described buffers (no market object): used by the
