@@ -438,21 +438,36 @@ __device__ __forceinline__ void chunk_topk(const uint32_t (&v)[32], const float*
   }
 }
 
-// Ranked lists with k <= kSharedTopK (kModeTopKShared): every epilogue
-// thread keeps the k best (score, column) pairs of its row and column half in
-// shared memory, entry i of thread t at [i * kEpiThreads + t] (a warp's
-// accesses to one entry are conflict-free), sorted by decreasing score, equal
-// scores in increasing column order (the order in which a column half's
-// columns arrive). The list starts as k (-inf, INT32_MAX) pairs, so the k-th
-// score is the threshold from the first column on. An insertion shifts at
-// most k - 1 entries in shared memory. Rows whose rankings differ (a
-// converged market, where the potentials cancel the popularity terms) insert
-// at different columns, and a warp runs every lane's insertion in turn; with
-// the list in shared memory each of those costs a few shared-memory round
-// trips instead of a chain through local memory.
+// Ranked lists with k <= kSharedTopK (kModeTopKShared): every epilogue thread
+// has kTopKSlots (score, column) slots in shared memory, slot i of thread t
+// at [i * kEpiThreads + t] (a warp's accesses to one slot are conflict-free).
+// The first k hold the k best of its row and column half, sorted by
+// decreasing score, equal scores in increasing column order (the order in
+// which a column half's columns arrive); they start as (-inf, INT32_MAX)
+// pairs, so the k-th score is the threshold from the first column on. The
+// other slots buffer candidates: columns that beat the threshold as of the
+// last merge, appended in column order. When a lane's buffer could overflow,
+// the whole warp merges: all 32 lanes insert their candidates side by side.
+// Rows whose rankings differ (a converged market, where the potentials cancel
+// the popularity terms) meet their candidates at different columns; inserting
+// each at once ran the lanes' insertions one after another (3 of 32 lanes per
+// chunk and more), which cost several times the pass itself.
+// (Top-10 lists of 100,000 users over 60,000 partners, d = 64, at solved
+// potentials: 4.23 ms with every candidate inserted at once, 2.93 with
+// buffers, 2.74 with the shared bound below, 2.71 without the scores kept
+// across the vote, 2.16 with the merges of all warps at the same tiles; a
+// half-sweep of that size takes 1.4.)
 constexpr int kSharedTopK = 14;
+constexpr int kTopKSlots = 20;
 constexpr int kEpiThreads = kEpiWarps * 32;
-constexpr int kTopKListBytes = kSharedTopK * kEpiThreads * 8;
+// (the slots, then one 8-byte word per thread: the bound that the two threads
+// of a row share, see chunk_topk_shared)
+constexpr int kTopKListBytes = (kTopKSlots + 1) * kEpiThreads * 8;
+// A group of kTopKGroup columns adds at most that many candidates, so a buffer
+// of kTopKSlots - k >= kTopKGroup + 1 slots is merged whenever fewer than
+// kTopKGroup are free.
+constexpr int kTopKGroup = 4;
+static_assert(kTopKSlots - kSharedTopK > kTopKGroup, "candidate slots");
 constexpr int kWideShiftBytes = 2 * kFusedOwnRows * 4;  // kModeSweepWide: the row hand-over's shifts
 // kModeMu: each epilogue warp turns its 32 rows x mu_width columns through
 // shared memory, so that its stores run along the rows of the output (rows of
@@ -468,56 +483,138 @@ constexpr int mode_extra_bytes(int mode, int KB) {
                                   : 0;
 }
 
-__device__ __forceinline__ float lds_f32(uint32_t a) {
-  float v;
-  asm volatile("ld.shared.f32 %0, [%1];" : "=f"(v) : "r"(a));
+__device__ __forceinline__ void sts_u64(uint32_t a, uint64_t v) {
+  asm volatile("st.volatile.shared.b64 [%0], %1;" ::"r"(a), "l"(v));
+}
+__device__ __forceinline__ uint64_t lds_u64(uint32_t a) {
+  uint64_t v;
+  asm volatile("ld.volatile.shared.b64 %0, [%1];" : "=l"(v) : "r"(a));
   return v;
 }
-__device__ __forceinline__ int32_t lds_s32(uint32_t a) {
-  int32_t v;
-  asm volatile("ld.shared.s32 %0, [%1];" : "=r"(v) : "r"(a));
-  return v;
-}
-__device__ __forceinline__ void sts_f32(uint32_t a, float v) { asm volatile("st.shared.f32 [%0], %1;" ::"r"(a), "f"(v)); }
-__device__ __forceinline__ void sts_s32(uint32_t a, int32_t v) { asm volatile("st.shared.s32 [%0], %1;" ::"r"(a), "r"(v)); }
 
-// Insert (s, col) into the list at shared addresses lv (scores) and li
-// (columns) of one thread; s beats the current k-th score. Returns the new
-// k-th score. Kept out of line: one copy serves every call site.
-__device__ __noinline__ float list_insert(uint32_t lv, uint32_t li, int k, float s, int32_t col) {
-  constexpr uint32_t kStride = kEpiThreads * 4;
-  uint32_t pos = (uint32_t)(k - 1);
-  while (pos > 0) {
-    const float above = lds_f32(lv + (pos - 1) * kStride);
-    if (!(s > above)) break;
-    sts_f32(lv + pos * kStride, above);
-    sts_s32(li + pos * kStride, lds_s32(li + (pos - 1) * kStride));
-    --pos;
+// A slot: the score in the low word, the column in the high one.
+__device__ __forceinline__ uint64_t slot_of(float s, int32_t col) {
+  return ((uint64_t)(uint32_t)col << 32) | __float_as_uint(s);
+}
+__device__ __forceinline__ float slot_score(uint64_t w) { return __uint_as_float((uint32_t)w); }
+__device__ __forceinline__ int32_t slot_col(uint64_t w) { return (int32_t)(w >> 32); }
+constexpr uint32_t kSlotStride = kEpiThreads * 8;
+
+// Merge a warp's candidate buffers (cnt candidates of this lane) into its
+// lists at shared address lv: round j inserts every lane's candidate j, where
+// it beats the lane's current k-th score. An insertion reads the entries above
+// it four at a time (independent loads: one shared-memory latency per four
+// shifts). Returns the new k-th score. Kept out of line: one copy serves every
+// call site.
+__device__ __noinline__ float list_merge(uint32_t lv, int k, int cnt) {
+  const uint32_t last = lv + (uint32_t)(k - 1) * kSlotStride;
+  float thr = slot_score(lds_u64(last));
+  const int rounds = __reduce_max_sync(0xffffffffu, cnt);
+  for (int j = 0; j < rounds; ++j) {
+    const uint64_t w = j < cnt ? lds_u64(last + (uint32_t)(j + 1) * kSlotStride) : slot_of(-INFINITY, 0);
+    const float s = slot_score(w);
+    if (s > thr) {
+      uint32_t pos = last;
+      bool go = pos != lv;
+      while (go) {
+        uint64_t e[4];
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+          const uint32_t a = pos - (uint32_t)(i + 1) * kSlotStride;
+          e[i] = (int32_t)(a - lv) >= 0 ? lds_u64(a) : slot_of(INFINITY, 0);
+        }
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+          go = go && s > slot_score(e[i]);
+          if (go) {
+            sts_u64(pos, e[i]);
+            pos -= kSlotStride;
+          }
+        }
+        go = go && pos != lv;
+      }
+      sts_u64(pos, w);
+      thr = slot_score(lds_u64(last));
+    }
+    __syncwarp();
   }
-  sts_f32(lv + pos * kStride, s);
-  sts_s32(li + pos * kStride, col);
-  return lds_f32(lv + (uint32_t)(k - 1) * kStride);
+  return thr;
 }
 
+// A row's columns are split over two threads (column halves), each with its own
+// list. If both lists hold ceil(k / 2) scores of at least b, the row's k-th
+// best is at least b: a column below b cannot be listed. So each thread
+// publishes, after every merge, the value just below its list's
+// ceil(k / 2)-th score (so that equal scores still pass), tagged with its own
+// tile, and takes as threshold the larger of its k-th score and the smaller
+// of the two published values: about the k-th best of both halves together,
+// which halves the candidates. A word of an older tile (or one read while the
+// other thread is a merge behind) only makes the bound weaker, never wrong, so
+// the lists do not depend on timing.
+struct SharedBound {
+  uint32_t mine, other;  // shared addresses of the two threads' words
+  uint32_t tag;          // the own tile, counted per CTA
+  float pub;             // this thread's published value
+  __device__ __forceinline__ void publish(uint32_t lv, int k) {
+    pub = nextafterf(slot_score(lds_u64(lv + (uint32_t)((k - 1) / 2) * kSlotStride)), -INFINITY);
+    sts_u64(mine, ((uint64_t)tag << 32) | __float_as_uint(pub));
+  }
+  __device__ __forceinline__ float bound() const {
+    const uint64_t w = lds_u64(other);
+    return (uint32_t)(w >> 32) == tag ? fminf(pub, __uint_as_float((uint32_t)w)) : -INFINITY;
+  }
+};
+
+// One 32-column chunk: the scores' maximum in every group of four columns; the
+// groups in which some lane beats its threshold form their scores again and
+// append them (keeping all 32 beside the next chunk's TMEM load in flight
+// would spill).
 template <bool RS>
-__device__ __forceinline__ void chunk_topk_shared(const uint32_t (&v)[32], const float* g, const float* fs, float c,
-                                                  int64_t colbase, int k, uint32_t lv, uint32_t li, float& thr) {
+__device__ __forceinline__ void chunk_topk_shared(const uint32_t (&v)[32], const float* g, const float* fs,
+                                                  uint64_t cc, int64_t colbase, int k, uint32_t lv, int& cnt,
+                                                  float& thr, SharedBound& sb) {
+  constexpr int kGroups = 32 / kTopKGroup;
+  static_assert(kTopKGroup == 4, "a group is one float4 of g");
   const float4* g4 = reinterpret_cast<const float4*>(g);
-  float s[32];
-  float mx = -INFINITY;
+  const float4* fs4 = reinterpret_cast<const float4*>(fs);
+  auto scores = [&](int i, float (&s)[4]) {
+    const float4 gg = g4[i];
+    float4 ff = make_float4(1.f, 1.f, 1.f, 1.f);
+    if constexpr (RS) ff = fs4[i];
+    const uint64_t t0 = pair_exponents<RS>(v[4 * i + 0], v[4 * i + 1], gg.x, gg.y, ff.x, ff.y, cc);
+    const uint64_t t1 = pair_exponents<RS>(v[4 * i + 2], v[4 * i + 3], gg.z, gg.w, ff.z, ff.w, cc);
+    s[0] = __uint_as_float((uint32_t)t0);
+    s[1] = __uint_as_float((uint32_t)(t0 >> 32));
+    s[2] = __uint_as_float((uint32_t)t1);
+    s[3] = __uint_as_float((uint32_t)(t1 >> 32));
+  };
+  thr = fmaxf(thr, sb.bound());
+  uint32_t hit = 0;
 #pragma unroll
-  for (int i4 = 0; i4 < 8; ++i4) {
-    const float4 gg = g4[i4];
-    s[4 * i4 + 0] = fmaf(scaled_phi<RS>(v[4 * i4 + 0], fs, 4 * i4 + 0), c, gg.x);
-    s[4 * i4 + 1] = fmaf(scaled_phi<RS>(v[4 * i4 + 1], fs, 4 * i4 + 1), c, gg.y);
-    s[4 * i4 + 2] = fmaf(scaled_phi<RS>(v[4 * i4 + 2], fs, 4 * i4 + 2), c, gg.z);
-    s[4 * i4 + 3] = fmaf(scaled_phi<RS>(v[4 * i4 + 3], fs, 4 * i4 + 3), c, gg.w);
-    mx = fmaxf(mx, fmaxf(fmaxf(s[4 * i4 + 0], s[4 * i4 + 1]), fmaxf(s[4 * i4 + 2], s[4 * i4 + 3])));
+  for (int i = 0; i < kGroups; ++i) {
+    float s[4];
+    scores(i, s);
+    if (fmaxf(fmaxf(s[0], s[1]), fmaxf(s[2], s[3])) > thr) hit |= 1u << i;
   }
-  if (mx > thr) {
+  hit = __reduce_or_sync(0xffffffffu, hit);
+  if (hit == 0) return;
 #pragma unroll
-    for (int e = 0; e < 32; ++e)
-      if (s[e] > thr) thr = list_insert(lv, li, k, s[e], (int32_t)(colbase + e));
+  for (int i = 0; i < kGroups; ++i) {
+    if ((hit & (1u << i)) == 0) continue;
+    float s[4];
+    scores(i, s);
+#pragma unroll
+    for (int e = 0; e < 4; ++e) {
+      if (s[e] > thr) {
+        sts_u64(lv + (uint32_t)(k + cnt) * kSlotStride, slot_of(s[e], (int32_t)(colbase + 4 * i + e)));
+        ++cnt;
+      }
+    }
+    if (__any_sync(0xffffffffu, cnt > kTopKSlots - k - kTopKGroup)) {
+      thr = list_merge(lv, k, cnt);
+      sb.publish(lv, k);
+      cnt = 0;
+    }
   }
 }
 
@@ -742,6 +839,11 @@ __global__ void __launch_bounds__(kThreads, 1)
     }
     asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
   }
+  if constexpr (MODE == kModeTopKShared) {
+    // no published bound yet (tags start at 1; shared memory may hold another launch's words)
+    if (threadIdx.x >= 64)
+      sts_u64(smem_u32(topk_list) + (uint32_t)(kTopKSlots * kEpiThreads + (int)threadIdx.x - 64) * 8u, 0ull);
+  }
   tc_fence_before();
   __syncthreads();
   tc_fence_after();
@@ -955,9 +1057,16 @@ __global__ void __launch_bounds__(kThreads, 1)
     float tv[MODE == kModeTopK ? kMaxTopK : 1];
     int32_t ti[MODE == kModeTopK ? kMaxTopK : 1];
     // shared-memory lists (k <= kSharedTopK): this thread's entry 0
-    const uint32_t lv = smem_u32(topk_list) + (uint32_t)(ew * 32 + lane) * 4u;
-    const uint32_t li = lv + (uint32_t)(kSharedTopK * kEpiThreads) * 4u;
+    const uint32_t lv = smem_u32(topk_list) + (uint32_t)(ew * 32 + lane) * 8u;
+    SharedBound sb{};
+    {
+      // (rows' other column half: epilogue warp ew ^ 8)
+      const uint32_t words = smem_u32(topk_list) + (uint32_t)(kTopKSlots * kEpiThreads) * 8u;
+      sb.mine = words + (uint32_t)(ew * 32 + lane) * 8u;
+      sb.other = words + (uint32_t)((ew ^ 8) * 32 + lane) * 8u;
+    }
     int tcnt = 0;
+    int merge_at = 0;  // the partner tile before which every warp merges its candidates
     float thr = -INFINITY;
     int tile_iter = 0;
     for (int it = item_begin<BATCH>(p); it < item_end<BATCH, SPLIT>(p) && ok; it += item_step<BATCH>(), ++tile_iter) {
@@ -1012,11 +1121,13 @@ __global__ void __launch_bounds__(kThreads, 1)
         thr = -INFINITY;
       }
       if constexpr (MODE == kModeTopKShared) {
-        for (int i = 0; i < p.k; ++i) {
-          sts_f32(lv + (uint32_t)(i * kEpiThreads) * 4u, -INFINITY);
-          sts_s32(li + (uint32_t)(i * kEpiThreads) * 4u, 0x7fffffff);
-        }
+        for (int i = 0; i < p.k; ++i) sts_u64(lv + (uint32_t)i * kSlotStride, slot_of(-INFINITY, 0x7fffffff));
         thr = -INFINITY;
+        tcnt = 0;
+        merge_at = jb + 1;
+        sb.tag = (uint32_t)tile_iter + 1u;
+        sb.pub = -INFINITY;
+        sts_u64(sb.mine, ((uint64_t)sb.tag << 32) | __float_as_uint(-INFINITY));
       }
       for (int j = jb; j < je; ++j) {
         // every lane waits; the outcome is made warp-uniform so that the
@@ -1047,7 +1158,7 @@ __global__ void __launch_bounds__(kThreads, 1)
           if constexpr (MODE == kModeSweepWide) chunk_sum_wide<RS>(va, gs4, fs4, cc, acc, wide_m, sum, comp);
           if constexpr (MODE == kModeTopK) chunk_topk<RS>(va, gsf, fsf, crow, colbase, p.k, tv, ti, &tcnt, thr);
           if constexpr (MODE == kModeTopKShared)
-            chunk_topk_shared<RS>(va, gsf, fsf, crow, colbase, p.k, lv, li, thr);
+            chunk_topk_shared<RS>(va, gsf, fsf, cc, colbase, p.k, lv, tcnt, thr, sb);
           if constexpr (MODE == kModeMu)
             chunk_mu<RS, mu_width(KB)>(va, gsf, fsf, crow, colbase, mu_lo, mu_hi, mu_s1, mu_s2, lane, mu_nrow, mu_row,
                          topk_list + ew * mu_stage_floats(KB), p);
@@ -1064,7 +1175,7 @@ __global__ void __launch_bounds__(kThreads, 1)
           if constexpr (MODE == kModeTopK)
             chunk_topk<RS>(vb, gsf + 32, fsf + 32, crow, colbase + 32, p.k, tv, ti, &tcnt, thr);
           if constexpr (MODE == kModeTopKShared)
-            chunk_topk_shared<RS>(vb, gsf + 32, fsf + 32, crow, colbase + 32, p.k, lv, li, thr);
+            chunk_topk_shared<RS>(vb, gsf + 32, fsf + 32, cc, colbase + 32, p.k, lv, tcnt, thr, sb);
           if constexpr (MODE == kModeMu)
             chunk_mu<RS, mu_width(KB)>(vb, gsf + 32, fsf + 32, crow, colbase + 32, mu_lo, mu_hi, mu_s1, mu_s2, lane, mu_nrow,
                          mu_row, topk_list + ew * mu_stage_floats(KB), p);
@@ -1081,6 +1192,20 @@ __global__ void __launch_bounds__(kThreads, 1)
           comp = (tsum - sum) - y;
           sum = tsum;
         }
+        if constexpr (MODE == kModeTopKShared) {
+          // All warps merge after the same tiles, each a quarter further into
+          // the row: a merge takes some thousand cycles, and the accumulator
+          // buffers let a warp run two tiles ahead of the slowest, so merges
+          // at different tiles would hold up the whole CTA one after another.
+          if (j + 1 == merge_at) {
+            merge_at += 1 + (merge_at - jb) / 4;
+            if (!idle) {
+              thr = list_merge(lv, p.k, tcnt);
+              sb.publish(lv, p.k);
+              tcnt = 0;
+            }
+          }
+        }
         buf ^= 1;
         if (buf == 0) tphase ^= 1u;
         if (++gs == kGSlots) {
@@ -1090,6 +1215,9 @@ __global__ void __launch_bounds__(kThreads, 1)
       }
       if (!ok) break;
       if constexpr (MODE == kModeMu) continue;
+      if constexpr (MODE == kModeTopKShared) {
+        if (!(SMALL && h == 1)) list_merge(lv, p.k, tcnt);
+      }
       // the two column halves of a row meet (double-buffered by own-tile
       // parity, handed over through bounded mbarrier waits)
       const int pb = tile_iter & 1;
@@ -1112,8 +1240,9 @@ __global__ void __launch_bounds__(kThreads, 1)
         if constexpr (MODE == kModeTopKShared) {
           if (row_ok)
             for (int i = 0; i < p.k; ++i) {
-              p.hand_v[r * p.k + i] = lds_f32(lv + (uint32_t)(i * kEpiThreads) * 4u);
-              p.hand_i[r * p.k + i] = lds_s32(li + (uint32_t)(i * kEpiThreads) * 4u);
+              const uint64_t w = lds_u64(lv + (uint32_t)i * kSlotStride);
+              p.hand_v[r * p.k + i] = slot_score(w);
+              p.hand_i[r * p.k + i] = slot_col(w);
             }
         }
         __syncwarp();
@@ -1149,8 +1278,9 @@ __global__ void __launch_bounds__(kThreads, 1)
           const double base = shift + p.ell[p.row0 + r];
           int a = 0, b = 0;
           for (int i = 0; i < p.k; ++i) {
-            const float av = lds_f32(lv + (uint32_t)(a * kEpiThreads) * 4u);
-            const int32_t ai = lds_s32(li + (uint32_t)(a * kEpiThreads) * 4u);
+            const uint64_t w = lds_u64(lv + (uint32_t)a * kSlotStride);
+            const float av = slot_score(w);
+            const int32_t ai = slot_col(w);
             const float bv = p.hand_v[r * p.k + b];
             const int32_t bi = p.hand_i[r * p.k + b];
             const bool take_a = av > bv || (av == bv && ai < bi);
