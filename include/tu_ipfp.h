@@ -26,8 +26,10 @@
  *                  256).
  *   TU_PATH_DENSE  batch IPFP (Alg. 1 / Eq. iteration_matrix): the FP32 kernel
  *                  A-hat = exp((Phi - b^X - b^Y) / (2 sigma)) is materialised
- *                  once, with its transpose (2*N*M*4 bytes), and one of the
- *                  two is streamed every half-sweep.
+ *                  once, with its transpose (2*N*M*4 bytes). A sweep streams
+ *                  A-hat once for both half-sweeps (512 to 81,920 users per
+ *                  side Y, at least 512 on side X, no over-relaxation), or
+ *                  else A-hat and its transpose in turn.
  *
  * Conventions shared by every entry point:
  *   - Return codes only; nothing is thrown across the ABI.
@@ -419,7 +421,7 @@ int64_t tu_market_footprint(int64_t N, int64_t M, int64_t d, int path);
 /* Kernel timing for benchmarks (no counterpart in the paper). While enabled,
  * every half-sweep pass records a CUDA event pair on the market's stream
  * around its main kernel (fused: the tcgen05 half-sweep; dense: the row pass,
- * or the two column-pass kernels), and sweeps are launched directly instead of
+ * or the one pass of a whole sweep), and sweeps are launched directly instead of
  * through a captured graph. tu_profile_read synchronises the stream, returns
  * the summed elapsed milliseconds and the number of timed passes since the
  * last read (either pointer may be NULL), and starts a new count. */

@@ -2,7 +2,8 @@
 // FP32 kernel. A-hat_xy = exp((Phi_xy - b^X_x - b^Y_y) / (2 sigma)) is built
 // once; the biases live in the potentials (ell = log u + b / (2 sigma)), so
 //     s_x = 1/2 exp(b^X_x / 2 sigma) sum_y A-hat_xy exp(ell_y)
-// and every half-sweep is one HBM stream over a row-major matrix.
+// and sweeps are HBM streams over a row-major matrix: one per sweep
+// (k_dense_sweep) where the market's shape allows it, else one per half-sweep.
 //
 // HBM layout: A-hat (N x ldA, ldA = M rounded up to 4) and its transpose
 // (M x ldN). With both resident, the v step (s = A^T u / 2) is the same row
@@ -345,6 +346,564 @@ __global__ void __launch_bounds__(kPassThreads) k_dense_rowpass(
   }
 }
 
+// One sweep from one pass over A-hat. The v step needs s_y = 1/2 sum_x A_xy u_x
+// with the new u, and row x of A-hat is all that u_x needs: so while a row is
+// in shared memory, its dot product with v gives u_x, and the row scaled by u_x
+// is added to the column sums. A-hat is read once per sweep instead of A-hat and
+// its transpose (at 20,000 x 10,000 two passes of 800 MB took 2 x 120 us).
+//
+// Roles of a CTA (a cluster of `cl` CTAs shares every row when it is longer
+// than kSweepWidth columns; each holds a slice of the columns):
+//   producer warp   streams units of `rows` rows (one slice of a row in a
+//                   cluster) into a ring in shared memory with bulk copies.
+//   dot warps       every thread owns fixed columns, its part of v in registers;
+//                   a row's dot product is parked per warp.
+//   update warp     (the cluster's first CTA) sums a unit's parked shares and
+//                   hands the rows' weights 2^(ell log2 e - R) to the sum warps
+//                   of the cluster, in FP32.
+//   sum warps       every thread owns fixed columns, their sums (compensated) in
+//                   registers: a unit is added once its weights are there, and
+//                   its slot released.
+//   row warp        (the cluster's first CTA) the rows' stored potentials in
+//                   FP64, residual and groups, 32 rows at a time, off the path.
+// The pass takes 127 us at 20,000 x 10,000 (6.3 TB/s, 0.93 of the measured copy
+// rate); a sweep 272 -> 161 us. Rows in clusters: 30,000 x 30,000 1,106 -> 755 us
+// per sweep, 3,000 x 40,000 208 -> 131. The shares and weights of a cluster travel
+// by asynchronous stores; with plain remote stores and releasing arrivals its
+// update warp took 1.5 us per row and the pass was slower than two.
+// A row passes through load, dot, update and sum one after another, about
+// 5,000 cycles; with one slot of the ring per row in flight the SM still takes
+// one 40 KB row per 1,700 cycles, its share of HBM. (One set of warps doing
+// both products in turn was the bound: 165 us per 800 MB pass.)
+// R is an integer per cluster, raised when a row's exponent passes it by 40
+// (weights up to 2^40 against A-hat up to e^40 stay in the FP32 range); the
+// column sums so far are then rescaled by a power of two, exactly. At the end
+// each CTA writes its column sums and R; k_dense_cols adds them up.
+// A unit is at most 40 KB and the ring takes what shared memory there is.
+// 2^d for any integer d, exactly, flushed to 0 below FP32's normal range and to infinity above it
+__device__ __forceinline__ float exp2_whole(int d) {
+  return d < -126 ? 0.0f : (d > 127 ? INFINITY : __int_as_float((127 + d) << 23));
+}
+
+constexpr int kSweepWidth = 10240;  // columns of a slice, at most
+constexpr int kSweepSums = 12;      // sum warps (28 columns per thread, at most)
+constexpr int kSweepDots = 5;       // dot warps (64 columns per thread, at most)
+constexpr int kSweepRows = 8;       // rows of a unit, at most
+constexpr int kSweepSlots = 24;     // ring slots, at most
+constexpr int kSweepCl = 8;         // cluster size, at most
+constexpr int kSweepUpdate = kSweepSums + kSweepDots;  // the update warp
+constexpr int kSweepProducer = kSweepUpdate + 1;       // the producer warp; then the row warp
+constexpr int kSweepThreads = (kSweepUpdate + 3) * 32;
+constexpr int kSweepMinCols = 512;  // fewer columns leave most threads without work
+
+// Packed pairs of floats, and four floats as two of them.
+struct __align__(16) Quad {
+  uint64_t x, y;
+};
+__device__ __forceinline__ uint64_t pack2(float a, float b) {
+  return ((uint64_t)__float_as_uint(b) << 32) | __float_as_uint(a);
+}
+__device__ __forceinline__ float low2(uint64_t v) { return __uint_as_float((uint32_t)v); }
+__device__ __forceinline__ float high2(uint64_t v) { return __uint_as_float((uint32_t)(v >> 32)); }
+__device__ __forceinline__ uint64_t fma2(uint64_t a, uint64_t b, uint64_t c) {
+  uint64_t d;
+  asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(d) : "l"(a), "l"(b), "l"(c));
+  return d;
+}
+__device__ __forceinline__ uint64_t add2(uint64_t a, uint64_t b) {
+  uint64_t d;
+  asm("add.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b));
+  return d;
+}
+__device__ __forceinline__ uint64_t sub2(uint64_t a, uint64_t b) {
+  uint64_t d;
+  asm("sub.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b));
+  return d;
+}
+__device__ __forceinline__ uint64_t mul2(uint64_t a, uint64_t b) {
+  uint64_t d;
+  asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b));
+  return d;
+}
+// kahan_fma on pairs; n is the compensation with its sign turned
+__device__ __forceinline__ void kahan_fma2(uint64_t& s, uint64_t& n, uint64_t x, uint64_t w) {
+  const uint64_t y = fma2(x, w, n);
+  const uint64_t t = add2(s, y);
+  n = sub2(y, sub2(t, s));
+  s = t;
+}
+
+struct SweepSmem {
+  // per slot of the ring: a unit's parked shares (the cluster's first CTA; a
+  // cluster's units are one row), its rows' weights, the factor that the column
+  // sums so far take before them (in a cluster: beside the one weight)
+  float part[kSweepSlots][kSweepRows][kSweepDots];
+  float weight[kSweepSlots][kSweepRows];
+  float scale[kSweepSlots];
+  float4 row[2][32];            // a batch's rows: log2 constants of their updates
+  float2 sum[2][32];            // and their sums (hi, lo)
+  uint64_t full[kSweepSlots];   // a unit has landed
+  uint64_t empty[kSweepSlots];  // every sum warp is done with it
+  uint64_t done[kSweepSlots];   // its shares are parked
+  uint64_t ready[kSweepSlots];  // its weights are here
+  uint64_t ahead[2];            // a batch's constants are here
+  uint64_t summed[2];           // a batch's sums are here
+  int abort;
+};
+static_assert(kSweepRows >= kSweepCl, "a cluster's shares of one row use the unit's rows");
+constexpr size_t kSweepRing = (sizeof(SweepSmem) + 127) / 128 * 128;  // the ring's offset
+constexpr size_t kSweepSmemMax = 232448;                              // shared memory of a CTA
+
+struct SweepArgs {
+  const float* A;
+  int64_t ld, rows;
+  const float* w;  // the partner vector exp(ell - shift), zero-padded
+  const double* st;
+  const float* b2s;
+  const double* mass;
+  double* log_u;
+  double* ell;
+  float4* grp;
+  int64_t grp_units;  // groups per cluster
+  double* partials;
+  int residual;
+  int* err;
+  float* colsum;  // clusters x ld
+  int* scale;     // R of each cluster
+  DensePlan plan;
+};
+
+// NA, ND: groups of four columns per thread of the sum and of the dot warps
+template <int NA, int ND, bool CLUSTER>
+__global__ void __launch_bounds__(kSweepThreads, 1) k_dense_sweep(const SweepArgs a) {
+  extern __shared__ __align__(128) uint8_t sweep_smem_raw[];
+  SweepSmem& S = *reinterpret_cast<SweepSmem*>(sweep_smem_raw);
+  float* ring = reinterpret_cast<float*>(sweep_smem_raw + kSweepRing);
+  const int warp = threadIdx.x / 32, lane = threadIdx.x % 32;
+  volatile int* abort_flag = &S.abort;
+  const int cl = CLUSTER ? a.plan.cl : 1;
+  const int rank = CLUSTER ? (int)cluster_rank() : 0;
+  const int64_t P = a.plan.clusters;
+  const int64_t cid = CLUSTER ? blockIdx.x / cl : blockIdx.x;
+  const int B = CLUSTER ? 1 : a.plan.rows;
+  const int slots = a.plan.slots;
+  const int64_t c0 = (int64_t)rank * a.plan.width;
+  const int width = (int)(a.ld - c0 < a.plan.width ? a.ld - c0 : a.plan.width);  // (never empty, see dense_plan)
+  const int slot_floats = B * a.plan.width;
+  const int64_t units = (a.rows + B - 1) / B;
+  const int64_t nu = (units - cid + P - 1) / P;  // this cluster's units: cid, cid + P, ...
+  if (threadIdx.x == 0) {
+    for (int t = 0; t < slots; ++t) {
+      mbar_init(&S.full[t], 1);
+      mbar_init(&S.empty[t], kSweepSums);
+      mbar_init(&S.done[t], CLUSTER ? 1 : kSweepDots);
+      mbar_init(&S.ready[t], 1);
+    }
+    for (int t = 0; t < 2; ++t) {
+      mbar_init(&S.ahead[t], 1);
+      mbar_init(&S.summed[t], 1);
+    }
+    S.abort = 0;
+    fence_mbar_init();
+  }
+  if constexpr (CLUSTER) {
+    cluster_sync();
+  } else {
+    __syncthreads();
+  }
+
+  if (warp == kSweepProducer) {
+    // ---------------------------------------------------------- producer
+    if (lane == 0) {
+      int t = 0;
+      uint32_t ph = 0, issued = 0, issued_ph = 0;
+      bool ok = true;
+      for (int64_t k = 0; k < nu; ++k) {
+        if (!mbar_wait(&S.empty[t], ph ^ 1u, abort_flag)) {
+          ok = false;
+          break;
+        }
+        const int64_t r0 = (cid + k * P) * B;
+        const int nb = (int)(a.rows - r0 < B ? a.rows - r0 : B);
+        // (outside a cluster a unit's rows are one run of memory)
+        const uint32_t bytes = (uint32_t)(CLUSTER ? width : nb * width) * 4u;
+        if constexpr (CLUSTER) {
+          // what the unit's barriers will count: the weight and scale, and in the
+          // first CTA every dot warp's share (both sent by asynchronous stores)
+          mbar_arrive_expect_tx(&S.ready[t], 8u);
+          if (rank == 0) mbar_arrive_expect_tx(&S.done[t], (uint32_t)(4 * kSweepDots * cl));
+        }
+        mbar_arrive_expect_tx(&S.full[t], bytes);
+        bulk_copy(ring + (size_t)t * slot_floats, a.A + r0 * a.ld + c0, bytes, &S.full[t]);
+        issued |= 1u << t;
+        issued_ph = (issued_ph & ~(1u << t)) | (ph << t);
+        if (++t == slots) {
+          t = 0;
+          ph ^= 1u;
+        }
+      }
+      if (!ok && !*abort_flag) pass_abort(a.err, abort_flag);
+      // copies in flight complete before the CTA's shared memory is released
+      for (int u = 0; u < slots; ++u)
+        if (issued & (1u << u)) mbar_wait_drain(&S.full[u], (issued_ph >> u) & 1u, 100000000ull);
+    }
+    __syncwarp();
+  } else if (warp < kSweepSums) {
+    // ---------------------------------------------------------- sum warps
+    constexpr int kStep = kSweepSums * 32;
+    const int nq = width / 4;
+    Quad s[NA], e[NA];  // the column sums and their compensations
+#pragma unroll
+    for (int j = 0; j < NA; ++j) s[j] = e[j] = Quad{0ull, 0ull};
+    int t = 0;
+    uint32_t ph = 0;
+    bool ok = true;
+    for (int64_t k = 0; k < nu; ++k) {
+      if (!__all_sync(0xffffffffu, mbar_wait(&S.ready[t], ph, abort_flag))) {
+        ok = false;
+        break;
+      }
+      // (the copy's own writes are made visible by its barrier)
+      if (!__all_sync(0xffffffffu, mbar_wait(&S.full[t], ph, abort_flag))) {
+        ok = false;
+        break;
+      }
+      const float sc = *reinterpret_cast<volatile float*>(CLUSTER ? &S.weight[t][1] : &S.scale[t]);
+      if (sc != 1.0f) {
+        const uint64_t sc2 = pack2(sc, sc);
+#pragma unroll
+        for (int j = 0; j < NA; ++j) {
+          s[j] = Quad{mul2(s[j].x, sc2), mul2(s[j].y, sc2)};
+          e[j] = Quad{mul2(e[j].x, sc2), mul2(e[j].y, sc2)};
+        }
+      }
+      const int64_t r0 = (cid + k * P) * B;
+      const int nb = (int)(a.rows - r0 < B ? a.rows - r0 : B);
+      const Quad* r4 = reinterpret_cast<const Quad*>(ring + (size_t)t * slot_floats) + threadIdx.x;
+      for (int b = 0; b < nb; ++b, r4 += nq) {
+        const float u = *reinterpret_cast<volatile float*>(&S.weight[t][b]);
+        const uint64_t uu = pack2(u, u);
+#pragma unroll
+        for (int j = 0; j < NA; ++j) {
+          if ((int)threadIdx.x + j * kStep < nq) {
+            const Quad x = r4[j * kStep];
+            kahan_fma2(s[j].x, e[j].x, x.x, uu);
+            kahan_fma2(s[j].y, e[j].y, x.y, uu);
+          }
+        }
+      }
+      __syncwarp();
+      if (lane == 0) mbar_arrive(&S.empty[t]);
+      if (++t == slots) {
+        t = 0;
+        ph ^= 1u;
+      }
+    }
+    if (ok) {
+      Quad* out = reinterpret_cast<Quad*>(a.colsum + cid * a.ld + c0) + threadIdx.x;
+#pragma unroll
+      for (int j = 0; j < NA; ++j)
+        if ((int)threadIdx.x + j * kStep < nq) out[j * kStep] = Quad{add2(s[j].x, e[j].x), add2(s[j].y, e[j].y)};
+    } else if (!*abort_flag) {
+      pass_abort(a.err, abort_flag);
+    }
+  } else if (warp < kSweepUpdate) {
+    // ---------------------------------------------------------- dot warps
+    constexpr int kStep = kSweepDots * 32;
+    const int dw = warp - kSweepSums, tid = dw * 32 + lane;
+    const int nq = width / 4;
+    const Quad* w4 = reinterpret_cast<const Quad*>(a.w + c0) + tid;
+    Quad w[ND];  // this thread's part of v
+#pragma unroll
+    for (int j = 0; j < ND; ++j) w[j] = tid + j * kStep < nq ? w4[j * kStep] : Quad{0ull, 0ull};
+    int t = 0;
+    uint32_t ph = 0;
+    bool ok = true;
+    for (int64_t k = 0; k < nu; ++k) {
+      if (!__all_sync(0xffffffffu, mbar_wait(&S.full[t], ph, abort_flag))) {
+        ok = false;
+        break;
+      }
+      const int64_t r0 = (cid + k * P) * B;
+      const int nb = (int)(a.rows - r0 < B ? a.rows - r0 : B);
+      const Quad* r4 = reinterpret_cast<const Quad*>(ring + (size_t)t * slot_floats) + tid;
+      for (int b = 0; b < nb; ++b, r4 += nq) {
+        uint64_t d0 = 0ull, d1 = 0ull;
+#pragma unroll
+        for (int j = 0; j < ND; ++j) {
+          if (tid + j * kStep < nq) {
+            const Quad x = r4[j * kStep];
+            d0 = fma2(x.x, w[j].x, d0);
+            d1 = fma2(x.y, w[j].y, d1);
+          }
+        }
+        d0 = add2(d0, d1);
+        float r = low2(d0) + high2(d0);
+        for (int o = 16; o > 0; o >>= 1) r += __shfl_xor_sync(0xffffffffu, r, o);
+        if (lane == 0) {
+          if constexpr (CLUSTER) {
+            cluster_store_async(cluster_addr(&S.part[t][rank][dw], 0), r, cluster_addr(&S.done[t], 0));
+          } else {
+            S.part[t][b][dw] = r;
+          }
+        }
+      }
+      if (!CLUSTER && lane == 0) mbar_arrive(&S.done[t]);
+      __syncwarp();
+      if (++t == slots) {
+        t = 0;
+        ph ^= 1u;
+      }
+    }
+    if (!ok && !*abort_flag) pass_abort(a.err, abort_flag);
+  } else if (warp == kSweepUpdate) {
+    // ---------------------------------------------------------- update warp
+    if (rank == 0) {
+      int R = 0, pb = 0;
+      uint32_t dph = 0;
+      bool ok = true;
+      for (int64_t k = 0; k < nu; ++k) {
+        const int64_t r0 = (cid + k * P) * B;
+        const int nb = (int)(a.rows - r0 < B ? a.rows - r0 : B);
+        const bool mine = lane < nb;
+        const int64_t batch = k * B / 32;
+        const int at = (int)(k * B % 32) + (mine ? lane : 0);  // this row in its batch
+        const int bb = (int)(batch & 1);
+        bool got = at - (mine ? lane : 0) != 0 || mbar_wait(&S.ahead[bb], (uint32_t)(batch >> 1) & 1u, abort_flag);
+        got = got && mbar_wait(&S.done[pb], dph, abort_flag);
+        if (!__all_sync(0xffffffffu, got)) {
+          ok = false;
+          break;
+        }
+        // the warps' shares of a row, added with their roundings kept
+        float hi = 0.0f, lo = 0.0f;
+        if constexpr (CLUSTER) {
+          const volatile float* p = S.part[pb][0];
+          for (int i = lane; i < kSweepDots * cl; i += 32) pair_add(hi, lo, p[i], 0.0f);
+          for (int o = 16; o > 0; o >>= 1)
+            pair_add(hi, lo, __shfl_xor_sync(0xffffffffu, hi, o), __shfl_xor_sync(0xffffffffu, lo, o));
+        } else {
+          const volatile float* p = S.part[pb][mine ? lane : 0];
+#pragma unroll
+          for (int i = 0; i < kSweepDots; ++i) pair_add(hi, lo, p[i], 0.0f);
+        }
+        // The row's weight u 2^-R in FP32: log2 of the sum and of u are each an
+        // integer plus a fraction, so that no digits go to their size
+        // (row_log_u's closed form with z = log s - 1/2 log n in log2 units).
+        const volatile float4* cst = reinterpret_cast<const volatile float4*>(&S.row[bb][at]);
+        const int nc = __float_as_int(cst->x), nB = __float_as_int(cst->z);
+        const float fc = cst->y, fB = cst->w;
+        int ex;
+        const float m = frexpf(hi, &ex);
+        const float rel = __fdividef(lo, hi) * kLog2e;
+        const float lm = log2f(m) + rel;
+        const float z2 = (float)(nc + ex) + (fc + lm);
+        int n;
+        float f;
+        if (z2 > 0.0f) {
+          const float c = log1pf(sqrtf(1.0f + exp2f(-2.0f * z2)));
+          n = nB - nc - ex;
+          f = ((fB - fc) - lm) - c * kLog2e;
+        } else {
+          n = nB;
+          f = fB - asinhf(exp2f(z2)) * kLog2e;
+        }
+        const int top = __reduce_max_sync(0xffffffffu, mine ? n : -0x40000000);
+        float sc = 1.0f;
+        if (k == 0 || top > R + 40) {
+          if (k > 0) sc = exp2_whole(R - top);
+          R = top;
+        }
+        // (a sum that is not finite makes the weight so, or 0 for an infinite one)
+        const float u = exp2f(f) * exp2_whole(n - R);
+        if constexpr (CLUSTER) {
+          const float u0 = __shfl_sync(0xffffffffu, u, 0);
+          if (lane < cl)
+            cluster_store_async2(cluster_addr(&S.weight[pb][0], lane), u0, sc, cluster_addr(&S.ready[pb], lane));
+        } else {
+          if (mine) S.weight[pb][lane] = u;
+          if (lane == 0) S.scale[pb] = sc;
+          __syncwarp();
+          if (lane == 0) mbar_arrive(&S.ready[pb]);
+        }
+        if (mine) S.sum[bb][at] = make_float2(hi, lo);
+        __syncwarp();
+        if (lane == 0 && ((k + 1) * B % 32 == 0 || k == nu - 1)) mbar_arrive(&S.summed[bb]);
+        if (++pb == slots) {
+          pb = 0;
+          dph ^= 1u;
+        }
+      }
+      if (ok && lane == 0) a.scale[cid] = R;
+      if (!ok && !*abort_flag) pass_abort(a.err, abort_flag);
+    }
+  } else if (rank == 0) {
+    // ---------------------------------------------------------- row warp
+    // Batches of 32 of the cluster's rows, one per lane: what the update warp
+    // needs of them, a batch ahead; then, from their sums, the FP64 update of
+    // the stored potentials, the residual and the batch's group. FP64 runs at a
+    // few operations per clock and SM: a row's chain of it takes microseconds,
+    // which the update warp cannot wait for.
+    PartialAcc acc;
+    const double shift = a.st[kStShift], own_off = a.st[kStOwnOff];
+    const int64_t last0 = (cid + (nu - 1) * P) * B;
+    const int64_t nr = (nu - 1) * B + (a.rows - last0 < B ? a.rows - last0 : B);  // this cluster's rows
+    const int64_t batches = (nr + 31) / 32;
+    auto row_of = [&](int64_t i) { return (cid + i / B * P) * B + i % B; };
+    auto ahead = [&](int64_t j) {
+      const int64_t i = j * 32 + lane;
+      if (i < nr) {
+        const int64_t row = row_of(i);
+        const double b = a.b2s != nullptr ? (double)a.b2s[row] : 0.0;
+        const double hl = 0.5 * (double)logf((float)a.mass[row]);
+        const double c2 = ((kLnHalf + b + shift) - hl) * 1.4426950408889634, b2 = (hl + b) * 1.4426950408889634;
+        const double cn = rint(c2), bn = rint(b2);
+        S.row[j & 1][lane] = make_float4(__int_as_float((int)cn), (float)(c2 - cn), __int_as_float((int)bn),
+                                         (float)(b2 - bn));
+      }
+      __syncwarp();
+      if (lane == 0) mbar_arrive(&S.ahead[j & 1]);
+    };
+    bool ok = true;
+    ahead(0);
+    for (int64_t j = 0; j < batches; ++j) {
+      if (j + 1 < batches) ahead(j + 1);  // (its buffers: batch j - 1 is done)
+      const bool got = mbar_wait(&S.summed[j & 1], (uint32_t)(j >> 1) & 1u, abort_flag, 2 * kWaitLimitNs);
+      if (!__all_sync(0xffffffffu, got)) {
+        ok = false;
+        break;
+      }
+      const int64_t i = j * 32 + lane;
+      const bool valid = i < nr;
+      double lu = 0.0, el = 0.0;
+      if (valid) {
+        const int64_t row = row_of(i);
+        const volatile float2* s2 = &S.sum[j & 1][lane];
+        const RowResult rr = row_update(log_row_sum(s2->x, s2->y, 0.0f), shift, a.b2s != nullptr ? a.b2s[row] : 0.0f,
+                                        a.mass[row], a.log_u[row] + own_off, a.residual);
+        a.log_u[row] = lu = rr.log_u;
+        a.ell[row] = el = rr.ell;
+        acc.add(rr);
+      }
+      const float4 gv = warp_group(lu, el, valid);
+      if (lane == 0) a.grp[j * P + cid] = gv;
+    }
+    if (ok && lane == 0)
+      for (int64_t j = batches; j < a.grp_units; ++j) a.grp[j * P + cid] = empty_group();
+    if (!ok && !*abort_flag) pass_abort(a.err, abort_flag);
+    for (int o = 16; o > 0; o >>= 1) {
+      acc.rmax = fmax(acc.rmax, __shfl_xor_sync(0xffffffffu, acc.rmax, o));
+      acc.rsum += __shfl_xor_sync(0xffffffffu, acc.rsum, o);
+      acc.sq += __shfl_xor_sync(0xffffffffu, acc.sq, o);
+      acc.nf += __shfl_xor_sync(0xffffffffu, acc.nf, o);
+    }
+    if (lane == 0) {
+      a.partials[4 * cid + 0] = acc.rmax;
+      a.partials[4 * cid + 1] = acc.rsum;
+      a.partials[4 * cid + 2] = acc.sq;
+      a.partials[4 * cid + 3] = acc.nf;
+    }
+  }
+  // no CTA of a cluster leaves while another may still write to its shared memory
+  if constexpr (CLUSTER) cluster_sync();
+}
+
+// The Y update from the clusters' column sums: 32 columns per block, the
+// clusters dealt to kColSegs threads per column, each sum kept with its
+// roundings and added in a fixed order.
+constexpr int kColSegs = 16;
+
+__global__ void __launch_bounds__(32 * kColSegs) k_dense_cols(const float* __restrict__ colsum,
+                                                             const int* __restrict__ scale, int64_t ld, int clusters,
+                                                             int64_t cols, const double* __restrict__ st,
+                                                             const float* __restrict__ b2s,
+                                                             const double* __restrict__ mass,
+                                                             double* __restrict__ log_u, double* __restrict__ ell,
+                                                             float4* __restrict__ grp, double* __restrict__ partials) {
+  __shared__ float2 seg[kColSegs][32];
+  const int lane = threadIdx.x % 32, sg = threadIdx.x / 32;
+  const int64_t c = (int64_t)blockIdx.x * 32 + lane;
+  int R = -0x40000000;
+  for (int p = 0; p < clusters; ++p) R = max(R, __ldg(scale + p));
+  float hi = 0.0f, lo = 0.0f;
+  if (c < cols)
+#pragma unroll 4
+    for (int p = sg; p < clusters; p += kColSegs)
+      pair_add(hi, lo, __ldg(colsum + p * ld + c) * exp2_whole(__ldg(scale + p) - R), 0.0f);
+  seg[sg][lane] = make_float2(hi, lo);
+  __syncthreads();
+  if (sg != 0) return;
+  for (int i = 1; i < kColSegs; ++i) pair_add(hi, lo, seg[i][lane].x, seg[i][lane].y);
+  PartialAcc acc;
+  double lu = 0.0, el = 0.0;
+  if (c < cols) {
+    // the rows' weights are relative to R instead of the side's shift: the
+    // pass's shift without the shift, plus R ln 2
+    const double shift = (st[kStShift] - st[kStLmax + 0]) + (double)R * 0.69314718055994530942;
+    const RowResult rr = row_update(log_row_sum(hi, lo, 0.0f), shift, b2s != nullptr ? b2s[c] : 0.0f, mass[c],
+                                    log_u[c] + st[kStOwnOff], kResidualNone);
+    log_u[c] = lu = rr.log_u;
+    ell[c] = el = rr.ell;
+    acc.add(rr);
+  }
+  const float4 gv = warp_group(lu, el, c < cols);
+  for (int o = 16; o > 0; o >>= 1) {
+    acc.sq += __shfl_xor_sync(0xffffffffu, acc.sq, o);
+    acc.nf += __shfl_xor_sync(0xffffffffu, acc.nf, o);
+  }
+  if (lane == 0) {
+    grp[blockIdx.x] = gv;
+    partials[4 * blockIdx.x + 0] = 0.0;
+    partials[4 * blockIdx.x + 1] = 0.0;
+    partials[4 * blockIdx.x + 2] = acc.sq;
+    partials[4 * blockIdx.x + 3] = acc.nf;
+  }
+}
+
+// The instantiation for a slice width.
+typedef void (*SweepKernel)(SweepArgs);
+template <bool CLUSTER>
+SweepKernel sweep_kernel_for(int width) {
+  const int na = (width / 4 + kSweepSums * 32 - 1) / (kSweepSums * 32);
+  if (na <= 1) return k_dense_sweep<1, 3, CLUSTER>;
+  if (na == 2) return k_dense_sweep<2, 5, CLUSTER>;
+  if (na == 3) return k_dense_sweep<3, 8, CLUSTER>;
+  if (na == 4) return k_dense_sweep<4, 10, CLUSTER>;
+  if (na == 5) return k_dense_sweep<5, 12, CLUSTER>;
+  if (na == 6) return k_dense_sweep<6, 15, CLUSTER>;
+  return k_dense_sweep<7, 16, CLUSTER>;
+}
+// (a slice of up to na * 1,536 columns needs na * 2.4 quads per dot thread, the longest 16)
+static_assert(7 * kSweepSums * 128 >= kSweepWidth && 16 * kSweepDots * 128 >= kSweepWidth, "columns per thread");
+static_assert(kSweepDots * 3 >= kSweepSums && kSweepDots * 5 >= kSweepSums * 2 && kSweepDots * 8 >= kSweepSums * 3 &&
+                  kSweepDots * 10 >= kSweepSums * 4 && kSweepDots * 12 >= kSweepSums * 5 &&
+                  kSweepDots * 15 >= kSweepSums * 6,
+              "columns per thread");
+SweepKernel sweep_kernel(const DensePlan& p) {
+  return p.cl > 1 ? sweep_kernel_for<true>(p.width) : sweep_kernel_for<false>(p.width);
+}
+size_t sweep_smem(const DensePlan& p) { return kSweepRing + (size_t)p.slots * p.rows * p.width * 4; }
+
+cudaError_t sweep_attributes(const DensePlan& p) {
+  return cudaFuncSetAttribute(sweep_kernel(p), cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSweepSmemMax);
+}
+
+cudaLaunchConfig_t sweep_config(const DensePlan& p, cudaLaunchAttribute* attr, cudaStream_t stream) {
+  cudaLaunchConfig_t c = {};
+  c.gridDim = dim3((unsigned)(p.clusters * p.cl));
+  c.blockDim = dim3(kSweepThreads);
+  c.dynamicSmemBytes = sweep_smem(p);
+  c.stream = stream;
+  if (p.cl > 1) {
+    attr->id = cudaLaunchAttributeClusterDimension;
+    attr->val.clusterDim.x = (unsigned)p.cl;
+    attr->val.clusterDim.y = attr->val.clusterDim.z = 1;
+    c.attrs = attr;
+    c.numAttrs = 1;
+  }
+  return c;
+}
+
 // CTAs of a pass: as many as fit on the device at once (the ring's shared
 // memory allows a few per SM), at most one per row.
 int rowpass_grid(tu_market* m, int64_t rows) {
@@ -375,6 +934,7 @@ cudaError_t launch_dense_build(tu_market* m) {
   if (e == cudaSuccess)
     e = cudaFuncSetAttribute(k_dense_rowpass<true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                              (int)sizeof(PassSmem));
+  if (e == cudaSuccess && m->dplan.cl > 0) e = sweep_attributes(m->dplan);
   if (e != cudaSuccess) return e;
   const int64_t row_tiles = (m->N + 63) / 64;
   dim3 grid((unsigned)((m->M + 63) / 64), (unsigned)(row_tiles < 65535 ? row_tiles : 65535));
@@ -404,6 +964,81 @@ cudaError_t launch_dense_colpass(tu_market* m, int update, int* nparts_out, int6
                                                          m->partials, 0, update, m->omega_dev, m->err_dev);
   *nparts_out = g;
   *ngroups_out = blocks * g;
+  return cudaGetLastError();
+}
+
+// The layout of a market's one-pass sweep. Markets with very short rows, or
+// rows longer than a cluster holds, take the two passes.
+DensePlan dense_plan(const tu_market* m) {
+  DensePlan p;
+  if (m->M < kSweepMinCols || m->N < kSweepMinCols || m->ldA > (int64_t)kSweepCl * kSweepWidth) return p;
+  int cl = 1;
+  while ((int64_t)cl * kSweepWidth < m->ldA) cl *= 2;
+  p.width = (int)(((m->ldA + cl - 1) / cl + 3) / 4 * 4);
+  p.rows = 1;
+  while (cl == 1 && 2 * p.rows <= kSweepRows && 2 * p.rows * p.width <= kSweepWidth) p.rows *= 2;
+  const size_t fit = (kSweepSmemMax - kSweepRing) / ((size_t)p.rows * p.width * 4);
+  p.slots = (int)(fit < (size_t)kSweepSlots ? fit : (size_t)kSweepSlots);
+  p.cl = cl;
+  p.clusters = m->num_sms / cl;
+  if (cl > 1) {
+    // clusters that fit on the device at once
+    cudaLaunchAttribute attr;
+    const cudaLaunchConfig_t c = sweep_config(p, &attr, nullptr);
+    int n = 0;
+    if (sweep_attributes(p) != cudaSuccess || cudaOccupancyMaxActiveClusters(&n, sweep_kernel(p), &c) != cudaSuccess ||
+        n < 1) {
+      cudaGetLastError();
+      return DensePlan();
+    }
+    if (n < p.clusters) p.clusters = n;
+  }
+  const int64_t units = (m->N + p.rows - 1) / p.rows;
+  if (units < p.clusters) p.clusters = (int)units;
+  return p;
+}
+
+size_t dense_plan_floats(const DensePlan& p) {
+  return (size_t)p.clusters * ((size_t)p.cl * p.width) + (size_t)p.clusters;
+}
+
+cudaError_t launch_dense_sweep(tu_market* m, int residual, int* nparts_out, int64_t* ngroups_out) {
+  const DensePlan& p = m->dplan;
+  SweepArgs a;
+  a.A = m->Ahat;
+  a.ld = m->ldA;
+  a.rows = m->N;
+  a.w = m->Y.pvec;
+  a.st = m->st;
+  a.b2s = m->X.b2s;
+  a.mass = m->X.mass;
+  a.log_u = m->X.log_u;
+  a.ell = m->X.ell;
+  a.grp = m->X.grp;
+  const int64_t units = (m->N + p.rows - 1) / p.rows;
+  const int64_t most = (units + p.clusters - 1) / p.clusters;  // units of the fullest cluster
+  a.grp_units = (most * p.rows + kGroupRows - 1) / kGroupRows;
+  a.partials = m->partials;
+  a.residual = residual;
+  a.err = m->err_dev;
+  a.colsum = m->colsum;
+  a.scale = reinterpret_cast<int*>(m->colsum + (size_t)p.clusters * m->ldA);
+  a.plan = p;
+  cudaLaunchAttribute attr;
+  const cudaLaunchConfig_t c = sweep_config(p, &attr, m->stream);
+  *nparts_out = p.clusters;
+  *ngroups_out = a.grp_units * p.clusters;
+  return cudaLaunchKernelEx(&c, sweep_kernel(p), a);
+}
+
+cudaError_t launch_dense_cols(tu_market* m, int* nparts_out, int64_t* ngroups_out) {
+  const DensePlan& p = m->dplan;
+  const int blocks = (int)((m->M + 31) / 32);
+  k_dense_cols<<<blocks, 32 * kColSegs, 0, m->stream>>>(
+      m->colsum, reinterpret_cast<const int*>(m->colsum + (size_t)p.clusters * m->ldA), m->ldA, p.clusters, m->M, m->st,
+      m->Y.b2s, m->Y.mass, m->Y.log_u, m->Y.ell, m->Y.grp, m->partials);
+  *nparts_out = blocks;
+  *ngroups_out = blocks;
   return cudaGetLastError();
 }
 

@@ -503,6 +503,19 @@ cudaError_t enqueue_half(tu_market* m, int side, int residual, int update) {
 // One sweep of Eq. iteration: u from v (with the residual of the entering
 // state), then v from the new u.
 cudaError_t enqueue_sweep(tu_market* m) {
+  // dense path, plain updates: both half-sweeps from one pass over A-hat
+  if (m->dplan.cl > 0 && m->omega_cfg == 1.0) {
+    int nparts = 0;
+    int64_t ngroups = 0;
+    cudaError_t e = launch_prep(m, m->Y, 0, m->translate ? 1 : 0);
+    if (e == cudaSuccess) e = profile_mark(m, true);
+    if (e == cudaSuccess) e = launch_dense_sweep(m, kResidualEstimate, &nparts, &ngroups);
+    if (e == cudaSuccess) e = profile_mark(m, false);
+    if (e == cudaSuccess) e = launch_finalize(m, nparts, 1, kResidualEstimate, 1, ngroups, m->translate ? 2 : 1);
+    if (e == cudaSuccess) e = launch_dense_cols(m, &nparts, &ngroups);
+    if (e == cudaSuccess) e = launch_finalize(m, nparts, 0, 0, 1, ngroups);
+    return e;
+  }
   cudaError_t e = enqueue_half(m, 0, kResidualEstimate, 1);
   if (e != cudaSuccess) return e;
   return enqueue_half(m, 1, 0, 1);
@@ -744,6 +757,7 @@ void tu_market_destroy(tu_market_t m) {
       *a = nullptr;
     }
   }
+  dev_free(m, m->colsum);
   dev_free(m, m->partials);
   dev_free(m, m->st);
   dev_free(m, m->split_part);
@@ -860,6 +874,10 @@ tu_status tu_market_create(const tu_market_desc* desc, tu_market_t* out) {
       if (e == cudaSuccess) e = cudaMalloc(&m->AhatT, (size_t)m->M * m->ldN * sizeof(float));
       if (e != cudaSuccess) return bail(fail_cuda(m, e, "cudaMalloc(A-hat)"));
     }
+  }
+  if (D.path == TU_PATH_DENSE) {
+    m->dplan = dense_plan(m);
+    if (m->dplan.cl > 0 && (st = dev_alloc(m, &m->colsum, dense_plan_floats(m->dplan))) != TU_OK) return bail(st);
   }
   // (allocated after the dense matrices: placing this small allocation before
   // them measurably slowed the dense row stream)
@@ -1311,6 +1329,7 @@ int64_t tu_market_footprint(int64_t N, int64_t M, int64_t d, int path) {
     if (kp == kKBlock) bytes += (np + mp) * 32;              // the extra MMA's g / c operand
   } else {
     bytes += (N + M) * kp * 4 + N * round_up(M, 4) * 4 + M * round_up(N, 4) * 4;
+    bytes += 8 << 20;  // column sums of the one-pass sweep
   }
   return bytes;
 }

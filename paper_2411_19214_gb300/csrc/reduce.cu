@@ -300,7 +300,7 @@ __global__ void k_flush_scalars(double* __restrict__ st) {
 // size as the batched finalize.
 __global__ void k_finalize(const double* __restrict__ partials, int nparts, int is_x, int residual, int update,
                            const float4* __restrict__ grp, int64_t ngroups, double dm_next, double* __restrict__ st,
-                           double* __restrict__ results) {
+                           double* __restrict__ results, int prep_next) {
   __shared__ double red[4][kThreads / 32];
   __shared__ float redf[2 * kThreads / 32];
   double mx = 0.0, l1 = 0.0, sq = 0.0, nf = 0.0;
@@ -344,6 +344,7 @@ __global__ void k_finalize(const double* __restrict__ partials, int nparts, int 
     }
     results[kResNonfin] += nf;
     if (update) finish_scalars(st, is_x ? 0 : 1, g, dm_next);
+    if (prep_next) prep_scalars(st, is_x ? 1 : 0, prep_next > 1);
   }
 }
 
@@ -480,15 +481,16 @@ cudaError_t launch_sum_sq(tu_market* m, Side& s, int is_x) {
   int g = grid_for(s.rows, m->num_sms, 4);
   if (g > kMaxPartials) g = kMaxPartials;
   k_sum_sq<<<g, kThreads, 0, m->stream>>>(s.log_u, s.rows, m->partials);
-  k_finalize<<<1, kThreads, 0, m->stream>>>(m->partials, g, is_x, 0, 0, nullptr, 0, 0.0, m->st, m->results);
+  k_finalize<<<1, kThreads, 0, m->stream>>>(m->partials, g, is_x, 0, 0, nullptr, 0, 0.0, m->st, m->results, 0);
   return cudaGetLastError();
 }
 
-cudaError_t launch_finalize(tu_market* m, int nparts, int is_x, int residual, int update, int64_t ngroups) {
+cudaError_t launch_finalize(tu_market* m, int nparts, int is_x, int residual, int update, int64_t ngroups,
+                            int prep_next) {
   Side& own = is_x ? m->X : m->Y;
   Side& par = is_x ? m->Y : m->X;
   k_finalize<<<1, kThreads, 0, m->stream>>>(m->partials, nparts, is_x, residual, update, own.grp, ngroups,
-                                            own.sum_mass - par.sum_mass, m->st, m->results);
+                                            own.sum_mass - par.sum_mass, m->st, m->results, prep_next);
   return cudaGetLastError();
 }
 

@@ -140,6 +140,16 @@ inline int plan_block(int last_k, double r_prev, double r, double tol, int cap) 
   return k < 1 ? 1 : k;
 }
 
+// How a dense sweep in one pass over A-hat is laid out (dense.cu); cl = 0: the
+// market takes two passes.
+struct DensePlan {
+  int cl = 0;        // CTAs of a cluster, each with a slice of every row's columns
+  int width = 0;     // columns of a slice (multiple of 4)
+  int rows = 1;      // rows of a pipeline unit
+  int slots = 0;     // units in the ring
+  int clusters = 0;  // clusters of the launch
+};
+
 }  // namespace tu
 
 struct tu_market {
@@ -160,6 +170,8 @@ struct tu_market {
   double* partials = nullptr;   // kMaxPartials x 4 doubles
   double* st = nullptr;          // device scalars (kSt*): shifts, sums, offsets and steps of both sides
   float* AhatT = nullptr;       // dense path: transpose of A-hat, M x ldN fp32
+  tu::DensePlan dplan;          // dense path: the one-pass sweep's layout
+  float* colsum = nullptr;      // its scratch: clusters x ldA column sums, then the clusters' scales (int)
   int64_t ldN = 0;
   double* results = nullptr;       // device, kResSlots
   double* results_host = nullptr;  // pinned, kResSlots
@@ -214,7 +226,10 @@ namespace tu {
 cudaError_t launch_prep(tu_market* m, Side& partner, int fused_mode, int translate);
 // Reduce a pass's partials; after an update, also the own side's groups into
 // the market scalars (ngroups: groups the pass wrote).
-cudaError_t launch_finalize(tu_market* m, int nparts, int is_x, int residual, int update, int64_t ngroups);
+// prep_next: also set the scalars of the half-sweep that follows, which updates
+// the other side (1: without, 2: with the translation step).
+cudaError_t launch_finalize(tu_market* m, int nparts, int is_x, int residual, int update, int64_t ngroups,
+                            int prep_next = 0);
 // Groups and scalars of both sides from their stored potentials (after the
 // potentials were set from outside a sweep).
 cudaError_t launch_rescan(tu_market* m);
@@ -241,6 +256,13 @@ cudaError_t launch_sum_sq(tu_market* m, Side& s, int is_x);  // results[kResXSq 
 cudaError_t launch_dense_build(tu_market* m);
 cudaError_t launch_dense_rowpass(tu_market* m, int residual, int update, int* nparts_out, int64_t* ngroups_out);
 cudaError_t launch_dense_colpass(tu_market* m, int update, int* nparts_out, int64_t* ngroups_out);
+// A whole sweep with one pass over A-hat (markets with a DensePlan): the X
+// half-sweep and the column sums of the new u, then (after the X half-sweep's
+// finalize has set the Y half-sweep's scalars) the Y update from them.
+cudaError_t launch_dense_sweep(tu_market* m, int residual, int* nparts_out, int64_t* ngroups_out);
+cudaError_t launch_dense_cols(tu_market* m, int* nparts_out, int64_t* ngroups_out);
+DensePlan dense_plan(const tu_market* m);
+size_t dense_plan_floats(const DensePlan& p);  // scratch of a plan, in floats
 
 // fused.cu
 cudaError_t fused_prepare(tu_market* m);  // tensor maps + kernel attributes
@@ -397,10 +419,8 @@ __device__ __forceinline__ double log_row_sum(float a, float b, float c) {
 //
 // omega != 1 over-relaxes the update in the log domain:
 // log u <- log u_old + omega * (update - log u_old) (same fixed point).
-__device__ __forceinline__ RowResult row_update(double ln_sum, double shift, float b2s, double mass,
-                                                double log_u_old, int residual, double omega = 1.0) {
-  RowResult o;
-  const double log_s = kLnHalf + (double)b2s + shift + ln_sum;
+// The residual part (r_rel, r_abs) of the entering state.
+__device__ __forceinline__ void row_residual(RowResult& o, double log_s, double mass, double log_u_old, int residual) {
   o.r_rel = 0.0;
   o.r_abs = 0.0;
   if (residual == kResidualExact) {
@@ -414,7 +434,10 @@ __device__ __forceinline__ RowResult row_update(double ln_sum, double shift, flo
     o.r_abs = fabs(r);
     o.r_rel = fabs(r) / mass;
   }
-  const double hl = 0.5 * (double)logf((float)mass);
+}
+
+// The updated log u, from log s and hl = 1/2 log n.
+__device__ __forceinline__ double row_log_u(double log_s, double hl, double log_u_old, double omega) {
   const double z = log_s - hl;
   double a;
   if (z > 0.0) {
@@ -424,7 +447,15 @@ __device__ __forceinline__ RowResult row_update(double ln_sum, double shift, flo
     a = (double)asinhf(expf((float)z));
   }
   const double lu_upd = hl - a;
-  const double lu = omega == 1.0 ? lu_upd : log_u_old + omega * (lu_upd - log_u_old);
+  return omega == 1.0 ? lu_upd : log_u_old + omega * (lu_upd - log_u_old);
+}
+
+__device__ __forceinline__ RowResult row_update(double ln_sum, double shift, float b2s, double mass,
+                                                double log_u_old, int residual, double omega = 1.0) {
+  RowResult o;
+  const double log_s = kLnHalf + (double)b2s + shift + ln_sum;
+  row_residual(o, log_s, mass, log_u_old, residual);
+  const double lu = row_log_u(log_s, 0.5 * (double)logf((float)mass), log_u_old, omega);
   o.log_u = lu;
   o.ell = lu + (double)b2s;
   o.u2 = (double)expf((float)(2.0 * lu));
@@ -683,6 +714,33 @@ __device__ __forceinline__ bool mbar_wait(uint64_t* bar, uint32_t parity, volati
     if (*abort_flag) return false;
     if (global_timer_ns() - t0 > limit_ns) return false;
   }
+}
+
+// The address of a shared-memory location in CTA `rank` of the cluster.
+__device__ __forceinline__ uint32_t cluster_addr(const void* p, uint32_t rank) {
+  uint32_t a;
+  asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(a) : "r"(smem_u32(p)), "r"(rank));
+  return a;
+}
+// Store to the shared memory of a CTA of the cluster, counted in bytes on an
+// mbarrier of that CTA (which orders it as it does a bulk copy's writes).
+__device__ __forceinline__ void cluster_store_async(uint32_t a, float v, uint32_t bar) {
+  asm volatile("st.async.shared::cluster.mbarrier::complete_tx::bytes.f32 [%0], %1, [%2];" ::"r"(a), "f"(v), "r"(bar)
+               : "memory");
+}
+__device__ __forceinline__ void cluster_store_async2(uint32_t a, float v0, float v1, uint32_t bar) {
+  asm volatile("st.async.shared::cluster.mbarrier::complete_tx::bytes.v2.f32 [%0], {%1, %2}, [%3];" ::"r"(a), "f"(v0),
+               "f"(v1), "r"(bar)
+               : "memory");
+}
+__device__ __forceinline__ uint32_t cluster_rank() {
+  uint32_t r;
+  asm volatile("mov.u32 %0, %%cluster_ctarank;" : "=r"(r));
+  return r;
+}
+// Every thread of every CTA of the cluster.
+__device__ __forceinline__ void cluster_sync() {
+  asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
 }
 
 // Bounded wait that ignores the abort flag: used while draining after an abort,
