@@ -88,15 +88,13 @@ __global__ void __launch_bounds__(256) k_dense_build(const float* __restrict__ A
   }
 }
 
-struct PartialAcc {
-  double rmax = 0.0, rsum = 0.0, sq = 0.0, nf = 0.0;
-  __device__ void add(const RowResult& rr) {
-    rmax = fmax(rmax, rr.r_rel);
-    rsum += rr.r_abs;
-    sq += rr.u2;
-    if (!isfinite(rr.log_u) || !isfinite(rr.ell)) nf += 1.0;
-  }
-};
+// A warp's partials to its CTA's place.
+__device__ __forceinline__ void store_partials(double* dst, const RowPartials& p) {
+  dst[0] = p.r_max;
+  dst[1] = p.r_sum;
+  dst[2] = p.sq;
+  dst[3] = p.nf;
+}
 
 // One half-sweep over a row-major matrix A (rows x ld): for every row r,
 // s_r = 1/2 exp(b_r / 2 sigma) exp(shift) sum_c A[r][c] w_c with
@@ -273,7 +271,7 @@ __global__ void __launch_bounds__(kPassThreads) k_dense_rowpass(
   }
 
   if (warp != kUpdateWarp) return;
-  PartialAcc acc;
+  RowPartials acc = {0.0, 0.0, 0.0, 0.0};
   // the pass's partner shift and own offset (market scalars set by the preparation)
   double shift = 0.0, own_off = 0.0;
   if constexpr (!RELAX) {
@@ -291,7 +289,7 @@ __global__ void __launch_bounds__(kPassThreads) k_dense_rowpass(
       break;
     }
     const int64_t k = blk * kSlots + lane;
-    double lu_new = 0.0, ell_new = 0.0;
+    RowResult rr{};
     if (k < nrows) {
       const int64_t row = blockIdx.x + k * G;
       // the eight warps' shares, added with their roundings kept (two-sum)
@@ -307,23 +305,22 @@ __global__ void __launch_bounds__(kPassThreads) k_dense_rowpass(
         own_off = __ldg(st + kStOwnOff);
         omega = (update && omega_p != nullptr) ? __ldg(omega_p) : 1.0;
       }
-      const RowResult rr = row_update(log_row_sum(sum, err, 0.0f), shift, b2s ? b2s[row] : 0.0f, mass[row],
-                                      log_u[row] + own_off, residual, omega);
+      int ex;
+      const float lm = log_row_sum_parts(sum, err, 0.0f, ex);
+      rr = row_update(ex, lm, shift, b2s ? b2s[row] : 0.0f, mass[row], log_u[row] + own_off, residual, omega);
       if (update) {
         log_u[row] = rr.log_u;
         ell[row] = rr.ell;
       }
-      lu_new = rr.log_u;
-      ell_new = rr.ell;
-      acc.add(rr);
     }
     __syncwarp();
     if (lane == 0) mbar_arrive(&S.freed[pb]);
     if (update) {
       // the block's rows (this CTA's rows blk * 32 .. blk * 32 + 31) form group blk * G + blockIdx.x
-      const float4 gv = warp_group(lu_new, ell_new, k < nrows);
+      const float4 gv = warp_group(rr.log_u, rr.ell, k < nrows);
       if (lane == 0) grp[blk * G + blockIdx.x] = gv;
     }
+    add_partials(acc, row_partials(rr, k < nrows, residual));
   }
   if (update && ok && lane == 0) {
     // groups of the blocks this CTA does not have (the grid's rows are
@@ -332,18 +329,7 @@ __global__ void __launch_bounds__(kPassThreads) k_dense_rowpass(
   }
   if (!ok && !*abort_flag) pass_abort(err, abort_flag);
   // this warp holds every partial of the CTA
-  for (int o = 16; o > 0; o >>= 1) {
-    acc.rmax = fmax(acc.rmax, __shfl_xor_sync(0xffffffffu, acc.rmax, o));
-    acc.rsum += __shfl_xor_sync(0xffffffffu, acc.rsum, o);
-    acc.sq += __shfl_xor_sync(0xffffffffu, acc.sq, o);
-    acc.nf += __shfl_xor_sync(0xffffffffu, acc.nf, o);
-  }
-  if (lane == 0) {
-    partials[4 * blockIdx.x + 0] = acc.rmax;
-    partials[4 * blockIdx.x + 1] = acc.rsum;
-    partials[4 * blockIdx.x + 2] = acc.sq;
-    partials[4 * blockIdx.x + 3] = acc.nf;
-  }
+  if (lane == 0) store_partials(partials + 4 * blockIdx.x, acc);
 }
 
 // One sweep from one pass over A-hat. The v step needs s_y = 1/2 sum_x A_xy u_x
@@ -689,7 +675,7 @@ __global__ void __launch_bounds__(kSweepThreads, 1) k_dense_sweep(const SweepArg
         }
         // The row's weight u 2^-R in FP32: log2 of the sum and of u are each an
         // integer plus a fraction, so that no digits go to their size
-        // (row_log_u's closed form with z = log s - 1/2 log n in log2 units).
+        // (row_update's closed form with z = log s - 1/2 log n in log2 units).
         const volatile float4* cst = reinterpret_cast<const volatile float4*>(&S.row[bb][at]);
         const int nc = __float_as_int(cst->x), nB = __float_as_int(cst->z);
         const float fc = cst->y, fB = cst->w;
@@ -744,7 +730,7 @@ __global__ void __launch_bounds__(kSweepThreads, 1) k_dense_sweep(const SweepArg
     // the stored potentials, the residual and the batch's group. FP64 runs at a
     // few operations per clock and SM: a row's chain of it takes microseconds,
     // which the update warp cannot wait for.
-    PartialAcc acc;
+    RowPartials acc = {0.0, 0.0, 0.0, 0.0};
     const double shift = a.st[kStShift], own_off = a.st[kStOwnOff];
     const int64_t last0 = (cid + (nu - 1) * P) * B;
     const int64_t nr = (nu - 1) * B + (a.rows - last0 < B ? a.rows - last0 : B);  // this cluster's rows
@@ -775,34 +761,25 @@ __global__ void __launch_bounds__(kSweepThreads, 1) k_dense_sweep(const SweepArg
       }
       const int64_t i = j * 32 + lane;
       const bool valid = i < nr;
-      double lu = 0.0, el = 0.0;
+      RowResult rr{};
       if (valid) {
         const int64_t row = row_of(i);
         const volatile float2* s2 = &S.sum[j & 1][lane];
-        const RowResult rr = row_update(log_row_sum(s2->x, s2->y, 0.0f), shift, a.b2s != nullptr ? a.b2s[row] : 0.0f,
-                                        a.mass[row], a.log_u[row] + own_off, a.residual);
-        a.log_u[row] = lu = rr.log_u;
-        a.ell[row] = el = rr.ell;
-        acc.add(rr);
+        int ex;
+        const float lm = log_row_sum_parts(s2->x, s2->y, 0.0f, ex);
+        rr = row_update(ex, lm, shift, a.b2s != nullptr ? a.b2s[row] : 0.0f, a.mass[row], a.log_u[row] + own_off,
+                        a.residual);
+        a.log_u[row] = rr.log_u;
+        a.ell[row] = rr.ell;
       }
-      const float4 gv = warp_group(lu, el, valid);
+      add_partials(acc, row_partials(rr, valid, a.residual));
+      const float4 gv = warp_group(rr.log_u, rr.ell, valid);
       if (lane == 0) a.grp[j * P + cid] = gv;
     }
     if (ok && lane == 0)
       for (int64_t j = batches; j < a.grp_units; ++j) a.grp[j * P + cid] = empty_group();
     if (!ok && !*abort_flag) pass_abort(a.err, abort_flag);
-    for (int o = 16; o > 0; o >>= 1) {
-      acc.rmax = fmax(acc.rmax, __shfl_xor_sync(0xffffffffu, acc.rmax, o));
-      acc.rsum += __shfl_xor_sync(0xffffffffu, acc.rsum, o);
-      acc.sq += __shfl_xor_sync(0xffffffffu, acc.sq, o);
-      acc.nf += __shfl_xor_sync(0xffffffffu, acc.nf, o);
-    }
-    if (lane == 0) {
-      a.partials[4 * cid + 0] = acc.rmax;
-      a.partials[4 * cid + 1] = acc.rsum;
-      a.partials[4 * cid + 2] = acc.sq;
-      a.partials[4 * cid + 3] = acc.nf;
-    }
+    if (lane == 0) store_partials(a.partials + 4 * cid, acc);
   }
   // no CTA of a cluster leaves while another may still write to its shared memory
   if constexpr (CLUSTER) cluster_sync();
@@ -834,29 +811,23 @@ __global__ void __launch_bounds__(32 * kColSegs) k_dense_cols(const float* __res
   __syncthreads();
   if (sg != 0) return;
   for (int i = 1; i < kColSegs; ++i) pair_add(hi, lo, seg[i][lane].x, seg[i][lane].y);
-  PartialAcc acc;
-  double lu = 0.0, el = 0.0;
+  RowResult rr{};
   if (c < cols) {
     // the rows' weights are relative to R instead of the side's shift: the
     // pass's shift without the shift, plus R ln 2
-    const double shift = (st[kStShift] - st[kStLmax + 0]) + (double)R * 0.69314718055994530942;
-    const RowResult rr = row_update(log_row_sum(hi, lo, 0.0f), shift, b2s != nullptr ? b2s[c] : 0.0f, mass[c],
-                                    log_u[c] + st[kStOwnOff], kResidualNone);
-    log_u[c] = lu = rr.log_u;
-    ell[c] = el = rr.ell;
-    acc.add(rr);
+    const double shift = st[kStShift] - st[kStLmax + 0];
+    int ex;
+    const float lm = log_row_sum_parts(hi, lo, 0.0f, ex);
+    rr = row_update(ex + R, lm, shift, b2s != nullptr ? b2s[c] : 0.0f, mass[c], log_u[c] + st[kStOwnOff],
+                    kResidualNone);
+    log_u[c] = rr.log_u;
+    ell[c] = rr.ell;
   }
-  const float4 gv = warp_group(lu, el, c < cols);
-  for (int o = 16; o > 0; o >>= 1) {
-    acc.sq += __shfl_xor_sync(0xffffffffu, acc.sq, o);
-    acc.nf += __shfl_xor_sync(0xffffffffu, acc.nf, o);
-  }
+  const float4 gv = warp_group(rr.log_u, rr.ell, c < cols);
+  const RowPartials p = row_partials(rr, c < cols, kResidualNone);
   if (lane == 0) {
     grp[blockIdx.x] = gv;
-    partials[4 * blockIdx.x + 0] = 0.0;
-    partials[4 * blockIdx.x + 1] = 0.0;
-    partials[4 * blockIdx.x + 2] = acc.sq;
-    partials[4 * blockIdx.x + 3] = acc.nf;
+    store_partials(partials + 4 * blockIdx.x, p);
   }
 }
 

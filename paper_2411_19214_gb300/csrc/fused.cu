@@ -784,7 +784,7 @@ __global__ void __launch_bounds__(kThreads, 1)
   uint64_t* rowfree = a_full + 11;  // [2] row hand-over buffer read
   uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(a_full + 13);
   volatile int* abort_flag = reinterpret_cast<volatile int*>(tmem_slot + 1);
-  double* red = reinterpret_cast<double*>(reinterpret_cast<uint8_t*>(bars) + 512);      // 4 x kEpiWarps doubles
+  double* red = reinterpret_cast<double*>(reinterpret_cast<uint8_t*>(bars) + 512);      // kEpiWarps x 4 doubles
   float* rowbuf = reinterpret_cast<float*>(reinterpret_cast<uint8_t*>(bars) + 1024);   // 2 x 256 floats
   // ranked lists in shared memory (kModeTopKShared only): after the tail area
   float* topk_list = reinterpret_cast<float*>(reinterpret_cast<uint8_t*>(bars) + kTailBytes);
@@ -1051,7 +1051,11 @@ __global__ void __launch_bounds__(kThreads, 1)
     int buf = 0, gs = 0;
     uint32_t tphase = 0, gphase = 0;
     bool ok = true;
-    double r_max = 0.0, r_sum = 0.0, sq = 0.0, nf = 0.0;
+    if constexpr (kSweepLike && !BATCH) {
+      // this warp's partials over its own tiles, in shared memory: carried in
+      // registers they would stay live across the tile loop
+      if (lane == 0) *reinterpret_cast<RowPartials*>(red + 4 * ew) = RowPartials{0.0, 0.0, 0.0, 0.0};
+    }
     uint32_t va[32], vb[32];
     // ranked lists: this thread's sorted candidates for its row and column half
     float tv[MODE == kModeTopK ? kMaxTopK : 1];
@@ -1337,87 +1341,58 @@ __global__ void __launch_bounds__(kThreads, 1)
               }
           }
         }
-        double lu_new = 0.0, ell_new = 0.0;
+        RowResult rr{};
         if (row_ok) {
           const float* b2s = BATCH ? bd->b2s : p.b2s;
           double* log_u = BATCH ? bd->log_u : p.log_u;
           double* ell = BATCH ? bd->ell : p.ell;
           const double omega = BATCH ? ((bd->omega != nullptr && p.update) ? *bd->omega : 1.0) : omega0;
           const double own_off = BATCH ? bd->st[kStOwnOff] : own_off0;
-          double ln_sum = log_row_sum(s_hi, s_lo, s_o);
+          int ex;
+          const float lm = log_row_sum_parts(s_hi, s_lo, s_o, ex);
           // wide markets: the row's shift comes back into the sum's logarithm
-          if constexpr (MODE == kModeSweepWide) ln_sum = __fma_rn((double)row_m, 0.69314718055994530942, ln_sum);
-          const RowResult rr = row_update(ln_sum, shift, b2s ? b2s[row] : 0.0f,
-                                          (BATCH ? bd->mass : p.mass)[row], log_u[row] + own_off,
-                                          p.residual, omega);
+          // (no finite exponent: the sum is 0 and its logarithm -inf whatever is added)
+          if constexpr (MODE == kModeSweepWide) ex += row_m > -1e9f ? (int)row_m : 0;
+          rr = row_update(ex, lm, shift, b2s ? b2s[row] : 0.0f, (BATCH ? bd->mass : p.mass)[row],
+                          log_u[row] + own_off, p.residual, omega);
           if (p.update) {
             log_u[row] = rr.log_u;
             ell[row] = rr.ell;
           }
-          lu_new = rr.log_u;
-          ell_new = rr.ell;
-          r_max = fmax(r_max, rr.r_rel);
-          r_sum += rr.r_abs;
-          sq += rr.u2;
-          if (!isfinite(rr.log_u) || !isfinite(rr.ell)) nf += 1.0;
         }
         // this warp's 32 rows form one group of the own side (the finalize
         // reduces the groups into the side's shift and sum of u^2)
         float4* grp = BATCH ? bd->grp : p.grp;
         const int64_t g = (int64_t)t * (kOwn / kGroupRows) + (h * 128 + q * 32) / kGroupRows;
-        if (p.update && grp != nullptr && !(SMALL && h == 1) &&
-            g * kGroupRows < (BATCH ? bd->rows : p.rows)) {
-          const float4 gv = warp_group(lu_new, ell_new, row_ok);
+        if (SMALL && h == 1) continue;  // (no rows)
+        if (p.update && grp != nullptr && g * kGroupRows < (BATCH ? bd->rows : p.rows)) {
+          const float4 gv = warp_group(rr.log_u, rr.ell, row_ok);
           if (lane == 0) grp[g] = gv;
         }
-        if constexpr (BATCH) {
-          // partials of this own tile and warp (warps ew = 0..7 own the row
-          // updates); the batched finalize sums them per market in a fixed order
-          for (int o = 16; o > 0; o >>= 1) {
-            r_max = fmax(r_max, __shfl_xor_sync(0xffffffffu, r_max, o));
-            r_sum += __shfl_xor_sync(0xffffffffu, r_sum, o);
-            sq += __shfl_xor_sync(0xffffffffu, sq, o);
-            nf += __shfl_xor_sync(0xffffffffu, nf, o);
+        const RowPartials rp = row_partials(rr, row_ok, p.residual);
+        if (lane == 0) {
+          if constexpr (BATCH) {
+            // partials of this own tile and warp (warps ew = 0..7 own the row
+            // updates); the batched finalize sums them per market in a fixed order
+            *reinterpret_cast<RowPartials*>(p.partials + ((int64_t)(bd->slot0 + t) * kBatchSlotWarps + ew) * 4) = rp;
+          } else {
+            add_partials(*reinterpret_cast<RowPartials*>(red + 4 * ew), rp);
           }
-          if (lane == 0) {
-            double* dst = p.partials + ((int64_t)(bd->slot0 + t) * kBatchSlotWarps + ew) * 4;
-            dst[0] = r_max;
-            dst[1] = r_sum;
-            dst[2] = sq;
-            dst[3] = nf;
-          }
-          r_max = r_sum = sq = nf = 0.0;
         }
       }
     }
     if (!ok && !*abort_flag) raise_error(p.err, abort_flag, kErrTimeout);
     if constexpr (kSweepLike && !BATCH) {
-      // reduce the CTA's partials over the epilogue threads
-      for (int o = 16; o > 0; o >>= 1) {
-        r_max = fmax(r_max, __shfl_xor_sync(0xffffffffu, r_max, o));
-        r_sum += __shfl_xor_sync(0xffffffffu, r_sum, o);
-        sq += __shfl_xor_sync(0xffffffffu, sq, o);
-        nf += __shfl_xor_sync(0xffffffffu, nf, o);
-      }
-      if (lane == 0) {
-        red[0 * kEpiWarps + ew] = r_max;
-        red[1 * kEpiWarps + ew] = r_sum;
-        red[2 * kEpiWarps + ew] = sq;
-        red[3 * kEpiWarps + ew] = nf;
-      }
+      // the CTA's partials: those of the warps that own the row updates
       named_bar_sync(1, kEpiWarps * 32);
-      if (ew == 0 && lane == 0) {
-        double m0 = 0.0, s1 = 0.0, s2 = 0.0, s3 = 0.0;
-        for (int w = 0; w < kEpiWarps; ++w) {
-          m0 = fmax(m0, red[w]);
-          s1 += red[kEpiWarps + w];
-          s2 += red[2 * kEpiWarps + w];
-          s3 += red[3 * kEpiWarps + w];
+      if (ew == 0 && lane < 8) {
+        RowPartials v = *reinterpret_cast<const RowPartials*>(red + 4 * lane);
+        for (int o = 4; o > 0; o >>= 1) {
+          const RowPartials w = {__shfl_xor_sync(0xffu, v.r_max, o), __shfl_xor_sync(0xffu, v.r_sum, o),
+                                 __shfl_xor_sync(0xffu, v.sq, o), __shfl_xor_sync(0xffu, v.nf, o)};
+          add_partials(v, w);
         }
-        p.partials[4 * blockIdx.x + 0] = m0;
-        p.partials[4 * blockIdx.x + 1] = s1;
-        p.partials[4 * blockIdx.x + 2] = s2;
-        p.partials[4 * blockIdx.x + 3] = s3;
+        if (lane == 0) *reinterpret_cast<RowPartials*>(p.partials + 4 * blockIdx.x) = v;
       }
     }
   }

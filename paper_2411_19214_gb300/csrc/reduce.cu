@@ -301,38 +301,32 @@ __global__ void k_flush_scalars(double* __restrict__ st) {
 __global__ void k_finalize(const double* __restrict__ partials, int nparts, int is_x, int residual, int update,
                            const float4* __restrict__ grp, int64_t ngroups, double dm_next, double* __restrict__ st,
                            double* __restrict__ results, int prep_next) {
-  __shared__ double red[4][kThreads / 32];
+  __shared__ double red[4];
   __shared__ float redf[2 * kThreads / 32];
-  double mx = 0.0, l1 = 0.0, sq = 0.0, nf = 0.0;
-  for (int i = threadIdx.x; i < nparts; i += blockDim.x) {
-    mx = fmax(mx, partials[4 * i + 0]);
-    l1 += partials[4 * i + 1];
-    sq += partials[4 * i + 2];
-    nf += partials[4 * i + 3];
-  }
-  for (int o = 16; o > 0; o >>= 1) {
-    mx = fmax(mx, __shfl_xor_sync(0xffffffffu, mx, o));
-    l1 += __shfl_xor_sync(0xffffffffu, l1, o);
-    sq += __shfl_xor_sync(0xffffffffu, sq, o);
-    nf += __shfl_xor_sync(0xffffffffu, nf, o);
-  }
-  const int w = threadIdx.x / 32;
-  if (threadIdx.x % 32 == 0) {
-    red[0][w] = mx;
-    red[1][w] = l1;
-    red[2][w] = sq;
-    red[3][w] = nf;
+  // one warp per quantity: an FP64 addition takes about 80 cycles, so four
+  // short chains side by side, and the groups meanwhile
+  const int w = threadIdx.x / 32, lane = threadIdx.x % 32;
+  if (w < 4) {
+    double v[4] = {0.0, 0.0, 0.0, 0.0};
+    for (int i = lane; i < nparts; i += 128) {
+#pragma unroll
+      for (int j = 0; j < 4; ++j) {
+        const double x = i + 32 * j < nparts ? partials[4 * (int64_t)(i + 32 * j) + w] : 0.0;
+        v[j] = w == 0 ? (x > v[j] ? x : v[j]) : v[j] + x;
+      }
+    }
+    double t = w == 0 ? fmax(fmax(v[0], v[1]), fmax(v[2], v[3])) : (v[0] + v[1]) + (v[2] + v[3]);
+    for (int o = 16; o > 0; o >>= 1) {
+      const double x = __shfl_xor_sync(0xffffffffu, t, o);
+      t = w == 0 ? (x > t ? x : t) : t + x;
+    }
+    if (lane == 0) red[w] = t;
   }
   GroupTotal g{};
   if (update) g = block_reduce_groups(grp, ngroups, redf);  // synchronises the block
   else __syncthreads();
   if (threadIdx.x == 0) {
-    for (int k = 1; k < kThreads / 32; ++k) {
-      mx = fmax(mx, red[0][k]);
-      l1 += red[1][k];
-      sq += red[2][k];
-      nf += red[3][k];
-    }
+    const double mx = red[0], l1 = red[1], sq = red[2], nf = red[3];
     if (is_x) {
       if (residual) {
         results[kResXInf] = mx;

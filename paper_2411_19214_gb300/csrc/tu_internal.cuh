@@ -367,7 +367,9 @@ constexpr float kLog2e = 1.4426950408889634f;
 
 struct RowResult {
   double log_u, ell;
-  double r_rel, r_abs, u2;
+  double r_rel, r_abs;  // residual of the entering state (0 without)
+  float u2;             // u^2
+  bool finite;          // the new potentials
 };
 
 // ln (a + b + c) of a positive row sum given as three FP32 parts, to an
@@ -384,21 +386,30 @@ __device__ __forceinline__ float two_sum(float a, float b, float& err) {
   err = __fadd_rn(__fsub_rn(a, __fsub_rn(s, bb)), __fsub_rn(b, bb));
   return s;
 }
-__device__ __forceinline__ double log_row_sum(float a, float b, float c) {
+// The logarithm as e ln 2 + the returned float, e an integer.
+__device__ __forceinline__ float log_row_sum_parts(float a, float b, float c, int& e) {
   float e1, e2;
   const float s1 = two_sum(a, b, e1);
   const float hi = two_sum(s1, c, e2);
   const float lo = __fadd_rn(e1, e2);
+  const float m = frexpf(hi, &e);
+  return __fadd_rn(logf(m), __fdividef(lo, hi));
+}
+__device__ __forceinline__ double log_row_sum(float a, float b, float c) {
   int ex;
-  const float m = frexpf(hi, &ex);
-  return __dadd_rn((double)ex * 0.69314718055994530942, (double)__fadd_rn(logf(m), __fdividef(lo, hi)));
+  const float lm = log_row_sum_parts(a, b, c, ex);
+  return __dadd_rn((double)ex * 0.69314718055994530942, (double)lm);
+}
+
+__device__ __forceinline__ bool finite64(double v) {
+  return ((uint32_t)__double2hiint(v) & 0x7ff00000u) != 0x7ff00000u;
 }
 
 // The closed-form update of Eq. iteration for one user, in logs.
-//   ln_sum   : log of sum_y exp(phi_hat_xy / (2 sigma) + ell_y - shift)
+//   ex, lm   : ex ln 2 + lm = log of sum_y exp(phi_hat_xy / (2 sigma) + ell_y - shift)
 //   shift    : the partner-side shift (max_y ell_y) taken out of the sum
 //   b2s      : this user's bias / (2 sigma)
-//   log_s    = log(1/2) + b2s + shift + ln_sum          (s = 1/2 sum_y A_xy v_y)
+//   log_s    = log(1/2) + b2s + shift + ex ln 2 + lm    (s = 1/2 sum_y A_xy v_y)
 //   log u    = 1/2 log n - asinh(exp(log s - 1/2 log n)) (= sqrt(n + s^2) - s)
 // With residual, r = u_old^2 + 2 u_old s - n is the row equation of Eq. IPFP
 // evaluated at the state entering the half-sweep.
@@ -419,47 +430,97 @@ __device__ __forceinline__ double log_row_sum(float a, float b, float c) {
 //
 // omega != 1 over-relaxes the update in the log domain:
 // log u <- log u_old + omega * (update - log u_old) (same fixed point).
-// The residual part (r_rel, r_abs) of the entering state.
-__device__ __forceinline__ void row_residual(RowResult& o, double log_s, double mass, double log_u_old, int residual) {
+// An FP64 operation has a latency of about 80 cycles here and issues at 2 per
+// clock and SM, conversions included, so the chain keeps to the additions that
+// need it: doublings, comparisons and tests of finiteness are FP32 or integer,
+// and the estimate's quotient r / n is FP32. (45 FP64 instructions per row and
+// FP64 butterflies over all epilogue warps ended a tile in 15,000 cycles: half
+// of the time of a 1,000 x 1,000 half-sweep. See row_partials.)
+__device__ __forceinline__ RowResult row_update(int ex, float lm, double shift, float b2s, double mass,
+                                                double log_u_old, int residual, double omega = 1.0) {
+  RowResult o;
+  const double b = (double)b2s;
+  const float nf = (float)mass;
+  const double ln = (double)logf(nf);  // log n
+  const double ls = fma((double)ex, 0.69314718055994530942, __dadd_rn(__dadd_rn(shift, kLnHalf), b));  // log s - lm
   o.r_rel = 0.0;
   o.r_abs = 0.0;
   if (residual == kResidualExact) {
     // r = u^2 + 2 u s - n with u^2 = e^{2 log u}, 2 u s = e^{log u + log s + ln 2}
-    const double r = exp(2.0 * log_u_old) + exp(log_u_old + log_s + 0.69314718055994530942) - mass;
+    const double r = exp(2.0 * log_u_old) + exp(log_u_old + (ls + (double)lm) + 0.69314718055994530942) - mass;
     o.r_abs = fabs(r);
     o.r_rel = fabs(r) / mass;
   } else if (residual == kResidualEstimate) {
-    const double r = (double)expf((float)(2.0 * log_u_old)) +
-                     (double)expf((float)(log_u_old + log_s + 0.69314718055994530942)) - mass;
+    const float e2 = expf((float)__dadd_rn(__dadd_rn(log_u_old, 0.69314718055994530942), ls) + lm);
+    const double r = __dadd_rn(__dadd_rn((double)expf(2.0f * (float)log_u_old), -mass), (double)e2);
     o.r_abs = fabs(r);
-    o.r_rel = fabs(r) / mass;
+    o.r_rel = (double)__fdiv_rn(fabsf((float)r), nf);
   }
-}
-
-// The updated log u, from log s and hl = 1/2 log n.
-__device__ __forceinline__ double row_log_u(double log_s, double hl, double log_u_old, double omega) {
-  const double z = log_s - hl;
-  double a;
-  if (z > 0.0) {
-    const float c = log1pf(sqrtf(1.0f + expf((float)(-2.0 * z))));
-    a = z + (double)c;
+  const float z = (float)fma(-0.5, ln, ls) + lm;
+  double lu;
+  if (z > 0.0f) {
+    const float c = log1pf(sqrtf(1.0f + expf(-2.0f * z)));
+    lu = __dadd_rn(__dadd_rn(__dadd_rn(ln, -ls), -(double)lm), -(double)c);
   } else {
-    a = (double)asinhf(expf((float)z));
+    lu = fma(0.5, ln, -(double)asinhf(expf(z)));
   }
-  const double lu_upd = hl - a;
-  return omega == 1.0 ? lu_upd : log_u_old + omega * (lu_upd - log_u_old);
+  if (omega != 1.0) lu = log_u_old + omega * (lu - log_u_old);
+  o.log_u = lu;
+  o.ell = __dadd_rn(lu, b);
+  o.u2 = expf(2.0f * (float)lu);
+  o.finite = finite64(o.log_u) && finite64(o.ell);
+  return o;
 }
 
-__device__ __forceinline__ RowResult row_update(double ln_sum, double shift, float b2s, double mass,
-                                                double log_u_old, int residual, double omega = 1.0) {
-  RowResult o;
-  const double log_s = kLnHalf + (double)b2s + shift + ln_sum;
-  row_residual(o, log_s, mass, log_u_old, residual);
-  const double lu = row_log_u(log_s, 0.5 * (double)logf((float)mass), log_u_old, omega);
-  o.log_u = lu;
-  o.ell = lu + (double)b2s;
-  o.u2 = (double)expf((float)(2.0 * lu));
-  return o;
+// Partials of one warp's rows (one per lane; lanes with valid = false
+// contribute nothing), on lane 0: max r / n, sum |r|, sum u^2, non-finite
+// count. The sums of u^2 (and of an estimate's |r|) add FP32 terms with their
+// roundings kept; a certifying pass's |r| is summed in FP64.
+struct RowPartials {
+  double r_max, r_sum, sq, nf;
+};
+__device__ __forceinline__ RowPartials row_partials(const RowResult& rr, bool valid, int residual) {
+  RowPartials p;
+  float hi = valid ? rr.u2 : 0.0f, lo = 0.0f;
+  for (int o = 16; o > 0; o >>= 1) {
+    const float h2 = __shfl_xor_sync(0xffffffffu, hi, o), l2 = __shfl_xor_sync(0xffffffffu, lo, o);
+    float e;
+    hi = two_sum(hi, h2, e);
+    lo = __fadd_rn(__fadd_rn(lo, l2), e);
+  }
+  // (an infinite u^2 makes the error term NaN; the sum itself says what it is)
+  p.sq = isfinite(lo) ? (double)hi + (double)lo : (double)hi;
+  p.nf = (double)__popc(__ballot_sync(0xffffffffu, valid && !rr.finite));
+  p.r_max = p.r_sum = 0.0;
+  if (residual == kResidualNone) return p;
+  // non-negative floating-point numbers order like their bits; a NaN is left out
+  const double rel = valid && rr.r_rel == rr.r_rel ? rr.r_rel : 0.0;
+  if (residual == kResidualExact) {
+    const unsigned h = (unsigned)__double2hiint(rel), top = __reduce_max_sync(0xffffffffu, h);
+    const unsigned l = __reduce_max_sync(0xffffffffu, h == top ? (unsigned)__double2loint(rel) : 0u);
+    p.r_max = __hiloint2double((int)top, (int)l);
+    double a = valid ? rr.r_abs : 0.0;
+    for (int o = 16; o > 0; o >>= 1) a += __shfl_xor_sync(0xffffffffu, a, o);
+    p.r_sum = a;
+  } else {
+    p.r_max = (double)__uint_as_float(__reduce_max_sync(0xffffffffu, __float_as_uint((float)rel)));
+    float ah = valid ? (float)rr.r_abs : 0.0f, al = 0.0f;
+    for (int o = 16; o > 0; o >>= 1) {
+      const float h2 = __shfl_xor_sync(0xffffffffu, ah, o), l2 = __shfl_xor_sync(0xffffffffu, al, o);
+      float e;
+      ah = two_sum(ah, h2, e);
+      al = __fadd_rn(__fadd_rn(al, l2), e);
+    }
+    p.r_sum = isfinite(al) ? (double)ah + (double)al : (double)ah;
+  }
+  return p;
+}
+// p += q (one thread)
+__device__ __forceinline__ void add_partials(RowPartials& p, const RowPartials& q) {
+  p.r_max = q.r_max > p.r_max ? q.r_max : p.r_max;
+  p.r_sum += q.r_sum;
+  p.sq += q.sq;
+  p.nf += q.nf;
 }
 
 // ---- translation step and the per-side scalars -------------------------------
@@ -475,35 +536,30 @@ __device__ __forceinline__ RowResult row_update(double ln_sum, double shift, flo
 // per-side offset and written to the arrays only when a side is next updated
 // (for the updated side) or at the end of a block of sweeps.
 
-// Block-wide reductions (every thread returns the result; `red` holds
-// blockDim.x / 32 doubles). Sums in a fixed order: a butterfly within each warp
-// (every lane ends with the same value), then the warps in order.
-__device__ __forceinline__ double block_reduce_max(double v, double* red) {
-  for (int o = 16; o > 0; o >>= 1) v = fmax(v, __shfl_xor_sync(0xffffffffu, v, o));
-  if (threadIdx.x % 32 == 0) red[threadIdx.x / 32] = v;
-  __syncthreads();
-  double b = -INFINITY;
-  for (int w = 0; w < (int)blockDim.x / 32; ++w) b = fmax(b, red[w]);
-  __syncthreads();
-  return b;
+// Order-preserving float <-> uint mapping for max on floats of any sign.
+__device__ __forceinline__ unsigned int float_to_ordered(float f) {
+  unsigned int u = __float_as_uint(f);
+  return (u & 0x80000000u) ? ~u : (u | 0x80000000u);
 }
-__device__ __forceinline__ float block_reduce_maxf(float v, float* red) {
-  for (int o = 16; o > 0; o >>= 1) v = fmaxf(v, __shfl_xor_sync(0xffffffffu, v, o));
-  if (threadIdx.x % 32 == 0) red[threadIdx.x / 32] = v;
-  __syncthreads();
-  float b = -INFINITY;
-  for (int w = 0; w < (int)blockDim.x / 32; ++w) b = fmaxf(b, red[w]);
-  __syncthreads();
-  return b;
+__device__ __forceinline__ float ordered_to_float(unsigned int u) {
+  return __uint_as_float((u & 0x80000000u) ? (u & 0x7fffffffu) : ~u);
 }
-__device__ __forceinline__ double block_reduce_sum(double v, double* red) {
-  for (int o = 16; o > 0; o >>= 1) v = __dadd_rn(v, __shfl_xor_sync(0xffffffffu, v, o));
-  if (threadIdx.x % 32 == 0) red[threadIdx.x / 32] = v;
+
+// Block-wide maxima of two floats (every thread returns them).
+// (red: 2 * blockDim.x / 32 floats; a NaN does not take part)
+__device__ __forceinline__ void block_reduce_max2(float& a, float& b, float* red) {
+  a = ordered_to_float(__reduce_max_sync(0xffffffffu, float_to_ordered(a)));
+  b = ordered_to_float(__reduce_max_sync(0xffffffffu, float_to_ordered(b)));
+  if (threadIdx.x % 32 == 0) {
+    red[2 * (threadIdx.x / 32)] = a;
+    red[2 * (threadIdx.x / 32) + 1] = b;
+  }
   __syncthreads();
-  double b = 0.0;
-  for (int w = 0; w < (int)blockDim.x / 32; ++w) b = __dadd_rn(b, red[w]);
+  for (int w = 0; w < (int)blockDim.x / 32; ++w) {
+    a = fmaxf(a, red[2 * w]);
+    b = fmaxf(b, red[2 * w + 1]);
+  }
   __syncthreads();
-  return b;
 }
 
 // The group of one warp's 32 rows (lanes with valid = false contribute
@@ -516,14 +572,13 @@ __device__ __forceinline__ double block_reduce_sum(double v, double* red) {
 // translation step then falls back to tau = 0). One FP64 operation per row:
 // FP64 throughput is a small fraction of FP32 on this part.
 __device__ __forceinline__ float4 warp_group(double lu, double ell, bool valid) {
-  float m = valid ? (float)(2.0 * lu) : -INFINITY;
-  float e = valid ? (float)ell : -INFINITY;
-  for (int o = 16; o > 0; o >>= 1) {
-    m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, o));
-    e = fmaxf(e, __shfl_xor_sync(0xffffffffu, e, o));
-  }
-  float t = (valid && m > -INFINITY) ? expf((float)__dadd_rn(2.0 * lu, -(double)m)) : 0.0f;
-  if (valid && isnan(lu)) t = NAN;
+  const float m2 = 2.0f * (float)lu, e1 = (float)ell;
+  const bool mok = valid && m2 == m2, eok = valid && e1 == e1;
+  // (a NaN does not take part in the maxima)
+  const float m = ordered_to_float(__reduce_max_sync(0xffffffffu, float_to_ordered(mok ? m2 : -INFINITY)));
+  const float e = ordered_to_float(__reduce_max_sync(0xffffffffu, float_to_ordered(eok ? e1 : -INFINITY)));
+  float t = (valid && m > -INFINITY) ? expf((float)fma(2.0, lu, -(double)m)) : 0.0f;
+  if (valid && !mok) t = NAN;
   for (int o = 16; o > 0; o >>= 1) t = __fadd_rn(t, __shfl_xor_sync(0xffffffffu, t, o));
   return make_float4(m, t, e, 0.0f);
 }
@@ -549,16 +604,21 @@ struct GroupTotal {
 };
 __device__ __forceinline__ GroupTotal block_reduce_groups(const float4* __restrict__ grp, int64_t ng, float* red) {
   float mm = -INFINITY, me = -INFINITY;
-  for (int64_t i = threadIdx.x; i < ng; i += blockDim.x) {
+  const float4 q0 = (int64_t)threadIdx.x < ng ? grp[threadIdx.x] : make_float4(-INFINITY, 0.0f, -INFINITY, 0.0f);
+  mm = fmaxf(mm, q0.x);
+  me = fmaxf(me, q0.z);
+  for (int64_t i = threadIdx.x + blockDim.x; i < ng; i += blockDim.x) {
     const float4 q = grp[i];
     mm = fmaxf(mm, q.x);
     me = fmaxf(me, q.z);
   }
   GroupTotal r;
-  r.top = block_reduce_maxf(mm, red);
-  r.lmax = block_reduce_maxf(me, red);
+  block_reduce_max2(mm, me, red);
+  r.top = mm;
+  r.lmax = me;
   float hi = 0.0f, lo = 0.0f;
-  for (int64_t i = threadIdx.x; i < ng; i += blockDim.x) {
+  if (q0.x > -INFINITY || isnan(q0.y)) pair_add(hi, lo, q0.y * expf(q0.x - r.top), 0.0f);
+  for (int64_t i = threadIdx.x + blockDim.x; i < ng; i += blockDim.x) {
     const float4 q = grp[i];
     if (q.x > -INFINITY || isnan(q.y)) pair_add(hi, lo, q.y * expf(q.x - r.top), 0.0f);
   }
@@ -926,12 +986,6 @@ __device__ __forceinline__ float ex2_approx(float x) {
 
 __device__ __forceinline__ void named_bar_sync(int id, int nthreads) {
   asm volatile("bar.sync %0, %1;" ::"r"(id), "r"(nthreads) : "memory");
-}
-
-// Order-preserving float <-> uint mapping for atomic max on floats of any sign.
-__device__ __forceinline__ unsigned int float_to_ordered(float f) {
-  unsigned int u = __float_as_uint(f);
-  return (u & 0x80000000u) ? ~u : (u | 0x80000000u);
 }
 
 }  // namespace tu
