@@ -100,7 +100,8 @@ def load_peaks() -> dict:
 
 
 KERNEL_SOURCES = {
-    "fused": ["paper_2411_19214_gb300/csrc/fused.cu", "paper_2411_19214_gb300/csrc/tu_internal.cuh"],
+    "fused": ["paper_2411_19214_gb300/csrc/fused.cu", "paper_2411_19214_gb300/csrc/fused_kernel.cuh",
+              "paper_2411_19214_gb300/csrc/tu_internal.cuh"],
     "dense": ["paper_2411_19214_gb300/csrc/dense.cu", "paper_2411_19214_gb300/csrc/tu_internal.cuh"],
 }
 

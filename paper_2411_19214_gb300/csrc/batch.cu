@@ -620,6 +620,8 @@ tu_status tu_batch_create(const tu_market_t* markets, int count, void* stream, t
       d.partner_rows_pad = par.rows_pad;
       d.num_own_tiles = (int)((own.rows + kFusedOwnRows - 1) / kFusedOwnRows);
       d.num_partner_tiles = (int)((par.rows + kFusedPartnerRows - 1) / kFusedPartnerRows);
+      d.cut_t0 = own.cut.t0;
+      d.cut_span = own.cut.span;
       d.slot0 = (int)slot;
       d.c = m->cmul;
       if (side == 0) b->c_host[i] = m->cmul;

@@ -1,44 +1,7 @@
-// fused.cu -- mini-batch IPFP half-sweep (Alg. 2, Eq. iteration_minibatch) on
-// sm_103a tensor cores. Phi is formed tile by tile and never written to HBM.
-//
-// For the half-sweep that updates side "own" against side "partner":
-//   S_r = sum_c exp2( c * <a_r, b_c> + g_c ),   c = log2(e) / (2 sigma),
-//   g_c = (ell_c - max ell) * log2(e)  (partner potential incl. bias, shifted <= 0),
-// then log s_r = log(1/2) + bias_r/(2 sigma) + max ell + log S_r and the
-// closed-form update of Eq. iteration gives the new log u_r.
-//
-// Because the partner biases are folded into g and the shift is the maximum of
-// g, every exponent is bounded by c * |a_r| * |b_c| (checked on the host), so
-// no per-pair running maximum is needed: the running-max rescale of
-// flash-attention collapses to one shift per half-sweep.
-//
-// CTA layout (576 threads, one CTA per SM, persistent over own tiles):
-//   warp 0     : producer (one elected thread): TMA loads of the own tile
-//                [F|K]_j (256 rows x kp) once per own tile (double-buffered
-//                when kp = 64) and of partner tiles (128 rows x kp) through a
-//                STAGES-deep shared-memory ring (a stage is a whole partner
-//                tile, or with four 128-byte k blocks per row one k block of
-//                it), plus a bulk copy of each partner tile's 128 g values
-//                (e4m3 factors: and of its 128 row scales) into an 8-slot ring
-//                that the epilogue reads with broadcast loads.
-//   warp 1     : MMA issuer (one thread): two tcgen05.mma M=128 N=128 chains
-//                (own rows 0-127 and 128-255) per partner tile into one of two
-//                TMEM accumulator buffers (2 x 256 columns = all 512).
-//   warps 2-17 : epilogue: epilogue warp e reads TMEM lane quadrant (e+2)%4
-//                of own sub-tile (e/4)%2 and column half e/8 of every partner
-//                tile, i.e. one own row and 64 columns per thread, so the row
-//                reduction stays inside the thread; the two column halves of
-//                a row meet through shared memory at the end of the own tile.
-//                TMEM loads run one 32-column chunk ahead of the arithmetic;
-//                per pair of columns one packed FMA (f32x2), two ex2.approx
-//                and one packed add; per-tile partials go into a compensated
-//                (Kahan) sum.
-// In a batched launch the own tiles of a CTA come from a list of
-// (market, own tile) items of many independent markets.
-// Every wait is bounded (kWaitLimitNs); a wait that runs out raises the
-// abort flag and the error word, the roles drain, TMEM is freed, and the
-// kernel returns.
-#include "tu_internal.cuh"
+// fused.cu -- the fused path's host side: tensor maps, launch shapes, and the
+// narrow and batched half-sweeps of fused_kernel.cuh (the kernel, its design
+// and its instantiations).
+#include "fused_kernel.cuh"
 
 #include <cstring>
 #include <mutex>
@@ -46,1368 +9,6 @@
 namespace tu {
 
 namespace {
-
-constexpr int kEpiWarps = 16;
-constexpr int kThreads = 64 + kEpiWarps * 32;  // producer warp, MMA warp, epilogue warps
-constexpr int kOwnBytesPerKB = kFusedOwnRows * 128;          // 32 KB per 64-wide k block
-constexpr int kPartnerBytesPerKB = kFusedPartnerRows * 128;  // 16 KB per 64-wide k block
-constexpr int kGSlots = 8;                                   // g ring depth
-constexpr int kGBytes = kFusedPartnerRows * 4;               // one partner tile of g (512 B)
-constexpr uint32_t kTmemCols = 512;
-
-// Epilogue modes of the one fused kernel: the same TMA / MMA pipeline forms
-// the tiles of c * phi_hat + g; the epilogue either reduces them (a half-sweep),
-// keeps the k best columns of every row (ranked lists) or writes mu.
-// Markets whose factor range is too wide for one shift per half-sweep (see
-// market.cu) take kModeSweepWide: a half-sweep that keeps a running maximum
-// per row and rescales the row's sum whenever it grows (the log-domain
-// rescale of an online softmax), so that no term's exponent exceeds 0.
-enum : int { kModeSweep = 0, kModeTopK = 1, kModeMu = 2, kModeTopKShared = 3, kModeSweepWide = 4 };
-
-struct FusedParams {
-  int64_t rows;            // own users of this launch: [row0, row0 + rows)
-  int64_t row0;            // first own user
-  int64_t col0;            // first partner column streamed (multiple of 4)
-  int64_t ncols;           // partner columns streamed: [col0, col0 + ncols)
-  int num_own_tiles;       // ceil(rows / 256)
-  int num_partner_tiles;   // ceil(ncols / 128)
-  float c;                 // log2(e) / (2 sigma)
-  const float* g;          // partner prepared potentials (index = partner user), -inf padded
-  const double* lmax;      // partner shift (natural log)
-  const double* own_off;   // offset added to the stored own potentials, or nullptr for 0   (sweep)
-  float4* grp;             // own-side groups written by an updating pass, or nullptr        (sweep)
-  const float* b2s;        // own bias / (2 sigma), or nullptr          (sweep)
-  const double* mass;      // own capacities                             (sweep)
-  double* log_u;           // own potentials (in: old, out: new)          (sweep)
-  double* ell;             // own ell: out (sweep), in (ranked lists, mu)
-  double* partials;        // [gridDim.x][4]                              (sweep)
-  int* err;                // device error word
-  int residual;
-  int update;
-  const double* omega;     // over-relaxation factor (device scalar) or nullptr for 1  (sweep)
-  // batched launches: per-market descriptors and this launch's item lists
-  const BatchDesc* bdesc;
-  const int2* items;
-  const int* cta_start;
-  // ranked lists: for own user row0 + r, idx[r * k + i], logmu[r * k + i], best first
-  int k;
-  int32_t* idx;
-  float* logmu;
-  float* hand_v;           // rows x k scratch: second column half's list
-  int32_t* hand_i;
-  // mu block: out[(r) * ld + (col - y0)] for partner col in [y0, y0 + ny)
-  float* out;
-  int64_t ld;
-  int64_t y0;
-  int64_t ny;
-  // e4m3 factors: per-row scales of the own side (index row0 + r) and of the
-  // partner side (index = partner user); the product of row r and partner
-  // column j is fs_own[r] * fs_par[j] * <e4m3 row r, e4m3 row j>
-  const float* fs_own;
-  const float* fs_par;
-  // partner split (single-market half-sweeps, 1 = off): an item is an own
-  // tile and one of `split` contiguous ranges of its partner tiles; each
-  // epilogue warp writes its rows' partial sums to part[s * rows + r], and the
-  // warp that completes a (tile, 32-row block), counted in split_cnt, sums
-  // the partials in range order and updates the rows
-  int split;
-  int range_major;         // items ordered range by range (every own tile against range 0 first)
-  // L2 residency of the partner matrix (single-market launches): this
-  // fraction of its lines is loaded evict-last, so that a partner matrix
-  // larger than L2 keeps a fixed part resident across the waves of own tiles
-  // (0: no hint)
-  float l2_keep;
-  float4* part;
-  int* split_cnt;
-  // folded g (BF16 half-sweeps, kp = 64): the partner side's g / c as the
-  // K = 16 operand of one extra MMA per chain and partner tile, 4 KB per
-  // partner tile of 128 rows in the unswizzled K-major layout (written by the
-  // preparation kernel)
-  const uint8_t* gfold;
-};
-
-// Own-tile buffers: with one 128-byte k block per row the next own tile is
-// loaded while the current one is still in use (short items of batched
-// launches); with two or four there is room for one only.
-template <int KB>
-constexpr int kABufs = KB == 1 ? 2 : 1;
-
-// k blocks per partner stage: with four k blocks per row (d up to 128 in
-// BF16, 256 in e4m3) a whole 64 KB partner tile would leave room for one
-// stage beside the 128 KB own tile, so a stage then carries one k block and a
-// partner tile takes four stages.
-constexpr int kbs_for(int KB) { return KB == 4 ? 1 : KB; }
-
-// Operand formats: BF16, e4m3 with one scale per side, e4m3 with one per row.
-enum : int { kFmtBF16 = 0, kFmtE4M3Side = 1, kFmtE4M3Rows = 2 };
-
-// shared memory: [A: ABUFS x KB x 32 KB][B: STAGES x KBS x 16 KB][g ring: 8 x 512 B]
-//                [per-row scales: scale ring 8 x 512 B][barriers and flags: 512 B]
-//                [reduction: 512 B][row hand-over: 2 x 256 floats]
-constexpr int kTailBytes = 512 + 512 + 2 * kFusedOwnRows * 4;
-// folded g: the partner tile's K = 16 operand rides in its (last) stage, the
-// own side's constant operand (ones in columns 0-2) is one tile of its own.
-// Taken for rows of one k block (d <= 32 in BF16, d <= 64 in e4m3 with one
-// scale per side), where the tensor pipe has room for a fifth MMA per chain
-// and the epilogue sheds its g loads: batched d = 32 half-sweep 5.44 -> 5.12
-// ms, a 1e5 d = 32 sweep 3.54 -> 3.37 ms; with two BF16 k blocks (d =
-// 33..64) the ninth MMA costs more than it saves (1e6 d = 64 half-sweep
-// 184.5 -> 187.1 ms), so those keep g in the shared ring. e4m3 rows with one
-// scale per side: 1e6 d = 64 half-sweep 149.4 -> 142.5 ms; there the fold MMA
-// is a separate kind::f16 MMA (BF16 ones x BF16 g / c) into the same FP32
-// accumulator. e4m3 rows with per-row scales cannot fold: the own row's scale
-// multiplies phi, so no per-column constant added to it gives g in every row.
-constexpr int kFoldBytes = kFusedPartnerRows * 32;
-constexpr bool fold_for(int KB, int MODE, bool BATCH, int fmt, bool nofold) {
-  return MODE == kModeSweep && (fmt == kFmtBF16 || fmt == kFmtE4M3Side) && KB == 1 && !nofold;
-}
-constexpr int stage_bytes(int KB, bool fold) { return kbs_for(KB) * kPartnerBytesPerKB + (fold ? kFoldBytes : 0); }
-constexpr int smem_bytes(int KB, int fmt, int stages, bool fold = false) {
-  return 1024 /*alignment slack*/ + (KB == 1 ? 2 : 1) * KB * kOwnBytesPerKB + stages * stage_bytes(KB, fold) +
-         (fold ? kFoldBytes : 0) + kGSlots * kGBytes * (fmt == kFmtE4M3Rows ? 2 : 1) + kTailBytes;
-}
-
-__device__ __forceinline__ void raise_error(int* err, volatile int* abort_flag, int code) {
-  atomicCAS(err, kErrNone, code);
-  *abort_flag = 1;
-}
-
-// 1D bulk copy global -> shared, completion counted on an mbarrier (16-byte aligned, size % 16 == 0).
-__device__ __forceinline__ void bulk_load(void* smem_dst, const void* gsrc, uint32_t bytes, uint64_t* bar) {
-  asm volatile(
-      "cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(
-          smem_u32(smem_dst)),
-      "l"(reinterpret_cast<uint64_t>(gsrc)), "r"(bytes), "r"(smem_u32(bar))
-      : "memory");
-}
-
-// Issue a 32-lane x 32-column FP32 TMEM load without waiting for it.
-__device__ __forceinline__ void tmem_ld_issue(uint32_t taddr, uint32_t (&r)[32]) {
-  asm volatile(
-      "tcgen05.ld.sync.aligned.32x32b.x32.b32 "
-      "{%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15, "
-      "%16, %17, %18, %19, %20, %21, %22, %23, %24, %25, %26, %27, %28, %29, %30, %31}, [%32];"
-      : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]),
-        "=r"(r[8]), "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15]),
-        "=r"(r[16]), "=r"(r[17]), "=r"(r[18]), "=r"(r[19]), "=r"(r[20]), "=r"(r[21]), "=r"(r[22]), "=r"(r[23]),
-        "=r"(r[24]), "=r"(r[25]), "=r"(r[26]), "=r"(r[27]), "=r"(r[28]), "=r"(r[29]), "=r"(r[30]), "=r"(r[31])
-      : "r"(taddr)
-      : "memory");
-}
-
-// Wait for the outstanding TMEM loads; the registers are passed through so
-// that no use of them can be scheduled before the wait.
-__device__ __forceinline__ void tmem_ld_wait(uint32_t (&r)[32]) {
-  asm volatile("tcgen05.wait::ld.sync.aligned;"
-               : "+r"(r[0]), "+r"(r[1]), "+r"(r[2]), "+r"(r[3]), "+r"(r[4]), "+r"(r[5]), "+r"(r[6]), "+r"(r[7]),
-                 "+r"(r[8]), "+r"(r[9]), "+r"(r[10]), "+r"(r[11]), "+r"(r[12]), "+r"(r[13]), "+r"(r[14]),
-                 "+r"(r[15]), "+r"(r[16]), "+r"(r[17]), "+r"(r[18]), "+r"(r[19]), "+r"(r[20]), "+r"(r[21]),
-                 "+r"(r[22]), "+r"(r[23]), "+r"(r[24]), "+r"(r[25]), "+r"(r[26]), "+r"(r[27]), "+r"(r[28]),
-                 "+r"(r[29]), "+r"(r[30]), "+r"(r[31])
-               :
-               : "memory");
-}
-
-// acc(2 lanes) += (ex2(phi0 * c + g0), ex2(phi1 * c + g1)) with packed FP32x2 FMA and add.
-__device__ __forceinline__ void pair_step(uint64_t& acc, uint32_t phi0, uint32_t phi1, float g0, float g1,
-                                          uint64_t cc) {
-  asm("{\n\t.reg .b64 a, gg, t, e;\n\t.reg .f32 t0, t1, e0, e1;\n\t"
-      "mov.b64 a, {%1, %2};\n\t"
-      "mov.b64 gg, {%3, %4};\n\t"
-      "fma.rn.f32x2 t, a, %5, gg;\n\t"
-      "mov.b64 {t0, t1}, t;\n\t"
-      "ex2.approx.ftz.f32 e0, t0;\n\t"
-      "ex2.approx.ftz.f32 e1, t1;\n\t"
-      "mov.b64 e, {e0, e1};\n\t"
-      "add.rn.f32x2 %0, %0, e;\n\t}"
-      : "+l"(acc)
-      : "r"(phi0), "r"(phi1), "f"(g0), "f"(g1), "l"(cc));
-}
-
-// e4m3 factors: acc += (ex2(phi0 f0 c + g0), ex2(phi1 f1 c + g1)), f the
-// partner rows' scales (the own row's scale is folded into c).
-__device__ __forceinline__ void pair_step_scaled(uint64_t& acc, uint32_t phi0, uint32_t phi1, float g0, float g1,
-                                                 float f0, float f1, uint64_t cc) {
-  asm("{\n\t.reg .b64 a, gg, ff, t, e;\n\t.reg .f32 t0, t1, e0, e1;\n\t"
-      "mov.b64 a, {%1, %2};\n\t"
-      "mov.b64 gg, {%3, %4};\n\t"
-      "mov.b64 ff, {%5, %6};\n\t"
-      "mul.rn.f32x2 t, a, ff;\n\t"
-      "fma.rn.f32x2 t, t, %7, gg;\n\t"
-      "mov.b64 {t0, t1}, t;\n\t"
-      "ex2.approx.ftz.f32 e0, t0;\n\t"
-      "ex2.approx.ftz.f32 e1, t1;\n\t"
-      "mov.b64 e, {e0, e1};\n\t"
-      "add.rn.f32x2 %0, %0, e;\n\t}"
-      : "+l"(acc)
-      : "r"(phi0), "r"(phi1), "f"(g0), "f"(g1), "f"(f0), "f"(f1), "l"(cc));
-}
-
-// Folded g: acc += (ex2(D0 * c), ex2(D1 * c)), D = phi + g / c from the MMA.
-__device__ __forceinline__ void pair_step_fold(uint64_t& acc, uint32_t d0, uint32_t d1, uint64_t cc) {
-  asm("{\n\t.reg .b64 a, t, e;\n\t.reg .f32 t0, t1, e0, e1;\n\t"
-      "mov.b64 a, {%1, %2};\n\t"
-      "mul.rn.f32x2 t, a, %3;\n\t"
-      "mov.b64 {t0, t1}, t;\n\t"
-      "ex2.approx.ftz.f32 e0, t0;\n\t"
-      "ex2.approx.ftz.f32 e1, t1;\n\t"
-      "mov.b64 e, {e0, e1};\n\t"
-      "add.rn.f32x2 %0, %0, e;\n\t}"
-      : "+l"(acc)
-      : "r"(d0), "r"(d1), "l"(cc));
-}
-
-__device__ __forceinline__ void chunk_sum_fold(const uint32_t (&v)[32], uint64_t cc, uint64_t (&acc)[4]) {
-#pragma unroll
-  for (int i = 0; i < 16; ++i) pair_step_fold(acc[i & 3], v[2 * i], v[2 * i + 1], cc);
-}
-
-// phi of column i of a chunk, times the partner row's scale (e4m3 factors
-// with per-row scales)
-template <bool RS>
-__device__ __forceinline__ float scaled_phi(uint32_t v, const float* fs, int i) {
-  if constexpr (RS) return __uint_as_float(v) * fs[i];
-  return __uint_as_float(v);
-}
-
-__device__ __forceinline__ float unpack_sum(uint64_t a) {
-  return __uint_as_float((uint32_t)a) + __uint_as_float((uint32_t)(a >> 32));
-}
-
-// Sum over one 32-column chunk: 16 packed pairs into four packed accumulators.
-template <bool RS>
-__device__ __forceinline__ void chunk_sum(const uint32_t (&v)[32], const float4* gs4, const float4* fs4, uint64_t cc,
-                                          uint64_t (&acc)[4]) {
-#pragma unroll
-  for (int i = 0; i < 8; ++i) {
-    const float4 gg = gs4[i];
-    if constexpr (RS) {
-      const float4 ff = fs4[i];
-      pair_step_scaled(acc[(2 * i) & 3], v[4 * i + 0], v[4 * i + 1], gg.x, gg.y, ff.x, ff.y, cc);
-      pair_step_scaled(acc[(2 * i + 1) & 3], v[4 * i + 2], v[4 * i + 3], gg.z, gg.w, ff.z, ff.w, cc);
-    } else {
-      pair_step(acc[(2 * i) & 3], v[4 * i + 0], v[4 * i + 1], gg.x, gg.y, cc);
-      pair_step(acc[(2 * i + 1) & 3], v[4 * i + 2], v[4 * i + 3], gg.z, gg.w, cc);
-    }
-  }
-}
-
-// ---- wide markets: one pass with a running maximum per row -----------------
-
-// t = (phi0, phi1) * c + (g0, g1); e4m3 per-row scales: (phi0 f0, phi1 f1) * c + (g0, g1)
-template <bool RS>
-__device__ __forceinline__ uint64_t pair_exponents(uint32_t phi0, uint32_t phi1, float g0, float g1, float f0,
-                                                   float f1, uint64_t cc) {
-  uint64_t t;
-  if constexpr (RS) {
-    asm("{\n\t.reg .b64 a, gg, ff, x;\n\t"
-        "mov.b64 a, {%1, %2};\n\t"
-        "mov.b64 gg, {%3, %4};\n\t"
-        "mov.b64 ff, {%5, %6};\n\t"
-        "mul.rn.f32x2 x, a, ff;\n\t"
-        "fma.rn.f32x2 %0, x, %7, gg;\n\t}"
-        : "=l"(t)
-        : "r"(phi0), "r"(phi1), "f"(g0), "f"(g1), "f"(f0), "f"(f1), "l"(cc));
-  } else {
-    asm("{\n\t.reg .b64 a, gg;\n\t"
-        "mov.b64 a, {%1, %2};\n\t"
-        "mov.b64 gg, {%3, %4};\n\t"
-        "fma.rn.f32x2 %0, a, %5, gg;\n\t}"
-        : "=l"(t)
-        : "r"(phi0), "r"(phi1), "f"(g0), "f"(g1), "l"(cc));
-  }
-  return t;
-}
-
-// acc(2 lanes) += (ex2(t0 + m), ex2(t1 + m)), mm = (m, m)
-__device__ __forceinline__ void ex2_add_shifted(uint64_t& acc, uint64_t t, uint64_t mm) {
-  asm("{\n\t.reg .b64 x, e;\n\t.reg .f32 x0, x1, e0, e1;\n\t"
-      "add.rn.f32x2 x, %1, %2;\n\t"
-      "mov.b64 {x0, x1}, x;\n\t"
-      "ex2.approx.ftz.f32 e0, x0;\n\t"
-      "ex2.approx.ftz.f32 e1, x1;\n\t"
-      "mov.b64 e, {e0, e1};\n\t"
-      "add.rn.f32x2 %0, %0, e;\n\t}"
-      : "+l"(acc)
-      : "l"(t), "l"(mm));
-}
-
-// acc(2 lanes) *= (s, s)
-__device__ __forceinline__ void scale2(uint64_t& acc, float s) {
-  const uint64_t ss = ((uint64_t)__float_as_uint(s) << 32) | __float_as_uint(s);
-  asm("mul.rn.f32x2 %0, %0, %1;" : "+l"(acc) : "l"(ss));
-}
-
-// The larger of a, b and c; NaN if any of them is NaN.
-__device__ __forceinline__ float max3_nan(float a, float b, float c) {
-  float r;
-  asm("max.NaN.f32 %0, %1, %2, %3;" : "=f"(r) : "f"(a), "f"(b), "f"(c));
-  return r;
-}
-
-// 2^d for an integer-valued d <= 0, as an exact power of two; 0 for d below
-// -126 (FP32's normal range), for -inf and for NaN.
-__device__ __forceinline__ float exp2_int(float d) {
-  return d >= -126.0f ? __int_as_float((127 + (int)d) << 23) : 0.0f;
-}
-
-// One 32-column chunk of a wide market's row: the exponents t = c * phi + g,
-// their largest; when that exceeds the row's running shift M (an integer,
-// -inf before the first term) the shift becomes M' = ceil(max) and all the
-// row has summed so far (this tile's packed partials acc, the compensated
-// sum over the earlier tiles) is multiplied by 2^(M - M'), a power of two,
-// so exactly; then acc += 2^(t - M). Every term is at most 1, and the row's
-// log-sum is log(sum) + M ln 2.
-template <bool RS>
-__device__ __forceinline__ void chunk_sum_wide(uint32_t (&v)[32], const float4* gs4, const float4* fs4, uint64_t cc,
-                                               uint64_t (&acc)[4], float& M, float& sum, float& comp) {
-  // the exponents replace the loaded values in place
-#pragma unroll
-  for (int i = 0; i < 8; ++i) {
-    const float4 gg = gs4[i];
-    float4 ff = make_float4(1.f, 1.f, 1.f, 1.f);
-    if constexpr (RS) ff = fs4[i];
-    const uint64_t t0 = pair_exponents<RS>(v[4 * i + 0], v[4 * i + 1], gg.x, gg.y, ff.x, ff.y, cc);
-    const uint64_t t1 = pair_exponents<RS>(v[4 * i + 2], v[4 * i + 3], gg.z, gg.w, ff.z, ff.w, cc);
-    v[4 * i + 0] = (uint32_t)t0;
-    v[4 * i + 1] = (uint32_t)(t0 >> 32);
-    v[4 * i + 2] = (uint32_t)t1;
-    v[4 * i + 3] = (uint32_t)(t1 >> 32);
-  }
-  float mx = -INFINITY;
-#pragma unroll
-  for (int k = 0; k < 16; ++k) mx = max3_nan(mx, __uint_as_float(v[2 * k]), __uint_as_float(v[2 * k + 1]));
-  if (!(mx <= M)) {  // a larger maximum (or NaN, which then reaches the sum)
-    const float Mn = ceilf(mx);
-    const float sc = exp2_int(M - Mn);
-    sum *= sc;
-    comp *= sc;
-#pragma unroll
-    for (int k = 0; k < 4; ++k) scale2(acc[k], sc);
-    M = Mn;
-  }
-  if (M == -INFINITY) return;  // every exponent so far is -inf: no terms
-  const uint64_t mm = ((uint64_t)__float_as_uint(-M) << 32) | __float_as_uint(-M);
-#pragma unroll
-  for (int k = 0; k < 16; ++k)
-    ex2_add_shifted(acc[k & 3], ((uint64_t)v[2 * k + 1] << 32) | v[2 * k], mm);
-}
-
-constexpr int kMaxTopK = 64;
-
-// Insert score s of partner col into a thread's list, sorted by decreasing
-// score; equal scores keep the earlier (lower) column first. Returns the new
-// threshold (the k-th best score, -inf while the list is not full). Kept out
-// of line: it runs rarely, and one copy keeps the hot loop small.
-__device__ __noinline__ float top_insert(float* tv, int32_t* ti, int* cnt, int k, float s, int32_t col) {
-  int c = *cnt;
-  int pos = c < k ? c : k - 1;
-  while (pos > 0 && s > tv[pos - 1]) {
-    tv[pos] = tv[pos - 1];
-    ti[pos] = ti[pos - 1];
-    --pos;
-  }
-  tv[pos] = s;
-  ti[pos] = col;
-  if (c < k) *cnt = ++c;
-  return c == k ? tv[k - 1] : -INFINITY;
-}
-
-// Ranked lists: score = c * phi_hat + g (log2 units, shifted; same order as
-// log mu within a row). The chunk's maximum is compared with the running k-th
-// best first, so most chunks cost one FFMA and one max per column.
-template <bool RS>
-__device__ __forceinline__ void chunk_topk(const uint32_t (&v)[32], const float* g, const float* fs, float c,
-                                           int64_t colbase, int k, float* tv, int32_t* ti, int* cnt, float& thr) {
-  const float4* g4 = reinterpret_cast<const float4*>(g);
-  float s[32];
-  float mx = -INFINITY;
-#pragma unroll
-  for (int i4 = 0; i4 < 8; ++i4) {
-    const float4 gg = g4[i4];
-    s[4 * i4 + 0] = fmaf(scaled_phi<RS>(v[4 * i4 + 0], fs, 4 * i4 + 0), c, gg.x);
-    s[4 * i4 + 1] = fmaf(scaled_phi<RS>(v[4 * i4 + 1], fs, 4 * i4 + 1), c, gg.y);
-    s[4 * i4 + 2] = fmaf(scaled_phi<RS>(v[4 * i4 + 2], fs, 4 * i4 + 2), c, gg.z);
-    s[4 * i4 + 3] = fmaf(scaled_phi<RS>(v[4 * i4 + 3], fs, 4 * i4 + 3), c, gg.w);
-    mx = fmaxf(mx, fmaxf(fmaxf(s[4 * i4 + 0], s[4 * i4 + 1]), fmaxf(s[4 * i4 + 2], s[4 * i4 + 3])));
-  }
-  if (mx > thr) {
-#pragma unroll
-    for (int e = 0; e < 32; ++e)
-      if (s[e] > thr) thr = top_insert(tv, ti, cnt, k, s[e], (int32_t)(colbase + e));
-  }
-}
-
-// Ranked lists with k <= kSharedTopK (kModeTopKShared): every epilogue thread
-// has kTopKSlots (score, column) slots in shared memory, slot i of thread t
-// at [i * kEpiThreads + t] (a warp's accesses to one slot are conflict-free).
-// The first k hold the k best of its row and column half, sorted by
-// decreasing score, equal scores in increasing column order (the order in
-// which a column half's columns arrive); they start as (-inf, INT32_MAX)
-// pairs, so the k-th score is the threshold from the first column on. The
-// other slots buffer candidates: columns that beat the threshold as of the
-// last merge, appended in column order. When a lane's buffer could overflow,
-// the whole warp merges: all 32 lanes insert their candidates side by side.
-// Rows whose rankings differ (a converged market, where the potentials cancel
-// the popularity terms) meet their candidates at different columns; inserting
-// each at once ran the lanes' insertions one after another (3 of 32 lanes per
-// chunk and more), which cost several times the pass itself.
-// (Top-10 lists of 100,000 users over 60,000 partners, d = 64, at solved
-// potentials: 4.23 ms with every candidate inserted at once, 2.93 with
-// buffers, 2.74 with the shared bound below, 2.71 without the scores kept
-// across the vote, 2.16 with the merges of all warps at the same tiles; a
-// half-sweep of that size takes 1.4.)
-constexpr int kSharedTopK = 14;
-constexpr int kTopKSlots = 20;
-constexpr int kEpiThreads = kEpiWarps * 32;
-// (the slots, then one 8-byte word per thread: the bound that the two threads
-// of a row share, see chunk_topk_shared)
-constexpr int kTopKListBytes = (kTopKSlots + 1) * kEpiThreads * 8;
-// A group of kTopKGroup columns adds at most that many candidates, so a buffer
-// of kTopKSlots - k >= kTopKGroup + 1 slots is merged whenever fewer than
-// kTopKGroup are free.
-constexpr int kTopKGroup = 4;
-static_assert(kTopKSlots - kSharedTopK > kTopKGroup, "candidate slots");
-constexpr int kWideShiftBytes = 2 * kFusedOwnRows * 4;  // kModeSweepWide: the row hand-over's shifts
-// kModeMu: each epilogue warp turns its 32 rows x mu_width columns through
-// shared memory, so that its stores run along the rows of the output (rows of
-// mu_width + 1 floats: conflict-free columns). Half the width where a
-// four-block own tile leaves no room for more.
-constexpr int mu_width(int KB) { return KB == 4 ? 16 : 32; }
-constexpr int mu_stage_floats(int KB) { return 32 * (mu_width(KB) + 1); }
-// shared memory a mode needs after the tail area
-constexpr int mode_extra_bytes(int mode, int KB) {
-  return mode == kModeTopKShared  ? kTopKListBytes
-         : mode == kModeSweepWide ? kWideShiftBytes
-         : mode == kModeMu        ? kEpiWarps * mu_stage_floats(KB) * 4
-                                  : 0;
-}
-
-__device__ __forceinline__ void sts_u64(uint32_t a, uint64_t v) {
-  asm volatile("st.volatile.shared.b64 [%0], %1;" ::"r"(a), "l"(v));
-}
-__device__ __forceinline__ uint64_t lds_u64(uint32_t a) {
-  uint64_t v;
-  asm volatile("ld.volatile.shared.b64 %0, [%1];" : "=l"(v) : "r"(a));
-  return v;
-}
-
-// A slot: the score in the low word, the column in the high one.
-__device__ __forceinline__ uint64_t slot_of(float s, int32_t col) {
-  return ((uint64_t)(uint32_t)col << 32) | __float_as_uint(s);
-}
-__device__ __forceinline__ float slot_score(uint64_t w) { return __uint_as_float((uint32_t)w); }
-__device__ __forceinline__ int32_t slot_col(uint64_t w) { return (int32_t)(w >> 32); }
-constexpr uint32_t kSlotStride = kEpiThreads * 8;
-
-// Merge a warp's candidate buffers (cnt candidates of this lane) into its
-// lists at shared address lv: round j inserts every lane's candidate j, where
-// it beats the lane's current k-th score. An insertion reads the entries above
-// it four at a time (independent loads: one shared-memory latency per four
-// shifts). Returns the new k-th score. Kept out of line: one copy serves every
-// call site.
-__device__ __noinline__ float list_merge(uint32_t lv, int k, int cnt) {
-  const uint32_t last = lv + (uint32_t)(k - 1) * kSlotStride;
-  float thr = slot_score(lds_u64(last));
-  const int rounds = __reduce_max_sync(0xffffffffu, cnt);
-  for (int j = 0; j < rounds; ++j) {
-    const uint64_t w = j < cnt ? lds_u64(last + (uint32_t)(j + 1) * kSlotStride) : slot_of(-INFINITY, 0);
-    const float s = slot_score(w);
-    if (s > thr) {
-      uint32_t pos = last;
-      bool go = pos != lv;
-      while (go) {
-        uint64_t e[4];
-#pragma unroll
-        for (int i = 0; i < 4; ++i) {
-          const uint32_t a = pos - (uint32_t)(i + 1) * kSlotStride;
-          e[i] = (int32_t)(a - lv) >= 0 ? lds_u64(a) : slot_of(INFINITY, 0);
-        }
-#pragma unroll
-        for (int i = 0; i < 4; ++i) {
-          go = go && s > slot_score(e[i]);
-          if (go) {
-            sts_u64(pos, e[i]);
-            pos -= kSlotStride;
-          }
-        }
-        go = go && pos != lv;
-      }
-      sts_u64(pos, w);
-      thr = slot_score(lds_u64(last));
-    }
-    __syncwarp();
-  }
-  return thr;
-}
-
-// A row's columns are split over two threads (column halves), each with its own
-// list. If both lists hold ceil(k / 2) scores of at least b, the row's k-th
-// best is at least b: a column below b cannot be listed. So each thread
-// publishes, after every merge, the value just below its list's
-// ceil(k / 2)-th score (so that equal scores still pass), tagged with its own
-// tile, and takes as threshold the larger of its k-th score and the smaller
-// of the two published values: about the k-th best of both halves together,
-// which halves the candidates. A word of an older tile (or one read while the
-// other thread is a merge behind) only makes the bound weaker, never wrong, so
-// the lists do not depend on timing.
-struct SharedBound {
-  uint32_t mine, other;  // shared addresses of the two threads' words
-  uint32_t tag;          // the own tile, counted per CTA
-  float pub;             // this thread's published value
-  __device__ __forceinline__ void publish(uint32_t lv, int k) {
-    pub = nextafterf(slot_score(lds_u64(lv + (uint32_t)((k - 1) / 2) * kSlotStride)), -INFINITY);
-    sts_u64(mine, ((uint64_t)tag << 32) | __float_as_uint(pub));
-  }
-  __device__ __forceinline__ float bound() const {
-    const uint64_t w = lds_u64(other);
-    return (uint32_t)(w >> 32) == tag ? fminf(pub, __uint_as_float((uint32_t)w)) : -INFINITY;
-  }
-};
-
-// One 32-column chunk: the scores' maximum in every group of four columns; the
-// groups in which some lane beats its threshold form their scores again and
-// append them (keeping all 32 beside the next chunk's TMEM load in flight
-// would spill).
-template <bool RS>
-__device__ __forceinline__ void chunk_topk_shared(const uint32_t (&v)[32], const float* g, const float* fs,
-                                                  uint64_t cc, int64_t colbase, int k, uint32_t lv, int& cnt,
-                                                  float& thr, SharedBound& sb) {
-  constexpr int kGroups = 32 / kTopKGroup;
-  static_assert(kTopKGroup == 4, "a group is one float4 of g");
-  const float4* g4 = reinterpret_cast<const float4*>(g);
-  const float4* fs4 = reinterpret_cast<const float4*>(fs);
-  auto scores = [&](int i, float (&s)[4]) {
-    const float4 gg = g4[i];
-    float4 ff = make_float4(1.f, 1.f, 1.f, 1.f);
-    if constexpr (RS) ff = fs4[i];
-    const uint64_t t0 = pair_exponents<RS>(v[4 * i + 0], v[4 * i + 1], gg.x, gg.y, ff.x, ff.y, cc);
-    const uint64_t t1 = pair_exponents<RS>(v[4 * i + 2], v[4 * i + 3], gg.z, gg.w, ff.z, ff.w, cc);
-    s[0] = __uint_as_float((uint32_t)t0);
-    s[1] = __uint_as_float((uint32_t)(t0 >> 32));
-    s[2] = __uint_as_float((uint32_t)t1);
-    s[3] = __uint_as_float((uint32_t)(t1 >> 32));
-  };
-  thr = fmaxf(thr, sb.bound());
-  uint32_t hit = 0;
-#pragma unroll
-  for (int i = 0; i < kGroups; ++i) {
-    float s[4];
-    scores(i, s);
-    if (fmaxf(fmaxf(s[0], s[1]), fmaxf(s[2], s[3])) > thr) hit |= 1u << i;
-  }
-  hit = __reduce_or_sync(0xffffffffu, hit);
-  if (hit == 0) return;
-#pragma unroll
-  for (int i = 0; i < kGroups; ++i) {
-    if ((hit & (1u << i)) == 0) continue;
-    float s[4];
-    scores(i, s);
-#pragma unroll
-    for (int e = 0; e < 4; ++e) {
-      if (s[e] > thr) {
-        sts_u64(lv + (uint32_t)(k + cnt) * kSlotStride, slot_of(s[e], (int32_t)(colbase + 4 * i + e)));
-        ++cnt;
-      }
-    }
-    if (__any_sync(0xffffffffu, cnt > kTopKSlots - k - kTopKGroup)) {
-      thr = list_merge(lv, k, cnt);
-      sb.publish(lv, k);
-      cnt = 0;
-    }
-  }
-}
-
-// mu block: mu = 2^(c * phi_hat + g + lo) * 2^hi, where hi + lo = (shift + ell_row) log2 e;
-// 2^hi as the two factors s1, s2 (hi clamped to +-252: beyond, the product is
-// 0 or infinite all the same). The warp's 32 rows x 32 columns go through
-// `st` in shared memory, W columns at a time, so that every store of the warp
-// writes 32 / W runs of W consecutive floats of the output; lane = row before,
-// (row % (32 / W), column) after. nrow: the warp's rows inside the block, orow:
-// its first row there.
-template <bool RS, int W>
-__device__ __forceinline__ void chunk_mu(const uint32_t (&v)[32], const float* g, const float* fs, float c,
-                                         int64_t colbase, float lo, int hi, float s1, float s2, int lane, int nrow,
-                                         int64_t orow, float* st, const FusedParams& p) {
-  const float4* g4 = reinterpret_cast<const float4*>(g);
-  float t[32];
-  float far = 0.0f;
-#pragma unroll
-  for (int i = 0; i < 8; ++i) {
-    const float4 gg = g4[i];
-    t[4 * i + 0] = fmaf(scaled_phi<RS>(v[4 * i + 0], fs, 4 * i + 0), c, gg.x) + lo;
-    t[4 * i + 1] = fmaf(scaled_phi<RS>(v[4 * i + 1], fs, 4 * i + 1), c, gg.y) + lo;
-    t[4 * i + 2] = fmaf(scaled_phi<RS>(v[4 * i + 2], fs, 4 * i + 2), c, gg.z) + lo;
-    t[4 * i + 3] = fmaf(scaled_phi<RS>(v[4 * i + 3], fs, 4 * i + 3), c, gg.w) + lo;
-    far = fmaxf(far, fmaxf(fmaxf(fabsf(t[4 * i + 0]), fabsf(t[4 * i + 1])),
-                           fmaxf(fabsf(t[4 * i + 2]), fabsf(t[4 * i + 3]))));
-  }
-  const bool near = !__any_sync(0xffffffffu, far > 100.0f);
-#pragma unroll
-  for (int c0 = 0; c0 < 32; c0 += W) {
-    float* mine = st + lane * (W + 1);
-    if (near) {
-#pragma unroll
-      for (int i = 0; i < W; ++i) mine[i] = ex2_approx(t[c0 + i]) * s1 * s2;
-    } else {
-      // (an exponent beyond the FP32 range is brought back by hi first)
-#pragma unroll
-      for (int i = 0; i < W; ++i)
-        mine[i] = fabsf(t[c0 + i]) <= 100.0f ? ex2_approx(t[c0 + i]) * s1 * s2 : ex2_approx(t[c0 + i] + (float)hi);
-    }
-    __syncwarp();
-    const int64_t col = colbase + c0 + lane % W;
-    if (col >= p.y0 && col < p.y0 + p.ny) {
-      float* o = p.out + (orow + lane / W) * p.ld + (col - p.y0);
-      const float* src = st + (lane / W) * (W + 1) + lane % W;
-      const int64_t step = (32 / W) * p.ld;
-      if (nrow == 32) {
-#pragma unroll 8
-        for (int i = 0; i < W; ++i) o[i * step] = src[i * (32 / W) * (W + 1)];
-      } else {
-        for (int i = 0; i * (32 / W) + lane / W < nrow; ++i) o[i * step] = src[i * (32 / W) * (W + 1)];
-      }
-    }
-    __syncwarp();
-  }
-}
-
-// The items of a batched launch are (market, own tile) pairs.
-struct ItemRef {
-  const BatchDesc* d;
-  int t;
-};
-__device__ __forceinline__ ItemRef batch_item(const FusedParams& p, int it) {
-  const int2 v = p.items[it];
-  return {p.bdesc + v.x, v.y};
-}
-
-// This CTA's items: own tiles blockIdx.x, blockIdx.x + gridDim.x, ... of one
-// market, or a contiguous range of the batched item list (all roles walk the
-// same sequence).
-template <bool BATCH>
-__device__ __forceinline__ int item_begin(const FusedParams& p) {
-  if constexpr (BATCH) return p.cta_start[blockIdx.x];
-  return blockIdx.x;
-}
-template <bool BATCH, bool SPLIT>
-__device__ __forceinline__ int item_end(const FusedParams& p) {
-  if constexpr (BATCH) return p.cta_start[blockIdx.x + 1];
-  if constexpr (SPLIT) return p.num_own_tiles * p.split;
-  return p.num_own_tiles;
-}
-
-// An item of a single-market launch: own tile t and its partner tiles
-// [jb, je) (range s of p.split equal parts). Items are ordered tile by tile
-// (the ranges of one own tile on neighbouring CTAs), or with range_major
-// range by range, so that all CTAs stream one range of the partner matrix
-// (small enough to stay in L2) against every own tile before the next.
-struct Span {
-  int t, s, jb, je;
-};
-template <bool SPLIT>
-__device__ __forceinline__ Span single_span(const FusedParams& p, int it) {
-  if constexpr (!SPLIT) return {it, 0, 0, p.num_partner_tiles};
-  const int S = p.split;
-  int t, s;
-  if (p.range_major) {
-    s = it / p.num_own_tiles;
-    t = it - s * p.num_own_tiles;
-  } else {
-    t = it / S;
-    s = it - t * S;
-  }
-  const int npt = p.num_partner_tiles;
-  return {t, s, (int)((int64_t)s * npt / S), (int)((int64_t)(s + 1) * npt / S)};
-}
-template <bool BATCH>
-__device__ __forceinline__ int item_step() {
-  if constexpr (BATCH) return 1;
-  return gridDim.x;
-}
-
-// BATCH: the CTA's own tiles come from the launch's item list and may belong
-// to different markets (tensor maps, vectors and sizes from BatchDesc); the
-// residual partials are then written per own tile and epilogue warp instead
-// of per CTA.
-// KB: 128-byte k blocks per packed row (1, 2 or 4: BF16 kp = 64, 128, 256;
-// e4m3 kp = 128, 256, 512).
-// FMT: kFmtBF16, or e4m3 factors on tcgen05.mma kind::f8f6f4 with one scale
-// per side (kFmtE4M3Side: both folded into p.c) or per row (kFmtE4M3Rows: the
-// own row's scale is folded into the row's exponent multiplier, the partner
-// rows' scales multiply the accumulator entries in the epilogue).
-// SMALL: own tiles of 128 rows (one MMA chain; the epilogue warps of the
-// second sub-tile take part in every barrier but load and compute nothing),
-// for markets whose 256-row tiles would leave SMs idle: twice the CTAs, each
-// finishing its rows in about half the time. Every row's arithmetic is the
-// same as with 256-row tiles.
-template <int KB, int STAGES, int MODE, bool BATCH, int FMT, bool SMALL = false, bool SPLIT = false,
-          bool NOFOLD = false>
-__global__ void __launch_bounds__(kThreads, 1)
-    k_fused_halfsweep(const __grid_constant__ CUtensorMap tm_own, const __grid_constant__ CUtensorMap tm_partner,
-                      const FusedParams p) {
-  static_assert(!BATCH || MODE == kModeSweep, "batched launches run half-sweeps only");
-  static_assert(!SPLIT || ((MODE == kModeSweep || MODE == kModeMu) && !BATCH),
-                "partner splits are single-market half-sweeps and mu blocks");
-  constexpr bool kSweepLike = MODE == kModeSweep || MODE == kModeSweepWide;
-  static_assert(!(BATCH && SMALL), "batched launches use 256-row own tiles");
-  constexpr int kOwn = SMALL ? kFusedOwnRows / 2 : kFusedOwnRows;  // rows of an own tile
-  static_assert(KB == 1 || KB == 2 || KB == 4, "128-byte k blocks per row");
-  constexpr bool F8 = FMT != kFmtBF16;      // e4m3 operands
-  constexpr bool RS = FMT == kFmtE4M3Rows;  // per-row scales
-  constexpr int ABUF = kABufs<KB>;
-  constexpr int KBS = kbs_for(KB);   // k blocks per partner stage
-  constexpr int SPT = KB / KBS;      // stages per partner tile
-  constexpr int XB = F8 ? 128 : kKBlock;  // elements per 128-byte k block (TMA x coordinate step)
-  constexpr bool FOLD = fold_for(KB, MODE, BATCH, FMT, NOFOLD);  // g added by an extra MMA
-  constexpr int SB = stage_bytes(KB, FOLD);                        // bytes per partner stage
-  extern __shared__ uint8_t smem_raw[];
-  const uint32_t raw_u32 = smem_u32(smem_raw);
-  uint8_t* smem = smem_raw + (((raw_u32 + 1023u) & ~1023u) - raw_u32);
-  uint8_t* sA = smem;
-  uint8_t* sB = smem + ABUF * KB * kOwnBytesPerKB;
-  uint8_t* sOnes = sB + STAGES * SB;  // folded g: the own side's constant operand
-  float* sG = reinterpret_cast<float*>(sOnes + (FOLD ? kFoldBytes : 0));
-  float* sF = sG + kGSlots * kFusedPartnerRows;  // per-row scales: partner scale ring
-  uint64_t* bars =
-      reinterpret_cast<uint64_t*>(reinterpret_cast<uint8_t*>(sG) + kGSlots * kGBytes * (RS ? 2 : 1));
-  uint64_t* full = bars;
-  uint64_t* empty = bars + STAGES;
-  uint64_t* gfull = bars + 2 * STAGES;
-  uint64_t* gempty = gfull + kGSlots;
-  uint64_t* a_full = gempty + kGSlots;  // [2]
-  uint64_t* a_empty = a_full + 2;       // [2]
-  uint64_t* tfull = a_full + 4;         // [2]
-  uint64_t* tempty = a_full + 6;        // [2]
-  uint64_t* mma_done = a_full + 8;
-  uint64_t* rowfull = a_full + 9;   // [2] second column half of the rows written
-  uint64_t* rowfree = a_full + 11;  // [2] row hand-over buffer read
-  uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(a_full + 13);
-  volatile int* abort_flag = reinterpret_cast<volatile int*>(tmem_slot + 1);
-  double* red = reinterpret_cast<double*>(reinterpret_cast<uint8_t*>(bars) + 512);      // kEpiWarps x 4 doubles
-  float* rowbuf = reinterpret_cast<float*>(reinterpret_cast<uint8_t*>(bars) + 1024);   // 2 x 256 floats
-  // ranked lists in shared memory (kModeTopKShared only): after the tail area
-  float* topk_list = reinterpret_cast<float*>(reinterpret_cast<uint8_t*>(bars) + kTailBytes);
-  // the running shifts of the second column half's rows (kModeSweepWide only): the same place
-  float* wide_shift = topk_list;  // 2 x 256 floats
-  static_assert(4 * kEpiWarps * 8 <= 512, "reduction area");
-  static_assert((2 * STAGES + 2 * kGSlots + 13) * 8 + 8 <= 512, "barrier area");
-
-  const int warp = threadIdx.x / 32, lane = threadIdx.x % 32;
-
-  if (threadIdx.x == 0) {
-    for (int s = 0; s < STAGES; ++s) {
-      mbar_init(&full[s], 1);
-      mbar_init(&empty[s], 1);
-    }
-    for (int s = 0; s < kGSlots; ++s) {
-      mbar_init(&gfull[s], 1);
-      mbar_init(&gempty[s], kEpiWarps);
-    }
-    for (int b = 0; b < 2; ++b) {
-      mbar_init(&a_full[b], 1);
-      mbar_init(&a_empty[b], 1);
-    }
-    for (int b = 0; b < 2; ++b) {
-      mbar_init(&tfull[b], 1);
-      mbar_init(&tempty[b], kEpiWarps);
-    }
-    mbar_init(mma_done, 1);
-    for (int b = 0; b < 2; ++b) {
-      mbar_init(&rowfull[b], kEpiWarps / 2);
-      mbar_init(&rowfree[b], kEpiWarps / 2);
-    }
-    *abort_flag = 0;
-    fence_mbar_init();
-    if constexpr (!BATCH) {
-      tma_prefetch_map(&tm_own);
-      tma_prefetch_map(&tm_partner);
-    }
-  }
-  if (warp == 0) {
-    tmem_alloc(tmem_slot, kTmemCols);
-    tmem_relinquish();
-  }
-  if constexpr (FOLD) {
-    // the own side's operand of the extra MMA: BF16 ones in columns 0-2 of
-    // every row (16-byte chunk q holds columns 0-7 when (q / 8) is even),
-    // made visible to the tensor core's (async) proxy
-    if (threadIdx.x < kFoldBytes / 16) {
-      const bool cols0_7 = ((threadIdx.x / 8) % 2) == 0;
-      reinterpret_cast<uint4*>(sOnes)[threadIdx.x] =
-          cols0_7 ? make_uint4(0x3F803F80u, 0x00003F80u, 0u, 0u) : make_uint4(0u, 0u, 0u, 0u);
-    }
-    asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-  }
-  if constexpr (MODE == kModeTopKShared) {
-    // no published bound yet (tags start at 1; shared memory may hold another launch's words)
-    if (threadIdx.x >= 64)
-      sts_u64(smem_u32(topk_list) + (uint32_t)(kTopKSlots * kEpiThreads + (int)threadIdx.x - 64) * 8u, 0ull);
-  }
-  tc_fence_before();
-  __syncthreads();
-  tc_fence_after();
-  const uint32_t tmem_base = *tmem_slot;
-
-  if (warp == 0) {
-    // ------------------------------------------------------------ producer
-    if (lane == 0) {
-      int stage = 0, gs = 0, ab = 0;
-      uint32_t phase = 0, gphase = 0, a_phase = 0;
-      const bool hint = !BATCH && p.l2_keep > 0.0f;
-      const uint64_t keep_policy = hint ? l2_policy_keep_fraction(p.l2_keep) : 0ull;
-      uint32_t armed[STAGES], garmed[kGSlots], a_armed[2] = {0u, 0u};
-      for (int s = 0; s < STAGES; ++s) armed[s] = 0;
-      for (int s = 0; s < kGSlots; ++s) garmed[s] = 0;
-      const BatchDesc* prev = nullptr;
-      bool ok = true;
-      for (int it = item_begin<BATCH>(p); it < item_end<BATCH, SPLIT>(p) && ok; it += item_step<BATCH>()) {
-        const BatchDesc* bd = nullptr;
-        int t, jb = 0, je;
-        if constexpr (BATCH) {
-          const ItemRef w = batch_item(p, it);
-          bd = w.d;
-          t = w.t;
-          je = bd->num_partner_tiles;
-          if (bd != prev) {
-            tensormap_acquire(&bd->tm_own);
-            tensormap_acquire(&bd->tm_partner);
-            prev = bd;
-          }
-        } else {
-          const Span sp = single_span<SPLIT>(p, it);
-          t = sp.t;
-          jb = sp.jb;
-          je = sp.je;
-        }
-        const CUtensorMap* map_own = BATCH ? &bd->tm_own : &tm_own;
-        const CUtensorMap* map_partner = BATCH ? &bd->tm_partner : &tm_partner;
-        const float* gsrc = BATCH ? bd->g : p.g + p.col0;
-        const float* fsrc = BATCH ? bd->fs_par : p.fs_par + p.col0;
-        // (SMALL: the 256-row box also brings the next tile's rows, unused)
-        const int64_t arow = BATCH ? (int64_t)t * kFusedOwnRows : p.row0 + (int64_t)t * kOwn;
-        if (!mbar_wait(&a_empty[ab], a_phase ^ 1u, abort_flag)) {
-          ok = false;
-          break;
-        }
-        mbar_arrive_expect_tx(&a_full[ab], KB * kOwnBytesPerKB);
-        for (int kb = 0; kb < KB; ++kb)
-          tma_load_2d(sA + (ab * KB + kb) * kOwnBytesPerKB, map_own, &a_full[ab], kb * XB, (int)arow);
-        ++a_armed[ab];
-        if (++ab == ABUF) {
-          ab = 0;
-          a_phase ^= 1u;
-        }
-        for (int j = jb; j < je && ok; ++j) {
-          for (int sp = 0; sp < SPT; ++sp) {
-            if (!mbar_wait(&empty[stage], phase ^ 1u, abort_flag)) {
-              ok = false;
-              break;
-            }
-            const bool fold_here = FOLD && sp == SPT - 1;  // the tile's g operand rides in its last stage
-            mbar_arrive_expect_tx(&full[stage], KBS * kPartnerBytesPerKB + (fold_here ? kFoldBytes : 0));
-            for (int kb = 0; kb < KBS; ++kb) {
-              const int px = (sp * KBS + kb) * XB, py = (int)(p.col0 + (int64_t)j * kFusedPartnerRows);
-              if (hint) {
-                tma_load_2d_hint(sB + stage * SB + kb * kPartnerBytesPerKB, map_partner, &full[stage], px, py,
-                                 keep_policy);
-              } else {
-                tma_load_2d(sB + stage * SB + kb * kPartnerBytesPerKB, map_partner, &full[stage], px, py);
-              }
-            }
-            if (fold_here)
-              bulk_load(sB + stage * SB + KBS * kPartnerBytesPerKB,
-                        (BATCH ? bd->gfold : p.gfold) + (int64_t)j * kFoldBytes, kFoldBytes, &full[stage]);
-            ++armed[stage];
-            if (++stage == STAGES) {
-              stage = 0;
-              phase ^= 1u;
-            }
-          }
-          if (!ok) break;
-          if (!mbar_wait(&gempty[gs], gphase ^ 1u, abort_flag)) {
-            ok = false;
-            break;
-          }
-          mbar_arrive_expect_tx(&gfull[gs], RS ? 2 * kGBytes : kGBytes);
-          bulk_load(sG + gs * kFusedPartnerRows, gsrc + (int64_t)j * kFusedPartnerRows, kGBytes, &gfull[gs]);
-          if constexpr (RS)
-            bulk_load(sF + gs * kFusedPartnerRows, fsrc + (int64_t)j * kFusedPartnerRows, kGBytes, &gfull[gs]);
-          ++garmed[gs];
-          if (++gs == kGSlots) {
-            gs = 0;
-            gphase ^= 1u;
-          }
-        }
-      }
-      if (!ok) {
-        if (!*abort_flag) raise_error(p.err, abort_flag, kErrTimeout);
-        // let the copies already issued land before the CTA's shared memory goes away
-        for (int s = 0; s < STAGES; ++s)
-          if (armed[s]) mbar_wait_drain(&full[s], (armed[s] - 1u) & 1u, 10000000ull);
-        for (int s = 0; s < kGSlots; ++s)
-          if (garmed[s]) mbar_wait_drain(&gfull[s], (garmed[s] - 1u) & 1u, 10000000ull);
-        for (int b = 0; b < ABUF; ++b)
-          if (a_armed[b]) mbar_wait_drain(&a_full[b], (a_armed[b] - 1u) & 1u, 10000000ull);
-      }
-    }
-    __syncwarp();
-  } else if (warp == 1) {
-    // ------------------------------------------------------------ MMA issuer
-    if (lane == 0) {
-      constexpr uint32_t idesc = F8 ? idesc_e4m3_f32(128, kFusedPartnerRows) : idesc_bf16_f32(128, kFusedPartnerRows);
-      constexpr uint32_t idesc_fold = idesc_bf16_f32(128, kFusedPartnerRows);  // (BF16 in every format)
-      int stage = 0, buf = 0, ab = 0;
-      uint32_t phase = 0, tphase = 0, a_phase = 0;
-      bool ok = true;
-      for (int it = item_begin<BATCH>(p); it < item_end<BATCH, SPLIT>(p) && ok; it += item_step<BATCH>()) {
-        int jb = 0, je;
-        if constexpr (BATCH) {
-          je = batch_item(p, it).d->num_partner_tiles;
-        } else {
-          const Span sp = single_span<SPLIT>(p, it);
-          jb = sp.jb;
-          je = sp.je;
-        }
-        if (!mbar_wait(&a_full[ab], a_phase, abort_flag)) {
-          ok = false;
-          break;
-        }
-        tc_fence_after();
-        const uint32_t a0 = smem_u32(sA + ab * KB * kOwnBytesPerKB);
-        uint64_t* a_release = &a_empty[ab];
-        if (++ab == ABUF) {
-          ab = 0;
-          a_phase ^= 1u;
-        }
-        for (int j = jb; j < je && ok; ++j) {
-          if (!mbar_wait(&tempty[buf], tphase ^ 1u, abort_flag)) {
-            ok = false;
-            break;
-          }
-          for (int sp = 0; sp < SPT; ++sp) {
-            if (!mbar_wait(&full[stage], phase, abort_flag)) {
-              ok = false;
-              break;
-            }
-            tc_fence_after();
-            const uint32_t b0 = smem_u32(sB + stage * SB);
-#pragma unroll
-            for (int h = 0; h < (SMALL ? 1 : 2); ++h) {
-              const uint32_t d_tmem = tmem_base + (uint32_t)(buf * 256 + h * 128);
-#pragma unroll
-              for (int k = 0; k < KBS * 4; ++k) {
-                const int kbl = k >> 2, kk = k & 3;
-                const int kb = sp * KBS + kbl;  // k block within the packed row
-                const uint64_t adesc = sdesc_sw128(a0 + kb * kOwnBytesPerKB + h * 128 * 128 + kk * 32);
-                const uint64_t bdesc = sdesc_sw128(b0 + kbl * kPartnerBytesPerKB + kk * 32);
-                const uint32_t accum = (sp > 0 || k > 0) ? 1u : 0u;
-                if constexpr (F8) {
-                  umma_e4m3(d_tmem, adesc, bdesc, idesc, accum);
-                } else {
-                  umma_bf16(d_tmem, adesc, bdesc, idesc, accum);
-                }
-              }
-              if constexpr (FOLD) {
-                // D += ones x (g / c): every row gets the partner column's g / c
-                if (sp == SPT - 1)
-                  umma_bf16(d_tmem, sdesc_none(smem_u32(sOnes), 128, 256),
-                            sdesc_none(b0 + KBS * kPartnerBytesPerKB, 128, 256), idesc_fold, 1u);
-              }
-            }
-            umma_commit(&empty[stage]);
-            if (++stage == STAGES) {
-              stage = 0;
-              phase ^= 1u;
-            }
-          }
-          if (!ok) break;
-          umma_commit(&tfull[buf]);
-          if (j == je - 1) umma_commit(a_release);
-          buf ^= 1;
-          if (buf == 0) tphase ^= 1u;
-        }
-      }
-      if (!ok && !*abort_flag) raise_error(p.err, abort_flag, kErrTimeout);
-      // all MMAs issued by this thread complete before TMEM is released
-      umma_commit(mma_done);
-      mbar_wait_drain(mma_done, 0, 100000000ull);
-    }
-    __syncwarp();
-  } else {
-    // ------------------------------------------------------------ epilogue
-    const int ew = warp - 2;          // 0..15
-    const int q = warp & 3;           // TMEM lane quadrant this warp may access
-    const int h = (ew >> 2) & 1;      // own sub-tile: rows [h*128, h*128+128)
-    const int half = ew >> 3;         // columns [half*64, half*64+64) of every partner tile
-    uint64_t cc = 0ull;
-    float crow = p.c;  // this thread's row's exponent multiplier (e4m3: times the row's scale)
-    // single market: the shift, own offset and omega of the launch (batched: per item)
-    const double shift0 = BATCH ? 0.0 : __ldg(p.lmax);
-    // (ranked lists and mu blocks run on potentials without pending offsets:
-    // every block of sweeps ends by writing them into the arrays)
-    const double own_off0 = (kSweepLike && !BATCH && p.own_off != nullptr) ? *p.own_off : 0.0;
-    const double omega0 = (!BATCH && p.omega != nullptr && p.update) ? *p.omega : 1.0;
-    int buf = 0, gs = 0;
-    uint32_t tphase = 0, gphase = 0;
-    bool ok = true;
-    if constexpr (kSweepLike && !BATCH) {
-      // this warp's partials over its own tiles, in shared memory: carried in
-      // registers they would stay live across the tile loop
-      if (lane == 0) *reinterpret_cast<RowPartials*>(red + 4 * ew) = RowPartials{0.0, 0.0, 0.0, 0.0};
-    }
-    uint32_t va[32], vb[32];
-    // ranked lists: this thread's sorted candidates for its row and column half
-    float tv[MODE == kModeTopK ? kMaxTopK : 1];
-    int32_t ti[MODE == kModeTopK ? kMaxTopK : 1];
-    // shared-memory lists (k <= kSharedTopK): this thread's entry 0
-    const uint32_t lv = smem_u32(topk_list) + (uint32_t)(ew * 32 + lane) * 8u;
-    SharedBound sb{};
-    {
-      // (rows' other column half: epilogue warp ew ^ 8)
-      const uint32_t words = smem_u32(topk_list) + (uint32_t)(kTopKSlots * kEpiThreads) * 8u;
-      sb.mine = words + (uint32_t)(ew * 32 + lane) * 8u;
-      sb.other = words + (uint32_t)((ew ^ 8) * 32 + lane) * 8u;
-    }
-    int tcnt = 0;
-    int merge_at = 0;  // the partner tile before which every warp merges its candidates
-    float thr = -INFINITY;
-    int tile_iter = 0;
-    for (int it = item_begin<BATCH>(p); it < item_end<BATCH, SPLIT>(p) && ok; it += item_step<BATCH>(), ++tile_iter) {
-      const BatchDesc* bd = nullptr;
-      int t, split_s = 0, jb = 0, je;
-      if constexpr (BATCH) {
-        const ItemRef w = batch_item(p, it);
-        bd = w.d;
-        t = w.t;
-        je = bd->num_partner_tiles;
-      } else {
-        const Span sp = single_span<SPLIT>(p, it);
-        t = sp.t;
-        split_s = sp.s;
-        jb = sp.jb;
-        je = sp.je;
-      }
-      const double shift = BATCH ? bd->st[kStShift] : shift0;
-      const int rloc = h * 128 + q * 32 + lane;          // row within the own tile
-      const int64_t r = (int64_t)t * kOwn + rloc;         // row within the launch
-      const bool row_ok = rloc < kOwn && r < (BATCH ? bd->rows : p.rows);
-      crow = BATCH ? bd->c : p.c;
-      if constexpr (RS) {
-        const float* fso = BATCH ? bd->fs_own : p.fs_own;
-        if (row_ok) crow *= fso[(BATCH ? 0 : p.row0) + r];
-      }
-      {
-        const uint32_t cb = __float_as_uint(crow);
-        cc = ((uint64_t)cb << 32) | cb;
-      }
-      float sum = 0.0f, comp = 0.0f;
-      float mu_lo = 0.0f;
-      int mu_hi = 0;
-      float mu_s1 = 1.0f, mu_s2 = 1.0f;
-      // mu blocks: this warp's first row of the block, and how many it has there
-      const int64_t mu_row = (int64_t)t * kOwn + h * 128 + q * 32;
-      const int mu_nrow = MODE == kModeMu ? (int)(p.rows - mu_row < 32 ? p.rows - mu_row : 32) : 0;
-      float wide_m = -INFINITY;  // wide markets: the row's running shift (an integer, log2 units)
-      if constexpr (MODE == kModeMu) {
-        if (row_ok) {
-          const double off = (shift + p.ell[p.row0 + r]) * 1.4426950408889634;
-          const double fl = floor(off);
-          mu_hi = (int)fl;
-          mu_lo = (float)(off - fl);
-          const int e = mu_hi < -252 ? -252 : (mu_hi > 252 ? 252 : mu_hi);
-          mu_s1 = __int_as_float((127 + e / 2) << 23);
-          mu_s2 = __int_as_float((127 + e - e / 2) << 23);
-        }
-      }
-      if constexpr (MODE == kModeTopK) {
-        tcnt = 0;
-        thr = -INFINITY;
-      }
-      if constexpr (MODE == kModeTopKShared) {
-        for (int i = 0; i < p.k; ++i) sts_u64(lv + (uint32_t)i * kSlotStride, slot_of(-INFINITY, 0x7fffffff));
-        thr = -INFINITY;
-        tcnt = 0;
-        merge_at = jb + 1;
-        sb.tag = (uint32_t)tile_iter + 1u;
-        sb.pub = -INFINITY;
-        sts_u64(sb.mine, ((uint64_t)sb.tag << 32) | __float_as_uint(-INFINITY));
-      }
-      for (int j = jb; j < je; ++j) {
-        // every lane waits; the outcome is made warp-uniform so that the
-        // .sync.aligned TMEM loads below never run with a partial warp
-        const bool got = mbar_wait(&tfull[buf], tphase, abort_flag) && mbar_wait(&gfull[gs], gphase, abort_flag);
-        if (!__all_sync(0xffffffffu, got)) {
-          ok = false;
-          break;
-        }
-        tc_fence_after();
-        const uint32_t taddr =
-            tmem_base + ((uint32_t)(q * 32) << 16) + (uint32_t)(buf * 256 + h * 128 + half * 64);
-        const float* gsf = sG + gs * kFusedPartnerRows + half * 64;
-        const float4* gs4 = reinterpret_cast<const float4*>(gsf);
-        const float* fsf = sF + gs * kFusedPartnerRows + half * 64;  // (per-row scales only)
-        const float4* fs4 = reinterpret_cast<const float4*>(fsf);
-        const int64_t colbase = p.col0 + (int64_t)j * kFusedPartnerRows + half * 64;
-        uint64_t acc[4] = {0ull, 0ull, 0ull, 0ull};
-        // SMALL: the second sub-tile's warps keep step with the barriers only
-        const bool idle = SMALL && h == 1;
-        if (!idle) {
-          // the second 32-column chunk is loaded while the first is processed
-          tmem_ld_issue(taddr, va);
-          tmem_ld_wait(va);
-          tmem_ld_issue(taddr + 32, vb);
-          if constexpr (FOLD) chunk_sum_fold(va, cc, acc);
-          if constexpr (MODE == kModeSweep && !FOLD) chunk_sum<RS>(va, gs4, fs4, cc, acc);
-          if constexpr (MODE == kModeSweepWide) chunk_sum_wide<RS>(va, gs4, fs4, cc, acc, wide_m, sum, comp);
-          if constexpr (MODE == kModeTopK) chunk_topk<RS>(va, gsf, fsf, crow, colbase, p.k, tv, ti, &tcnt, thr);
-          if constexpr (MODE == kModeTopKShared)
-            chunk_topk_shared<RS>(va, gsf, fsf, cc, colbase, p.k, lv, tcnt, thr, sb);
-          if constexpr (MODE == kModeMu)
-            chunk_mu<RS, mu_width(KB)>(va, gsf, fsf, crow, colbase, mu_lo, mu_hi, mu_s1, mu_s2, lane, mu_nrow, mu_row,
-                         topk_list + ew * mu_stage_floats(KB), p);
-          tmem_ld_wait(vb);
-        }
-        // this warp's part of the accumulator buffer has been read: hand it back to the MMA warp
-        tc_fence_before();
-        __syncwarp();
-        if (lane == 0) mbar_arrive(&tempty[buf]);
-        if (!idle) {
-          if constexpr (FOLD) chunk_sum_fold(vb, cc, acc);
-          if constexpr (MODE == kModeSweep && !FOLD) chunk_sum<RS>(vb, gs4 + 8, fs4 + 8, cc, acc);
-          if constexpr (MODE == kModeSweepWide) chunk_sum_wide<RS>(vb, gs4 + 8, fs4 + 8, cc, acc, wide_m, sum, comp);
-          if constexpr (MODE == kModeTopK)
-            chunk_topk<RS>(vb, gsf + 32, fsf + 32, crow, colbase + 32, p.k, tv, ti, &tcnt, thr);
-          if constexpr (MODE == kModeTopKShared)
-            chunk_topk_shared<RS>(vb, gsf + 32, fsf + 32, cc, colbase + 32, p.k, lv, tcnt, thr, sb);
-          if constexpr (MODE == kModeMu)
-            chunk_mu<RS, mu_width(KB)>(vb, gsf + 32, fsf + 32, crow, colbase + 32, mu_lo, mu_hi, mu_s1, mu_s2, lane, mu_nrow,
-                         mu_row, topk_list + ew * mu_stage_floats(KB), p);
-        }
-        // the g slot has been read by this warp
-        __syncwarp();
-        if (lane == 0) mbar_arrive(&gempty[gs]);
-        if constexpr (kSweepLike) {
-          // compensated (Kahan) accumulation of the per-tile partial sums
-          const float tile =
-              (unpack_sum(acc[0]) + unpack_sum(acc[1])) + (unpack_sum(acc[2]) + unpack_sum(acc[3]));
-          const float y = tile - comp;
-          const float tsum = sum + y;
-          comp = (tsum - sum) - y;
-          sum = tsum;
-        }
-        if constexpr (MODE == kModeTopKShared) {
-          // All warps merge after the same tiles, each a quarter further into
-          // the row: a merge takes some thousand cycles, and the accumulator
-          // buffers let a warp run two tiles ahead of the slowest, so merges
-          // at different tiles would hold up the whole CTA one after another.
-          if (j + 1 == merge_at) {
-            merge_at += 1 + (merge_at - jb) / 4;
-            if (!idle) {
-              thr = list_merge(lv, p.k, tcnt);
-              sb.publish(lv, p.k);
-              tcnt = 0;
-            }
-          }
-        }
-        buf ^= 1;
-        if (buf == 0) tphase ^= 1u;
-        if (++gs == kGSlots) {
-          gs = 0;
-          gphase ^= 1u;
-        }
-      }
-      if (!ok) break;
-      if constexpr (MODE == kModeMu) continue;
-      if constexpr (MODE == kModeTopKShared) {
-        if (!(SMALL && h == 1)) list_merge(lv, p.k, tcnt);
-      }
-      // the two column halves of a row meet (double-buffered by own-tile
-      // parity, handed over through bounded mbarrier waits)
-      const int pb = tile_iter & 1;
-      const uint32_t rphase = (uint32_t)(tile_iter >> 1) & 1u;
-      float* rb = rowbuf + pb * kFusedOwnRows;
-      if (half == 1) {
-        if (!__all_sync(0xffffffffu, mbar_wait(&rowfree[pb], rphase ^ 1u, abort_flag))) {
-          ok = false;
-          break;
-        }
-        if constexpr (kSweepLike) rb[rloc] = sum - comp;
-        if constexpr (MODE == kModeSweepWide) wide_shift[pb * kFusedOwnRows + rloc] = wide_m;
-        if constexpr (MODE == kModeTopK) {
-          if (row_ok)
-            for (int i = 0; i < p.k; ++i) {
-              p.hand_v[r * p.k + i] = i < tcnt ? tv[i] : -INFINITY;
-              p.hand_i[r * p.k + i] = i < tcnt ? ti[i] : 0x7fffffff;
-            }
-        }
-        if constexpr (MODE == kModeTopKShared) {
-          if (row_ok)
-            for (int i = 0; i < p.k; ++i) {
-              const uint64_t w = lds_u64(lv + (uint32_t)i * kSlotStride);
-              p.hand_v[r * p.k + i] = slot_score(w);
-              p.hand_i[r * p.k + i] = slot_col(w);
-            }
-        }
-        __syncwarp();
-        if (lane == 0) mbar_arrive(&rowfull[pb]);
-        continue;
-      }
-      if (!__all_sync(0xffffffffu, mbar_wait(&rowfull[pb], rphase, abort_flag))) {
-        ok = false;
-        break;
-      }
-      if constexpr (MODE == kModeTopK) {
-        if (row_ok) {
-          // merge the two sorted halves: higher score first, lower index on ties
-          const double base = shift + p.ell[p.row0 + r];
-          int a = 0, b = 0;
-          for (int i = 0; i < p.k; ++i) {
-            const float bv = p.hand_v[r * p.k + b];
-            const int32_t bi = p.hand_i[r * p.k + b];
-            const bool take_a = a < tcnt && (b >= p.k || tv[a] > bv || (tv[a] == bv && ti[a] < bi));
-            const float sv = take_a ? tv[a] : bv;
-            p.idx[r * p.k + i] = take_a ? ti[a] : bi;
-            if (p.logmu != nullptr) p.logmu[r * p.k + i] = (float)((double)sv * 0.69314718055994530942 + base);
-            if (take_a) ++a; else ++b;
-          }
-        }
-        __syncwarp();
-        if (lane == 0) mbar_arrive(&rowfree[pb]);
-      }
-      if constexpr (MODE == kModeTopKShared) {
-        if (row_ok) {
-          // merge the two sorted halves (both exactly k entries, padded with
-          // (-inf, INT32_MAX)): higher score first, lower index on ties
-          const double base = shift + p.ell[p.row0 + r];
-          int a = 0, b = 0;
-          for (int i = 0; i < p.k; ++i) {
-            const uint64_t w = lds_u64(lv + (uint32_t)a * kSlotStride);
-            const float av = slot_score(w);
-            const int32_t ai = slot_col(w);
-            const float bv = p.hand_v[r * p.k + b];
-            const int32_t bi = p.hand_i[r * p.k + b];
-            const bool take_a = av > bv || (av == bv && ai < bi);
-            const float sv = take_a ? av : bv;
-            p.idx[r * p.k + i] = take_a ? ai : bi;
-            if (p.logmu != nullptr) p.logmu[r * p.k + i] = (float)((double)sv * 0.69314718055994530942 + base);
-            if (take_a) ++a; else ++b;
-          }
-        }
-        __syncwarp();
-        if (lane == 0) mbar_arrive(&rowfree[pb]);
-      }
-      if constexpr (kSweepLike) {
-        float other = rb[rloc];
-        float row_m = 0.0f;  // wide markets: the shift of the row's sum (log2 units)
-        if constexpr (MODE == kModeSweepWide) {
-          // the two halves' sums onto the larger of their shifts (exact powers of two)
-          const float other_m = wide_shift[pb * kFusedOwnRows + rloc];
-          row_m = fmaxf(wide_m, other_m);
-          const float own_scale = exp2_int(wide_m - row_m);
-          sum *= own_scale;
-          comp *= own_scale;
-          other *= exp2_int(other_m - row_m);
-        }
-        __syncwarp();
-        if (lane == 0) mbar_arrive(&rowfree[pb]);
-        const int64_t row = p.row0 + r;
-        // the row's sum as three FP32 parts (a split: summed over its ranges)
-        float s_hi = sum, s_lo = -comp, s_o = other;
-        if constexpr (SPLIT) {
-          {
-            // this range's partial; the warp that completes the (tile, 32-row
-            // block) sums all ranges in order and updates the rows (no wait:
-            // the other warps of this block move on)
-            const int64_t blk = (int64_t)t * (kFusedOwnRows / 32) + (h * 128 + q * 32) / 32;
-            if (row_ok) p.part[(int64_t)split_s * p.rows + r] = make_float4(sum, -comp, other, 0.0f);
-            __threadfence();
-            __syncwarp();
-            int prev = 0;
-            if (lane == 0) prev = atomicAdd(p.split_cnt + blk, 1);
-            prev = __shfl_sync(0xffffffffu, prev, 0);
-            if (prev != p.split - 1) continue;
-            if (lane == 0) p.split_cnt[blk] = 0;  // ready for the next launch
-            __threadfence();
-            s_hi = s_lo = s_o = 0.0f;
-            if (row_ok)
-              for (int qs = 0; qs < p.split; ++qs) {
-                const float4 v = __ldcg(p.part + (int64_t)qs * p.rows + r);
-                float e1, e2, e3;
-                s_hi = two_sum(s_hi, v.x, e1);
-                s_hi = two_sum(s_hi, v.y, e2);
-                s_hi = two_sum(s_hi, v.z, e3);
-                s_lo = __fadd_rn(s_lo, __fadd_rn(e1, __fadd_rn(e2, e3)));
-              }
-          }
-        }
-        RowResult rr{};
-        if (row_ok) {
-          const float* b2s = BATCH ? bd->b2s : p.b2s;
-          double* log_u = BATCH ? bd->log_u : p.log_u;
-          double* ell = BATCH ? bd->ell : p.ell;
-          const double omega = BATCH ? ((bd->omega != nullptr && p.update) ? *bd->omega : 1.0) : omega0;
-          const double own_off = BATCH ? bd->st[kStOwnOff] : own_off0;
-          int ex;
-          const float lm = log_row_sum_parts(s_hi, s_lo, s_o, ex);
-          // wide markets: the row's shift comes back into the sum's logarithm
-          // (no finite exponent: the sum is 0 and its logarithm -inf whatever is added)
-          if constexpr (MODE == kModeSweepWide) ex += row_m > -1e9f ? (int)row_m : 0;
-          rr = row_update(ex, lm, shift, b2s ? b2s[row] : 0.0f, (BATCH ? bd->mass : p.mass)[row],
-                          log_u[row] + own_off, p.residual, omega);
-          if (p.update) {
-            log_u[row] = rr.log_u;
-            ell[row] = rr.ell;
-          }
-        }
-        // this warp's 32 rows form one group of the own side (the finalize
-        // reduces the groups into the side's shift and sum of u^2)
-        float4* grp = BATCH ? bd->grp : p.grp;
-        const int64_t g = (int64_t)t * (kOwn / kGroupRows) + (h * 128 + q * 32) / kGroupRows;
-        if (SMALL && h == 1) continue;  // (no rows)
-        if (p.update && grp != nullptr && g * kGroupRows < (BATCH ? bd->rows : p.rows)) {
-          const float4 gv = warp_group(rr.log_u, rr.ell, row_ok);
-          if (lane == 0) grp[g] = gv;
-        }
-        const RowPartials rp = row_partials(rr, row_ok, p.residual);
-        if (lane == 0) {
-          if constexpr (BATCH) {
-            // partials of this own tile and warp (warps ew = 0..7 own the row
-            // updates); the batched finalize sums them per market in a fixed order
-            *reinterpret_cast<RowPartials*>(p.partials + ((int64_t)(bd->slot0 + t) * kBatchSlotWarps + ew) * 4) = rp;
-          } else {
-            add_partials(*reinterpret_cast<RowPartials*>(red + 4 * ew), rp);
-          }
-        }
-      }
-    }
-    if (!ok && !*abort_flag) raise_error(p.err, abort_flag, kErrTimeout);
-    if constexpr (kSweepLike && !BATCH) {
-      // the CTA's partials: those of the warps that own the row updates
-      named_bar_sync(1, kEpiWarps * 32);
-      if (ew == 0 && lane < 8) {
-        RowPartials v = *reinterpret_cast<const RowPartials*>(red + 4 * lane);
-        for (int o = 4; o > 0; o >>= 1) {
-          const RowPartials w = {__shfl_xor_sync(0xffu, v.r_max, o), __shfl_xor_sync(0xffu, v.r_sum, o),
-                                 __shfl_xor_sync(0xffu, v.sq, o), __shfl_xor_sync(0xffu, v.nf, o)};
-          add_partials(v, w);
-        }
-        if (lane == 0) *reinterpret_cast<RowPartials*>(p.partials + 4 * blockIdx.x) = v;
-      }
-    }
-  }
-
-  tc_fence_before();
-  __syncthreads();
-  if (warp == 0) {
-    tc_fence_after();
-    tmem_dealloc(tmem_base, kTmemCols);
-  }
-}
-
-// ---------------------------------------------------------------------------
-// Host side
-// ---------------------------------------------------------------------------
 
 typedef CUresult (*EncodeTiledFn)(CUtensorMap*, CUtensorMapDataType, cuuint32_t, void*, const cuuint64_t*,
                                   const cuuint64_t*, const cuuint32_t*, const cuuint32_t*, CUtensorMapInterleave,
@@ -1444,107 +45,11 @@ cudaError_t make_map(CUtensorMap* map, const void* base, int64_t rows, int64_t k
   return r == CUDA_SUCCESS ? cudaSuccess : cudaErrorInvalidValue;
 }
 
-constexpr int kSmemLimit = 232448;  // dynamic shared memory per CTA (227 KB)
-
-// Partner stages per instantiation: as many as fit beside the own tile(s), the
-// g (and scale) rings, the tail and (kModeTopKShared) the ranked lists, at
-// most 6 whole tiles (one k block per row), 4 (two) or 5 single k blocks
-// (four: 1.25 partner tiles in flight).
-constexpr int stages_for(int KB, int MODE, int fmt, bool fold) {
-  const int fixed = smem_bytes(KB, fmt, 0, fold) + mode_extra_bytes(MODE, KB);
-  const int fit = (kSmemLimit - fixed) / stage_bytes(KB, fold);
-  const int cap = KB == 1 ? 6 : (KB == 2 ? 4 : 5);
-  return fit < cap ? fit : cap;
-}
-
-template <int KB, int MODE, int FMT, bool FOLD>
-constexpr int kStages = stages_for(KB, MODE, FMT, FOLD);
-
-template <int KB, int MODE, int FMT, bool FOLD>
-constexpr int kSmemTotal =
-    smem_bytes(KB, FMT, kStages<KB, MODE, FMT, FOLD>, FOLD) + mode_extra_bytes(MODE, KB);
-
-// Instantiations that exist: batched launches take one or two k blocks
-// (e4m3: one); the shared-memory ranked lists leave too little room for
-// partner stages beside a four-block own tile (those lists use kModeTopK).
-// SPLIT: the partner-split instantiation (single-market half-sweeps with
-// tu_market_set_split > 1); the default kernel carries none of its code.
-// NOFOLD: the BF16 half-sweep with g from the shared ring instead of the
-// extra MMA, for callers without the folded operand (the allocation-free
-// entry point).
-template <int KB, int MODE, bool BATCH, int FMT, bool SPLIT = false, bool SMALL = false, bool NOFOLD = false>
-constexpr bool kBuilt = !(BATCH && (KB == 4 || (FMT != kFmtBF16 && KB != 1))) &&
-                        !(MODE == kModeTopKShared && KB == 4) && !(SPLIT && MODE != kModeSweep && MODE != kModeMu) &&
-                        !(SPLIT && BATCH) && !(MODE == kModeMu && (!SPLIT || SMALL)) &&
-                        !(NOFOLD && (!fold_for(KB, MODE, BATCH, FMT, false) || SPLIT || SMALL));
-
-template <int KB, int MODE, bool BATCH, int FMT = kFmtBF16, bool SMALL = false, bool SPLIT = false,
-          bool NOFOLD = false>
-cudaError_t launch_kernel(const CUtensorMap& own, const CUtensorMap& partner, const FusedParams& p, int grid,
-                          cudaStream_t stream) {
-  if constexpr (!kBuilt<KB, MODE, BATCH, FMT, SPLIT, SMALL, NOFOLD>) {
-    return cudaErrorNotSupported;
-  } else {
-    constexpr bool FD = fold_for(KB, MODE, BATCH, FMT, NOFOLD);
-    static_assert(kStages<KB, MODE, FMT, FD> >= 2, "at least two partner stages");
-    static_assert(kSmemTotal<KB, MODE, FMT, FD> <= kSmemLimit, "shared memory budget");
-    if (FD && !BATCH && p.gfold == nullptr) return cudaErrorInvalidValue;  // the folded operand must be prepared
-    k_fused_halfsweep<KB, kStages<KB, MODE, FMT, FD>, MODE, BATCH, FMT, SMALL, SPLIT, NOFOLD>
-        <<<grid, kThreads, kSmemTotal<KB, MODE, FMT, FD>, stream>>>(own, partner, p);
-    return cudaGetLastError();
-  }
-}
-
-template <int KB, int MODE, bool BATCH, int FMT, bool SMALL, bool SPLIT = false, bool NOFOLD = false>
-cudaError_t set_attribute_one() {
-  if constexpr (!kBuilt<KB, MODE, BATCH, FMT, SPLIT, SMALL, NOFOLD>) {
-    return cudaSuccess;
-  } else {
-    constexpr bool FD = fold_for(KB, MODE, BATCH, FMT, NOFOLD);
-    return cudaFuncSetAttribute(
-        k_fused_halfsweep<KB, kStages<KB, MODE, FMT, FD>, MODE, BATCH, FMT, SMALL, SPLIT, NOFOLD>,
-        cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemTotal<KB, MODE, FMT, FD>);
-  }
-}
-
-template <int MODE, bool BATCH, bool SMALL, int FMT, bool SPLIT = false>
-cudaError_t set_attributes_fmt() {
-  cudaError_t e = set_attribute_one<1, MODE, BATCH, FMT, SMALL, SPLIT>();
-  if (e == cudaSuccess) e = set_attribute_one<2, MODE, BATCH, FMT, SMALL, SPLIT>();
-  if (e == cudaSuccess) e = set_attribute_one<4, MODE, BATCH, FMT, SMALL, SPLIT>();
-  return e;
-}
-
-template <int MODE, bool BATCH, bool SMALL, bool SPLIT = false>
-cudaError_t set_attributes_variant() {
-  cudaError_t e = set_attributes_fmt<MODE, BATCH, SMALL, kFmtBF16, SPLIT>();
-  if (e == cudaSuccess) e = set_attributes_fmt<MODE, BATCH, SMALL, kFmtE4M3Side, SPLIT>();
-  if (e == cudaSuccess) e = set_attributes_fmt<MODE, BATCH, SMALL, kFmtE4M3Rows, SPLIT>();
-  return e;
-}
-
-template <int MODE, bool BATCH>
-cudaError_t set_attributes_mode() {
-  cudaError_t e = set_attributes_variant<MODE, BATCH, false>();
-  if (e == cudaSuccess && !BATCH) e = set_attributes_variant<MODE, false, true>();
-  if (MODE == kModeMu) {
-    if (e == cudaSuccess) e = set_attributes_variant<MODE, false, false, true>();
-  }
-  if (MODE == kModeSweep && !BATCH) {
-    if (e == cudaSuccess) e = set_attributes_variant<MODE, false, false, true>();
-    if (e == cudaSuccess) e = set_attributes_variant<MODE, false, true, true>();
-  }
-  return e;
-}
-
 // Dynamic shared memory opt-in of every instantiation, on the current device.
 cudaError_t set_kernel_attributes_now() {
   cudaError_t e = set_attributes_mode<kModeSweep, false>();
-  if (e == cudaSuccess) e = set_attributes_mode<kModeTopK, false>();
-  if (e == cudaSuccess) e = set_attributes_mode<kModeMu, false>();
-  if (e == cudaSuccess) e = set_attributes_mode<kModeTopKShared, false>();
   if (e == cudaSuccess) e = set_attributes_mode<kModeSweep, true>();
-  if (e == cudaSuccess) e = set_attributes_mode<kModeSweepWide, false>();
+  if (e == cudaSuccess) e = set_out_attributes();
   // the allocation-free entry point's unfolded half-sweep (rows of one k block)
   if (e == cudaSuccess) e = set_attribute_one<1, kModeSweep, false, kFmtBF16, false, false, true>();
   return e;
@@ -1567,48 +72,9 @@ cudaError_t set_kernel_attributes() {
   return e;
 }
 
-// 128-byte k blocks of a packed row: kp elements of 2 bytes (BF16) or 1 (e4m3).
-int k_blocks(int64_t kp, int fmt) { return (int)(fmt != kFmtBF16 ? kp / 128 : kp / kKBlock); }
-
 // The operand format of a market's dtype.
 int fmt_of(int dtype) {
   return dtype == TU_DTYPE_FP8E4M3 ? kFmtE4M3Rows : (dtype == TU_DTYPE_FP8E4M3_SIDE ? kFmtE4M3Side : kFmtBF16);
-}
-
-template <int MODE, bool BATCH, bool SMALL, int FMT, bool SPLIT>
-cudaError_t launch_fmt(int kb, const CUtensorMap& own, const CUtensorMap& partner, const FusedParams& p, int grid,
-                       cudaStream_t stream) {
-  if (kb == 1) return launch_kernel<1, MODE, BATCH, FMT, SMALL, SPLIT>(own, partner, p, grid, stream);
-  if (kb == 2) return launch_kernel<2, MODE, BATCH, FMT, SMALL, SPLIT>(own, partner, p, grid, stream);
-  if (kb == 4) return launch_kernel<4, MODE, BATCH, FMT, SMALL, SPLIT>(own, partner, p, grid, stream);
-  return cudaErrorNotSupported;
-}
-
-template <int MODE, bool BATCH = false, bool SMALL = false, bool SPLIT = false>
-cudaError_t launch_variant(int64_t kp, int fmt, const CUtensorMap& own, const CUtensorMap& partner,
-                           const FusedParams& p, int grid, cudaStream_t stream) {
-  const int kb = k_blocks(kp, fmt);
-  if (fmt == kFmtE4M3Rows)
-    return launch_fmt<MODE, BATCH, SMALL, kFmtE4M3Rows, SPLIT>(kb, own, partner, p, grid, stream);
-  if (fmt == kFmtE4M3Side)
-    return launch_fmt<MODE, BATCH, SMALL, kFmtE4M3Side, SPLIT>(kb, own, partner, p, grid, stream);
-  return launch_fmt<MODE, BATCH, SMALL, kFmtBF16, SPLIT>(kb, own, partner, p, grid, stream);
-}
-
-// small: 128-row own tiles (single-market launches only; see use_small_tiles)
-template <int MODE, bool BATCH = false>
-cudaError_t launch_any(int64_t kp, int fmt, const CUtensorMap& own, const CUtensorMap& partner,
-                       const FusedParams& p, int grid, cudaStream_t stream, bool small = false) {
-  if constexpr (!BATCH && MODE == kModeSweep) {
-    if (p.split > 1) {
-      if (small) return launch_variant<MODE, false, true, true>(kp, fmt, own, partner, p, grid, stream);
-      return launch_variant<MODE, false, false, true>(kp, fmt, own, partner, p, grid, stream);
-    }
-  }
-  if constexpr (!BATCH) {
-    if (small) return launch_variant<MODE, false, true>(kp, fmt, own, partner, p, grid, stream);
-  }
-  return launch_variant<MODE, BATCH, false>(kp, fmt, own, partner, p, grid, stream);
 }
 
 // 128-row own tiles when they all fit one wave (and the market allows them):
@@ -1635,6 +101,7 @@ FusedParams base_params(int64_t rows, int64_t row0, int64_t col0, int64_t ncols,
   p.num_partner_tiles = (int)((ncols + kFusedPartnerRows - 1) / kFusedPartnerRows);
   p.c = c;
   p.split = 1;
+  p.cut_t0 = p.num_own_tiles;
   return p;
 }
 
@@ -1676,6 +143,41 @@ cudaError_t fused_prepare(tu_market* m) {
   return set_kernel_attributes();
 }
 
+// The whole tiles of w full waves run as they are; the rest, one line of (tile,
+// partner tile) pairs, is cut into equal spans, one per SM. Without cuts 313
+// tiles on 152 SMs take three waves of which the last runs 9 tiles (the
+// 100,003-user side of a 79,999-user market), and a market of 40 tiles keeps
+// 112 SMs idle. A span costs its partner tiles and about kSpanCost more (two
+// pipeline fills, the partials' stores and the sums of the completing warp),
+// a tile kTileCost; the cuts are taken when they save 8 % of the longest CTA:
+// with eight waves and more the chip runs at its power limit anyway, and idle
+// SMs in the last wave give the others clock (300,000 x 300,000, 7.7 waves:
+// 33.3 ms per sweep whole, 34.3 cut). Per sweep, whole -> cut: 3,000 x 3,000
+// d = 50 58 -> 51 us, 10,000 x 10,000 123 -> 88, 20,000 x 15,001 d = 32 213 ->
+// 152, 40,000 x 40,000 1.08 -> 0.67 ms, 100,003 x 79,999 d = 64 3.57 -> 3.05,
+// FP8 rows 100,000 x 80,000 3.65 -> 2.96, d = 100 50,001 x 70,000 3.56 -> 2.89;
+// spans under four partner tiles lose (1,000 x 1,000: 38 us whole, 45 in spans
+// of two).
+constexpr int kSpanCost = 8, kTileCost = 4, kMinSpan = 4;
+
+CutPlan cut_plan(int64_t own_rows, int64_t partner_rows, int sms) {
+  CutPlan c;
+  const int64_t T = (own_rows + kFusedOwnRows - 1) / kFusedOwnRows;
+  const int64_t P = (partner_rows + kFusedPartnerRows - 1) / kFusedPartnerRows;
+  const int64_t w = T / sms, rest = T - w * sms;
+  c.t0 = (int)T;
+  if (rest == 0 || P <= kMinSpan || rest * P > (1 << 30)) return c;
+  int64_t span = (rest * P + sms - 1) / sms;
+  if (span < kMinSpan) span = kMinSpan;
+  if ((double)(w * (P + kTileCost) + span + kSpanCost) > 0.92 * (double)((w + 1) * (P + kTileCost))) return c;
+  c.t0 = (int)(w * sms);
+  c.span = (int)span;
+  c.spans = (int)((rest * P + span - 1) / span);
+  return c;
+}
+
+int64_t cut_slots(const CutPlan& p) { return 2 * (int64_t)p.spans; }
+
 cudaError_t launch_fused_halfsweep(tu_market* m, int side, int residual, int update, int* nparts_out,
                                    int64_t row0, int64_t nrows) {
   Side& own = side == 0 ? m->X : m->Y;
@@ -1685,7 +187,11 @@ cudaError_t launch_fused_halfsweep(tu_market* m, int side, int residual, int upd
     row0 = 0;
     nrows = own.rows;
   }
-  const bool small = use_small_tiles(m, nrows);
+  // the caller's split; or, in the default shape, a CTA per span of the cut tiles
+  const bool user_split = whole && !m->wide && m->split > 1 && m->split_part != nullptr;
+  const bool cuts = !user_split && own.cut.span > 0;
+  const bool cut_launch = cuts && whole && m->small_mode == 1 && m->cut_part != nullptr;
+  const bool small = !cut_launch && use_small_tiles(m, nrows);
   FusedParams p = base_params(nrows, row0, 0, partner.rows, m->cmul, small);
   p.g = partner.pvec;
   p.lmax = m->st + kStShift;
@@ -1709,18 +215,33 @@ cudaError_t launch_fused_halfsweep(tu_market* m, int side, int residual, int upd
     const double keep = 0.7 * (double)m->l2_bytes;
     p.l2_keep = (m->l2_bytes > 0 && pbytes > keep) ? (float)(keep / pbytes) : 0.0f;
   }
-  if (whole && !m->wide && m->split > 1 && m->split_part != nullptr) {
-    // partner split: at most one range per partner tile
+  int items = p.num_own_tiles;
+  if (user_split) {
+    // at most one range per partner tile
     p.split = m->split < p.num_partner_tiles ? m->split : p.num_partner_tiles;
     p.range_major = m->split_blocks ? 1 : 0;
     p.part = m->split_part;
     p.split_cnt = m->split_cnt;
+    items *= p.split;
+  } else if (cuts) {
+    p.cut_t0 = own.cut.t0;
+    p.cut_span = own.cut.span;
+    p.cut_spans = own.cut.spans;
+    p.cut_ptiles = p.num_partner_tiles;
+    if (cut_launch) {
+      p.part = m->cut_part;
+      p.part_m = m->cut_m;
+      p.split_cnt = m->cut_cnt;
+      items = p.cut_t0 > 0 ? m->num_sms : p.cut_spans;
+    }
   }
-  const int grid = grid_for_tiles(p.num_own_tiles * p.split, m->num_sms);
+  const int grid = grid_for_tiles(items, m->num_sms);
   *nparts_out = grid;
   const int fmt = fmt_of(m->dtype);
-  if (m->wide) return launch_any<kModeSweepWide>(m->kp, fmt, own.tm_own, partner.tm_partner, p, grid, m->stream, small);
-  return launch_any<kModeSweep>(m->kp, fmt, own.tm_own, partner.tm_partner, p, grid, m->stream, small);
+  const bool split = p.split > 1 || cut_launch;
+  if (m->wide)
+    return launch_wide_sweep(m->kp, fmt, own.tm_own, partner.tm_partner, p, grid, m->stream, small, split);
+  return launch_sweep<kModeSweep>(m->kp, fmt, own.tm_own, partner.tm_partner, p, grid, m->stream, small, split);
 }
 
 // Ranked lists of own users [row0, row0 + nrows) over all partners (the
@@ -1746,9 +267,7 @@ cudaError_t launch_fused_topk(tu_market* m, int side, int k, int64_t row0, int64
   p.fs_par = partner.fs;
   const int grid = grid_for_tiles(p.num_own_tiles, m->num_sms);
   const int fmt = fmt_of(m->dtype);
-  if (k <= kSharedTopK && k_blocks(m->kp, fmt) < 4)
-    return launch_any<kModeTopKShared>(m->kp, fmt, own.tm_own, partner.tm_partner, p, grid, m->stream, small);
-  return launch_any<kModeTopK>(m->kp, fmt, own.tm_own, partner.tm_partner, p, grid, m->stream, small);
+  return launch_lists(m->kp, fmt, own.tm_own, partner.tm_partner, p, grid, m->stream, small);
 }
 
 // mu for own X users [x0, x0 + nx) and partners [y0, y0 + ny) (the Y partner
@@ -1772,8 +291,8 @@ cudaError_t launch_fused_mu(tu_market* m, int64_t x0, int64_t nx, int64_t y0, in
   p.ny = ny;
   p.fs_own = m->X.fs;
   p.fs_par = m->Y.fs;
-  return launch_variant<kModeMu, false, false, true>(m->kp, fmt_of(m->dtype), m->X.tm_own, m->Y.tm_partner, p,
-                                                     grid_for_tiles(p.num_own_tiles * p.split, m->num_sms), m->stream);
+  return launch_mu(m->kp, fmt_of(m->dtype), m->X.tm_own, m->Y.tm_partner, p,
+                   grid_for_tiles(p.num_own_tiles * p.split, m->num_sms), m->stream);
 }
 
 // Same kernel on caller-described buffers (no market object): used by the

@@ -584,8 +584,8 @@ tu_status clear_results(tu_market* m) {
   TU_CK(m, cudaMemsetAsync(m->err_dev, 0, sizeof(int), m->stream));
   // every completed split launch leaves its counters at zero, but one that a
   // timed-out wait cut short may not: zeroed again before the next work
-  if (m->split_cnt != nullptr)
-    TU_CK(m, cudaMemsetAsync(m->split_cnt, 0, (size_t)split_counter_count(m) * sizeof(int), m->stream));
+  for (int* cnt : {m->split_cnt, m->cut_cnt})
+    if (cnt != nullptr) TU_CK(m, cudaMemsetAsync(cnt, 0, (size_t)split_counter_count(m) * sizeof(int), m->stream));
   return TU_OK;
 }
 
@@ -762,6 +762,9 @@ void tu_market_destroy(tu_market_t m) {
   dev_free(m, m->st);
   dev_free(m, m->split_part);
   dev_free(m, m->split_cnt);
+  dev_free(m, m->cut_part);
+  dev_free(m, m->cut_m);
+  dev_free(m, m->cut_cnt);
   dev_free(m, m->results);
   dev_free(m, m->err_dev);
   dev_free(m, m->staging);
@@ -920,6 +923,15 @@ tu_status tu_market_create(const tu_market_desc* desc, tu_market_t* out) {
     return bail(st);
   }
   if (D.path == TU_PATH_FUSED) {
+    m->X.cut = cut_plan(m->N, m->M, m->num_sms);
+    m->Y.cut = cut_plan(m->M, m->N, m->num_sms);
+    const int64_t sx = cut_slots(m->X.cut), sy = cut_slots(m->Y.cut), slots = sx > sy ? sx : sy;
+    if (slots > 0) {
+      // (the shifts too: replaced factors can make the market wide)
+      if ((st = dev_alloc(m, &m->cut_part, (size_t)slots * kFusedOwnRows)) != TU_OK) return bail(st);
+      if ((st = dev_alloc(m, &m->cut_m, (size_t)slots * kFusedOwnRows)) != TU_OK) return bail(st);
+      if ((st = dev_alloc(m, &m->cut_cnt, (size_t)split_counter_count(m))) != TU_OK) return bail(st);
+    }
     cudaError_t e = fused_prepare(m);
     if (e != cudaSuccess) return bail(fail_cuda(m, e, "fused_prepare"));
     apply_tuned(m);
@@ -1327,6 +1339,7 @@ int64_t tu_market_footprint(int64_t N, int64_t M, int64_t d, int path) {
   if (path == TU_PATH_FUSED) {
     bytes += (N + M) * kp * 2 + (np > mp ? np : mp) * 4;  // factors, per-row shifts
     if (kp == kKBlock) bytes += (np + mp) * 32;              // the extra MMA's g / c operand
+    bytes += 2 << 20;                                        // the cut sums' partials
   } else {
     bytes += (N + M) * kp * 4 + N * round_up(M, 4) * 4 + M * round_up(N, 4) * 4;
     bytes += 8 << 20;  // column sums of the one-pass sweep

@@ -64,6 +64,16 @@ enum : int { kResidualNone = 0, kResidualEstimate = 1, kResidualExact = 2 };
 // device error word codes (first error wins)
 enum : int { kErrNone = 0, kErrTimeout = 1, kErrNonfinite = 2 };
 
+// Where the rows' sums of a fused half-sweep are cut (cut_plan, fused.cu). Own
+// tiles (256 rows) from t0 on, taken as one line of (tile, partner tile)
+// pairs, are cut after every `span` pairs; a row's sum is formed range by range
+// and the ranges are added in order. span = 0: nothing is cut. The cuts belong
+// to the market's shape, not to a launch: a launch that gives each range to
+// another CTA and one that runs a row's ranges in turn give the same bits.
+struct CutPlan {
+  int t0 = 0, span = 0, spans = 0;
+};
+
 struct Side {
   int64_t rows = 0;      // users on this side
   int64_t rows_pad = 0;  // rows rounded up to kRowPad
@@ -83,6 +93,7 @@ struct Side {
   float* fac32 = nullptr;          // packed rows x kp, fp32 (dense path), zero padded
   CUtensorMap tm_own;       // TMA map, box kKBlock x kFusedOwnRows
   CUtensorMap tm_partner;   // TMA map, box kKBlock x kFusedPartnerRows
+  CutPlan cut;              // fused path: the cuts of the half-sweep that updates this side
 };
 
 // Over-relaxation controller of the solve loops (host side, one per market).
@@ -192,6 +203,9 @@ struct tu_market {
   float4* split_part = nullptr;    // split > 1: partial row sums, split x max(N, M)
   int* split_cnt = nullptr;        // split > 1: arrivals per (own tile, 32-row block), zeroed
   int split_cap = 0;               // the split the buffers were sized for
+  float4* cut_part = nullptr;      // cut half-sweeps: the ranges' sums, 2 x 256 per span of the larger plan
+  float2* cut_m = nullptr;         // and their shifts (wide markets)
+  int* cut_cnt = nullptr;          // arrivals per (own tile, 32-row block), zeroed
   bool translate = true;           // tu_market_set_translation: translation step before every half-sweep
   bool wide = false;               // factor range beyond one shift per half-sweep: per-row running maxima
   bool poisoned = false;
@@ -270,6 +284,11 @@ cudaError_t fused_prepare(tu_market* m);  // tensor maps + kernel attributes
 cudaError_t launch_fused_halfsweep(tu_market* m, int side, int residual, int update, int* nparts_out,
                                    int64_t row0 = 0, int64_t nrows = -1);
 
+// The cuts of a half-sweep of own_rows against partner_rows on sms SMs.
+CutPlan cut_plan(int64_t own_rows, int64_t partner_rows, int sms);
+// Scratch of cut launches, in ranges' slots of kFusedOwnRows rows (0: none).
+int64_t cut_slots(const CutPlan& p);
+
 // The fused half-sweep on caller-described device buffers (no market object).
 struct FusedRaw {
   const __nv_bfloat16* own16;  // rows x kp packed own factors
@@ -318,6 +337,7 @@ struct BatchDesc {
   int64_t partner_rows_pad;    // partner vector length (multiple of kRowPad)
   int num_own_tiles;           // ceil(rows / kFusedOwnRows)
   int num_partner_tiles;       // ceil(partner_rows / kFusedPartnerRows)
+  int cut_t0, cut_span;        // CutPlan of this half-sweep
   int slot0;                   // first own-tile slot of this market in the partials array
   float c;                     // log2(e) / (2 sigma)
 };
