@@ -995,6 +995,7 @@ __global__ void __launch_bounds__(kThreads, 1)
             }
           }
           if (!ok) break;
+          if constexpr (FOLD) continue;  // g rides in the MMA
           if (!mbar_wait(&gempty[gs], gphase ^ 1u, abort_flag)) {
             ok = false;
             break;
@@ -1212,7 +1213,8 @@ __global__ void __launch_bounds__(kThreads, 1)
       for (int j = jb; j < je; ++j) {
         // every lane waits; the outcome is made warp-uniform so that the
         // .sync.aligned TMEM loads below never run with a partial warp
-        const bool got = mbar_wait(&tfull[buf], tphase, abort_flag) && mbar_wait(&gfull[gs], gphase, abort_flag);
+        bool got = mbar_wait(&tfull[buf], tphase, abort_flag);
+        if constexpr (!FOLD) got = got && mbar_wait(&gfull[gs], gphase, abort_flag);
         if (!__all_sync(0xffffffffu, got)) {
           ok = false;
           break;
@@ -1260,9 +1262,11 @@ __global__ void __launch_bounds__(kThreads, 1)
             chunk_mu<RS, mu_width(KB)>(vb, gsf + 32, fsf + 32, crow, colbase + 32, mu_lo, mu_hi, mu_s1, mu_s2, lane, mu_nrow,
                          mu_row, topk_list + ew * mu_stage_floats(KB), p);
         }
-        // the g slot has been read by this warp
-        __syncwarp();
-        if (lane == 0) mbar_arrive(&gempty[gs]);
+        if constexpr (!FOLD) {
+          // the g slot has been read by this warp
+          __syncwarp();
+          if (lane == 0) mbar_arrive(&gempty[gs]);
+        }
         if constexpr (kSweepLike) {
           // compensated (Kahan) accumulation of the per-tile partial sums
           const float tile =
