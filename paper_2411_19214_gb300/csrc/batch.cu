@@ -163,7 +163,7 @@ __global__ void __launch_bounds__(kFinThreads) k_batch_finalize(const BatchDesc*
   }
   if (update) {
     const GroupTotal g = block_reduce_groups(d.grp, (d.rows + kGroupRows - 1) / kGroupRows, redf);
-    if (threadIdx.x == 0) finish_scalars(d.st, d.own_side, g, d.dm_next);
+    if (threadIdx.x == 0) finish_scalars(d.st, d.own_side, g, d.dm_next, d.log_dm);
   }
 }
 
@@ -197,7 +197,7 @@ __global__ void __launch_bounds__(kFinThreads) k_batch_reset(const BatchDesc* __
     tot[s] = block_reduce_groups(d.grp, ng, redf);
   }
   // the next half-sweep updates X against Y: dm = sum m - sum n
-  if (threadIdx.x == 0) rescan_scalars(desc_x[mk].st, tot[0], tot[1], -desc_x[mk].dm_next);
+  if (threadIdx.x == 0) rescan_scalars(desc_x[mk].st, tot[0], tot[1], -desc_x[mk].dm_next, desc_x[mk].log_dm);
 }
 
 // End of a block of batched sweeps: the listed markets' pending offsets
@@ -609,6 +609,7 @@ tu_status tu_batch_create(const tu_market_t* markets, int count, void* stream, t
       d.ell = own.ell;
       d.partner_ell = par.ell;
       d.dm_next = own.sum_mass - par.sum_mass;
+      d.log_dm = log_abs(d.dm_next);
       d.own_side = side;
       d.st = m->st;
       d.grp = own.grp;

@@ -798,10 +798,16 @@ __global__ void __launch_bounds__(32 * kColSegs) k_dense_cols(const float* __res
                                                              double* __restrict__ log_u, double* __restrict__ ell,
                                                              float4* __restrict__ grp, double* __restrict__ partials) {
   __shared__ float2 seg[kColSegs][32];
+  __shared__ int top[kColSegs];
   const int lane = threadIdx.x % 32, sg = threadIdx.x / 32;
   const int64_t c = (int64_t)blockIdx.x * 32 + lane;
   int R = -0x40000000;
-  for (int p = 0; p < clusters; ++p) R = max(R, __ldg(scale + p));
+  for (int p = threadIdx.x; p < clusters; p += 32 * kColSegs) R = max(R, __ldg(scale + p));
+  R = __reduce_max_sync(0xffffffffu, R);
+  if (lane == 0) top[sg] = R;
+  __syncthreads();
+#pragma unroll
+  for (int i = 0; i < kColSegs; ++i) R = max(R, top[i]);
   float hi = 0.0f, lo = 0.0f;
   if (c < cols)
 #pragma unroll 4

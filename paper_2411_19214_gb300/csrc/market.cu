@@ -220,10 +220,9 @@ void dev_free(tu_market* m, T*& p) {
 // word) share one block from slabs of kSlabBlocks: page-locked allocations
 // serialise the device like cudaMalloc. Slabs live for the process.
 struct HostMirror {
-  double results[kResSlots];
+  double results[kResSlots + 1];  // and the error word, as on the device
   double query[kResSlots + 1];
   double omega;
-  int err;
 };
 constexpr size_t kMirrorBytes = (sizeof(HostMirror) + 63) / 64 * 64;
 constexpr int kSlabBlocks = 64;
@@ -450,6 +449,8 @@ tu_status load_factors(tu_market* m, const void* F, const void* K, const void* G
   return TU_OK;
 }
 
+constexpr size_t kResBytes = (kResSlots + 1) * sizeof(double);  // the results and the error word behind them
+
 tu_status check_device_error(tu_market* m) {
   if (*m->err_host == kErrTimeout) return fail(m, TU_ERR_TIMEOUT, "a device-side wait ran out of its time limit");
   if (*m->err_host != kErrNone) return fail(m, TU_ERR_CUDA, "device error word set");
@@ -478,6 +479,23 @@ cudaError_t profile_mark(tu_market* m, bool start) {
   return e;
 }
 
+// The pass of one half-sweep, whose partner and scalars are prepared. nparts,
+// ngroups: the partials and groups it writes.
+cudaError_t enqueue_pass(tu_market* m, int side, int residual, int update, int* nparts, int64_t* ngroups) {
+  cudaError_t e;
+  if ((e = profile_mark(m, true)) != cudaSuccess) return e;
+  *ngroups = ((side == 0 ? m->N : m->M) + kGroupRows - 1) / kGroupRows;
+  if (m->path == TU_PATH_FUSED) {
+    e = launch_fused_halfsweep(m, side, residual, update, nparts);
+  } else if (side == 0) {
+    e = launch_dense_rowpass(m, residual, update, nparts, ngroups);
+  } else {
+    e = launch_dense_colpass(m, update, nparts, ngroups);
+  }
+  if (e != cudaSuccess) return e;
+  return profile_mark(m, false);
+}
+
 // One half-sweep: prepare the partner potentials and the pass's scalars, run
 // the pass, reduce its partials (and, after an update, the own side's groups).
 cudaError_t enqueue_half(tu_market* m, int side, int residual, int update) {
@@ -485,57 +503,54 @@ cudaError_t enqueue_half(tu_market* m, int side, int residual, int update) {
   // sweeps (update = 1) take the translation step; a certifying pass leaves the state as it is
   cudaError_t e = launch_prep(m, partner, m->path == TU_PATH_FUSED ? 1 : 0, update && m->translate ? 1 : 0);
   if (e != cudaSuccess) return e;
-  if ((e = profile_mark(m, true)) != cudaSuccess) return e;
   int nparts = 0;
-  int64_t ngroups = ((side == 0 ? m->N : m->M) + kGroupRows - 1) / kGroupRows;
-  if (m->path == TU_PATH_FUSED) {
-    e = launch_fused_halfsweep(m, side, residual, update, &nparts);
-  } else if (side == 0) {
-    e = launch_dense_rowpass(m, residual, update, &nparts, &ngroups);
-  } else {
-    e = launch_dense_colpass(m, update, &nparts, &ngroups);
-  }
-  if (e != cudaSuccess) return e;
-  if ((e = profile_mark(m, false)) != cudaSuccess) return e;
+  int64_t ngroups = 0;
+  if ((e = enqueue_pass(m, side, residual, update, &nparts, &ngroups)) != cudaSuccess) return e;
   return launch_finalize(m, nparts, side == 0 ? 1 : 0, residual, update, ngroups);
-}
-
-// One sweep of Eq. iteration: u from v (with the residual of the entering
-// state), then v from the new u.
-cudaError_t enqueue_sweep(tu_market* m) {
-  // dense path, plain updates: both half-sweeps from one pass over A-hat
-  if (m->dplan.cl > 0 && m->omega_cfg == 1.0) {
-    int nparts = 0;
-    int64_t ngroups = 0;
-    cudaError_t e = launch_prep(m, m->Y, 0, m->translate ? 1 : 0);
-    if (e == cudaSuccess) e = profile_mark(m, true);
-    if (e == cudaSuccess) e = launch_dense_sweep(m, kResidualEstimate, &nparts, &ngroups);
-    if (e == cudaSuccess) e = profile_mark(m, false);
-    if (e == cudaSuccess) e = launch_finalize(m, nparts, 1, kResidualEstimate, 1, ngroups, m->translate ? 2 : 1);
-    if (e == cudaSuccess) e = launch_dense_cols(m, &nparts, &ngroups);
-    if (e == cudaSuccess) e = launch_finalize(m, nparts, 0, 0, 1, ngroups);
-    return e;
-  }
-  cudaError_t e = enqueue_half(m, 0, kResidualEstimate, 1);
-  if (e != cudaSuccess) return e;
-  return enqueue_half(m, 1, 0, 1);
 }
 
 bool stream_capturable(cudaStream_t s) { return s != nullptr && s != cudaStreamLegacy && s != cudaStreamPerThread; }
 
-// k sweeps, then the translation steps still pending as offsets written into
-// the potentials (so every other call sees plain arrays).
+// k sweeps of Eq. iteration, each u from v (with the residual of the entering
+// state), then v from the new u; then the translation steps still pending as
+// offsets written into the potentials (so every other call sees plain arrays).
 cudaError_t enqueue_block(tu_market* m, int k) {
-  cudaError_t e = cudaSuccess;
-  for (int i = 0; i < k && e == cudaSuccess; ++i) e = enqueue_sweep(m);
-  if (e == cudaSuccess && k > 0) e = launch_flush(m);
-  return e;
+  if (k <= 0) return cudaSuccess;
+  const int fused = m->path == TU_PATH_FUSED ? 1 : 0, translate = m->translate ? 1 : 0;
+  // dense path, plain updates: both half-sweeps from one pass over A-hat
+  const bool one_pass = m->dplan.cl > 0 && m->omega_cfg == 1.0;
+  cudaError_t e = launch_prep(m, m->Y, fused, translate);
+  for (int i = 0; i < k && e == cudaSuccess; ++i) {
+    int nparts = 0;
+    int64_t ngroups = 0;
+    if (one_pass) {
+      e = profile_mark(m, true);
+      if (e == cudaSuccess) e = launch_dense_sweep(m, kResidualEstimate, &nparts, &ngroups);
+      if (e == cudaSuccess) e = profile_mark(m, false);
+      if (e == cudaSuccess) e = launch_finalize(m, nparts, 1, kResidualEstimate, 1, ngroups, translate ? 2 : 1);
+      if (e == cudaSuccess) e = launch_dense_cols(m, &nparts, &ngroups);
+    } else {
+      e = enqueue_pass(m, 0, kResidualEstimate, 1, &nparts, &ngroups);
+      if (e == cudaSuccess) e = launch_between(m, nparts, 1, kResidualEstimate, ngroups, fused, translate);
+      if (e == cudaSuccess) e = enqueue_pass(m, 1, kResidualNone, 1, &nparts, &ngroups);
+    }
+    if (e != cudaSuccess) break;
+    e = i + 1 < k ? launch_between(m, nparts, 0, kResidualNone, ngroups, fused, translate)
+                  : launch_finalize(m, nparts, 0, kResidualNone, 1, ngroups);
+  }
+  return e == cudaSuccess ? launch_flush(m) : e;
 }
 
 // Enqueue k sweeps, replaying a captured graph of k sweeps when possible.
-tu_status enqueue_sweeps(tu_market* m, int k) {
+// A solve's block lengths follow its market, and a capture costs as much as
+// launching some ten sweeps: with `again` a length is captured when it comes
+// the second time.
+tu_status enqueue_sweeps(tu_market* m, int k, bool again = false) {
   if (k <= 0) return TU_OK;
-  if (m->use_graphs && stream_capturable(m->stream) && k > 1 && !m->profiling) {
+  const bool seen = m->last_block == k;
+  m->last_block = k;
+  if (m->use_graphs && stream_capturable(m->stream) && k > 1 && !m->profiling &&
+      (!again || seen || (m->graph != nullptr && m->graph_sweeps == k))) {
     if (m->graph == nullptr || m->graph_sweeps != k) {
       if (m->graph != nullptr) {
         cudaGraphExecDestroy(m->graph);
@@ -563,9 +578,7 @@ tu_status enqueue_sweeps(tu_market* m, int k) {
 }
 
 tu_status read_results(tu_market* m) {
-  TU_CK(m, cudaMemcpyAsync(m->results_host, m->results, kResSlots * sizeof(double), cudaMemcpyDeviceToHost,
-                           m->stream));
-  TU_CK(m, cudaMemcpyAsync(m->err_host, m->err_dev, sizeof(int), cudaMemcpyDeviceToHost, m->stream));
+  TU_CK(m, cudaMemcpyAsync(m->results_host, m->results, kResBytes, cudaMemcpyDeviceToHost, m->stream));
   TU_CK(m, cudaStreamSynchronize(m->stream));
   TU_TRY(check_device_error(m));
   if (m->results_host[kResNonfin] > 0.0) return fail(m, TU_ERR_NONFINITE, "a computed potential is not finite");
@@ -580,8 +593,7 @@ int64_t split_counter_count(const tu_market* m) {
 }
 
 tu_status clear_results(tu_market* m) {
-  TU_CK(m, cudaMemsetAsync(m->results, 0, kResSlots * sizeof(double), m->stream));
-  TU_CK(m, cudaMemsetAsync(m->err_dev, 0, sizeof(int), m->stream));
+  TU_CK(m, cudaMemsetAsync(m->results, 0, kResBytes, m->stream));
   // every completed split launch leaves its counters at zero, but one that a
   // timed-out wait cut short may not: zeroed again before the next work
   for (int* cnt : {m->split_cnt, m->cut_cnt})
@@ -589,9 +601,11 @@ tu_status clear_results(tu_market* m) {
   return TU_OK;
 }
 
-// Residual of the current potentials (one X pass without update).
-tu_status certify(tu_market* m, double* res_inf, double* res_l1) {
+// Residual of the current potentials (one X pass without update); with match,
+// also the match count's sum of v^2 in FP64.
+tu_status certify(tu_market* m, double* res_inf, double* res_l1, bool match = false) {
   TU_CK(m, enqueue_half(m, 0, kResidualExact, 0));
+  if (match) TU_CK(m, launch_sum_sq(m, m->Y, 0));
   TU_TRY(read_results(m));
   if (res_inf) *res_inf = m->results_host[kResXInf];
   if (res_l1) *res_l1 = m->results_host[kResXL1] / m->X.sum_mass;
@@ -766,7 +780,6 @@ void tu_market_destroy(tu_market_t m) {
   dev_free(m, m->cut_m);
   dev_free(m, m->cut_cnt);
   dev_free(m, m->results);
-  dev_free(m, m->err_dev);
   dev_free(m, m->staging);
   dev_free(m, m->aux);
   dev_free(m, m->omega_dev);
@@ -855,15 +868,15 @@ tu_status tu_market_create(const tu_market_desc* desc, tu_market_t* out) {
   if ((st = side_alloc(m, m->Y, D.M, D.bias_y != nullptr)) != TU_OK) return bail(st);
   if ((st = dev_alloc(m, &m->partials, (size_t)kMaxPartials * 4)) != TU_OK) return bail(st);
   if ((st = dev_alloc(m, &m->st, (size_t)kStSlots)) != TU_OK) return bail(st);
-  if ((st = dev_alloc(m, &m->results, (size_t)kResSlots)) != TU_OK) return bail(st);
-  if ((st = dev_alloc(m, &m->err_dev, 1)) != TU_OK) return bail(st);
+  if ((st = dev_alloc(m, &m->results, (size_t)kResSlots + 1)) != TU_OK) return bail(st);
+  m->err_dev = reinterpret_cast<int*>(m->results + kResSlots);
   {
     HostMirror* hm = mirror_alloc();
     if (hm == nullptr) return bail(TU_ERR_OOM);
     m->results_host = hm->results;
     m->query_host = hm->query;
     m->omega_host = &hm->omega;
-    m->err_host = &hm->err;
+    m->err_host = reinterpret_cast<int*>(hm->results + kResSlots);
   }
   *m->err_host = 0;
   if (D.path == TU_PATH_DENSE) {
@@ -974,10 +987,7 @@ tu_status tu_ipfp_sweep(tu_market_t m, int nsweeps, double* residual_out) {
     TU_TRY(certify(m, residual_out, nullptr));
   } else if (nsweeps > 0) {
     // snapshot of the FP64 results for tu_market_query, then the completion event
-    TU_CK(m, cudaMemcpyAsync(m->query_host, m->results, kResSlots * sizeof(double), cudaMemcpyDeviceToHost,
-                             m->stream));
-    TU_CK(m, cudaMemcpyAsync(m->query_host + kResSlots, m->err_dev, sizeof(int), cudaMemcpyDeviceToHost,
-                             m->stream));
+    TU_CK(m, cudaMemcpyAsync(m->query_host, m->results, kResBytes, cudaMemcpyDeviceToHost, m->stream));
     if (m->done_ev == nullptr) TU_CK(m, cudaEventCreateWithFlags(&m->done_ev, cudaEventDisableTiming));
     TU_CK(m, cudaEventRecord(m->done_ev, m->stream));
     m->query_sweeps = m->sweeps_enqueued;
@@ -1351,11 +1361,7 @@ tu_status tu_ipfp_solve(tu_market_t m, double tol, int max_iter, int warm_start,
   TU_TRACE("tu_ipfp_solve");
   TU_TRY(check_live(m));
   if (!(tol >= 0.0) || max_iter < 0) return fail(m, TU_ERR_INVALID_ARG, "tol < 0 or max_iter < 0");
-  if (!warm_start) {
-    TU_CK(m, launch_reset_potentials(m, m->X));
-    TU_CK(m, launch_reset_potentials(m, m->Y));
-    TU_CK(m, launch_rescan(m));
-  }
+  if (!warm_start) TU_CK(m, launch_reset(m));
   TU_TRY(clear_results(m));
   // sweeps between host checks: planned from the measured decay (plan_block),
   // at most about 2e9 pair evaluations per check and 64 sweeps
@@ -1374,7 +1380,9 @@ tu_status tu_ipfp_solve(tu_market_t m, double tol, int max_iter, int warm_start,
   double omega = 1.0;
   if (relax) TU_TRY(set_omega(m, 1.0));
   while (true) {
-    TU_TRY(certify(m, &res_inf, &res_l1));
+    // match count from the column equations (they hold after every v update):
+    // sum_xy mu_xy = sum m - sum v^2
+    TU_TRY(certify(m, &res_inf, &res_l1, true));
     if (res_inf <= tol) {
       status = TU_OK;
       break;
@@ -1385,7 +1393,7 @@ tu_status tu_ipfp_solve(tu_market_t m, double tol, int max_iter, int warm_start,
     while (done < max_iter) {
       int k = plan_block(last_k, r_prev, r_last, tol, block);
       if (k > max_iter - done) k = max_iter - done;
-      TU_TRY(enqueue_sweeps(m, k));
+      TU_TRY(enqueue_sweeps(m, k, true));
       m->sweeps_enqueued += k;
       TU_TRY(read_results(m));
       done += k;
@@ -1403,11 +1411,6 @@ tu_status tu_ipfp_solve(tu_market_t m, double tol, int max_iter, int warm_start,
     }
   }
   if (relax) TU_TRY(set_omega(m, m->omega_cfg > 1.0 ? m->omega_cfg : 1.0));
-  // match count from the column equations (they hold after every v update):
-  // sum_xy mu_xy = sum m - sum v^2
-  TU_TRY(clear_results(m));
-  TU_CK(m, launch_sum_sq(m, m->Y, 0));
-  TU_TRY(read_results(m));
   const double match = m->Y.sum_mass - m->results_host[kResYSq];
   if (info != nullptr) {
     info->sweeps = done;
@@ -1428,11 +1431,7 @@ tu_status tu_ipfp_solve_ranking(tu_market_t m, int k, int64_t sample, int check_
   if (k < 1 || k > 63 || k > m->N || k > m->M || sample < 1 || check_every < 1 || patience < 1 ||
       !(score_eps >= 0.0) || max_iter < 0)
     return fail(m, TU_ERR_INVALID_ARG, "ranking-stability arguments out of range");
-  if (!warm_start) {
-    TU_CK(m, launch_reset_potentials(m, m->X));
-    TU_CK(m, launch_reset_potentials(m, m->Y));
-    TU_CK(m, launch_rescan(m));
-  }
+  if (!warm_start) TU_CK(m, launch_reset(m));
   TU_TRY(clear_results(m));
   // per side: the users checked and the list length (k + 1 when there is a next partner)
   const int64_t rows[2] = {sample < m->N ? sample : m->N, sample < m->M ? sample : m->M};
@@ -1513,10 +1512,7 @@ tu_status tu_ipfp_solve_ranking(tu_market_t m, int k, int64_t sample, int check_
   if (st != TU_OK) return st;
   if (ctl.enabled()) TU_TRY(set_omega(m, m->omega_cfg > 1.0 ? m->omega_cfg : 1.0));
   double res_inf = INFINITY, res_l1 = INFINITY;
-  TU_TRY(certify(m, &res_inf, &res_l1));
-  TU_TRY(clear_results(m));
-  TU_CK(m, launch_sum_sq(m, m->Y, 0));
-  TU_TRY(read_results(m));
+  TU_TRY(certify(m, &res_inf, &res_l1, true));
   if (info != nullptr) {
     info->sweeps = done;
     info->status = status;

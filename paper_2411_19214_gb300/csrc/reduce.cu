@@ -160,7 +160,7 @@ __global__ void k_set_potentials(const float* __restrict__ src, const float* __r
                                  double* __restrict__ log_u, double* __restrict__ ell) {
   for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < rows;
        i += (int64_t)gridDim.x * blockDim.x) {
-    const double lu = (src != nullptr) ? (double)src[i] : 0.0;
+    const double lu = (double)src[i];
     log_u[i] = lu;
     ell[i] = (b2s != nullptr) ? lu + (double)b2s[i] : lu;
   }
@@ -223,6 +223,21 @@ __global__ void k_row_norm_max(const float* __restrict__ f32, const __nv_bfloat1
 // of block 0 records the pass's scalars (prep_scalars: its translation step,
 // the partner shift it adds back and the own offset). No other thread reads
 // the scalars it writes.
+__device__ __forceinline__ void prep_row(int64_t i, int64_t rows, const double* __restrict__ ell, double top,
+                                        int fused_mode, float* __restrict__ out, uint4* __restrict__ fold,
+                                        float inv_c) {
+  float v;
+  if (i < rows) {
+    // the FP64 state is rounded once, to the FP32 vector the half-sweep streams
+    const double z = ell[i] - top;
+    v = fused_mode ? (float)(z * 1.4426950408889634) : (float)exp(z);
+  } else {
+    v = fused_mode ? -INFINITY : 0.0f;
+  }
+  out[i] = v;
+  if (fold != nullptr) write_fold_row(fold, i, v, inv_c);
+}
+
 __global__ void k_prep(const double* __restrict__ ell, int64_t rows, int64_t rows_pad, double* __restrict__ st,
                        int own, int translate, int fused_mode, float* __restrict__ out, uint4* __restrict__ fold,
                        float inv_c) {
@@ -230,49 +245,57 @@ __global__ void k_prep(const double* __restrict__ ell, int64_t rows, int64_t row
   if (blockIdx.x == 0 && threadIdx.x == 0) prep_scalars(st, own, translate);
   for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < rows_pad;
        i += (int64_t)gridDim.x * blockDim.x) {
-    float v;
-    if (i < rows) {
-      // the FP64 state is rounded once, to the FP32 vector the half-sweep streams
-      const double z = ell[i] - top;
-      v = fused_mode ? (float)(z * 1.4426950408889634) : (float)exp(z);
-    } else {
-      v = fused_mode ? -INFINITY : 0.0f;
-    }
-    out[i] = v;
-    if (fold != nullptr) write_fold_row(fold, i, v, inv_c);
+    prep_row(i, rows, ell, top, fused_mode, out, fold, inv_c);
   }
 }
 
-// Groups of a side's stored potentials (one warp per 32 rows), as a half-sweep
-// writes them for the rows it updates.
-__global__ void k_scan_groups(const double* __restrict__ log_u, const double* __restrict__ ell, int64_t rows,
-                              float4* __restrict__ grp) {
-  const int64_t ng = (rows + kGroupRows - 1) / kGroupRows;
+// Groups of both sides' stored potentials (one warp per 32 rows), as a
+// half-sweep writes them for the rows it updates; with reset, of u = v = 1,
+// which it stores (Alg. 1 / Alg. 2 initialisation).
+struct ScanSide {
+  double* log_u;
+  double* ell;
+  const float* b2s;
+  float4* grp;
+  int64_t rows;
+};
+__global__ void k_scan_groups(const ScanSide x, const ScanSide y, int reset) {
+  const int64_t nx = (x.rows + kGroupRows - 1) / kGroupRows, ng = nx + (y.rows + kGroupRows - 1) / kGroupRows;
   const int lane = threadIdx.x % 32;
-  for (int64_t g = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) / 32; g < ng;
-       g += (int64_t)gridDim.x * blockDim.x / 32) {
-    const int64_t r = g * kGroupRows + lane;
-    const bool valid = r < rows;
-    const float4 gv = warp_group(valid ? log_u[r] : 0.0, valid ? ell[r] : 0.0, valid);
-    if (lane == 0) grp[g] = gv;
+  for (int64_t i = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) / 32; i < ng;
+       i += (int64_t)gridDim.x * blockDim.x / 32) {
+    const ScanSide& s = i < nx ? x : y;
+    const int64_t g = i < nx ? i : i - nx, r = g * kGroupRows + lane;
+    const bool valid = r < s.rows;
+    double lu = 0.0, el = 0.0;
+    if (valid && reset) {
+      el = s.b2s != nullptr ? (double)s.b2s[r] : 0.0;
+      s.log_u[r] = lu;
+      s.ell[r] = el;
+    } else if (valid) {
+      lu = s.log_u[r];
+      el = s.ell[r];
+    }
+    const float4 gv = warp_group(lu, el, valid);
+    if (lane == 0) s.grp[g] = gv;
   }
 }
 
 // Scalars of both sides from their groups (one block): shifts and sums,
 // offsets cleared, and tau for the next half-sweep, which updates X against Y.
 __global__ void k_rescan_scalars(const float4* __restrict__ grp_x, int64_t ng_x, const float4* __restrict__ grp_y,
-                                 int64_t ng_y, double dm_next, double* __restrict__ st) {
+                                 int64_t ng_y, double dm_next, double log_dm, double* __restrict__ st) {
   __shared__ float red[2 * kThreads / 32];
   const GroupTotal x = block_reduce_groups(grp_x, ng_x, red);
   const GroupTotal y = block_reduce_groups(grp_y, ng_y, red);
-  if (threadIdx.x == 0) rescan_scalars(st, x, y, dm_next);
+  if (threadIdx.x == 0) rescan_scalars(st, x, y, dm_next, log_dm);
 }
 
-// End of a block of sweeps: write the sides' offsets into their arrays (the
-// scalars are folded by k_flush_scalars afterwards, so every block reads the
-// offsets before any is cleared).
+// End of a block of sweeps: write the sides' offsets into their arrays and fold
+// them into the scalars (by the last block to finish: every block has read the
+// offsets by then; the counter, in a spare scalar slot, wraps to 0).
 __global__ void k_flush(double* __restrict__ lu_x, double* __restrict__ ell_x, int64_t nx, double* __restrict__ lu_y,
-                        double* __restrict__ ell_y, int64_t ny, const double* __restrict__ st) {
+                        double* __restrict__ ell_y, int64_t ny, double* __restrict__ st) {
   const double ox = st[kStOff + 0], oy = st[kStOff + 1];
   const int64_t n = nx > ny ? nx : ny;
   for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
@@ -285,22 +308,36 @@ __global__ void k_flush(double* __restrict__ lu_x, double* __restrict__ ell_x, i
       ell_y[i] += oy;
     }
   }
-}
-
-__global__ void k_flush_scalars(double* __restrict__ st) {
-  for (int s = 0; s < 2; ++s) {
-    st[kStLmax + s] += st[kStOff + s];
-    st[kStOff + s] = 0.0;
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    __threadfence();
+    if (atomicInc(reinterpret_cast<unsigned*>(st + kStCount), gridDim.x - 1) == gridDim.x - 1) {
+      st[kStLmax + 0] += ox;
+      st[kStLmax + 1] += oy;
+      st[kStOff + 0] = 0.0;
+      st[kStOff + 1] = 0.0;
+    }
   }
 }
 
+// What the finalize of a pass needs.
+struct FinalizeArgs {
+  const double* partials;
+  int nparts, is_x, residual, update;
+  const float4* grp;
+  int64_t ngroups;
+  double dm_next;   // sum of own capacities - sum of partner capacities
+  double log_dm;    // log |dm_next|
+  double* st;
+  double* results;
+  int prep_next;    // also the scalars of the half-sweep that follows (2: with the translation step)
+};
+
 // FP64 reduction of the per-CTA partials (max r/n, sum |r|, sum u^2, non-finite
-// count). After a pass that updated its side (update), also that side's groups
-// into the market scalars (finish_scalars), with the same routine and block
-// size as the batched finalize.
-__global__ void k_finalize(const double* __restrict__ partials, int nparts, int is_x, int residual, int update,
-                           const float4* __restrict__ grp, int64_t ngroups, double dm_next, double* __restrict__ st,
-                           double* __restrict__ results, int prep_next) {
+// count), by one block. After a pass that updated its side (update), also that
+// side's groups into the market scalars (finish_scalars), with the same routine
+// and block size as the batched finalize.
+__device__ __forceinline__ void finalize_pass(const FinalizeArgs& a) {
   __shared__ double red[4];
   __shared__ float redf[2 * kThreads / 32];
   // one warp per quantity: an FP64 addition takes about 80 cycles, so four
@@ -308,10 +345,10 @@ __global__ void k_finalize(const double* __restrict__ partials, int nparts, int 
   const int w = threadIdx.x / 32, lane = threadIdx.x % 32;
   if (w < 4) {
     double v[4] = {0.0, 0.0, 0.0, 0.0};
-    for (int i = lane; i < nparts; i += 128) {
+    for (int i = lane; i < a.nparts; i += 128) {
 #pragma unroll
       for (int j = 0; j < 4; ++j) {
-        const double x = i + 32 * j < nparts ? partials[4 * (int64_t)(i + 32 * j) + w] : 0.0;
+        const double x = i + 32 * j < a.nparts ? a.partials[4 * (int64_t)(i + 32 * j) + w] : 0.0;
         v[j] = w == 0 ? (x > v[j] ? x : v[j]) : v[j] + x;
       }
     }
@@ -323,23 +360,49 @@ __global__ void k_finalize(const double* __restrict__ partials, int nparts, int 
     if (lane == 0) red[w] = t;
   }
   GroupTotal g{};
-  if (update) g = block_reduce_groups(grp, ngroups, redf);  // synchronises the block
+  if (a.update) g = block_reduce_groups(a.grp, a.ngroups, redf);  // synchronises the block
   else __syncthreads();
   if (threadIdx.x == 0) {
     const double mx = red[0], l1 = red[1], sq = red[2], nf = red[3];
-    if (is_x) {
-      if (residual) {
-        results[kResXInf] = mx;
-        results[kResXL1] = l1;
+    if (a.is_x) {
+      if (a.residual) {
+        a.results[kResXInf] = mx;
+        a.results[kResXL1] = l1;
       }
-      results[kResXSq] = sq;
+      a.results[kResXSq] = sq;
     } else {
-      results[kResYSq] = sq;
+      a.results[kResYSq] = sq;
     }
-    results[kResNonfin] += nf;
-    if (update) finish_scalars(st, is_x ? 0 : 1, g, dm_next);
-    if (prep_next) prep_scalars(st, is_x ? 1 : 0, prep_next > 1);
+    if (nf != 0.0) a.results[kResNonfin] += nf;
+    if (a.update) finish_scalars(a.st, a.is_x ? 0 : 1, g, a.dm_next, a.log_dm);
+    if (a.prep_next) prep_scalars(a.st, a.is_x ? 1 : 0, a.prep_next > 1);
   }
+}
+
+__global__ void __launch_bounds__(kThreads) k_finalize(const FinalizeArgs a) { finalize_pass(a); }
+
+// Between two half-sweeps: block 0 finalizes the pass before (results,
+// scalars, the step and scalars of the next half-sweep); the others form the
+// shift of the side just updated from its groups, as block 0 does, and write its
+// vector for the pass that follows. The finalize is a chain of FP64 operations
+// on one thread (5 us and more, log and exp at about 80 cycles per operation),
+// which the pass needs only at its end and the vector not at all, so finalize
+// and preparation one after the other took 12 us of a 10,000-user half-sweep.
+__global__ void __launch_bounds__(kThreads) k_between(const FinalizeArgs a, const double* __restrict__ ell,
+                                                     int64_t rows, int64_t rows_pad, int fused_mode,
+                                                     float* __restrict__ out, uint4* __restrict__ fold, float inv_c) {
+  if (blockIdx.x == 0) {
+    finalize_pass(a);
+    return;
+  }
+  __shared__ float red[2 * kThreads / 32];
+  float mm = -INFINITY, me = -INFINITY;
+  for (int64_t i = threadIdx.x; i < a.ngroups; i += kThreads) me = fmaxf(me, a.grp[i].z);
+  block_reduce_max2(mm, me, red);
+  const double top = finite_or_zero((double)me);
+  for (int64_t i = (blockIdx.x - 1) * (int64_t)kThreads + threadIdx.x; i < rows_pad;
+       i += (int64_t)(gridDim.x - 1) * kThreads)
+    prep_row(i, rows, ell, top, fused_mode, out, fold, inv_c);
 }
 
 // sum_i exp(2 log u_i) in FP64 as per-block partials in the common format.
@@ -382,12 +445,6 @@ cudaError_t launch_init_side(tu_market* m, Side& s, const float* bias_dev, int h
   const int g = grid_for(s.rows_pad, m->num_sms);
   k_init_side<<<g, kThreads, 0, m->stream>>>(bias_dev, has_bias, (float)(0.5 / m->sigma), s.rows,
                                                s.rows_pad, s.b2s, s.log_u, s.ell);
-  return cudaGetLastError();
-}
-
-cudaError_t launch_reset_potentials(tu_market* m, Side& s) {
-  const int g = grid_for(s.rows, m->num_sms);
-  k_set_potentials<<<g, kThreads, 0, m->stream>>>(nullptr, s.b2s, s.rows, s.log_u, s.ell);
   return cudaGetLastError();
 }
 
@@ -450,24 +507,24 @@ cudaError_t launch_prep(tu_market* m, Side& partner, int fused_mode, int transla
   return cudaGetLastError();
 }
 
-cudaError_t launch_rescan(tu_market* m) {
-  for (Side* s : {&m->X, &m->Y}) {
-    const int64_t ng = (s->rows + kGroupRows - 1) / kGroupRows;
-    int g = (int)((ng * 32 + kThreads - 1) / kThreads);
-    if (g > m->num_sms * 8) g = m->num_sms * 8;
-    k_scan_groups<<<g < 1 ? 1 : g, kThreads, 0, m->stream>>>(s->log_u, s->ell, s->rows, s->grp);
-  }
-  k_rescan_scalars<<<1, kThreads, 0, m->stream>>>(m->X.grp, (m->X.rows + kGroupRows - 1) / kGroupRows, m->Y.grp,
-                                                  (m->Y.rows + kGroupRows - 1) / kGroupRows,
-                                                  m->Y.sum_mass - m->X.sum_mass, m->st);
+static cudaError_t scan_sides(tu_market* m, int reset) {
+  const ScanSide x = {m->X.log_u, m->X.ell, m->X.b2s, m->X.grp, m->X.rows};
+  const ScanSide y = {m->Y.log_u, m->Y.ell, m->Y.b2s, m->Y.grp, m->Y.rows};
+  const int64_t nx = (x.rows + kGroupRows - 1) / kGroupRows, ny = (y.rows + kGroupRows - 1) / kGroupRows;
+  const double dm = m->Y.sum_mass - m->X.sum_mass;
+  k_scan_groups<<<grid_for((nx + ny) * 32, m->num_sms, 8), kThreads, 0, m->stream>>>(x, y, reset);
+  k_rescan_scalars<<<1, kThreads, 0, m->stream>>>(x.grp, nx, y.grp, ny, dm, log_abs(dm), m->st);
   return cudaGetLastError();
 }
+
+cudaError_t launch_rescan(tu_market* m) { return scan_sides(m, 0); }
+
+cudaError_t launch_reset(tu_market* m) { return scan_sides(m, 1); }
 
 cudaError_t launch_flush(tu_market* m) {
   const int64_t n = m->X.rows > m->Y.rows ? m->X.rows : m->Y.rows;
   k_flush<<<grid_for(n, m->num_sms, 4), kThreads, 0, m->stream>>>(m->X.log_u, m->X.ell, m->X.rows, m->Y.log_u,
                                                                    m->Y.ell, m->Y.rows, m->st);
-  k_flush_scalars<<<1, 1, 0, m->stream>>>(m->st);
   return cudaGetLastError();
 }
 
@@ -475,7 +532,8 @@ cudaError_t launch_sum_sq(tu_market* m, Side& s, int is_x) {
   int g = grid_for(s.rows, m->num_sms, 4);
   if (g > kMaxPartials) g = kMaxPartials;
   k_sum_sq<<<g, kThreads, 0, m->stream>>>(s.log_u, s.rows, m->partials);
-  k_finalize<<<1, kThreads, 0, m->stream>>>(m->partials, g, is_x, 0, 0, nullptr, 0, 0.0, m->st, m->results, 0);
+  const FinalizeArgs a = {m->partials, g, is_x, 0, 0, nullptr, 0, 0.0, 0.0, m->st, m->results, 0};
+  k_finalize<<<1, kThreads, 0, m->stream>>>(a);
   return cudaGetLastError();
 }
 
@@ -483,8 +541,28 @@ cudaError_t launch_finalize(tu_market* m, int nparts, int is_x, int residual, in
                             int prep_next) {
   Side& own = is_x ? m->X : m->Y;
   Side& par = is_x ? m->Y : m->X;
-  k_finalize<<<1, kThreads, 0, m->stream>>>(m->partials, nparts, is_x, residual, update, own.grp, ngroups,
-                                            own.sum_mass - par.sum_mass, m->st, m->results, prep_next);
+  const double dm = own.sum_mass - par.sum_mass;
+  const FinalizeArgs a = {m->partials, nparts, is_x, residual, update, own.grp, ngroups, dm, log_abs(dm), m->st,
+                          m->results, prep_next};
+  k_finalize<<<1, kThreads, 0, m->stream>>>(a);
+  return cudaGetLastError();
+}
+
+cudaError_t launch_between(tu_market* m, int nparts, int is_x, int residual, int64_t ngroups, int fused_mode,
+                           int translate) {
+  // (every block reads the groups: past a few thousand the two kernels are better)
+  if (ngroups > 4096) {
+    cudaError_t e = launch_finalize(m, nparts, is_x, residual, 1, ngroups);
+    return e != cudaSuccess ? e : launch_prep(m, is_x ? m->X : m->Y, fused_mode, translate);
+  }
+  Side& own = is_x ? m->X : m->Y;
+  Side& par = is_x ? m->Y : m->X;
+  const double dm = own.sum_mass - par.sum_mass;
+  const FinalizeArgs a = {m->partials, nparts, is_x, residual, 1, own.grp, ngroups, dm, log_abs(dm), m->st,
+                          m->results, translate ? 2 : 1};
+  k_between<<<1 + grid_for(own.rows_pad, m->num_sms, 4), kThreads, 0, m->stream>>>(
+      a, own.ell, own.rows, own.rows_pad, fused_mode, own.pvec,
+      fused_mode ? reinterpret_cast<uint4*>(own.fold) : nullptr, 1.0f / m->cmul);
   return cudaGetLastError();
 }
 

@@ -48,6 +48,7 @@ enum : int {
   kStTauUsed = 7,  // the translation step the current half-sweep's preparation applied
   kStShift = 8,    // the current half-sweep's partner shift: lmax + offset + tau (natural log)
   kStOwnOff = 9,   // the current half-sweep's own-side offset: offset - tau
+  kStCount = 10,   // a counter (int) of the flush's finished blocks
   kStSlots = 16
 };
 
@@ -119,6 +120,9 @@ struct RelaxControl {
   double observe(int done, double r, double tol);
 };
 
+// log |dm| of the translation step (0 for dm = 0, where it is not used)
+inline double log_abs(double dm) { return dm == 0.0 ? 0.0 : std::log(std::fabs(dm)); }
+
 // e4m3 markets (per-row or per-side scales)
 inline bool is_fp8(int dtype) { return dtype == TU_DTYPE_FP8E4M3 || dtype == TU_DTYPE_FP8E4M3_SIDE; }
 
@@ -184,16 +188,17 @@ struct tu_market {
   tu::DensePlan dplan;          // dense path: the one-pass sweep's layout
   float* colsum = nullptr;      // its scratch: clusters x ldA column sums, then the clusters' scales (int)
   int64_t ldN = 0;
-  double* results = nullptr;       // device, kResSlots
-  double* results_host = nullptr;  // pinned, kResSlots
-  int* err_dev = nullptr;          // device error word
-  int* err_host = nullptr;         // pinned
+  double* results = nullptr;       // device, kResSlots, then the error word
+  double* results_host = nullptr;  // pinned, likewise
+  int* err_dev = nullptr;          // device error word (behind results)
+  int* err_host = nullptr;         // pinned (behind results_host)
   void* staging = nullptr;         // device staging buffer for host-memory arguments
   size_t staging_bytes = 0;
   void* aux = nullptr;             // ranked-list hand-over scratch (grow-only)
   size_t aux_bytes = 0;
   cudaGraphExec_t graph = nullptr; // captured block of sweeps
   int graph_sweeps = 0;
+  int last_block = 0;              // sweeps of the last block
   bool use_graphs = true;          // tu_market_use_graphs
   int small_mode = 1;              // tu_market_set_small_tiles: 0 256-row own tiles, 1 128-row when they
                                    // fit one wave, 2 always 128-row
@@ -247,11 +252,15 @@ cudaError_t launch_finalize(tu_market* m, int nparts, int is_x, int residual, in
 // Groups and scalars of both sides from their stored potentials (after the
 // potentials were set from outside a sweep).
 cudaError_t launch_rescan(tu_market* m);
+// Finalize a pass that updated a side (is_x: X) and prepare the half-sweep of the
+// other side against it.
+cudaError_t launch_between(tu_market* m, int nparts, int is_x, int residual, int64_t ngroups, int fused_mode,
+                           int translate);
 // Write the sides' pending offsets into their arrays (end of a block of sweeps).
 cudaError_t launch_flush(tu_market* m);
 cudaError_t launch_pack_factors(tu_market* m, Side& s, const void* A, const void* B, int src_dtype);
 cudaError_t launch_init_side(tu_market* m, Side& s, const float* bias_dev, int has_bias);
-cudaError_t launch_reset_potentials(tu_market* m, Side& s);
+cudaError_t launch_reset(tu_market* m);  // u = v = 1 on both sides, with their groups and scalars
 cudaError_t launch_set_potentials(tu_market* m, Side& s, const float* log_u_dev);
 cudaError_t launch_set_potentials64(tu_market* m, Side& s, const double* log_u_dev);
 cudaError_t launch_get_potentials(tu_market* m, Side& s, float* out_dev);  // FP64 state -> FP32
@@ -330,6 +339,7 @@ struct BatchDesc {
   float4* grp;                 // own-side groups (written by the pass, reduced by the finalize)
   const double* omega;         // over-relaxation factor of this market (device scalar)
   double dm_next;              // sum of own capacities - sum of partner capacities (the next step's tau)
+  double log_dm;               // log |dm_next|
   int own_side;                // 0: X is own, 1: Y is own
   int translate;               // the market's translation-step setting at batch creation
   int64_t rows;                // own users
@@ -680,13 +690,13 @@ __device__ __forceinline__ double group_log_sum(const GroupTotal& t) {
 // with no cancellation; for |w| > 60, q = w / 2 or log 2 to double precision.
 // Non-finite inputs (non-finite potentials, which the half-sweep reports)
 // give tau = 0.
-__device__ __forceinline__ double translation_tau(double log_p, double log_o, double dm) {
+// (L, of the two sides' capacities alone, comes from the host.)
+__device__ __forceinline__ double translation_tau(double log_p, double log_o, double dm, double L) {
   const double ln2 = 0.69314718055994530942;
   double log_z;
   if (dm == 0.0) {
     log_z = 0.5 * __dadd_rn(log_o, -log_p);
   } else {
-    const double L = log(fabs(dm));
     const double w = __dadd_rn(__dadd_rn(__dadd_rn(2.0 * ln2, log_p), log_o), -2.0 * L);
     const double q = w > 60.0 ? 0.5 * w : (w < -60.0 ? ln2 : log1p(sqrt(1.0 + exp(w))));
     log_z = dm > 0.0 ? __dadd_rn(__dadd_rn(__dadd_rn(L, q), -ln2), -log_p)
@@ -714,7 +724,8 @@ __device__ __forceinline__ void prep_scalars(double* st, int own, int translate)
 // half-sweep, which updates the partner against this side
 // (dm_next = sum mass_own - sum mass_partner).
 __device__ __forceinline__ double finite_or_zero(double v) { return (v > -INFINITY && v < INFINITY) ? v : 0.0; }
-__device__ __forceinline__ void finish_scalars(double* st, int own, const GroupTotal& g, double dm_next) {
+__device__ __forceinline__ void finish_scalars(double* st, int own, const GroupTotal& g, double dm_next,
+                                               double log_dm) {
   const int par = 1 - own;
   const double tau = st[kStTauUsed];
   const double log_s_own = group_log_sum(g);
@@ -725,14 +736,14 @@ __device__ __forceinline__ void finish_scalars(double* st, int own, const GroupT
   st[kStOff + par] += tau;
   st[kStLogS + par] += 2.0 * tau;
   st[kStTauUsed] = 0.0;
-  st[kStTauNext] = translation_tau(log_s_own, st[kStLogS + par], dm_next);
+  st[kStTauNext] = translation_tau(log_s_own, st[kStLogS + par], dm_next, log_dm);
 }
 
 // Scalars of both sides from their reduced groups (one thread; potentials set
 // from outside a sweep): shifts, sums, no offsets, and tau for the next
 // half-sweep, which updates X against Y (dm = sum m - sum n).
 __device__ __forceinline__ void rescan_scalars(double* st, const GroupTotal& x, const GroupTotal& y,
-                                               double dm_y_minus_x) {
+                                               double dm_y_minus_x, double log_dm) {
   const double sx = group_log_sum(x), sy = group_log_sum(y);
   st[kStLmax + 0] = finite_or_zero((double)x.lmax);
   st[kStLmax + 1] = finite_or_zero((double)y.lmax);
@@ -741,7 +752,7 @@ __device__ __forceinline__ void rescan_scalars(double* st, const GroupTotal& x, 
   st[kStOff + 0] = 0.0;
   st[kStOff + 1] = 0.0;
   st[kStTauUsed] = 0.0;
-  st[kStTauNext] = translation_tau(sy, sx, dm_y_minus_x);
+  st[kStTauNext] = translation_tau(sy, sx, dm_y_minus_x, log_dm);
 }
 
 __device__ __forceinline__ uint64_t global_timer_ns() {
