@@ -71,6 +71,7 @@ struct tu_batch {
   int64_t tiles[2] = {0, 0};        // own tiles of all markets, per side
   double* partials = nullptr;       // [slot][kBatchSlotWarps][4]
   double* results = nullptr;        // [market][kResSlots]
+  double* sums = nullptr;           // [market][kMarketBlocks]: the sum of squares' block sums
   double* results_host = nullptr;   // pinned
   int* err_dev = nullptr;
   int* err_host = nullptr;          // pinned
@@ -88,8 +89,33 @@ struct tu_batch {
 namespace {
 
 // ---------------------------------------------------------------------------
-// Kernels: one CTA per listed market
+// Kernels over the listed markets: blockIdx.x a market, blockIdx.y one of up to
+// kMarketBlocks blocks that share its users
 // ---------------------------------------------------------------------------
+
+// A block has about kBlockRows users: with one block per market the largest
+// (50,000 users) kept a block busy for 50 to 220 us while the rest of the chip
+// was idle (flush 163 us, preparation 57, sum of squares 224; 56 markets).
+constexpr int kMarketBlocks = 32;
+constexpr int kBlockRows = 2048;
+__device__ __forceinline__ int market_blocks(int64_t rows) {
+  const int64_t n = (rows + kBlockRows - 1) / kBlockRows;
+  return n < 1 ? 1 : (n > kMarketBlocks ? kMarketBlocks : (int)n);
+}
+// Whether this block is the last of the market's `blocks` to get here (on every
+// thread); what the others wrote before is then visible. The counter is a
+// spare scalar slot of the market and wraps to 0.
+__device__ __forceinline__ bool last_block(double* st, int blocks) {
+  __shared__ int last;
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    __threadfence();
+    last = atomicInc(reinterpret_cast<unsigned*>(st + kStCount), (unsigned)blocks - 1u) == (unsigned)blocks - 1u;
+    __threadfence();
+  }
+  __syncthreads();
+  return last != 0;
+}
 
 // Partner preparation of a listed market: the FP32 vector
 // g = (ell - max ell) log2(e), -inf padded, from the partner's shift kept in
@@ -101,10 +127,13 @@ __global__ void __launch_bounds__(kPrepThreads) k_batch_prep(const BatchDesc* __
                                                             const int* __restrict__ n_list, int sweep) {
   if ((int)blockIdx.x >= *n_list) return;
   const BatchDesc& d = desc[list[blockIdx.x]];
+  const int blocks = market_blocks(d.partner_rows_pad);
+  if ((int)blockIdx.y >= blocks) return;
   const double top = d.st[kStLmax + (1 - d.own_side)];  // not written by prep_scalars
-  if (threadIdx.x == 0) prep_scalars(d.st, d.own_side, sweep && d.translate);
+  if (blockIdx.y == 0 && threadIdx.x == 0) prep_scalars(d.st, d.own_side, sweep && d.translate);
   const float inv_c = 1.0f / d.c;  // (the single-market preparation's 1 / c, rounded alike)
-  for (int64_t i = threadIdx.x; i < d.partner_rows_pad; i += blockDim.x) {
+  for (int64_t i = (int64_t)blockIdx.y * kPrepThreads + threadIdx.x; i < d.partner_rows_pad;
+       i += (int64_t)blocks * kPrepThreads) {
     const float v = i < d.partner_rows ? (float)((d.partner_ell[i] - top) * 1.4426950408889634) : -INFINITY;
     d.g[i] = v;
     if (d.gfold != nullptr) write_fold_row(reinterpret_cast<uint4*>(d.gfold), i, v, inv_c);
@@ -123,43 +152,48 @@ __global__ void __launch_bounds__(kFinThreads) k_batch_finalize(const BatchDesc*
   if ((int)blockIdx.x >= *n_list) return;
   const int mk = list[blockIdx.x];
   const BatchDesc& d = desc[mk];
-  __shared__ double s_max[kFinThreads], s_l1[kFinThreads], s_sq[kFinThreads], s_nf[kFinThreads];
+  __shared__ double red[8];
   __shared__ float redf[2 * kFinThreads / 32];
-  const int64_t s0 = (int64_t)d.slot0 * kBatchSlotWarps;
-  const int64_t s1 = s0 + (int64_t)d.num_own_tiles * kBatchSlotWarps;
-  double mx = 0.0, l1 = 0.0, sq = 0.0, nf = 0.0;
-  for (int64_t i = s0 + threadIdx.x; i < s1; i += blockDim.x) {
-    mx = fmax(mx, partials[4 * i + 0]);
-    l1 += partials[4 * i + 1];
-    sq += partials[4 * i + 2];
-    nf += partials[4 * i + 3];
-  }
-  s_max[threadIdx.x] = mx;
-  s_l1[threadIdx.x] = l1;
-  s_sq[threadIdx.x] = sq;
-  s_nf[threadIdx.x] = nf;
-  __syncthreads();
-  for (int w = blockDim.x / 2; w > 0; w >>= 1) {
-    if ((int)threadIdx.x < w) {
-      s_max[threadIdx.x] = fmax(s_max[threadIdx.x], s_max[threadIdx.x + w]);
-      s_l1[threadIdx.x] += s_l1[threadIdx.x + w];
-      s_sq[threadIdx.x] += s_sq[threadIdx.x + w];
-      s_nf[threadIdx.x] += s_nf[threadIdx.x + w];
+  // two warps per quantity, eight chains side by side (an FP64 addition takes
+  // about 80 cycles, a load several hundred)
+  const int w = threadIdx.x / 32, lane = threadIdx.x % 32, what = w & 3;
+  const double* pm = partials + (int64_t)d.slot0 * kBatchSlotWarps * 4;
+  const int np = d.num_own_tiles * kBatchSlotWarps;
+  {
+    double v[8] = {0.0, 0.0, 0.0, 0.0, 0.0, 0.0, 0.0, 0.0};
+    for (int i = (w >> 2) * 32 + lane; i < np; i += 512) {
+      double x[8];
+#pragma unroll
+      for (int j = 0; j < 8; ++j) x[j] = i + 64 * j < np ? pm[4 * (i + 64 * j) + what] : 0.0;
+#pragma unroll
+      for (int j = 0; j < 8; ++j) v[j] = what == 0 ? (x[j] > v[j] ? x[j] : v[j]) : v[j] + x[j];
     }
-    __syncthreads();
+#pragma unroll
+    for (int o = 4; o > 0; o >>= 1)
+#pragma unroll
+      for (int j = 0; j < o; ++j) v[j] = what == 0 ? (v[j + o] > v[j] ? v[j + o] : v[j]) : v[j] + v[j + o];
+    double t = v[0];
+    for (int o = 16; o > 0; o >>= 1) {
+      const double x = __shfl_xor_sync(0xffffffffu, t, o);
+      t = what == 0 ? (x > t ? x : t) : t + x;
+    }
+    if (lane == 0) red[w] = t;
   }
+  __syncthreads();
   if (threadIdx.x == 0) {
     double* r = results + (int64_t)mk * kResSlots;
+    red[0] = red[4] > red[0] ? red[4] : red[0];
+    for (int k = 1; k < 4; ++k) red[k] += red[4 + k];
     if (is_x) {
       if (residual) {
-        r[kResXInf] = s_max[0];
-        r[kResXL1] = s_l1[0];
+        r[kResXInf] = red[0];
+        r[kResXL1] = red[1];
       }
-      r[kResXSq] = s_sq[0];
+      r[kResXSq] = red[2];
     } else {
-      r[kResYSq] = s_sq[0];
+      r[kResYSq] = red[2];
     }
-    r[kResNonfin] += s_nf[0];
+    r[kResNonfin] += red[3];
   }
   if (update) {
     const GroupTotal g = block_reduce_groups(d.grp, (d.rows + kGroupRows - 1) / kGroupRows, redf);
@@ -176,13 +210,17 @@ __global__ void __launch_bounds__(kFinThreads) k_batch_reset(const BatchDesc* __
   if ((int)blockIdx.x >= *n_list) return;
   const int mk = list[blockIdx.x];
   __shared__ float redf[2 * kFinThreads / 32];
-  const int warp = threadIdx.x / 32, lane = threadIdx.x % 32;
-  GroupTotal tot[2];
+  const BatchDesc& x = desc_x[mk];
+  const BatchDesc& y = desc_y[mk];
+  const int blocks = market_blocks(x.rows > y.rows ? x.rows : y.rows);
+  if ((int)blockIdx.y >= blocks) return;
+  const int lane = threadIdx.x % 32;
+  const int64_t warp = (int64_t)blockIdx.y * (kFinThreads / 32) + threadIdx.x / 32;
   for (int s = 0; s < 2; ++s) {
-    const BatchDesc& d = (s == 0 ? desc_x : desc_y)[mk];
+    const BatchDesc& d = s == 0 ? x : y;
     // each warp resets the rows of the groups it then forms
     const int64_t ng = (d.rows + kGroupRows - 1) / kGroupRows;
-    for (int64_t g = warp; g < ng; g += kFinThreads / 32) {
+    for (int64_t g = warp; g < ng; g += (int64_t)blocks * (kFinThreads / 32)) {
       const int64_t i = g * kGroupRows + lane;
       const bool valid = i < d.rows;
       const double e = (valid && d.b2s != nullptr) ? (double)d.b2s[i] : 0.0;
@@ -193,11 +231,12 @@ __global__ void __launch_bounds__(kFinThreads) k_batch_reset(const BatchDesc* __
       const float4 gv = warp_group(0.0, e, valid);
       if (lane == 0) d.grp[g] = gv;
     }
-    __syncthreads();
-    tot[s] = block_reduce_groups(d.grp, ng, redf);
   }
+  if (!last_block(x.st, blocks)) return;
+  const GroupTotal tx = block_reduce_groups(x.grp, (x.rows + kGroupRows - 1) / kGroupRows, redf);
+  const GroupTotal ty = block_reduce_groups(y.grp, (y.rows + kGroupRows - 1) / kGroupRows, redf);
   // the next half-sweep updates X against Y: dm = sum m - sum n
-  if (threadIdx.x == 0) rescan_scalars(desc_x[mk].st, tot[0], tot[1], -desc_x[mk].dm_next, desc_x[mk].log_dm);
+  if (threadIdx.x == 0) rescan_scalars(x.st, tx, ty, -x.dm_next, x.log_dm);
 }
 
 // End of a block of batched sweeps: the listed markets' pending offsets
@@ -210,16 +249,19 @@ __global__ void __launch_bounds__(kFinThreads) k_batch_flush(const BatchDesc* __
   const int mk = list[blockIdx.x];
   double* st = desc_x[mk].st;
   const double off[2] = {st[kStOff + 0], st[kStOff + 1]};
+  const int64_t rx = desc_x[mk].rows, ry = desc_y[mk].rows;
+  const int blocks = market_blocks(rx > ry ? rx : ry);
+  if ((int)blockIdx.y >= blocks) return;
   for (int s = 0; s < 2; ++s) {
     if (off[s] == 0.0) continue;
     const BatchDesc& d = (s == 0 ? desc_x : desc_y)[mk];
-    for (int64_t i = threadIdx.x; i < d.rows; i += blockDim.x) {
+    for (int64_t i = (int64_t)blockIdx.y * kFinThreads + threadIdx.x; i < d.rows; i += (int64_t)blocks * kFinThreads) {
       d.log_u[i] += off[s];
       d.ell[i] += off[s];
     }
   }
-  __syncthreads();  // every thread has read the offsets
-  if (threadIdx.x == 0) {
+  // (every block has read the offsets by then)
+  if (last_block(st, blocks) && threadIdx.x == 0) {
     for (int s = 0; s < 2; ++s) {
       st[kStLmax + s] += off[s];
       st[kStOff + s] = 0.0;
@@ -227,23 +269,33 @@ __global__ void __launch_bounds__(kFinThreads) k_batch_flush(const BatchDesc* __
   }
 }
 
-// results[kResYSq] = sum_y v_y^2 in FP64 for the listed markets.
+// results[kResYSq] = sum_y v_y^2 in FP64 for the listed markets (the blocks'
+// sums in `part`, kMarketBlocks per market, added in order).
 __global__ void __launch_bounds__(kFinThreads) k_batch_sum_sq(const BatchDesc* __restrict__ desc_y,
                                                              const int* __restrict__ list,
-                                                             const int* __restrict__ n_list,
+                                                             const int* __restrict__ n_list, double* part,
                                                              double* __restrict__ results) {
   if ((int)blockIdx.x >= *n_list) return;
   const int mk = list[blockIdx.x];
   const BatchDesc& d = desc_y[mk];
+  const int blocks = market_blocks(d.rows);
+  if ((int)blockIdx.y >= blocks) return;
   __shared__ double red[kFinThreads / 32];
   double s = 0.0;
-  for (int64_t i = threadIdx.x; i < d.rows; i += blockDim.x) s += exp(2.0 * d.log_u[i]);
+  for (int64_t i = (int64_t)blockIdx.y * kFinThreads + threadIdx.x; i < d.rows; i += (int64_t)blocks * kFinThreads)
+    s += exp(2.0 * d.log_u[i]);
   for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
   if (threadIdx.x % 32 == 0) red[threadIdx.x / 32] = s;
   __syncthreads();
+  double* mine = part + (int64_t)mk * kMarketBlocks;
   if (threadIdx.x == 0) {
     double b = 0.0;
     for (int w = 0; w < kFinThreads / 32; ++w) b += red[w];
+    mine[blockIdx.y] = b;
+  }
+  if (last_block(d.st, blocks) && threadIdx.x == 0) {
+    double b = 0.0;
+    for (int w = 0; w < blocks; ++w) b += __ldcg(mine + w);
     results[(int64_t)mk * kResSlots + kResYSq] = b;
   }
 }
@@ -405,7 +457,7 @@ cudaError_t enqueue_half(tu_batch* b, int si, int side, int residual, int update
   const Schedule& S = b->sched[si];
   const int* n = S.dev;
   const int* list = S.dev + S.off_list;
-  k_batch_prep<<<b->count, kPrepThreads, 0, b->stream>>>(b->desc_dev[side], list, n, update);
+  k_batch_prep<<<dim3(b->count, kMarketBlocks), kPrepThreads, 0, b->stream>>>(b->desc_dev[side], list, n, update);
   cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess) return e;
   if ((e = profile_mark(b, true)) != cudaSuccess) return e;
@@ -436,7 +488,7 @@ cudaError_t enqueue_sweep(tu_batch* b) {
 // After a block of sweeps over schedule 0: pending offsets into the arrays.
 cudaError_t enqueue_flush(tu_batch* b) {
   const Schedule& S = b->sched[0];
-  k_batch_flush<<<b->count, kFinThreads, 0, b->stream>>>(b->desc_dev[0], b->desc_dev[1], S.dev + S.off_list, S.dev);
+  k_batch_flush<<<dim3(b->count, kMarketBlocks), kFinThreads, 0, b->stream>>>(b->desc_dev[0], b->desc_dev[1], S.dev + S.off_list, S.dev);
   return cudaGetLastError();
 }
 
@@ -536,6 +588,7 @@ void tu_batch_destroy(tu_batch_t b) {
   }
   cudaFree(b->partials);
   cudaFree(b->results);
+  cudaFree(b->sums);
   cudaFree(b->err_dev);
   cudaFree(b->omega_dev);
   cudaFreeHost(b->results_host);
@@ -647,6 +700,7 @@ tu_status tu_batch_create(const tu_market_t* markets, int count, void* stream, t
         const int64_t slots = std::max(b->tiles[0], b->tiles[1]) * kBatchSlotWarps;
         TB_CK(b, cudaMalloc(&b->partials, (size_t)slots * 4 * sizeof(double)));
         TB_CK(b, cudaMalloc(&b->results, (size_t)count * kResSlots * sizeof(double)));
+        TB_CK(b, cudaMalloc(&b->sums, (size_t)count * kMarketBlocks * sizeof(double)));
         TB_CK(b, cudaMalloc(&b->err_dev, sizeof(int)));
         TB_CK(b, cudaMallocHost(&b->results_host, (size_t)count * kResSlots * sizeof(double)));
         TB_CK(b, cudaMallocHost(&b->err_host, sizeof(int)));
@@ -718,8 +772,8 @@ tu_status tu_batch_solve(tu_batch_t b, double tol, int max_iter, int warm_start,
   for (int i = 0; i < count; ++i) all[i] = i;
   if (!warm_start) {
     TB_TRY(sched_set(b, b->sched[0], all));
-    k_batch_reset<<<count, kFinThreads, 0, b->stream>>>(b->desc_dev[0], b->desc_dev[1], b->sched[0].dev + 4,
-                                                          b->sched[0].dev);
+    k_batch_reset<<<dim3(count, kMarketBlocks), kFinThreads, 0, b->stream>>>(b->desc_dev[0], b->desc_dev[1],
+                                                                             b->sched[0].dev + 4, b->sched[0].dev);
     TB_CK(b, cudaGetLastError());
   }
   TB_TRY(reset_omega(b, true));
@@ -821,8 +875,8 @@ tu_status tu_batch_solve(tu_batch_t b, double tol, int max_iter, int warm_start,
   TB_TRY(reset_omega(b));
   // match counts from the column equations: sum_xy mu_xy = sum m - sum v^2
   TB_TRY(sched_set(b, b->sched[1], all));
-  k_batch_sum_sq<<<count, kFinThreads, 0, b->stream>>>(b->desc_dev[1], b->sched[1].dev + 4, b->sched[1].dev,
-                                                         b->results);
+  k_batch_sum_sq<<<dim3(count, kMarketBlocks), kFinThreads, 0, b->stream>>>(
+      b->desc_dev[1], b->sched[1].dev + 4, b->sched[1].dev, b->sums, b->results);
   TB_CK(b, cudaGetLastError());
   TB_TRY(read_results(b));
   tu_status overall = TU_OK;

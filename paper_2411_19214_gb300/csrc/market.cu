@@ -1597,18 +1597,19 @@ tu_status tu_get_potentials(tu_market_t m, float* log_u, float* log_v) {
   TU_TRY(check_live(m));
   Side* sides[2] = {&m->X, &m->Y};
   float* outs[2] = {log_u, log_v};
-  for (int i = 0; i < 2; ++i) {
-    if (outs[i] == nullptr) continue;
-    const size_t bytes = (size_t)sides[i]->rows * sizeof(float);
-    void* dst;
-    bool host;
-    TU_TRY(output_view(m, outs[i], bytes, 0, &dst, &host));
-    TU_CK(m, launch_get_potentials(m, *sides[i], static_cast<float*>(dst)));
-    if (host) {
-      TU_CK(m, cudaMemcpyAsync(outs[i], dst, bytes, cudaMemcpyDeviceToHost, m->stream));
-      TU_CK(m, cudaStreamSynchronize(m->stream));
-    }
-  }
+  // host outputs share the staging buffer: sized for both before either view points into it
+  const size_t second = (size_t)round_up(m->N * (int64_t)sizeof(float), 256);
+  bool host[2] = {log_u != nullptr && !is_device_ptr(log_u), log_v != nullptr && !is_device_ptr(log_v)};
+  if (host[0] || host[1]) TU_TRY(ensure_staging(m, second + (size_t)m->M * sizeof(float)));
+  float* dst[2];
+  for (int i = 0; i < 2; ++i)
+    dst[i] = host[i] ? reinterpret_cast<float*>(static_cast<char*>(m->staging) + (i == 0 ? 0 : second)) : outs[i];
+  TU_CK(m, launch_get_potentials(m, dst[0], dst[1]));
+  for (int i = 0; i < 2; ++i)
+    if (host[i])
+      TU_CK(m, cudaMemcpyAsync(outs[i], dst[i], (size_t)sides[i]->rows * sizeof(float), cudaMemcpyDeviceToHost,
+                               m->stream));
+  if (host[0] || host[1]) TU_CK(m, cudaStreamSynchronize(m->stream));
   return TU_OK;
 }
 

@@ -176,10 +176,14 @@ __global__ void k_set_potentials64(const double* __restrict__ src, const float* 
   }
 }
 
-__global__ void k_get_potentials(const double* __restrict__ log_u, int64_t rows, float* __restrict__ out) {
-  for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < rows;
-       i += (int64_t)gridDim.x * blockDim.x)
-    out[i] = (float)log_u[i];
+// FP32 copies of the potentials (either output may be null)
+__global__ void k_get_potentials(const double* __restrict__ lu, int64_t nx, float* __restrict__ out_x,
+                                 const double* __restrict__ lv, int64_t ny, float* __restrict__ out_y) {
+  const int64_t n = nx > ny ? nx : ny;
+  for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
+    if (out_x != nullptr && i < nx) out_x[i] = (float)lu[i];
+    if (out_y != nullptr && i < ny) out_y[i] = (float)lv[i];
+  }
 }
 
 __global__ void k_row_norm_max(const float* __restrict__ f32, const __nv_bfloat16* __restrict__ f16,
@@ -448,9 +452,10 @@ cudaError_t launch_init_side(tu_market* m, Side& s, const float* bias_dev, int h
   return cudaGetLastError();
 }
 
-cudaError_t launch_get_potentials(tu_market* m, Side& s, float* out_dev) {
-  const int g = grid_for(s.rows, m->num_sms);
-  k_get_potentials<<<g, kThreads, 0, m->stream>>>(s.log_u, s.rows, out_dev);
+cudaError_t launch_get_potentials(tu_market* m, float* out_x, float* out_y) {
+  const int64_t n = m->X.rows > m->Y.rows ? m->X.rows : m->Y.rows;
+  k_get_potentials<<<grid_for(n, m->num_sms), kThreads, 0, m->stream>>>(m->X.log_u, m->X.rows, out_x, m->Y.log_u,
+                                                                      m->Y.rows, out_y);
   return cudaGetLastError();
 }
 

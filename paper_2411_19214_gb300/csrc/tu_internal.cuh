@@ -263,7 +263,8 @@ cudaError_t launch_init_side(tu_market* m, Side& s, const float* bias_dev, int h
 cudaError_t launch_reset(tu_market* m);  // u = v = 1 on both sides, with their groups and scalars
 cudaError_t launch_set_potentials(tu_market* m, Side& s, const float* log_u_dev);
 cudaError_t launch_set_potentials64(tu_market* m, Side& s, const double* log_u_dev);
-cudaError_t launch_get_potentials(tu_market* m, Side& s, float* out_dev);  // FP64 state -> FP32
+// FP64 state -> FP32 (either may be null)
+cudaError_t launch_get_potentials(tu_market* m, float* out_x, float* out_y);
 cudaError_t launch_row_norms(tu_market* m, Side& s, float* out_max);
 // FP8 markets: max |entry| of the FP32 factor pair (A, B: rows x d each) into *out_max
 cudaError_t launch_max_abs(tu_market* m, const float* A, const float* B, int64_t count, float* out_max);
@@ -632,13 +633,13 @@ __device__ __forceinline__ void pair_add(float& hi, float& lo, float h2, float l
 struct GroupTotal {
   float lmax, top, hi, lo;
 };
-__device__ __forceinline__ GroupTotal block_reduce_groups(const float4* __restrict__ grp, int64_t ng, float* red) {
+__device__ __forceinline__ GroupTotal block_reduce_groups(const float4* grp, int64_t ng, float* red) {
   float mm = -INFINITY, me = -INFINITY;
-  const float4 q0 = (int64_t)threadIdx.x < ng ? grp[threadIdx.x] : make_float4(-INFINITY, 0.0f, -INFINITY, 0.0f);
+  const float4 q0 = (int64_t)threadIdx.x < ng ? __ldcg(grp + threadIdx.x) : make_float4(-INFINITY, 0.0f, -INFINITY, 0.0f);
   mm = fmaxf(mm, q0.x);
   me = fmaxf(me, q0.z);
   for (int64_t i = threadIdx.x + blockDim.x; i < ng; i += blockDim.x) {
-    const float4 q = grp[i];
+    const float4 q = __ldcg(grp + i);
     mm = fmaxf(mm, q.x);
     me = fmaxf(me, q.z);
   }
@@ -649,7 +650,7 @@ __device__ __forceinline__ GroupTotal block_reduce_groups(const float4* __restri
   float hi = 0.0f, lo = 0.0f;
   if (q0.x > -INFINITY || isnan(q0.y)) pair_add(hi, lo, q0.y * expf(q0.x - r.top), 0.0f);
   for (int64_t i = threadIdx.x + blockDim.x; i < ng; i += blockDim.x) {
-    const float4 q = grp[i];
+    const float4 q = __ldcg(grp + i);
     if (q.x > -INFINITY || isnan(q.y)) pair_add(hi, lo, q.y * expf(q.x - r.top), 0.0f);
   }
   for (int o = 16; o > 0; o >>= 1)
