@@ -21,7 +21,7 @@
 //                it), plus a bulk copy of each partner tile's 128 g values
 //                (e4m3 factors: and of its 128 row scales) into an 8-slot ring
 //                that the epilogue reads with broadcast loads.
-//   warp 1     : MMA issuer (one thread): two tcgen05.mma M=128 N=128 chains
+//   warp 1     : MMA issuer: two tcgen05.mma M=128 N=128 chains
 //                (own rows 0-127 and 128-255) per partner tile into one of two
 //                TMEM accumulator buffers (2 x 256 columns = all 512).
 //   warps 2-17 : epilogue: epilogue warp e reads TMEM lane quadrant (e+2)%4
@@ -1025,9 +1025,22 @@ __global__ void __launch_bounds__(kThreads, 1)
     __syncwarp();
   } else if (warp == 1) {
     // ------------------------------------------------------------ MMA issuer
-    if (lane == 0) {
-      constexpr uint32_t idesc = F8 ? idesc_e4m3_f32(128, kFusedPartnerRows) : idesc_bf16_f32(128, kFusedPartnerRows);
-      constexpr uint32_t idesc_fold = idesc_bf16_f32(128, kFusedPartnerRows);  // (BF16 in every format)
+    // The whole warp runs the loop, and one elected lane the tensor-core
+    // instructions: what they are given (descriptors as a base per operand and
+    // constants added to it, addresses) then stays in uniform registers. With the
+    // loop on one lane each of them was moved there before every MMA, and issuing
+    // was the bound: about 100 cycles per MMA that takes 64.
+    {
+      constexpr int M = 128;
+      constexpr uint32_t idesc = F8 ? idesc_e4m3_f32(M, kFusedPartnerRows) : idesc_bf16_f32(M, kFusedPartnerRows);
+      constexpr uint32_t idesc_fold = idesc_bf16_f32(M, kFusedPartnerRows);  // (BF16 in every format)
+      auto ready = [&](uint64_t* bar, uint32_t ph) {
+        const bool got = __all_sync(0xffffffffu, mbar_wait(bar, ph, abort_flag));
+        tc_fence_after();
+        return got;
+      };
+      const uint64_t a_base = sdesc_sw128(smem_u32(sA)), b_base = sdesc_sw128(smem_u32(sB));
+      const uint64_t ones = sdesc_none(smem_u32(sOnes), 128, 256), gc_base = sdesc_none(smem_u32(sB), 128, 256);
       int stage = 0, buf = 0, ab = 0;
       uint32_t phase = 0, tphase = 0, a_phase = 0;
       bool ok = true;
@@ -1040,68 +1053,75 @@ __global__ void __launch_bounds__(kThreads, 1)
           jb = sg.jb;
           je = sg.je;
         }
-        if (!mbar_wait(&a_full[ab], a_phase, abort_flag)) {
+        if (!ready(&a_full[ab], a_phase)) {
           ok = false;
           break;
         }
-        tc_fence_after();
-        const uint32_t a0 = smem_u32(sA + ab * KB * kOwnBytesPerKB);
+        // (descriptors hold shared addresses in units of 16 bytes in their low bits)
+        const uint64_t a0 = a_base + (uint32_t)(ab * KB * (kOwnBytesPerKB >> 4));
         uint64_t* a_release = &a_empty[ab];
         if (++ab == ABUF) {
           ab = 0;
           a_phase ^= 1u;
         }
         for (int j = jb; j < je && ok; ++j) {
-          if (!mbar_wait(&tempty[buf], tphase ^ 1u, abort_flag)) {
+          if (!ready(&tempty[buf], tphase ^ 1u)) {
             ok = false;
             break;
           }
           for (int sp = 0; sp < SPT; ++sp) {
-            if (!mbar_wait(&full[stage], phase, abort_flag)) {
+            if (!ready(&full[stage], phase)) {
               ok = false;
               break;
             }
-            tc_fence_after();
-            const uint32_t b0 = smem_u32(sB + stage * SB);
+            if (elect_one()) {
+              const uint64_t b0 = b_base + (uint32_t)(stage * (SB >> 4));
 #pragma unroll
-            for (int h = 0; h < (SMALL ? 1 : 2); ++h) {
-              const uint32_t d_tmem = tmem_base + (uint32_t)(buf * 256 + h * 128);
+              for (int h = 0; h < (SMALL ? 1 : 2); ++h) {
+                const uint32_t d_tmem = tmem_base + (uint32_t)(buf * 256 + h * 128);
 #pragma unroll
-              for (int k = 0; k < KBS * 4; ++k) {
-                const int kbl = k >> 2, kk = k & 3;
-                const int kb = sp * KBS + kbl;  // k block within the packed row
-                const uint64_t adesc = sdesc_sw128(a0 + kb * kOwnBytesPerKB + h * 128 * 128 + kk * 32);
-                const uint64_t bdesc = sdesc_sw128(b0 + kbl * kPartnerBytesPerKB + kk * 32);
-                const uint32_t accum = (sp > 0 || k > 0) ? 1u : 0u;
-                if constexpr (F8) {
-                  umma_e4m3(d_tmem, adesc, bdesc, idesc, accum);
-                } else {
-                  umma_bf16(d_tmem, adesc, bdesc, idesc, accum);
+                for (int k = 0; k < KBS * 4; ++k) {
+                  const int kbl = k >> 2, kk = k & 3;
+                  const uint64_t adesc =
+                      a0 + (uint32_t)(sp * KBS * (kOwnBytesPerKB >> 4)) +
+                      (uint32_t)((kbl * kOwnBytesPerKB + h * 128 * 128 + kk * 32) >> 4);
+                  const uint64_t bdesc = b0 + (uint32_t)((kbl * kPartnerBytesPerKB + kk * 32) >> 4);
+                  const uint32_t accum = (sp > 0 || k > 0) ? 1u : 0u;
+                  if constexpr (F8) {
+                    umma_e4m3(d_tmem, adesc, bdesc, idesc, accum);
+                  } else {
+                    umma_bf16(d_tmem, adesc, bdesc, idesc, accum);
+                  }
+                }
+                if constexpr (FOLD) {
+                  // D += ones x (g / c): every row gets the partner column's g / c
+                  if (sp == SPT - 1) {
+                    const uint64_t gc = gc_base + (uint32_t)((stage * SB + KBS * kPartnerBytesPerKB) >> 4);
+                    umma_bf16(d_tmem, ones, gc, idesc_fold, 1u);
+                  }
                 }
               }
-              if constexpr (FOLD) {
-                // D += ones x (g / c): every row gets the partner column's g / c
-                if (sp == SPT - 1)
-                  umma_bf16(d_tmem, sdesc_none(smem_u32(sOnes), 128, 256),
-                            sdesc_none(b0 + KBS * kPartnerBytesPerKB, 128, 256), idesc_fold, 1u);
+              umma_commit(&empty[stage]);
+              if (sp == SPT - 1) {
+                umma_commit(&tfull[buf]);
+                if (j == je - 1) umma_commit(a_release);
               }
             }
-            umma_commit(&empty[stage]);
+            __syncwarp();
             if (++stage == STAGES) {
               stage = 0;
               phase ^= 1u;
             }
           }
           if (!ok) break;
-          umma_commit(&tfull[buf]);
-          if (j == je - 1) umma_commit(a_release);
           buf ^= 1;
           if (buf == 0) tphase ^= 1u;
         }
       }
-      if (!ok && !*abort_flag) raise_error(p.err, abort_flag, kErrTimeout);
-      // all MMAs issued by this thread complete before TMEM is released
-      umma_commit(mma_done);
+      if (!ok && lane == 0 && !*abort_flag) raise_error(p.err, abort_flag, kErrTimeout);
+      // all MMAs issued by this warp complete before TMEM is released
+      if (elect_one()) umma_commit(mma_done);
+      __syncwarp();
       mbar_wait_drain(mma_done, 0, 100000000ull);
     }
     __syncwarp();
