@@ -676,6 +676,7 @@ tu_status tu_batch_create(const tu_market_t* markets, int count, void* stream, t
       d.num_partner_tiles = (int)((par.rows + kFusedPartnerRows - 1) / kFusedPartnerRows);
       d.cut_t0 = own.cut.t0;
       d.cut_span = own.cut.span;
+      d.cut_rows = own.cut.pair ? 2 * kFusedOwnRows : kFusedOwnRows;
       d.slot0 = (int)slot;
       d.c = m->cmul;
       if (side == 0) b->c_host[i] = m->cmul;

@@ -49,9 +49,11 @@ cudaError_t make_map(CUtensorMap* map, const void* base, int64_t rows, int64_t k
 cudaError_t set_kernel_attributes_now() {
   cudaError_t e = set_attributes_mode<kModeSweep, false>();
   if (e == cudaSuccess) e = set_attributes_mode<kModeSweep, true>();
+  if (e == cudaSuccess) e = set_pair_attributes<kModeSweep>();
   if (e == cudaSuccess) e = set_out_attributes();
-  // the allocation-free entry point's unfolded half-sweep (rows of one k block)
+  // the allocation-free entry point's unfolded half-sweep 
   if (e == cudaSuccess) e = set_attribute_one<1, kModeSweep, false, kFmtBF16, false, false, true>();
+  if (e == cudaSuccess) e = set_attribute_one<2, kModeSweep, false, kFmtBF16, false, false, true>();
   return e;
 }
 
@@ -75,6 +77,23 @@ cudaError_t set_kernel_attributes() {
 // The operand format of a market's dtype.
 int fmt_of(int dtype) {
   return dtype == TU_DTYPE_FP8E4M3 ? kFmtE4M3Rows : (dtype == TU_DTYPE_FP8E4M3_SIDE ? kFmtE4M3Side : kFmtBF16);
+}
+
+// Tensor map over a side's folded operand (4 KB per 128 users) as rows of 256
+// bytes, 8 to a box: the half of a tile that one CTA of a pair loads.
+cudaError_t make_fold_map(Side* sd) {
+  memset(&sd->tm_fold, 0, sizeof(sd->tm_fold));
+  if (sd->fold == nullptr) return cudaSuccess;
+  EncodeTiledFn enc = get_encode_fn();
+  if (enc == nullptr) return cudaErrorNotSupported;
+  const cuuint64_t dims[2] = {64, (cuuint64_t)(sd->rows_pad / 8)};
+  const cuuint64_t strides[1] = {256};
+  const cuuint32_t box[2] = {64, 8};
+  const cuuint32_t estr[2] = {1, 1};
+  const CUresult r = enc(&sd->tm_fold, CU_TENSOR_MAP_DATA_TYPE_UINT32, 2, sd->fold, dims, strides, box, estr,
+                         CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_NONE, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
+                         CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
+  return r == CUDA_SUCCESS ? cudaSuccess : cudaErrorInvalidValue;
 }
 
 // 128-row own tiles when they all fit one wave (and the market allows them):
@@ -102,6 +121,7 @@ FusedParams base_params(int64_t rows, int64_t row0, int64_t col0, int64_t ncols,
   p.c = c;
   p.split = 1;
   p.cut_t0 = p.num_own_tiles;
+  p.cut_rows = kFusedOwnRows;
   return p;
 }
 
@@ -138,6 +158,10 @@ cudaError_t fused_prepare(tu_market* m) {
   cudaError_t e;
   if ((e = make_map(&m->X.tm_own, x, m->X.rows, m->kp, kFusedOwnRows, f8)) != cudaSuccess) return e;
   if ((e = make_map(&m->X.tm_partner, x, m->X.rows, m->kp, kFusedPartnerRows, f8)) != cudaSuccess) return e;
+  for (Side* sd : {&m->X, &m->Y})
+    if ((e = make_fold_map(sd)) != cudaSuccess) return e;
+  if ((e = make_map(&m->X.tm_half, x, m->X.rows, m->kp, kFusedPartnerRows / 2, f8)) != cudaSuccess) return e;
+  if ((e = make_map(&m->Y.tm_half, y, m->Y.rows, m->kp, kFusedPartnerRows / 2, f8)) != cudaSuccess) return e;
   if ((e = make_map(&m->Y.tm_own, y, m->Y.rows, m->kp, kFusedOwnRows, f8)) != cudaSuccess) return e;
   if ((e = make_map(&m->Y.tm_partner, y, m->Y.rows, m->kp, kFusedPartnerRows, f8)) != cudaSuccess) return e;
   return set_kernel_attributes();
@@ -160,9 +184,15 @@ cudaError_t fused_prepare(tu_market* m) {
 // of two).
 constexpr int kSpanCost = 8, kTileCost = 4, kMinSpan = 4;
 
-CutPlan cut_plan(int64_t own_rows, int64_t partner_rows, int sms) {
+// Own sides of more rows run on pairs of CTAs.
+constexpr int kPairRows = 512;
+
+CutPlan cut_plan(int64_t own_rows, int64_t partner_rows, int kblocks, int sms) {
   CutPlan c;
-  const int64_t T = (own_rows + kFusedOwnRows - 1) / kFusedOwnRows;
+  c.pair = kblocks > 1 && sms % 2 == 0 && own_rows > kPairRows;
+  if (c.pair) sms /= 2;
+  const int tile = c.pair ? 2 * kFusedOwnRows : kFusedOwnRows;
+  const int64_t T = (own_rows + tile - 1) / tile;
   const int64_t P = (partner_rows + kFusedPartnerRows - 1) / kFusedPartnerRows;
   const int64_t w = T / sms, rest = T - w * sms;
   c.t0 = (int)T;
@@ -176,7 +206,7 @@ CutPlan cut_plan(int64_t own_rows, int64_t partner_rows, int sms) {
   return c;
 }
 
-int64_t cut_slots(const CutPlan& p) { return 2 * (int64_t)p.spans; }
+int64_t cut_slots(const CutPlan& p) { return (p.pair ? 4 : 2) * (int64_t)p.spans; }
 
 cudaError_t launch_fused_halfsweep(tu_market* m, int side, int residual, int update, int* nparts_out,
                                    int64_t row0, int64_t nrows) {
@@ -191,7 +221,8 @@ cudaError_t launch_fused_halfsweep(tu_market* m, int side, int residual, int upd
   const bool user_split = whole && !m->wide && m->split > 1 && m->split_part != nullptr;
   const bool cuts = !user_split && own.cut.span > 0;
   const bool cut_launch = cuts && whole && m->small_mode == 1 && m->cut_part != nullptr;
-  const bool small = !cut_launch && use_small_tiles(m, nrows);
+  const bool pair = !user_split && whole && own.cut.pair && m->small_mode == 1 && cuts == cut_launch;
+  const bool small = !cut_launch && !pair && use_small_tiles(m, nrows);
   FusedParams p = base_params(nrows, row0, 0, partner.rows, m->cmul, small);
   p.g = partner.pvec;
   p.lmax = m->st + kStShift;
@@ -228,17 +259,29 @@ cudaError_t launch_fused_halfsweep(tu_market* m, int side, int residual, int upd
     p.cut_span = own.cut.span;
     p.cut_spans = own.cut.spans;
     p.cut_ptiles = p.num_partner_tiles;
+    p.cut_rows = own.cut.pair ? 2 * kFusedOwnRows : kFusedOwnRows;
     if (cut_launch) {
       p.part = m->cut_part;
       p.part_m = m->cut_m;
       p.split_cnt = m->cut_cnt;
-      items = p.cut_t0 > 0 ? m->num_sms : p.cut_spans;
+      items = p.cut_t0 > 0 ? m->num_sms : (pair ? 2 : 1) * p.cut_spans;
     }
+  }
+  if (pair && !cut_launch) {
+    items = (items + 1) / 2 * 2;
+    p.cut_t0 = items / 2;
   }
   const int grid = grid_for_tiles(items, m->num_sms);
   *nparts_out = grid;
   const int fmt = fmt_of(m->dtype);
   const bool split = p.split > 1 || cut_launch;
+  if (pair) {
+    if (m->wide)
+      return launch_wide_pair(k_blocks(m->kp, fmt), fmt, split, &own.tm_own, &partner.tm_half, &partner.tm_fold, &p,
+                              grid, m->stream);
+    return launch_pair<kModeSweep>(k_blocks(m->kp, fmt), fmt, split, &own.tm_own, &partner.tm_half, &partner.tm_fold, &p,
+                              grid, m->stream);
+  }
   if (m->wide)
     return launch_wide_sweep(m->kp, fmt, own.tm_own, partner.tm_partner, p, grid, m->stream, small, split);
   return launch_sweep<kModeSweep>(m->kp, fmt, own.tm_own, partner.tm_partner, p, grid, m->stream, small, split);
@@ -319,7 +362,7 @@ cudaError_t launch_fused_halfsweep_raw(const FusedRaw& r, cudaStream_t stream, i
   // (no folded operand here: the instantiation with g from the shared ring)
   if (r.kp == kKBlock) return launch_kernel<1, kModeSweep, false, kFmtBF16, false, false, true>(own_map, partner_map, p,
                                                                                               grid, stream);
-  return launch_any<kModeSweep>(r.kp, kFmtBF16, own_map, partner_map, p, grid, stream);
+  return launch_kernel<2, kModeSweep, false, kFmtBF16, false, false, true>(own_map, partner_map, p, grid, stream);
 }
 
 // One half-sweep over the items of many markets (batched launch). The

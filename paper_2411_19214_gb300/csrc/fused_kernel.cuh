@@ -119,7 +119,8 @@ struct FusedParams {
   int cut_span;
   int cut_spans;
   int cut_ptiles;          // partner tiles of the market
-  // folded g (BF16 half-sweeps, kp = 64): the partner side's g / c as the
+  int cut_rows;            // rows of the tiles that are cut
+  // folded g (see fold_for): the partner side's g / c as the
   // K = 16 operand of one extra MMA per chain and partner tile, 4 KB per
   // partner tile of 128 rows in the unswizzled K-major layout (written by the
   // preparation kernel)
@@ -148,7 +149,8 @@ constexpr int kABufs = KB == 1 ? 2 : 1;
 // BF16, 256 in e4m3) a whole 64 KB partner tile would leave room for one
 // stage beside the 128 KB own tile, so a stage then carries one k block and a
 // partner tile takes four stages.
-constexpr int kbs_for(int KB) { return KB == 4 ? 1 : KB; }
+// A pair's CTAs hold half of a partner tile each, so two k blocks fit there.
+constexpr int kbs_for(int KB, bool pair = false) { return KB == 4 ? (pair ? 2 : 1) : KB; }
 
 
 // shared memory: [A: ABUFS x KB x 32 KB][B: STAGES x KBS x 16 KB][g ring: 8 x 512 B]
@@ -157,23 +159,25 @@ constexpr int kbs_for(int KB) { return KB == 4 ? 1 : KB; }
 constexpr int kTailBytes = 512 + 512 + 2 * kFusedOwnRows * 4;
 // folded g: the partner tile's K = 16 operand rides in its (last) stage, the
 // own side's constant operand (ones in columns 0-2) is one tile of its own.
-// Taken for rows of one k block (d <= 32 in BF16, d <= 64 in e4m3 with one
-// scale per side), where the tensor pipe has room for a fifth MMA per chain
-// and the epilogue sheds its g loads: batched d = 32 half-sweep 5.44 -> 5.12
-// ms, a 1e5 d = 32 sweep 3.54 -> 3.37 ms; with two BF16 k blocks (d =
-// 33..64) the ninth MMA costs more than it saves (1e6 d = 64 half-sweep
-// 184.5 -> 187.1 ms), so those keep g in the shared ring. e4m3 rows with one
-// scale per side: 1e6 d = 64 half-sweep 149.4 -> 142.5 ms; there the fold MMA
-// is a separate kind::f16 MMA (BF16 ones x BF16 g / c) into the same FP32
-// accumulator. e4m3 rows with per-row scales cannot fold: the own row's scale
-// multiplies phi, so no per-column constant added to it gives g in every row.
+// Taken for rows of one and two k blocks (d <= 64 in BF16, d <= 128 in e4m3 with
+// one scale per side), where the tensor pipe has room for one more MMA per
+// chain and the epilogue, which bounds these kernels, sheds its g loads.
+// One block: batched d = 32 half-sweep 5.44 -> 5.12 ms, a 1e5 d = 32 sweep
+// 3.54 -> 3.37 ms. Two blocks, on pairs of CTAs: a 100,003 x 79,999 d = 64 sweep
+// 2.74 -> 2.60 ms (without pairs 2.73 -> 2.80: shared memory is short). With four
+// blocks the tensor pipe is the bound. e4m3: the fold MMA is a separate
+// kind::f16 MMA (BF16 ones x BF16 g / c) into the same FP32 accumulator. e4m3
+// rows with per-row scales cannot fold: the own row's scale multiplies phi, so
+// no per-column constant added to it gives g in every row.
 constexpr int kFoldBytes = kFusedPartnerRows * 32;
 constexpr bool fold_for(int KB, int MODE, bool BATCH, int fmt, bool nofold) {
-  return MODE == kModeSweep && (fmt == kFmtBF16 || fmt == kFmtE4M3Side) && KB == 1 && !nofold;
+  return MODE == kModeSweep && (fmt == kFmtBF16 || fmt == kFmtE4M3Side) && KB <= 2 && !nofold;
 }
-constexpr int stage_bytes(int KB, bool fold) { return kbs_for(KB) * kPartnerBytesPerKB + (fold ? kFoldBytes : 0); }
-constexpr int smem_bytes(int KB, int fmt, int stages, bool fold = false) {
-  return 1024 /*alignment slack*/ + (KB == 1 ? 2 : 1) * KB * kOwnBytesPerKB + stages * stage_bytes(KB, fold) +
+constexpr int stage_bytes(int KB, bool fold, bool pair = false) {
+  return (kbs_for(KB, pair) * kPartnerBytesPerKB + (fold ? kFoldBytes : 0)) / (pair ? 2 : 1);
+}
+constexpr int smem_bytes(int KB, int fmt, int stages, bool fold = false, bool pair = false) {
+  return 1024 /*alignment slack*/ + (KB == 1 ? 2 : 1) * KB * kOwnBytesPerKB + stages * stage_bytes(KB, fold, pair) +
          (fold ? kFoldBytes : 0) + kGSlots * kGBytes * (fmt == kFmtE4M3Rows ? 2 : 1) + kTailBytes;
 }
 
@@ -716,17 +720,20 @@ __device__ __forceinline__ int cut_slot(const FusedParams& p, int u, int k) {
 // to stay in L2) against every own tile before the next; SPLIT with p.split =
 // 1, the whole tiles and then the CTA's span of the cut ones. False past the
 // last one. (Batched: the market's descriptor comes from batch_item.)
-template <bool BATCH, bool SPLIT>
+// PAIR: the same for both CTAs of a pair, in tiles of 512 rows.
+template <bool BATCH, bool SPLIT, bool PAIR>
 __device__ __forceinline__ bool item_at(const FusedParams& p, int i, Seg& sg) {
   const int npt = p.num_partner_tiles;
+  const int tiles = PAIR ? (p.num_own_tiles + 1) / 2 : p.num_own_tiles;
+  const int cta = PAIR ? (int)blockIdx.x / 2 : (int)blockIdx.x, ctas = PAIR ? (int)gridDim.x / 2 : (int)gridDim.x;
   if constexpr (BATCH) {
     sg.t = p.cta_start[blockIdx.x] + i;  // the index in the item list
     return sg.t < p.cta_start[blockIdx.x + 1];
   }
-  const int it = (int)blockIdx.x + i * (int)gridDim.x;
+  const int it = cta + i * ctas;
   if constexpr (!SPLIT) {
     sg = {it, 0, npt, 0, 1};
-    return it < p.num_own_tiles;
+    return it < tiles;
   }
   if (p.split > 1) {
     const int S = p.split;
@@ -747,9 +754,9 @@ __device__ __forceinline__ bool item_at(const FusedParams& p, int i, Seg& sg) {
     return true;
   }
   // (with whole tiles the grid divides cut_t0, so every CTA has the same number of them)
-  const int q = i - p.cut_t0 / (int)gridDim.x, k = (int)blockIdx.x;
+  const int q = i - p.cut_t0 / ctas, k = cta;
   if (p.cut_span == 0 || k >= p.cut_spans || q > 1) return false;
-  const int lo = k * p.cut_span, end = (p.num_own_tiles - p.cut_t0) * npt;
+  const int lo = k * p.cut_span, end = (tiles - p.cut_t0) * npt;
   const int hi = lo + p.cut_span < end ? lo + p.cut_span : end;
   const int u = lo / npt + q, u0 = u * npt;
   if (u0 >= hi) return false;
@@ -781,8 +788,8 @@ struct RangeSum {
 // The partner tile before which a row's sum is next cut at or after `from`
 // (none: a number that no tile has).
 constexpr int kNoCut = 0x7fffffff;
-__device__ __forceinline__ int next_cut(int64_t row, int t0, int span, int ptiles) {
-  const int64_t t = row / kFusedOwnRows;
+__device__ __forceinline__ int next_cut(int64_t row, int rows, int t0, int span, int ptiles) {
+  const int64_t t = row / rows;
   if (span == 0 || t < t0) return kNoCut;
   const int u0 = (int)(t - t0) * ptiles, c = (u0 / span + 1) * span - u0;
   return c < ptiles ? c : kNoCut;
@@ -804,11 +811,23 @@ __device__ __forceinline__ int next_cut(int64_t row, int t0, int span, int ptile
 // finishing its rows in about half the time. Every row's arithmetic is the
 // same as with 256-row tiles.
 // CUTS (and BATCH): launches that run a cut row's ranges in turn.
+// PAIR: the CTAs of a cluster of two share every partner tile. The first one's
+// MMA warp issues M = 256 MMAs (cta_group::2) over both CTAs' own rows; each
+// CTA loads and holds half of the tile's rows, so the tensor core's reads of
+// shared memory per tile and SM fall from 128 KB to 96 (A's 128 rows and B's
+// 64 per instruction instead of 128 and 128) and the copies from 32 KB to 16.
+// That pays where the operands are long (d = 100, 50,001 x 70,000: 2.18 -> 1.75
+// ms per sweep) and makes room for the folded g at d = 64 (100,003 x 79,999:
+// 2.73 -> 2.60, 300,000 x 300,000: 31.3 -> 29.4). The epilogue warps of the
+// second CTA announce a read buffer by a plain remote arrival; a releasing one at
+// cluster scope stalled them (300,000 x 300,000: 41.7 ms). Handing each sub-tile
+// over by itself was slower (33.2 -> 35.4), releasing a buffer before its
+// arithmetic and eight stages instead of six made no difference.
 template <int KB, int STAGES, int MODE, bool BATCH, int FMT, bool SMALL = false, bool SPLIT = false,
-          bool NOFOLD = false, bool CUTS = false>
+          bool NOFOLD = false, bool CUTS = false, bool PAIR = false>
 __global__ void __launch_bounds__(kThreads, 1)
     k_fused_halfsweep(const __grid_constant__ CUtensorMap tm_own, const __grid_constant__ CUtensorMap tm_partner,
-                      const FusedParams p) {
+                      const __grid_constant__ CUtensorMap tm_fold, const FusedParams p) {
   static_assert(!BATCH || MODE == kModeSweep, "batched launches run half-sweeps only");
   constexpr bool WIDE = MODE == kModeSweepWide;
   constexpr bool kSweepLike = MODE == kModeSweep || WIDE;
@@ -817,16 +836,17 @@ __global__ void __launch_bounds__(kThreads, 1)
                 "partner splits are single-market half-sweeps and mu blocks");
   static_assert(!CUTS || (kSweepLike && !SPLIT && !BATCH), "ranges in turn: unsplit half-sweeps");
   static_assert(!(BATCH && SMALL), "batched launches use 256-row own tiles");
+  static_assert(!PAIR || (kSweepLike && KB > 1 && !BATCH && !SMALL && !NOFOLD && !CUTS), "pairs: half-sweeps");
   constexpr int kOwn = SMALL ? kFusedOwnRows / 2 : kFusedOwnRows;  // rows of an own tile
   static_assert(KB == 1 || KB == 2 || KB == 4, "128-byte k blocks per row");
   constexpr bool F8 = FMT != kFmtBF16;      // e4m3 operands
   constexpr bool RS = FMT == kFmtE4M3Rows;  // per-row scales
   constexpr int ABUF = kABufs<KB>;
-  constexpr int KBS = kbs_for(KB);   // k blocks per partner stage
+  constexpr int KBS = kbs_for(KB, PAIR);  // k blocks per partner stage
   constexpr int SPT = KB / KBS;      // stages per partner tile
   constexpr int XB = F8 ? 128 : kKBlock;  // elements per 128-byte k block (TMA x coordinate step)
   constexpr bool FOLD = fold_for(KB, MODE, BATCH, FMT, NOFOLD);  // g added by an extra MMA
-  constexpr int SB = stage_bytes(KB, FOLD);                        // bytes per partner stage
+  constexpr int SB = stage_bytes(KB, FOLD, PAIR);                        // bytes per partner stage
   extern __shared__ uint8_t smem_raw[];
   const uint32_t raw_u32 = smem_u32(smem_raw);
   uint8_t* smem = smem_raw + (((raw_u32 + 1023u) & ~1023u) - raw_u32);
@@ -864,6 +884,8 @@ __global__ void __launch_bounds__(kThreads, 1)
   static_assert((2 * STAGES + 2 * kGSlots + 13) * 8 + 8 <= 512, "barrier area");
 
   const int warp = threadIdx.x / 32, lane = threadIdx.x % 32;
+  const int rank = PAIR ? (int)cluster_rank() : 0;
+  constexpr int kParBytes = PAIR ? kPartnerBytesPerKB / 2 : kPartnerBytesPerKB;  // of a partner tile's k block here
 
   if (threadIdx.x == 0) {
     for (int s = 0; s < STAGES; ++s) {
@@ -880,7 +902,7 @@ __global__ void __launch_bounds__(kThreads, 1)
     }
     for (int b = 0; b < 2; ++b) {
       mbar_init(&tfull[b], 1);
-      mbar_init(&tempty[b], kEpiWarps);
+      mbar_init(&tempty[b], PAIR ? 2 * kEpiWarps : kEpiWarps);
     }
     mbar_init(mma_done, 1);
     for (int b = 0; b < 2; ++b) {
@@ -895,8 +917,13 @@ __global__ void __launch_bounds__(kThreads, 1)
     }
   }
   if (warp == 0) {
-    tmem_alloc(tmem_slot, kTmemCols);
-    tmem_relinquish();
+    if constexpr (PAIR) {
+      tmem_alloc_pair(tmem_slot, kTmemCols);
+      tmem_relinquish_pair();
+    } else {
+      tmem_alloc(tmem_slot, kTmemCols);
+      tmem_relinquish();
+    }
   }
   if constexpr (FOLD) {
     // the own side's operand of the extra MMA: BF16 ones in columns 0-2 of
@@ -915,7 +942,11 @@ __global__ void __launch_bounds__(kThreads, 1)
       sts_u64(smem_u32(topk_list) + (uint32_t)(kTopKSlots * kEpiThreads + (int)threadIdx.x - 64) * 8u, 0ull);
   }
   tc_fence_before();
-  __syncthreads();
+  if constexpr (PAIR) {
+    cluster_sync();  // (the other CTA's barriers are initialised, too)
+  } else {
+    __syncthreads();
+  }
   tc_fence_after();
   const uint32_t tmem_base = *tmem_slot;
 
@@ -932,7 +963,7 @@ __global__ void __launch_bounds__(kThreads, 1)
       const BatchDesc* prev = nullptr;
       bool ok = true;
       Seg sg;
-      for (int i = 0; ok && item_at<BATCH, SPLIT>(p, i, sg); ++i) {
+      for (int i = 0; ok && item_at<BATCH, SPLIT, PAIR>(p, i, sg); ++i) {
         const BatchDesc* bd = nullptr;
         int t, jb = 0, je;
         if constexpr (BATCH) {
@@ -946,7 +977,7 @@ __global__ void __launch_bounds__(kThreads, 1)
             prev = bd;
           }
         } else {
-          t = sg.t;
+          t = PAIR ? 2 * sg.t + rank : sg.t;
           jb = sg.jb;
           je = sg.je;
         }
@@ -960,9 +991,15 @@ __global__ void __launch_bounds__(kThreads, 1)
           ok = false;
           break;
         }
-        mbar_arrive_expect_tx(&a_full[ab], KB * kOwnBytesPerKB);
-        for (int kb = 0; kb < KB; ++kb)
-          tma_load_2d(sA + (ab * KB + kb) * kOwnBytesPerKB, map_own, &a_full[ab], kb * XB, (int)arow);
+        if (rank == 0) mbar_arrive_expect_tx(&a_full[ab], (PAIR ? 2 : 1) * KB * kOwnBytesPerKB);
+        for (int kb = 0; kb < KB; ++kb) {
+          if constexpr (PAIR) {
+            tma_load_2d_pair(sA + (ab * KB + kb) * kOwnBytesPerKB, map_own, cluster_addr(&a_full[ab], 0), kb * XB,
+                             (int)arow);
+          } else {
+            tma_load_2d(sA + (ab * KB + kb) * kOwnBytesPerKB, map_own, &a_full[ab], kb * XB, (int)arow);
+          }
+        }
         ++a_armed[ab];
         if (++ab == ABUF) {
           ab = 0;
@@ -975,17 +1012,29 @@ __global__ void __launch_bounds__(kThreads, 1)
               break;
             }
             const bool fold_here = FOLD && sp == SPT - 1;  // the tile's g operand rides in its last stage
-            mbar_arrive_expect_tx(&full[stage], KBS * kPartnerBytesPerKB + (fold_here ? kFoldBytes : 0));
+            if (rank == 0) mbar_arrive_expect_tx(&full[stage], KBS * kPartnerBytesPerKB + (fold_here ? kFoldBytes : 0));
             for (int kb = 0; kb < KBS; ++kb) {
               const int px = (sp * KBS + kb) * XB, py = (int)(p.col0 + (int64_t)j * kFusedPartnerRows);
-              if (hint) {
-                tma_load_2d_hint(sB + stage * SB + kb * kPartnerBytesPerKB, map_partner, &full[stage], px, py,
-                                 keep_policy);
+              uint8_t* dst = sB + stage * SB + kb * kParBytes;
+              if constexpr (PAIR) {
+                const uint32_t bar = cluster_addr(&full[stage], 0);
+                const int y = py + rank * (kFusedPartnerRows / 2);
+                if (hint) {
+                  tma_load_2d_pair_hint(dst, map_partner, bar, px, y, keep_policy);
+                } else {
+                  tma_load_2d_pair(dst, map_partner, bar, px, y);
+                }
+              } else if (hint) {
+                tma_load_2d_hint(dst, map_partner, &full[stage], px, py, keep_policy);
               } else {
-                tma_load_2d(sB + stage * SB + kb * kPartnerBytesPerKB, map_partner, &full[stage], px, py);
+                tma_load_2d(dst, map_partner, &full[stage], px, py);
               }
             }
-            if (fold_here)
+            if (PAIR && fold_here) {
+              // (a plain bulk copy cannot be counted in the other CTA: through a tensor map, in rows of 256 bytes)
+              tma_load_2d_pair(sB + stage * SB + KBS * kParBytes, &tm_fold, cluster_addr(&full[stage], 0), 0,
+                               (j * 2 + rank) * (kFoldBytes / 512));
+            } else if (fold_here)
               bulk_load(sB + stage * SB + KBS * kPartnerBytesPerKB,
                         (BATCH ? bd->gfold : p.gfold) + (int64_t)j * kFoldBytes, kFoldBytes, &full[stage]);
             ++armed[stage];
@@ -1013,27 +1062,41 @@ __global__ void __launch_bounds__(kThreads, 1)
       }
       if (!ok) {
         if (!*abort_flag) raise_error(p.err, abort_flag, kErrTimeout);
-        // let the copies already issued land before the CTA's shared memory goes away
-        for (int s = 0; s < STAGES; ++s)
+        // let the copies already issued land before the CTA's shared memory goes
+        // away (a pair's second CTA cannot see the barriers they are counted on:
+        // it waits for longer than any copy takes)
+        if (PAIR && rank != 0) {
+          const uint64_t t0 = global_timer_ns();
+          while (global_timer_ns() - t0 < 10000000ull) {
+          }
+        }
+        for (int s = 0; s < STAGES && rank == 0; ++s)
           if (armed[s]) mbar_wait_drain(&full[s], (armed[s] - 1u) & 1u, 10000000ull);
         for (int s = 0; s < kGSlots; ++s)
           if (garmed[s]) mbar_wait_drain(&gfull[s], (garmed[s] - 1u) & 1u, 10000000ull);
-        for (int b = 0; b < ABUF; ++b)
+        for (int b = 0; b < ABUF && rank == 0; ++b)
           if (a_armed[b]) mbar_wait_drain(&a_full[b], (a_armed[b] - 1u) & 1u, 10000000ull);
       }
     }
     __syncwarp();
   } else if (warp == 1) {
-    // ------------------------------------------------------------ MMA issuer
+    // ------------------------------------------------------------ MMA issuer (a pair's: in its first CTA)
     // The whole warp runs the loop, and one elected lane the tensor-core
     // instructions: what they are given (descriptors as a base per operand and
     // constants added to it, addresses) then stays in uniform registers. With the
     // loop on one lane each of them was moved there before every MMA, and issuing
     // was the bound: about 100 cycles per MMA that takes 64.
-    {
-      constexpr int M = 128;
+    if (rank == 0) {
+      constexpr int M = PAIR ? 256 : 128;
       constexpr uint32_t idesc = F8 ? idesc_e4m3_f32(M, kFusedPartnerRows) : idesc_bf16_f32(M, kFusedPartnerRows);
       constexpr uint32_t idesc_fold = idesc_bf16_f32(M, kFusedPartnerRows);  // (BF16 in every format)
+      auto commit = [](uint64_t* bar) {
+        if constexpr (PAIR) {
+          umma_commit_pair(bar);
+        } else {
+          umma_commit(bar);
+        }
+      };
       auto ready = [&](uint64_t* bar, uint32_t ph) {
         const bool got = __all_sync(0xffffffffu, mbar_wait(bar, ph, abort_flag));
         tc_fence_after();
@@ -1045,7 +1108,7 @@ __global__ void __launch_bounds__(kThreads, 1)
       uint32_t phase = 0, tphase = 0, a_phase = 0;
       bool ok = true;
       Seg sg;
-      for (int i = 0; ok && item_at<BATCH, SPLIT>(p, i, sg); ++i) {
+      for (int i = 0; ok && item_at<BATCH, SPLIT, PAIR>(p, i, sg); ++i) {
         int jb = 0, je;
         if constexpr (BATCH) {
           je = batch_item(p, sg.t).d->num_partner_tiles;
@@ -1085,9 +1148,13 @@ __global__ void __launch_bounds__(kThreads, 1)
                   const uint64_t adesc =
                       a0 + (uint32_t)(sp * KBS * (kOwnBytesPerKB >> 4)) +
                       (uint32_t)((kbl * kOwnBytesPerKB + h * 128 * 128 + kk * 32) >> 4);
-                  const uint64_t bdesc = b0 + (uint32_t)((kbl * kPartnerBytesPerKB + kk * 32) >> 4);
+                  const uint64_t bdesc = b0 + (uint32_t)((kbl * kParBytes + kk * 32) >> 4);
                   const uint32_t accum = (sp > 0 || k > 0) ? 1u : 0u;
-                  if constexpr (F8) {
+                  if constexpr (PAIR && F8) {
+                    umma_e4m3_pair(d_tmem, adesc, bdesc, idesc, accum);
+                  } else if constexpr (PAIR) {
+                    umma_bf16_pair(d_tmem, adesc, bdesc, idesc, accum);
+                  } else if constexpr (F8) {
                     umma_e4m3(d_tmem, adesc, bdesc, idesc, accum);
                   } else {
                     umma_bf16(d_tmem, adesc, bdesc, idesc, accum);
@@ -1096,15 +1163,19 @@ __global__ void __launch_bounds__(kThreads, 1)
                 if constexpr (FOLD) {
                   // D += ones x (g / c): every row gets the partner column's g / c
                   if (sp == SPT - 1) {
-                    const uint64_t gc = gc_base + (uint32_t)((stage * SB + KBS * kPartnerBytesPerKB) >> 4);
-                    umma_bf16(d_tmem, ones, gc, idesc_fold, 1u);
+                    const uint64_t gc = gc_base + (uint32_t)((stage * SB + KBS * kParBytes) >> 4);
+                    if constexpr (PAIR) {
+                      umma_bf16_pair(d_tmem, ones, gc, idesc_fold, 1u);
+                    } else {
+                      umma_bf16(d_tmem, ones, gc, idesc_fold, 1u);
+                    }
                   }
                 }
               }
-              umma_commit(&empty[stage]);
+              commit(&empty[stage]);
               if (sp == SPT - 1) {
-                umma_commit(&tfull[buf]);
-                if (j == je - 1) umma_commit(a_release);
+                commit(&tfull[buf]);
+                if (j == je - 1) commit(a_release);
               }
             }
             __syncwarp();
@@ -1120,7 +1191,7 @@ __global__ void __launch_bounds__(kThreads, 1)
       }
       if (!ok && lane == 0 && !*abort_flag) raise_error(p.err, abort_flag, kErrTimeout);
       // all MMAs issued by this warp complete before TMEM is released
-      if (elect_one()) umma_commit(mma_done);
+      if (elect_one()) commit(mma_done);
       __syncwarp();
       mbar_wait_drain(mma_done, 0, 100000000ull);
     }
@@ -1165,7 +1236,7 @@ __global__ void __launch_bounds__(kThreads, 1)
     float thr = -INFINITY;
     int tile_iter = 0;
     Seg sg;
-    for (; ok && item_at<BATCH, SPLIT>(p, tile_iter, sg); ++tile_iter) {
+    for (; ok && item_at<BATCH, SPLIT, PAIR>(p, tile_iter, sg); ++tile_iter) {
       const BatchDesc* bd = nullptr;
       int t, jb = 0, je;
       if constexpr (BATCH) {
@@ -1174,7 +1245,7 @@ __global__ void __launch_bounds__(kThreads, 1)
         t = w.t;
         je = bd->num_partner_tiles;
       } else {
-        t = sg.t;
+        t = PAIR ? 2 * sg.t + rank : sg.t;
         jb = sg.jb;
         je = sg.je;
       }
@@ -1203,8 +1274,8 @@ __global__ void __launch_bounds__(kThreads, 1)
       int cut_at = kNoCut;
       bool was_cut = false;
       if constexpr (RANGES) {
-        cut_at = BATCH ? next_cut((int64_t)t * kFusedOwnRows, bd->cut_t0, bd->cut_span, je)
-                       : next_cut(p.row0 + r, p.cut_t0, p.cut_span, p.cut_ptiles);
+        cut_at = BATCH ? next_cut((int64_t)t * kFusedOwnRows, bd->cut_rows, bd->cut_t0, bd->cut_span, je)
+                       : next_cut(p.row0 + r, p.cut_rows, p.cut_t0, p.cut_span, p.cut_ptiles);
       }
       if constexpr (MODE == kModeMu) {
         if (row_ok) {
@@ -1269,7 +1340,13 @@ __global__ void __launch_bounds__(kThreads, 1)
         // this warp's part of the accumulator buffer has been read: hand it back to the MMA warp
         tc_fence_before();
         __syncwarp();
-        if (lane == 0) mbar_arrive(&tempty[buf]);
+        if (lane == 0) {
+          if constexpr (PAIR) {
+            cluster_arrive(cluster_addr(&tempty[buf], 0));
+          } else {
+            mbar_arrive(&tempty[buf]);
+          }
+        }
         if (!idle) {
           if constexpr (FOLD) chunk_sum_fold(vb, cc, acc);
           if constexpr (MODE == kModeSweep && !FOLD) chunk_sum<RS>(vb, gs4 + 8, fs4 + 8, cc, acc);
@@ -1434,9 +1511,10 @@ __global__ void __launch_bounds__(kThreads, 1)
             // the other warps of this block move on)
             const int64_t blk = (int64_t)t * (kFusedOwnRows / 32) + (h * 128 + q * 32) / 32;
             const bool cuts = p.split == 1;
-            const int u = t - p.cut_t0, k0 = cuts ? cut_first(p, u) : 0;
+            const int u = sg.t - p.cut_t0, k0 = cuts ? cut_first(p, u) : 0;
             auto slot = [&](int c) -> int64_t {
-              return cuts ? (int64_t)cut_slot(p, u, k0 + c) * kFusedOwnRows + rloc : (int64_t)c * p.rows + r;
+              return cuts ? ((int64_t)cut_slot(p, u, k0 + c) * (PAIR ? 2 : 1) + rank) * kFusedOwnRows + rloc
+                          : (int64_t)c * p.rows + r;
             };
             if (row_ok) {
               p.part[slot(sg.me)] = make_float4(sum, comp, other, other_comp);
@@ -1546,10 +1624,18 @@ __global__ void __launch_bounds__(kThreads, 1)
   }
 
   tc_fence_before();
-  __syncthreads();
+  if constexpr (PAIR) {
+    cluster_sync();  // the pair's MMAs read and write both CTAs
+  } else {
+    __syncthreads();
+  }
   if (warp == 0) {
     tc_fence_after();
-    tmem_dealloc(tmem_base, kTmemCols);
+    if constexpr (PAIR) {
+      tmem_dealloc_pair(tmem_base, kTmemCols);
+    } else {
+      tmem_dealloc(tmem_base, kTmemCols);
+    }
   }
 }
 
@@ -1561,19 +1647,19 @@ constexpr int kSmemLimit = 232448;  // dynamic shared memory per CTA (227 KB)
 // g (and scale) rings, the tail and (kModeTopKShared) the ranked lists, at
 // most 6 whole tiles (one k block per row), 4 (two) or 5 single k blocks
 // (four: 1.25 partner tiles in flight).
-constexpr int stages_for(int KB, int MODE, int fmt, bool fold, bool split, bool ranges) {
-  const int fixed = smem_bytes(KB, fmt, 0, fold) + mode_extra_bytes(MODE, KB, split, ranges);
-  const int fit = (kSmemLimit - fixed) / stage_bytes(KB, fold);
-  const int cap = KB == 1 ? 6 : (KB == 2 ? 4 : 5);
+constexpr int stages_for(int KB, int MODE, int fmt, bool fold, bool split, bool ranges, bool pair) {
+  const int fixed = smem_bytes(KB, fmt, 0, fold, pair) + mode_extra_bytes(MODE, KB, split, ranges);
+  const int fit = (kSmemLimit - fixed) / stage_bytes(KB, fold, pair);
+  const int cap = KB == 1 ? 6 : (KB == 2 ? (pair ? 6 : 4) : 5);
   return fit < cap ? fit : cap;
 }
 
-template <int KB, int MODE, int FMT, bool FOLD, bool SPLIT, bool RANGES>
-constexpr int kStages = stages_for(KB, MODE, FMT, FOLD, SPLIT, RANGES);
+template <int KB, int MODE, int FMT, bool FOLD, bool SPLIT, bool RANGES, bool PAIR = false>
+constexpr int kStages = stages_for(KB, MODE, FMT, FOLD, SPLIT, RANGES, PAIR);
 
-template <int KB, int MODE, int FMT, bool FOLD, bool SPLIT, bool RANGES>
+template <int KB, int MODE, int FMT, bool FOLD, bool SPLIT, bool RANGES, bool PAIR = false>
 constexpr int kSmemTotal =
-    smem_bytes(KB, FMT, kStages<KB, MODE, FMT, FOLD, SPLIT, RANGES>, FOLD) + mode_extra_bytes(MODE, KB, SPLIT, RANGES);
+    smem_bytes(KB, FMT, kStages<KB, MODE, FMT, FOLD, SPLIT, RANGES, PAIR>, FOLD, PAIR) + mode_extra_bytes(MODE, KB, SPLIT, RANGES);
 
 // Instantiations that exist: batched launches take one or two k blocks
 // (e4m3: one); the shared-memory ranked lists leave too little room for
@@ -1607,7 +1693,7 @@ cudaError_t launch_kernel(const CUtensorMap& own, const CUtensorMap& partner, co
     static_assert(kSmem <= kSmemLimit, "shared memory budget");
     if (FD && !BATCH && p.gfold == nullptr) return cudaErrorInvalidValue;  // the folded operand must be prepared
     k_fused_halfsweep<KB, kStages<KB, MODE, FMT, FD, SPLIT, CUTS || BATCH>, MODE, BATCH, FMT, SMALL, SPLIT, NOFOLD, CUTS>
-        <<<grid, kThreads, kSmem, stream>>>(own, partner, p);
+        <<<grid, kThreads, kSmem, stream>>>(own, partner, partner, p);
     return cudaGetLastError();
   }
 }
@@ -1690,6 +1776,60 @@ cudaError_t launch_any(int64_t kp, int fmt, const CUtensorMap& own, const CUtens
   return launch_variant<MODE, BATCH, false>(kp, fmt, own, partner, p, grid, stream);
 }
 
+// Pairs of CTAs (kb > 1): the pair kernel's attributes and launch.
+template <int KB, int MODE, int FMT, bool SPLIT>
+cudaError_t pair_kernel(const CUtensorMap* own, const CUtensorMap* half, const CUtensorMap* fold, const FusedParams* p,
+                        int grid, cudaStream_t stream) {
+  constexpr bool FD = fold_for(KB, MODE, false, FMT, false);
+  constexpr int kSt = kStages<KB, MODE, FMT, FD, SPLIT, false, true>;
+  constexpr int kSmem = kSmemTotal<KB, MODE, FMT, FD, SPLIT, false, true>;
+  static_assert(kSt >= 4 && kSmem <= kSmemLimit, "shared memory budget");
+  auto kern = k_fused_halfsweep<KB, kSt, MODE, false, FMT, false, SPLIT, false, false, true>;
+  if (p == nullptr) return cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmem);
+  cudaLaunchAttribute attr;
+  attr.id = cudaLaunchAttributeClusterDimension;
+  attr.val.clusterDim.x = 2;
+  attr.val.clusterDim.y = attr.val.clusterDim.z = 1;
+  cudaLaunchConfig_t c = {};
+  c.gridDim = dim3((unsigned)grid);
+  c.blockDim = dim3(kThreads);
+  c.dynamicSmemBytes = kSmem;
+  c.stream = stream;
+  c.attrs = &attr;
+  c.numAttrs = 1;
+  return cudaLaunchKernelEx(&c, kern, *own, *half, *fold, *p);
+}
+template <int MODE, int FMT>
+cudaError_t pair_fmt(int kb, bool split, const CUtensorMap* own, const CUtensorMap* half, const CUtensorMap* fold,
+                     const FusedParams* p, int grid,
+                     cudaStream_t stream) {
+  if (kb == 2)
+    return split ? pair_kernel<2, MODE, FMT, true>(own, half, fold, p, grid, stream)
+                 : pair_kernel<2, MODE, FMT, false>(own, half, fold, p, grid, stream);
+  if (kb == 4)
+    return split ? pair_kernel<4, MODE, FMT, true>(own, half, fold, p, grid, stream)
+                 : pair_kernel<4, MODE, FMT, false>(own, half, fold, p, grid, stream);
+  return cudaErrorNotSupported;
+}
+// p == nullptr: set the attributes
+template <int MODE>
+cudaError_t launch_pair(int kb, int fmt, bool split, const CUtensorMap* own, const CUtensorMap* half,
+                        const CUtensorMap* fold, const FusedParams* p, int grid, cudaStream_t stream) {
+  if (fmt == kFmtE4M3Rows) return pair_fmt<MODE, kFmtE4M3Rows>(kb, split, own, half, fold, p, grid, stream);
+  if (fmt == kFmtE4M3Side) return pair_fmt<MODE, kFmtE4M3Side>(kb, split, own, half, fold, p, grid, stream);
+  return pair_fmt<MODE, kFmtBF16>(kb, split, own, half, fold, p, grid, stream);
+}
+template <int MODE>
+cudaError_t set_pair_attributes() {
+  for (int kb : {2, 4})
+    for (int fmt : {(int)kFmtBF16, (int)kFmtE4M3Side, (int)kFmtE4M3Rows})
+      for (bool split : {false, true}) {
+        const cudaError_t e = launch_pair<MODE>(kb, fmt, split, nullptr, nullptr, nullptr, nullptr, 0, nullptr);
+        if (e != cudaSuccess) return e;
+      }
+  return cudaSuccess;
+}
+
 // Half-sweeps of one market: split over CTAs (by the caller's ranges or the
 // market's cuts), a cut row's ranges in turn, or plain.
 template <int MODE>
@@ -1711,6 +1851,8 @@ cudaError_t launch_sweep(int64_t kp, int fmt, const CUtensorMap& own, const CUte
 cudaError_t set_out_attributes();
 cudaError_t launch_wide_sweep(int64_t kp, int fmt, const CUtensorMap& own, const CUtensorMap& partner,
                               const FusedParams& p, int grid, cudaStream_t stream, bool small, bool split);
+cudaError_t launch_wide_pair(int kb, int fmt, bool split, const CUtensorMap* own, const CUtensorMap* half,
+                             const CUtensorMap* fold, const FusedParams* p, int grid, cudaStream_t stream);
 cudaError_t launch_lists(int64_t kp, int fmt, const CUtensorMap& own, const CUtensorMap& partner,
                          const FusedParams& p, int grid, cudaStream_t stream, bool small);
 cudaError_t launch_mu(int64_t kp, int fmt, const CUtensorMap& own, const CUtensorMap& partner, const FusedParams& p,

@@ -9,12 +9,18 @@ cudaError_t set_out_attributes() {
   if (e == cudaSuccess) e = set_attributes_mode<kModeMu, false>();
   if (e == cudaSuccess) e = set_attributes_mode<kModeTopKShared, false>();
   if (e == cudaSuccess) e = set_attributes_mode<kModeSweepWide, false>();
+  if (e == cudaSuccess) e = set_pair_attributes<kModeSweepWide>();
   return e;
 }
 
 cudaError_t launch_wide_sweep(int64_t kp, int fmt, const CUtensorMap& own, const CUtensorMap& partner,
                               const FusedParams& p, int grid, cudaStream_t stream, bool small, bool split) {
   return launch_sweep<kModeSweepWide>(kp, fmt, own, partner, p, grid, stream, small, split);
+}
+
+cudaError_t launch_wide_pair(int kb, int fmt, bool split, const CUtensorMap* own, const CUtensorMap* half,
+                             const CUtensorMap* fold, const FusedParams* p, int grid, cudaStream_t stream) {
+  return launch_pair<kModeSweepWide>(kb, fmt, split, own, half, fold, p, grid, stream);
 }
 
 cudaError_t launch_lists(int64_t kp, int fmt, const CUtensorMap& own, const CUtensorMap& partner,

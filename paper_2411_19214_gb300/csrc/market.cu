@@ -286,12 +286,12 @@ tu_status side_alloc(tu_market* m, Side& s, int64_t rows, bool has_bias) {
   if (m->path == TU_PATH_FUSED && is_fp8(m->dtype)) {
     TU_TRY(dev_alloc(m, &s.fac8, (size_t)rows * m->kp));
     TU_TRY(dev_alloc(m, &s.fs, s.rows_pad));
-    // one scale per side and 128-byte rows: the extra MMA's g / c operand
-    if (m->dtype == TU_DTYPE_FP8E4M3_SIDE && m->kp == 128) TU_TRY(dev_alloc(m, &s.fold, (size_t)s.rows_pad * 32));
+    // one scale per side and up to two 128-byte blocks: the extra MMA's g / c operand
+    if (m->dtype == TU_DTYPE_FP8E4M3_SIDE && m->kp <= 256) TU_TRY(dev_alloc(m, &s.fold, (size_t)s.rows_pad * 32));
   } else if (m->path == TU_PATH_FUSED) {
     TU_TRY(dev_alloc(m, &s.fac16, (size_t)rows * m->kp));
     // the partner tiles' g / c operand of the fused kernel's extra MMA
-    if (m->kp == kKBlock) TU_TRY(dev_alloc(m, &s.fold, (size_t)s.rows_pad * 32));
+    if (m->kp <= 2 * kKBlock) TU_TRY(dev_alloc(m, &s.fold, (size_t)s.rows_pad * 32));
   } else {
     TU_TRY(dev_alloc(m, &s.fac32, (size_t)rows * m->kp));
   }
@@ -936,8 +936,9 @@ tu_status tu_market_create(const tu_market_desc* desc, tu_market_t* out) {
     return bail(st);
   }
   if (D.path == TU_PATH_FUSED) {
-    m->X.cut = cut_plan(m->N, m->M, m->num_sms);
-    m->Y.cut = cut_plan(m->M, m->N, m->num_sms);
+    const int kblocks = (int)(is_fp8(m->dtype) ? m->kp / 128 : m->kp / kKBlock);
+    m->X.cut = cut_plan(m->N, m->M, kblocks, m->num_sms);
+    m->Y.cut = cut_plan(m->M, m->N, kblocks, m->num_sms);
     const int64_t sx = cut_slots(m->X.cut), sy = cut_slots(m->Y.cut), slots = sx > sy ? sx : sy;
     if (slots > 0) {
       // (the shifts too: replaced factors can make the market wide)
@@ -1348,7 +1349,7 @@ int64_t tu_market_footprint(int64_t N, int64_t M, int64_t d, int path) {
   bytes += 2 * (N > M ? N : M) * d * 4;
   if (path == TU_PATH_FUSED) {
     bytes += (N + M) * kp * 2 + (np > mp ? np : mp) * 4;  // factors, per-row shifts
-    if (kp == kKBlock) bytes += (np + mp) * 32;              // the extra MMA's g / c operand
+    if (kp <= 2 * kKBlock) bytes += (np + mp) * 32;              // the extra MMA's g / c operand
     bytes += 2 << 20;                                        // the cut sums' partials
   } else {
     bytes += (N + M) * kp * 4 + N * round_up(M, 4) * 4 + M * round_up(N, 4) * 4;

@@ -66,13 +66,15 @@ enum : int { kResidualNone = 0, kResidualEstimate = 1, kResidualExact = 2 };
 enum : int { kErrNone = 0, kErrTimeout = 1, kErrNonfinite = 2 };
 
 // Where the rows' sums of a fused half-sweep are cut (cut_plan, fused.cu). Own
-// tiles (256 rows) from t0 on, taken as one line of (tile, partner tile)
+// tiles (256 rows; pair: 512) from t0 on, taken as one line of (tile, partner tile)
 // pairs, are cut after every `span` pairs; a row's sum is formed range by range
 // and the ranges are added in order. span = 0: nothing is cut. The cuts belong
 // to the market's shape, not to a launch: a launch that gives each range to
 // another CTA and one that runs a row's ranges in turn give the same bits.
+// `pair`: the half-sweep runs on pairs of CTAs, and the tiles are 512 rows.
 struct CutPlan {
   int t0 = 0, span = 0, spans = 0;
+  bool pair = false;
 };
 
 struct Side {
@@ -88,12 +90,14 @@ struct Side {
   __nv_bfloat16* fac16 = nullptr;  // packed [F | K] (or [G | L]) rows x kp, bf16, zero padded
   uint8_t* fac8 = nullptr;         // FP8 markets: packed rows x kp e4m3 of [F | K] / fs (zero padded)
   float* fs = nullptr;             // FP8 markets: per-row scales, rows_pad (padding 1)
-  uint8_t* fold = nullptr;         // BF16 fused markets, kp = 64: this side's g / c as the K = 16 operand of
+  uint8_t* fold = nullptr;         // BF16 fused markets, kp <= 128: this side's g / c as the K = 16 operand of
                                    // the partner tiles' extra MMA (rows_pad x 32 bytes, tcgen05 layout)
   int fp8_exp = 0;                 // FP8 markets with one scale per side: its exponent (fs = 2^fp8_exp)
   float* fac32 = nullptr;          // packed rows x kp, fp32 (dense path), zero padded
   CUtensorMap tm_own;       // TMA map, box kKBlock x kFusedOwnRows
   CUtensorMap tm_partner;   // TMA map, box kKBlock x kFusedPartnerRows
+  CUtensorMap tm_half;      // TMA map, box kKBlock x kFusedPartnerRows / 2 (pairs of CTAs)
+  CUtensorMap tm_fold;      // TMA map of `fold` (pairs of CTAs)
   CutPlan cut;              // fused path: the cuts of the half-sweep that updates this side
 };
 
@@ -294,8 +298,9 @@ cudaError_t fused_prepare(tu_market* m);  // tensor maps + kernel attributes
 cudaError_t launch_fused_halfsweep(tu_market* m, int side, int residual, int update, int* nparts_out,
                                    int64_t row0 = 0, int64_t nrows = -1);
 
-// The cuts of a half-sweep of own_rows against partner_rows on sms SMs.
-CutPlan cut_plan(int64_t own_rows, int64_t partner_rows, int sms);
+// The cuts of a half-sweep of own_rows against partner_rows on sms SMs; kblocks:
+// 128-byte k blocks of a packed row.
+CutPlan cut_plan(int64_t own_rows, int64_t partner_rows, int kblocks, int sms);
 // Scratch of cut launches, in ranges' slots of kFusedOwnRows rows (0: none).
 int64_t cut_slots(const CutPlan& p);
 
@@ -349,6 +354,7 @@ struct BatchDesc {
   int num_own_tiles;           // ceil(rows / kFusedOwnRows)
   int num_partner_tiles;       // ceil(partner_rows / kFusedPartnerRows)
   int cut_t0, cut_span;        // CutPlan of this half-sweep
+  int cut_rows;                // rows of its tiles
   int slot0;                   // first own-tile slot of this market in the partials array
   float c;                     // log2(e) / (2 sigma)
 };
@@ -830,6 +836,12 @@ __device__ __forceinline__ uint32_t cluster_rank() {
   asm volatile("mov.u32 %0, %%cluster_ctarank;" : "=r"(r));
   return r;
 }
+// Arrive on an mbarrier of a CTA of the cluster, ordering no memory of other
+// proxies or CTAs (what it announces here are TMEM reads, which
+// tcgen05.fence::before_thread_sync orders).
+__device__ __forceinline__ void cluster_arrive(uint32_t bar) {
+  asm volatile("mbarrier.arrive.shared::cluster.b64 _, [%0];" ::"r"(bar) : "memory");
+}
 // Every thread of every CTA of the cluster.
 __device__ __forceinline__ void cluster_sync() {
   asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
@@ -881,7 +893,66 @@ __device__ __forceinline__ void tensormap_acquire(const CUtensorMap* map) {
                : "memory");
 }
 
+// A load by one CTA of a pair, counted on an mbarrier of the pair's first CTA
+// (bar: its cluster address).
+__device__ __forceinline__ void tma_load_2d_pair(void* smem_dst, const CUtensorMap* map, uint32_t bar, int x, int y) {
+  asm volatile(
+      "cp.async.bulk.tensor.2d.cta_group::2.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1, {%3, "
+      "%4}], [%2];" ::"r"(smem_u32(smem_dst)),
+      "l"(reinterpret_cast<uint64_t>(map)), "r"(bar), "r"(x), "r"(y)
+      : "memory");
+}
+__device__ __forceinline__ void tma_load_2d_pair_hint(void* smem_dst, const CUtensorMap* map, uint32_t bar, int x,
+                                                      int y, uint64_t policy) {
+  asm volatile(
+      "cp.async.bulk.tensor.2d.cta_group::2.shared::cluster.global.mbarrier::complete_tx::bytes.L2::cache_hint [%0], "
+      "[%1, {%3, %4}], [%2], %5;" ::"r"(smem_u32(smem_dst)),
+      "l"(reinterpret_cast<uint64_t>(map)), "r"(bar), "r"(x), "r"(y), "l"(policy)
+      : "memory");
+}
+
 // ---- tcgen05 ---------------------------------------------------------------
+// Pairs of CTAs (cta_group::2): both CTAs of the pair allocate and free; the
+// first one issues. D's rows 0-127 (A's, from the first CTA's shared memory)
+// are in the first CTA's TMEM, rows 128-255 in the second's; each CTA's shared
+// memory holds half of B's rows, at the same offset.
+__device__ __forceinline__ void tmem_alloc_pair(uint32_t* smem_dst, uint32_t ncols) {
+  asm volatile("tcgen05.alloc.cta_group::2.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(smem_dst)),
+               "r"(ncols)
+               : "memory");
+}
+__device__ __forceinline__ void tmem_relinquish_pair() {
+  asm volatile("tcgen05.relinquish_alloc_permit.cta_group::2.sync.aligned;" ::: "memory");
+}
+__device__ __forceinline__ void tmem_dealloc_pair(uint32_t taddr, uint32_t ncols) {
+  asm volatile("tcgen05.dealloc.cta_group::2.sync.aligned.b32 %0, %1;" ::"r"(taddr), "r"(ncols) : "memory");
+}
+__device__ __forceinline__ void umma_bf16_pair(uint32_t d_tmem, uint64_t adesc, uint64_t bdesc, uint32_t idesc,
+                                               uint32_t accumulate) {
+  asm volatile(
+      "{\n\t.reg .pred p;\n\t"
+      "setp.ne.b32 p, %4, 0;\n\t"
+      "tcgen05.mma.cta_group::2.kind::f16 [%0], %1, %2, %3, p;\n\t}" ::"r"(d_tmem),
+      "l"(adesc), "l"(bdesc), "r"(idesc), "r"(accumulate)
+      : "memory");
+}
+__device__ __forceinline__ void umma_e4m3_pair(uint32_t d_tmem, uint64_t adesc, uint64_t bdesc, uint32_t idesc,
+                                               uint32_t accumulate) {
+  asm volatile(
+      "{\n\t.reg .pred p;\n\t"
+      "setp.ne.b32 p, %4, 0;\n\t"
+      "tcgen05.mma.cta_group::2.kind::f8f6f4 [%0], %1, %2, %3, p;\n\t}" ::"r"(d_tmem),
+      "l"(adesc), "l"(bdesc), "r"(idesc), "r"(accumulate)
+      : "memory");
+}
+// Arrive on the mbarrier at this offset in both CTAs.
+__device__ __forceinline__ void umma_commit_pair(uint64_t* bar) {
+  asm volatile(
+      "tcgen05.commit.cta_group::2.mbarrier::arrive::one.shared::cluster.multicast::cluster.b64 [%0], %1;" ::"r"(
+          smem_u32(bar)),
+      "h"((unsigned short)3)
+      : "memory");
+}
 __device__ __forceinline__ void tmem_alloc(uint32_t* smem_dst, uint32_t ncols) {
   asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(smem_dst)),
                "r"(ncols)
