@@ -313,17 +313,27 @@ cudaError_t launch_fused_topk(tu_market* m, int side, int k, int64_t row0, int64
   return launch_lists(m->kp, fmt, own.tm_own, partner.tm_partner, p, grid, m->stream, small);
 }
 
+// Where the partner vector of a mu block from column y0 starts in pvec.
+int mu_vector_offset(const tu_market* m, int64_t y0) {
+  return m->dtype == TU_DTYPE_FP8E4M3 ? 0 : (int)((4 - (y0 & 3)) & 3);
+}
+
 // mu for own X users [x0, x0 + nx) and partners [y0, y0 + ny) (the Y partner
 // vector must have been prepared in log2 mode).
 cudaError_t launch_fused_mu(tu_market* m, int64_t x0, int64_t nx, int64_t y0, int64_t ny, float* out, int64_t ld) {
-  const int64_t c0 = y0 & ~(int64_t)3;  // the g bulk copies start 16-byte aligned
+  // The bulk copies of g start 16-byte aligned: the vector is prepared with the
+  // block's first column there. (Row scales are where they are: the block then
+  // starts at the multiple of four before it, and its stores are single floats.)
+  const bool scales = m->dtype == TU_DTYPE_FP8E4M3;
+  const int64_t c0 = scales ? y0 & ~(int64_t)3 : y0;
   FusedParams p = base_params(nx, x0, c0, y0 + ny - c0, m->cmul);
   // A block is bounded by its stores (128 KB per 256 x 128 tile), so every SM
   // takes part: the partner tiles of an own tile go to several CTAs.
   // (7,150 x 9,336 at d = 50: 795 us on 56 CTAs with each thread storing along
   // its own row, 109 us with the stores turned through shared memory on 140.)
   p.split = best_split(p.num_own_tiles, p.num_partner_tiles, m->num_sms, 64, 1.0);
-  p.g = m->Y.pvec;
+  p.vec = !scales && (ld & 3) == 0 && (reinterpret_cast<uintptr_t>(out) & 15) == 0;
+  p.g = m->Y.pvec + mu_vector_offset(m, y0);
   p.lmax = m->st + kStShift;
   p.ell = m->X.ell;
   p.partials = m->partials;

@@ -92,6 +92,7 @@ struct FusedParams {
   int64_t ld;
   int64_t y0;
   int64_t ny;
+  int vec;                 // out, ld and the columns allow 16-byte stores
   // e4m3 factors: per-row scales of the own side (index row0 + r) and of the
   // partner side (index = partner user); the product of row r and partner
   // column j is fs_own[r] * fs_par[j] * <e4m3 row r, e4m3 row j>
@@ -494,10 +495,10 @@ static_assert(kTopKSlots - kSharedTopK > kTopKGroup, "candidate slots");
 constexpr int kWideShiftBytes = 2 * kFusedOwnRows * 4;  // kModeSweepWide: the row hand-over's shifts
 // kModeMu: each epilogue warp turns its 32 rows x mu_width columns through
 // shared memory, so that its stores run along the rows of the output (rows of
-// mu_width + 1 floats: conflict-free columns). Half the width where a
-// four-block own tile leaves no room for more.
+// mu_width + 4 floats: 16-byte accesses along and across them are free of bank
+// conflicts). Half the width where a four-block own tile leaves no room for more.
 constexpr int mu_width(int KB) { return KB == 4 ? 16 : 32; }
-constexpr int mu_stage_floats(int KB) { return 32 * (mu_width(KB) + 1); }
+constexpr int mu_stage_floats(int KB) { return 32 * (mu_width(KB) + 4); }
 // shared memory a mode needs after the tail area
 constexpr int mode_extra_bytes(int mode, int KB, bool split, bool ranges) {
   return mode == kModeTopKShared ? kTopKListBytes
@@ -646,10 +647,9 @@ __device__ __forceinline__ void chunk_topk_shared(const uint32_t (&v)[32], const
 // mu block: mu = 2^(c * phi_hat + g + lo) * 2^hi, where hi + lo = (shift + ell_row) log2 e;
 // 2^hi as the two factors s1, s2 (hi clamped to +-252: beyond, the product is
 // 0 or infinite all the same). The warp's 32 rows x 32 columns go through
-// `st` in shared memory, W columns at a time, so that every store of the warp
-// writes 32 / W runs of W consecutive floats of the output; lane = row before,
-// (row % (32 / W), column) after. nrow: the warp's rows inside the block, orow:
-// its first row there.
+// `st` in shared memory, W columns at a time, so that the warp's stores run along
+// the output's rows: four floats per lane and store (p.vec), or one. nrow: the
+// warp's rows inside the block, orow: its first row there.
 template <bool RS, int W>
 __device__ __forceinline__ void chunk_mu(const uint32_t (&v)[32], const float* g, const float* fs, float c,
                                          int64_t colbase, float lo, int hi, float s1, float s2, int lane, int nrow,
@@ -670,28 +670,35 @@ __device__ __forceinline__ void chunk_mu(const uint32_t (&v)[32], const float* g
   const bool near = !__any_sync(0xffffffffu, far > 100.0f);
 #pragma unroll
   for (int c0 = 0; c0 < 32; c0 += W) {
-    float* mine = st + lane * (W + 1);
+    float4* mine = reinterpret_cast<float4*>(st + lane * (W + 4));
     if (near) {
 #pragma unroll
-      for (int i = 0; i < W; ++i) mine[i] = ex2_approx(t[c0 + i]) * s1 * s2;
+      for (int i = 0; i < W; i += 4)
+        mine[i / 4] = make_float4(ex2_approx(t[c0 + i]) * s1 * s2, ex2_approx(t[c0 + i + 1]) * s1 * s2,
+                                  ex2_approx(t[c0 + i + 2]) * s1 * s2, ex2_approx(t[c0 + i + 3]) * s1 * s2);
     } else {
       // (an exponent beyond the FP32 range is brought back by hi first)
+      float* m = reinterpret_cast<float*>(mine);
 #pragma unroll
       for (int i = 0; i < W; ++i)
-        mine[i] = fabsf(t[c0 + i]) <= 100.0f ? ex2_approx(t[c0 + i]) * s1 * s2 : ex2_approx(t[c0 + i] + (float)hi);
+        m[i] = fabsf(t[c0 + i]) <= 100.0f ? ex2_approx(t[c0 + i]) * s1 * s2 : ex2_approx(t[c0 + i] + (float)hi);
     }
     __syncwarp();
-    const int64_t col = colbase + c0 + lane % W;
-    if (col >= p.y0 && col < p.y0 + p.ny) {
-      float* o = p.out + (orow + lane / W) * p.ld + (col - p.y0);
-      const float* src = st + (lane / W) * (W + 1) + lane % W;
-      const int64_t step = (32 / W) * p.ld;
-      if (nrow == 32) {
-#pragma unroll 8
-        for (int i = 0; i < W; ++i) o[i * step] = src[i * (32 / W) * (W + 1)];
-      } else {
-        for (int i = 0; i * (32 / W) + lane / W < nrow; ++i) o[i * step] = src[i * (32 / W) * (W + 1)];
+    const int64_t ocol = colbase + c0 - p.y0;  // (the chunk's first column of the output)
+    float* o = p.out + orow * p.ld + ocol;
+    if (p.vec && ocol >= 0 && ocol + W <= p.ny) {
+      constexpr int kLanes = W / 4, kRows = 32 / kLanes;  // lanes along a row, rows per store
+      const int rr = lane / kLanes, cq = lane % kLanes;
+#pragma unroll
+      for (int i = 0; i < W / 4; ++i) {
+        const int row = i * kRows + rr;
+        const float4 v4 = *reinterpret_cast<const float4*>(st + row * (W + 4) + 4 * cq);
+        if (row < nrow) *reinterpret_cast<float4*>(o + row * p.ld + 4 * cq) = v4;
       }
+    } else {
+      const int64_t col = ocol + lane % W;
+      if (col >= 0 && col < p.ny)
+        for (int i = lane / W; i < nrow; i += 32 / W) o[i * p.ld + lane % W] = st[i * (W + 4) + lane % W];
     }
     __syncwarp();
   }

@@ -277,7 +277,8 @@ tu_status side_alloc(tu_market* m, Side& s, int64_t rows, bool has_bias) {
   s.rows_pad = round_up(rows, kRowPad);
   TU_TRY(dev_alloc(m, &s.log_u, s.rows_pad));
   TU_TRY(dev_alloc(m, &s.ell, s.rows_pad));
-  TU_TRY(dev_alloc(m, &s.pvec, s.rows_pad));
+  // (a mu block's vector starts up to 3 later, and its last tile reads up to 127 past the side)
+  TU_TRY(dev_alloc(m, &s.pvec, s.rows_pad + 256));
   TU_TRY(dev_alloc(m, &s.mass, s.rows_pad));
   // groups of 32 rows; the dense pass's layout (rows dealt round-robin over up
   // to kMaxPartials CTAs) needs at most rows / 32 + 2 * kMaxPartials of them
@@ -285,7 +286,7 @@ tu_status side_alloc(tu_market* m, Side& s, int64_t rows, bool has_bias) {
   if (has_bias) TU_TRY(dev_alloc(m, &s.b2s, s.rows_pad));
   if (m->path == TU_PATH_FUSED && is_fp8(m->dtype)) {
     TU_TRY(dev_alloc(m, &s.fac8, (size_t)rows * m->kp));
-    TU_TRY(dev_alloc(m, &s.fs, s.rows_pad));
+    TU_TRY(dev_alloc(m, &s.fs, s.rows_pad + 256));
     // one scale per side and up to two 128-byte blocks: the extra MMA's g / c operand
     if (m->dtype == TU_DTYPE_FP8E4M3_SIDE && m->kp <= 256) TU_TRY(dev_alloc(m, &s.fold, (size_t)s.rows_pad * 32));
   } else if (m->path == TU_PATH_FUSED) {
@@ -1537,7 +1538,7 @@ tu_status tu_mu_block(tu_market_t m, int64_t x0, int64_t nx, int64_t y0, int64_t
   TU_TRY(output_view(m, out, bytes, 0, &dst, &host));
   if (m->path == TU_PATH_FUSED) {
     // Y potentials prepared in log2 mode, then the tensor-core mu epilogue
-    TU_CK(m, launch_prep(m, m->Y, 1, 0));
+    TU_CK(m, launch_prep(m, m->Y, 1, 0, mu_vector_offset(m, y0)));
     TU_CK(m, launch_fused_mu(m, x0, nx, y0, ny, static_cast<float*>(dst), ld));
   } else {
     TU_CK(m, launch_mu_block(m, x0, nx, y0, ny, static_cast<float*>(dst), ld));

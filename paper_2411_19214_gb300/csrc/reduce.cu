@@ -503,11 +503,11 @@ cudaError_t launch_pack_fp8_bytes(tu_market* m, Side& s, const uint8_t* A, const
   return cudaGetLastError();
 }
 
-cudaError_t launch_prep(tu_market* m, Side& partner, int fused_mode, int translate) {
+cudaError_t launch_prep(tu_market* m, Side& partner, int fused_mode, int translate, int offset) {
   const int own = &partner == &m->Y ? 0 : 1;
   const int g = grid_for(partner.rows_pad, m->num_sms, 4);
   k_prep<<<g, kThreads, 0, m->stream>>>(partner.ell, partner.rows, partner.rows_pad, m->st, own, translate, fused_mode,
-                                        partner.pvec, fused_mode ? reinterpret_cast<uint4*>(partner.fold) : nullptr,
+                                        partner.pvec + offset, fused_mode ? reinterpret_cast<uint4*>(partner.fold) : nullptr,
                                         1.0f / m->cmul);  // (the batched preparation rounds 1 / c alike)
   return cudaGetLastError();
 }

@@ -246,7 +246,8 @@ namespace tu {
 // reduce.cu
 // Prepare the partner's FP32 vector for a half-sweep of the other side and the
 // pass's scalars (with translate, the translation step taken before it).
-cudaError_t launch_prep(tu_market* m, Side& partner, int fused_mode, int translate);
+// (offset: where in pvec the vector starts, 0 to 3)
+cudaError_t launch_prep(tu_market* m, Side& partner, int fused_mode, int translate, int offset = 0);
 // Reduce a pass's partials; after an update, also the own side's groups into
 // the market scalars (ngroups: groups the pass wrote).
 // prep_next: also set the scalars of the half-sweep that follows, which updates
@@ -381,6 +382,7 @@ cudaError_t launch_fused_batch(const BatchLaunch& b, cudaStream_t stream);
 // ranked lists / mu block through the tensor-core pipeline (partner vector prepared in log2 mode)
 cudaError_t launch_fused_topk(tu_market* m, int side, int k, int64_t row0, int64_t nrows, int32_t* idx, float* logmu,
                               float* hand_v, int32_t* hand_i);
+int mu_vector_offset(const tu_market* m, int64_t y0);
 cudaError_t launch_fused_mu(tu_market* m, int64_t x0, int64_t nx, int64_t y0, int64_t ny, float* out, int64_t ld);
 
 // topk.cu (dense-path outputs, read from A-hat)
