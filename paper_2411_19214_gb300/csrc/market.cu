@@ -84,6 +84,7 @@ constexpr int kMaxDevices = 64;
 std::mutex g_pool_mu;
 cudaMemPool_t g_pools[kMaxDevices] = {};
 int g_live_markets = 0;
+constexpr size_t kPoolKeep = 64u << 20;  // kept mapped when the last market goes away
 
 cudaMemPool_t market_pool(int device) {
   if (device < 0 || device >= kMaxDevices) return nullptr;
@@ -155,9 +156,25 @@ void verify_guards(void* p, const GuardedBlock& g, cudaStream_t stream) {
   }
 }
 
+// The buffers that a market has from its creation on are parts of one block
+// (alloc_buffers runs twice: once to add up their sizes): an allocation costs
+// a few microseconds of the host, and a market has some twenty. (Checked mode:
+// a block and guard bands each.)
+constexpr size_t kArenaAlign = 256;
+
 tu_status dev_alloc_bytes(tu_market* m, void** p, size_t bytes) {
   *p = nullptr;
   if (bytes == 0) return TU_OK;
+  const size_t part = (bytes + kArenaAlign - 1) / kArenaAlign * kArenaAlign;
+  if (m->measuring) {
+    m->arena_bytes += part;
+    return TU_OK;
+  }
+  if (m->arena != nullptr && m->arena_used + part <= m->arena_bytes) {
+    *p = m->arena + m->arena_used;
+    m->arena_used += part;
+    return TU_OK;
+  }
   cudaMemPool_t pool = market_pool(m->device);
   if (pool == nullptr) return fail(m, TU_ERR_CUDA, "device memory pool unavailable");
   const bool guarded = g_checked.load();
@@ -184,6 +201,7 @@ tu_status dev_alloc_bytes(tu_market* m, void** p, size_t bytes) {
 // buffers: after their bands were checked).
 void dev_free_bytes(tu_market* m, void* p) {
   if (p == nullptr) return;
+  if (m->arena != nullptr && p >= m->arena && p < m->arena + m->arena_bytes) return;  // freed with the arena
   GuardedBlock g{nullptr, 0};
   {
     std::lock_guard<std::mutex> lk(g_guard_mu);
@@ -250,6 +268,10 @@ void mirror_free(void* b) {
   g_mirror_free.push_back(b);
 }
 
+// tu_market::scratch: the largest |bias| of the two sides, their largest row
+// norms, and two words of the FP8 packing
+constexpr int kScratchNorms = 2, kScratchBad = 4, kScratch = 6;
+
 tu_status ensure_staging(tu_market* m, size_t bytes) {
   if (m->staging_bytes >= bytes) return TU_OK;
   dev_free(m, m->staging);  // stream-ordered: after the copies that used it
@@ -260,12 +282,15 @@ tu_status ensure_staging(tu_market* m, size_t bytes) {
 }
 
 // Device view of a caller pointer: the pointer itself if it is device memory,
-// else a copy in the staging buffer at byte offset `off`.
-tu_status device_view(tu_market* m, const void* src, size_t bytes, size_t off, const void** out) {
+// else a copy in the staging buffer at byte offset `off` (*staged is set: the
+// buffer may be reused only after the work that reads it).
+tu_status device_view(tu_market* m, const void* src, size_t bytes, size_t off, const void** out,
+                      bool* staged = nullptr) {
   if (is_device_ptr(src)) {
     *out = src;
     return TU_OK;
   }
+  if (staged != nullptr) *staged = true;
   void* dst = static_cast<char*>(m->staging) + off;
   TU_CK(m, cudaMemcpyAsync(dst, src, bytes, cudaMemcpyHostToDevice, m->stream));
   *out = dst;
@@ -323,17 +348,6 @@ tu_status upload_masses(tu_market* m, Side& s, const double* host) {
   }
   s.sum_mass = sum;
   TU_CK(m, cudaMemcpyAsync(s.mass, host, (size_t)s.rows * sizeof(double), cudaMemcpyHostToDevice, m->stream));
-  // padding capacities are 1 so that padded rows never produce log(0)
-  if (s.rows_pad > s.rows) {
-    const size_t npad = (size_t)(s.rows_pad - s.rows);
-    double* ones = new (std::nothrow) double[npad];
-    if (ones == nullptr) return fail(m, TU_ERR_OOM, "host allocation");
-    for (size_t i = 0; i < npad; ++i) ones[i] = 1.0;
-    cudaError_t e = cudaMemcpyAsync(s.mass + s.rows, ones, npad * sizeof(double), cudaMemcpyHostToDevice, m->stream);
-    if (e == cudaSuccess) e = cudaStreamSynchronize(m->stream);  // `ones` is pageable and freed below
-    delete[] ones;
-    if (e != cudaSuccess) return fail_cuda(m, e, "mass padding");
-  }
   return TU_OK;
 }
 
@@ -390,41 +404,48 @@ tu_status load_factors(tu_market* m, const void* F, const void* K, const void* G
   // (caller scales follow the two factor matrices in the staging buffer)
   const size_t sx = prescaled ? round_up((int64_t)(2 * bx), 256) : 0, sy = prescaled ? round_up((int64_t)(2 * by), 256) : 0;
   const size_t stage = 2 * (bx > by ? bx : by) + (prescaled ? 256 + 4 * (size_t)(m->N > m->M ? m->N : m->M) : 0);
-  TU_TRY(ensure_staging(m, stage));
-  unsigned int* bad = nullptr;  // [0]: the pack kernels' flag, [1]: a float scratch
-  if (fp8) TU_TRY(dev_alloc(m, &bad, 2));
+  for (const void* q : {F, K, G, L, (const void*)(prescaled ? fsx : nullptr), (const void*)(prescaled ? fsy : nullptr)})
+    if (q != nullptr && !is_device_ptr(q)) {  // (nothing to stage otherwise)
+      TU_TRY(ensure_staging(m, stage));
+      break;
+    }
+  unsigned int* bad = reinterpret_cast<unsigned int*>(m->scratch + kScratchBad);  // the pack kernels' flag, a float
   auto pack = [&](Side& s, const void* a, const void* b, const float* sc) -> tu_status {
     if (fp8) return pack_side_fp8(m, s, a, b, sc, bad);
     TU_CK(m, launch_pack_factors(m, s, a, b, m->dtype));
     return TU_OK;
   };
   const void *a = nullptr, *b = nullptr, *sc = nullptr;
-  tu_status st = device_view(m, F, bx, 0, &a);
-  if (st == TU_OK) st = device_view(m, K, bx, bx, &b);
-  if (st == TU_OK && prescaled) st = device_view(m, fsx, (size_t)m->N * 4, sx, &sc);
+  bool staged = false;
+  tu_status st = device_view(m, F, bx, 0, &a, &staged);
+  if (st == TU_OK) st = device_view(m, K, bx, bx, &b, &staged);
+  if (st == TU_OK && prescaled) st = device_view(m, fsx, (size_t)m->N * 4, sx, &sc, &staged);
   if (st == TU_OK) st = pack(m->X, a, b, static_cast<const float*>(sc));
-  if (st == TU_OK && cudaStreamSynchronize(m->stream) != cudaSuccess)  // the staging buffer is reused
+  if (st == TU_OK && staged && cudaStreamSynchronize(m->stream) != cudaSuccess)  // the staging buffer is reused
     st = fail_cuda(m, cudaGetLastError(), "cudaStreamSynchronize");
   if (st == TU_OK) st = device_view(m, G, by, 0, &a);
   if (st == TU_OK) st = device_view(m, L, by, by, &b);
   if (st == TU_OK && prescaled) st = device_view(m, fsy, (size_t)m->M * 4, sy, &sc);
   if (st == TU_OK) st = pack(m->Y, a, b, static_cast<const float*>(sc));
-  dev_free(m, bad);
   if (st != TU_OK) return st;
   // the multiplier of <a_x, b_y> in the exponent (log2 units; FP8 with per-row
   // scales: those are applied in the kernels; with one scale per side: folded in)
   m->cmul = (float)std::ldexp(1.4426950408889634 / (2.0 * m->sigma),
                               m->dtype == TU_DTYPE_FP8E4M3_SIDE ? m->X.fp8_exp + m->Y.fp8_exp : 0);
   // exponent-range check (Cauchy-Schwarz bound of |phi_hat| / (2 sigma))
-  float* norms = nullptr;
-  TU_TRY(dev_alloc(m, &norms, 2));
-  float hn[2] = {0.f, 0.f};
-  cudaError_t e = launch_row_norms(m, m->X, norms);
+  // (every input has been read when this read-back returns; at creation it also
+  // brings the biases' largest entries)
+  float* norms = m->scratch + kScratchNorms;
+  float read[kScratchBad] = {};
+  cudaError_t e = cudaMemsetAsync(norms, 0, 2 * sizeof(float), m->stream);
+  if (e == cudaSuccess) e = launch_row_norms(m, m->X, norms);
   if (e == cudaSuccess) e = launch_row_norms(m, m->Y, norms + 1);
-  if (e == cudaSuccess) e = cudaMemcpyAsync(hn, norms, sizeof(hn), cudaMemcpyDeviceToHost, m->stream);
+  if (e == cudaSuccess) e = cudaMemcpyAsync(read, m->scratch, sizeof(read), cudaMemcpyDeviceToHost, m->stream);
   if (e == cudaSuccess) e = cudaStreamSynchronize(m->stream);
-  dev_free(m, norms);
   if (e != cudaSuccess) return fail_cuda(m, e, "factor norms");
+  const float* hn = read + kScratchNorms;
+  if (!std::isfinite(read[0]) || !std::isfinite(read[1]))
+    return fail(m, TU_ERR_NONFINITE, "popularity biases contain NaN or Inf");
   if (!std::isfinite(hn[0]) || !std::isfinite(hn[1]))
     return fail(m, TU_ERR_NONFINITE, "factor matrices contain NaN or Inf");
   const double bound = (double)hn[0] * (double)hn[1] / (2.0 * m->sigma);  // FP8: norms of the quantized rows
@@ -441,7 +462,6 @@ tu_status load_factors(tu_market* m, const void* F, const void* K, const void* G
   }
   m->wide = wide;
   if (m->path == TU_PATH_DENSE) TU_CK(m, launch_dense_build(m));
-  TU_CK(m, cudaStreamSynchronize(m->stream));
   if (m->graph != nullptr) {
     cudaGraphExecDestroy(m->graph);
     m->graph = nullptr;
@@ -784,15 +804,19 @@ void tu_market_destroy(tu_market_t m) {
   dev_free(m, m->staging);
   dev_free(m, m->aux);
   dev_free(m, m->omega_dev);
+  dev_free(m, m->scratch);
+  if (m->arena != nullptr) cudaFreeAsync(m->arena, m->stream);
   if (m->done_ev) cudaEventDestroy(m->done_ev);
   mirror_free(m->results_host);  // the block that holds all four host mirrors
   {
     // every market that reaches this point was counted by tu_market_create
     std::lock_guard<std::mutex> lk(g_pool_mu);
     if (--g_live_markets == 0 && m->device >= 0 && m->device < kMaxDevices && g_pools[m->device] != nullptr) {
-      // the last market: return the pool's memory once its frees have run
+      // the last market: return the pool's memory once its frees have run, but
+      // for what a small market takes (mapping it anew costs a program that
+      // makes one market after another 0.2 ms each)
       if (m->stream) cudaStreamSynchronize(m->stream);
-      cudaMemPoolTrimTo(g_pools[m->device], 0);
+      cudaMemPoolTrimTo(g_pools[m->device], kPoolKeep);
     }
   }
   delete m;
@@ -800,6 +824,26 @@ void tu_market_destroy(tu_market_t m) {
 
 namespace {
 void apply_tuned(tu_market* m);  // (the autotuner, below)
+
+// The buffers a market keeps from its creation on (but for A-hat and its transpose).
+tu_status alloc_buffers(tu_market* m, const tu_market_desc& D) {
+  TU_TRY(side_alloc(m, m->X, D.N, D.bias_x != nullptr));
+  TU_TRY(side_alloc(m, m->Y, D.M, D.bias_y != nullptr));
+  TU_TRY(dev_alloc(m, &m->partials, (size_t)kMaxPartials * 4));
+  TU_TRY(dev_alloc(m, &m->st, (size_t)kStSlots));
+  TU_TRY(dev_alloc(m, &m->results, (size_t)kResSlots + 1));
+  TU_TRY(dev_alloc(m, &m->omega_dev, 1));
+  TU_TRY(dev_alloc(m, &m->scratch, (size_t)kScratch));
+  if (m->dplan.cl > 0) TU_TRY(dev_alloc(m, &m->colsum, dense_plan_floats(m->dplan)));
+  const int64_t sx = cut_slots(m->X.cut), sy = cut_slots(m->Y.cut), slots = sx > sy ? sx : sy;
+  if (slots > 0) {
+    // (the shifts too: replaced factors can make the market wide)
+    TU_TRY(dev_alloc(m, &m->cut_part, (size_t)slots * kFusedOwnRows));
+    TU_TRY(dev_alloc(m, &m->cut_m, (size_t)slots * kFusedOwnRows));
+    TU_TRY(dev_alloc(m, &m->cut_cnt, (size_t)split_counter_count(m)));
+  }
+  return TU_OK;
+}
 }  // namespace
 
 tu_status tu_market_create(const tu_market_desc* desc, tu_market_t* out) {
@@ -865,11 +909,27 @@ tu_status tu_market_create(const tu_market_desc* desc, tu_market_t* out) {
     std::lock_guard<std::mutex> lk(g_pool_mu);
     ++g_live_markets;  // from here on every exit goes through tu_market_destroy
   }
-  if ((st = side_alloc(m, m->X, D.N, D.bias_x != nullptr)) != TU_OK) return bail(st);
-  if ((st = side_alloc(m, m->Y, D.M, D.bias_y != nullptr)) != TU_OK) return bail(st);
-  if ((st = dev_alloc(m, &m->partials, (size_t)kMaxPartials * 4)) != TU_OK) return bail(st);
-  if ((st = dev_alloc(m, &m->st, (size_t)kStSlots)) != TU_OK) return bail(st);
-  if ((st = dev_alloc(m, &m->results, (size_t)kResSlots + 1)) != TU_OK) return bail(st);
+  if (D.path == TU_PATH_FUSED) {
+    const int kblocks = (int)(is_fp8(m->dtype) ? m->kp / 128 : m->kp / kKBlock);
+    m->X.cut = cut_plan(m->N, m->M, kblocks, m->num_sms);
+    m->Y.cut = cut_plan(m->M, m->N, kblocks, m->num_sms);
+  } else {
+    m->ldA = round_up(D.M, 4);
+    m->ldN = round_up(D.N, 4);
+    m->dplan = dense_plan(m);
+  }
+  if (!g_checked.load()) {
+    m->measuring = true;
+    alloc_buffers(m, D);
+    m->measuring = false;
+    cudaMemPool_t pool = market_pool(m->device);
+    if (pool == nullptr) return bail(TU_ERR_CUDA);
+    void* base = nullptr;
+    const cudaError_t e = cudaMallocFromPoolAsync(&base, m->arena_bytes, pool, m->stream);
+    if (e != cudaSuccess) return bail(fail_cuda(m, e, "cudaMallocFromPoolAsync"));
+    m->arena = static_cast<char*>(base);
+  }
+  if ((st = alloc_buffers(m, D)) != TU_OK) return bail(st);
   m->err_dev = reinterpret_cast<int*>(m->results + kResSlots);
   {
     HostMirror* hm = mirror_alloc();
@@ -881,8 +941,6 @@ tu_status tu_market_create(const tu_market_desc* desc, tu_market_t* out) {
   }
   *m->err_host = 0;
   if (D.path == TU_PATH_DENSE) {
-    m->ldA = round_up(D.M, 4);
-    m->ldN = round_up(D.N, 4);
     if (g_checked.load()) {  // checked mode: guarded like the other buffers
       if ((st = dev_alloc(m, &m->Ahat, (size_t)m->N * m->ldA)) != TU_OK) return bail(st);
       if ((st = dev_alloc(m, &m->AhatT, (size_t)m->M * m->ldN)) != TU_OK) return bail(st);
@@ -892,13 +950,6 @@ tu_status tu_market_create(const tu_market_desc* desc, tu_market_t* out) {
       if (e != cudaSuccess) return bail(fail_cuda(m, e, "cudaMalloc(A-hat)"));
     }
   }
-  if (D.path == TU_PATH_DENSE) {
-    m->dplan = dense_plan(m);
-    if (m->dplan.cl > 0 && (st = dev_alloc(m, &m->colsum, dense_plan_floats(m->dplan))) != TU_OK) return bail(st);
-  }
-  // (allocated after the dense matrices: placing this small allocation before
-  // them measurably slowed the dense row stream)
-  if ((st = dev_alloc(m, &m->omega_dev, 1)) != TU_OK) return bail(st);
   *m->omega_host = 1.0;
   if (cudaMemcpyAsync(m->omega_dev, m->omega_host, sizeof(double), cudaMemcpyHostToDevice, m->stream) !=
       cudaSuccess)
@@ -908,28 +959,23 @@ tu_status tu_market_create(const tu_market_desc* desc, tu_market_t* out) {
   // biases -> b / (2 sigma); potentials start at u = v = 1. A non-finite
   // bias is refused (TU_ERR_NONFINITE) like a non-finite factor.
   {
-    const size_t bbytes = (size_t)(D.N > D.M ? D.N : D.M) * sizeof(float);
-    if ((st = ensure_staging(m, bbytes)) != TU_OK) return bail(st);
-    float* bmax = nullptr;
-    if ((D.bias_x || D.bias_y) && (st = dev_alloc(m, &bmax, 1)) != TU_OK) return bail(st);
-    auto init = [&](Side& s, const float* bias, int64_t rows, const char* what) -> tu_status {
+    auto init = [&](Side& s, const float* bias, int64_t rows, float* max_abs) -> tu_status {
       const void* bdev = nullptr;
+      bool staged = false;
       if (bias) {
-        TU_TRY(device_view(m, bias, (size_t)rows * 4, 0, &bdev));
-        float hm = 0.0f;
+        if (!is_device_ptr(bias)) TU_TRY(ensure_staging(m, (size_t)(D.N > D.M ? D.N : D.M) * sizeof(float)));
+        TU_TRY(device_view(m, bias, (size_t)rows * 4, 0, &bdev, &staged));
         const float* b = static_cast<const float*>(bdev);
-        TU_CK(m, launch_max_abs(m, b, b, rows, bmax));
-        TU_CK(m, cudaMemcpyAsync(&hm, bmax, sizeof(float), cudaMemcpyDeviceToHost, m->stream));
-        TU_CK(m, cudaStreamSynchronize(m->stream));
-        if (!std::isfinite(hm)) return fail(m, TU_ERR_NONFINITE, std::string(what) + " contains NaN or Inf");
+        TU_CK(m, launch_max_abs(m, b, b, rows, max_abs));  // (checked with the factors' norms)
       }
       TU_CK(m, launch_init_side(m, s, static_cast<const float*>(bdev), bias != nullptr));
-      TU_CK(m, cudaStreamSynchronize(m->stream));  // the staging buffer is reused
+      if (staged) TU_CK(m, cudaStreamSynchronize(m->stream));  // the staging buffer is reused
       return TU_OK;
     };
-    st = init(m->X, D.bias_x, D.N, "bias_x");
-    if (st == TU_OK) st = init(m->Y, D.bias_y, D.M, "bias_y");
-    dev_free(m, bmax);
+    if (cudaMemsetAsync(m->scratch, 0, kScratch * sizeof(float), m->stream) != cudaSuccess)
+      return bail(fail_cuda(m, cudaGetLastError(), "scratch"));
+    st = init(m->X, D.bias_x, D.N, m->scratch);
+    if (st == TU_OK) st = init(m->Y, D.bias_y, D.M, m->scratch + 1);
     if (st != TU_OK) return bail(st);
   }
   if ((st = load_factors(m, D.F, D.K, D.G, D.L, D.fscale_x, D.fscale_y)) != TU_OK) {
@@ -937,16 +983,6 @@ tu_status tu_market_create(const tu_market_desc* desc, tu_market_t* out) {
     return bail(st);
   }
   if (D.path == TU_PATH_FUSED) {
-    const int kblocks = (int)(is_fp8(m->dtype) ? m->kp / 128 : m->kp / kKBlock);
-    m->X.cut = cut_plan(m->N, m->M, kblocks, m->num_sms);
-    m->Y.cut = cut_plan(m->M, m->N, kblocks, m->num_sms);
-    const int64_t sx = cut_slots(m->X.cut), sy = cut_slots(m->Y.cut), slots = sx > sy ? sx : sy;
-    if (slots > 0) {
-      // (the shifts too: replaced factors can make the market wide)
-      if ((st = dev_alloc(m, &m->cut_part, (size_t)slots * kFusedOwnRows)) != TU_OK) return bail(st);
-      if ((st = dev_alloc(m, &m->cut_m, (size_t)slots * kFusedOwnRows)) != TU_OK) return bail(st);
-      if ((st = dev_alloc(m, &m->cut_cnt, (size_t)split_counter_count(m))) != TU_OK) return bail(st);
-    }
     cudaError_t e = fused_prepare(m);
     if (e != cudaSuccess) return bail(fail_cuda(m, e, "fused_prepare"));
     apply_tuned(m);
@@ -954,7 +990,7 @@ tu_status tu_market_create(const tu_market_desc* desc, tu_market_t* out) {
   if (cudaMemsetAsync(m->st, 0, kStSlots * sizeof(double), m->stream) != cudaSuccess ||
       launch_rescan(m) != cudaSuccess)
     return bail(fail_cuda(m, cudaGetLastError(), "scalars of the initial potentials"));
-  if (clear_results(m) != TU_OK || cudaStreamSynchronize(m->stream) != cudaSuccess) return bail(TU_ERR_CUDA);
+  if (clear_results(m) != TU_OK) return bail(TU_ERR_CUDA);
   *out = m;
   return TU_OK;
 }

@@ -145,7 +145,7 @@ __global__ void k_pack_fp8_bytes(const uint8_t* __restrict__ A, const uint8_t* _
 
 __global__ void k_init_side(const float* __restrict__ bias, int has_bias, float inv2s, int64_t rows,
                             int64_t rows_pad, float* __restrict__ b2s, double* __restrict__ log_u,
-                            double* __restrict__ ell) {
+                            double* __restrict__ ell, double* __restrict__ mass) {
   for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < rows_pad;
        i += (int64_t)gridDim.x * blockDim.x) {
     float b = 0.0f;
@@ -153,6 +153,7 @@ __global__ void k_init_side(const float* __restrict__ bias, int has_bias, float 
     if (b2s != nullptr) b2s[i] = b;
     log_u[i] = 0.0;  // u = 1 (Alg. 1 / Alg. 2 initialisation)
     ell[i] = (i < rows) ? (double)b : 0.0;
+    if (i >= rows) mass[i] = 1.0;  // padding capacities: padded rows never produce log(0)
   }
 }
 
@@ -448,7 +449,7 @@ cudaError_t launch_pack_factors(tu_market* m, Side& s, const void* A, const void
 cudaError_t launch_init_side(tu_market* m, Side& s, const float* bias_dev, int has_bias) {
   const int g = grid_for(s.rows_pad, m->num_sms);
   k_init_side<<<g, kThreads, 0, m->stream>>>(bias_dev, has_bias, (float)(0.5 / m->sigma), s.rows,
-                                               s.rows_pad, s.b2s, s.log_u, s.ell);
+                                               s.rows_pad, s.b2s, s.log_u, s.ell, s.mass);
   return cudaGetLastError();
 }
 
@@ -472,8 +473,6 @@ cudaError_t launch_set_potentials(tu_market* m, Side& s, const float* log_u_dev)
 }
 
 cudaError_t launch_row_norms(tu_market* m, Side& s, float* out_max) {
-  cudaError_t e = cudaMemsetAsync(out_max, 0, sizeof(float), m->stream);
-  if (e != cudaSuccess) return e;
   int64_t blocks = (s.rows + (kThreads / 32) - 1) / (kThreads / 32);
   if (blocks > (int64_t)m->num_sms * 8) blocks = (int64_t)m->num_sms * 8;
   k_row_norm_max<<<(int)blocks, kThreads, 0, m->stream>>>(s.fac32, s.fac16, s.fac8, s.fs, s.rows, m->kp,

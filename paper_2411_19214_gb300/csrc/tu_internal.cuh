@@ -196,6 +196,10 @@ struct tu_market {
   double* results_host = nullptr;  // pinned, likewise
   int* err_dev = nullptr;          // device error word (behind results)
   int* err_host = nullptr;         // pinned (behind results_host)
+  char* arena = nullptr;           // one block that holds the buffers made at creation
+  size_t arena_bytes = 0, arena_used = 0;
+  bool measuring = false;          // dev_alloc only adds up arena_bytes
+  float* scratch = nullptr;        // kScratch floats: maxima read back after factor and bias loads
   void* staging = nullptr;         // device staging buffer for host-memory arguments
   size_t staging_bytes = 0;
   void* aux = nullptr;             // ranked-list hand-over scratch (grow-only)
@@ -264,12 +268,13 @@ cudaError_t launch_between(tu_market* m, int nparts, int is_x, int residual, int
 // Write the sides' pending offsets into their arrays (end of a block of sweeps).
 cudaError_t launch_flush(tu_market* m);
 cudaError_t launch_pack_factors(tu_market* m, Side& s, const void* A, const void* B, int src_dtype);
-cudaError_t launch_init_side(tu_market* m, Side& s, const float* bias_dev, int has_bias);
+cudaError_t launch_init_side(tu_market* m, Side& s, const float* bias_dev, int has_bias);  // and the mass padding
 cudaError_t launch_reset(tu_market* m);  // u = v = 1 on both sides, with their groups and scalars
 cudaError_t launch_set_potentials(tu_market* m, Side& s, const float* log_u_dev);
 cudaError_t launch_set_potentials64(tu_market* m, Side& s, const double* log_u_dev);
 // FP64 state -> FP32 (either may be null)
 cudaError_t launch_get_potentials(tu_market* m, float* out_x, float* out_y);
+// the largest row norm into *out_max (zeroed by the caller)
 cudaError_t launch_row_norms(tu_market* m, Side& s, float* out_max);
 // FP8 markets: max |entry| of the FP32 factor pair (A, B: rows x d each) into *out_max
 cudaError_t launch_max_abs(tu_market* m, const float* A, const float* B, int64_t count, float* out_max);
