@@ -294,7 +294,7 @@ cudaError_t launch_fused_topk(tu_market* m, int side, int k, int64_t row0, int64
                               float* logmu, float* hand_v, int32_t* hand_i) {
   Side& own = side == 0 ? m->X : m->Y;
   Side& partner = side == 0 ? m->Y : m->X;
-  const bool small = use_small_tiles(m, nrows);
+  const bool small = use_small_tiles(m, nrows) || lists_want_small(k, m->kp, fmt_of(m->dtype));
   FusedParams p = base_params(nrows, row0, 0, partner.rows, m->cmul, small);
   p.g = partner.pvec;
   p.lmax = m->st + kStShift;

@@ -462,9 +462,9 @@ __device__ __forceinline__ void chunk_topk(const uint32_t (&v)[32], const float*
   }
 }
 
-// Ranked lists with k <= kSharedTopK (kModeTopKShared): every epilogue thread
-// has kTopKSlots (score, column) slots in shared memory, slot i of thread t
-// at [i * kEpiThreads + t] (a warp's accesses to one slot are conflict-free).
+// Ranked lists in shared memory (kModeTopKShared): every epilogue thread
+// has list_slots (score, column) slots in shared memory, slot i of thread t
+// at [i * list_threads + t] (a warp's accesses to one slot are conflict-free).
 // The first k hold the k best of its row and column half, sorted by
 // decreasing score, equal scores in increasing column order (the order in
 // which a column half's columns arrive); they start as (-inf, INT32_MAX)
@@ -481,17 +481,29 @@ __device__ __forceinline__ void chunk_topk(const uint32_t (&v)[32], const float*
 // buffers, 2.74 with the shared bound below, 2.71 without the scores kept
 // across the vote, 2.16 with the merges of all warps at the same tiles; a
 // half-sweep of that size takes 1.4.)
+// With own tiles of 128 rows (SMALL) half of the epilogue threads have rows, and
+// twice the slots each: lists longer than kSharedTopK, up to kSharedTopKSmall,
+// run on such tiles. (Half of the epilogue is idle then, and every partner tile
+// is read by twice as many own tiles; the lists of kModeTopK, in local memory
+// and entered one lane at a time, cost far more. 60,000 x 50,000, kModeTopK ->
+// here: k = 20, d = 64 34.8 -> 2.80 ms; k = 32, d = 32 74.1 -> 5.53; 5,000 x
+// 7,000, d = 32, k = 20 1.39 -> 0.31. Longer ones would need more than the
+// 41 slots: kModeTopK.)
 constexpr int kSharedTopK = 14;
+constexpr int kSharedTopKSmall = 32;
 constexpr int kTopKSlots = 20;
 constexpr int kEpiThreads = kEpiWarps * 32;
+constexpr int list_threads(bool small) { return small ? kEpiThreads / 2 : kEpiThreads; }
+constexpr int list_slots(bool small) { return small ? 2 * kTopKSlots + 1 : kTopKSlots; }
 // (the slots, then one 8-byte word per thread: the bound that the two threads
 // of a row share, see chunk_topk_shared)
 constexpr int kTopKListBytes = (kTopKSlots + 1) * kEpiThreads * 8;
 // A group of kTopKGroup columns adds at most that many candidates, so a buffer
-// of kTopKSlots - k >= kTopKGroup + 1 slots is merged whenever fewer than
+// of list_slots - k >= kTopKGroup + 1 slots is merged whenever fewer than
 // kTopKGroup are free.
 constexpr int kTopKGroup = 4;
-static_assert(kTopKSlots - kSharedTopK > kTopKGroup, "candidate slots");
+static_assert(kTopKSlots - kSharedTopK > kTopKGroup && list_slots(true) - kSharedTopKSmall > kTopKGroup,
+              "candidate slots");
 constexpr int kWideShiftBytes = 2 * kFusedOwnRows * 4;  // kModeSweepWide: the row hand-over's shifts
 // kModeMu: each epilogue warp turns its 32 rows x mu_width columns through
 // shared memory, so that its stores run along the rows of the output (rows of
@@ -524,7 +536,6 @@ __device__ __forceinline__ uint64_t slot_of(float s, int32_t col) {
 }
 __device__ __forceinline__ float slot_score(uint64_t w) { return __uint_as_float((uint32_t)w); }
 __device__ __forceinline__ int32_t slot_col(uint64_t w) { return (int32_t)(w >> 32); }
-constexpr uint32_t kSlotStride = kEpiThreads * 8;
 
 // Merge a warp's candidate buffers (cnt candidates of this lane) into its
 // lists at shared address lv: round j inserts every lane's candidate j, where
@@ -532,6 +543,7 @@ constexpr uint32_t kSlotStride = kEpiThreads * 8;
 // it four at a time (independent loads: one shared-memory latency per four
 // shifts). Returns the new k-th score. Kept out of line: one copy serves every
 // call site.
+template <uint32_t kSlotStride>
 __device__ __noinline__ float list_merge(uint32_t lv, int k, int cnt) {
   const uint32_t last = lv + (uint32_t)(k - 1) * kSlotStride;
   float thr = slot_score(lds_u64(last));
@@ -581,7 +593,7 @@ struct SharedBound {
   uint32_t mine, other;  // shared addresses of the two threads' words
   uint32_t tag;          // the own tile, counted per CTA
   float pub;             // this thread's published value
-  __device__ __forceinline__ void publish(uint32_t lv, int k) {
+  __device__ __forceinline__ void publish(uint32_t lv, int k, uint32_t kSlotStride) {
     pub = nextafterf(slot_score(lds_u64(lv + (uint32_t)((k - 1) / 2) * kSlotStride)), -INFINITY);
     sts_u64(mine, ((uint64_t)tag << 32) | __float_as_uint(pub));
   }
@@ -595,11 +607,12 @@ struct SharedBound {
 // groups in which some lane beats its threshold form their scores again and
 // append them (keeping all 32 beside the next chunk's TMEM load in flight
 // would spill).
-template <bool RS>
+template <bool RS, bool SMALL>
 __device__ __forceinline__ void chunk_topk_shared(const uint32_t (&v)[32], const float* g, const float* fs,
                                                   uint64_t cc, int64_t colbase, int k, uint32_t lv, int& cnt,
                                                   float& thr, SharedBound& sb) {
   constexpr int kGroups = 32 / kTopKGroup;
+  constexpr uint32_t kSlotStride = list_threads(SMALL) * 8;
   static_assert(kTopKGroup == 4, "a group is one float4 of g");
   const float4* g4 = reinterpret_cast<const float4*>(g);
   const float4* fs4 = reinterpret_cast<const float4*>(fs);
@@ -636,9 +649,9 @@ __device__ __forceinline__ void chunk_topk_shared(const uint32_t (&v)[32], const
         ++cnt;
       }
     }
-    if (__any_sync(0xffffffffu, cnt > kTopKSlots - k - kTopKGroup)) {
-      thr = list_merge(lv, k, cnt);
-      sb.publish(lv, k);
+    if (__any_sync(0xffffffffu, cnt > list_slots(SMALL) - k - kTopKGroup)) {
+      thr = list_merge<kSlotStride>(lv, k, cnt);
+      sb.publish(lv, k, kSlotStride);
       cnt = 0;
     }
   }
@@ -954,8 +967,9 @@ __global__ void __launch_bounds__(kThreads, 1)
   }
   if constexpr (MODE == kModeTopKShared) {
     // no published bound yet (tags start at 1; shared memory may hold another launch's words)
-    if (threadIdx.x >= 64)
-      sts_u64(smem_u32(topk_list) + (uint32_t)(kTopKSlots * kEpiThreads + (int)threadIdx.x - 64) * 8u, 0ull);
+    if ((int)threadIdx.x >= 64 && (int)threadIdx.x < 64 + list_threads(SMALL))
+      sts_u64(smem_u32(topk_list) + (uint32_t)(list_slots(SMALL) * list_threads(SMALL) + (int)threadIdx.x - 64) * 8u,
+              0ull);
   }
   tc_fence_before();
   if constexpr (PAIR) {
@@ -1238,14 +1252,17 @@ __global__ void __launch_bounds__(kThreads, 1)
     // ranked lists: this thread's sorted candidates for its row and column half
     float tv[MODE == kModeTopK ? kMaxTopK : 1];
     int32_t ti[MODE == kModeTopK ? kMaxTopK : 1];
-    // shared-memory lists (k <= kSharedTopK): this thread's entry 0
-    const uint32_t lv = smem_u32(topk_list) + (uint32_t)(ew * 32 + lane) * 8u;
+    // shared-memory lists: this thread's entry 0 (128-row tiles: warps 0-3
+    // and 8-11 have rows; the others share their addresses and touch none)
+    constexpr uint32_t kSlotStride = list_threads(SMALL) * 8;
+    const int lt = (SMALL ? (ew >> 3) * 4 + (ew & 3) : ew) * 32 + lane;
+    const uint32_t lv = smem_u32(topk_list) + (uint32_t)lt * 8u;
     SharedBound sb{};
     {
-      // (rows' other column half: epilogue warp ew ^ 8)
-      const uint32_t words = smem_u32(topk_list) + (uint32_t)(kTopKSlots * kEpiThreads) * 8u;
-      sb.mine = words + (uint32_t)(ew * 32 + lane) * 8u;
-      sb.other = words + (uint32_t)((ew ^ 8) * 32 + lane) * 8u;
+      // (a row's other column half: epilogue warp ew ^ 8)
+      const uint32_t words = smem_u32(topk_list) + (uint32_t)(list_slots(SMALL) * list_threads(SMALL)) * 8u;
+      sb.mine = words + (uint32_t)lt * 8u;
+      sb.other = words + (uint32_t)(lt ^ (list_threads(SMALL) / 2)) * 8u;
     }
     int tcnt = 0;
     int merge_at = 0;  // the partner tile before which every warp merges its candidates
@@ -1309,13 +1326,14 @@ __global__ void __launch_bounds__(kThreads, 1)
         thr = -INFINITY;
       }
       if constexpr (MODE == kModeTopKShared) {
-        for (int i = 0; i < p.k; ++i) sts_u64(lv + (uint32_t)i * kSlotStride, slot_of(-INFINITY, 0x7fffffff));
+        if (!(SMALL && h == 1))
+          for (int i = 0; i < p.k; ++i) sts_u64(lv + (uint32_t)i * kSlotStride, slot_of(-INFINITY, 0x7fffffff));
         thr = -INFINITY;
         tcnt = 0;
         merge_at = jb + 1;
         sb.tag = (uint32_t)tile_iter + 1u;
         sb.pub = -INFINITY;
-        sts_u64(sb.mine, ((uint64_t)sb.tag << 32) | __float_as_uint(-INFINITY));
+        if (!(SMALL && h == 1)) sts_u64(sb.mine, ((uint64_t)sb.tag << 32) | __float_as_uint(-INFINITY));
       }
       for (int j = jb; j < je; ++j) {
         // every lane waits; the outcome is made warp-uniform so that the
@@ -1347,7 +1365,7 @@ __global__ void __launch_bounds__(kThreads, 1)
           if constexpr (MODE == kModeSweepWide) chunk_sum_wide<RS, FOLD>(va, gs4, fs4, cc, acc, wide_m, sum, comp);
           if constexpr (MODE == kModeTopK) chunk_topk<RS>(va, gsf, fsf, crow, colbase, p.k, tv, ti, &tcnt, thr);
           if constexpr (MODE == kModeTopKShared)
-            chunk_topk_shared<RS>(va, gsf, fsf, cc, colbase, p.k, lv, tcnt, thr, sb);
+            chunk_topk_shared<RS, SMALL>(va, gsf, fsf, cc, colbase, p.k, lv, tcnt, thr, sb);
           if constexpr (MODE == kModeMu)
             chunk_mu<RS, mu_width(KB)>(va, gsf, fsf, crow, colbase, mu_lo, mu_hi, mu_s1, mu_s2, lane, mu_nrow, mu_row,
                          topk_list + ew * mu_stage_floats(KB), p);
@@ -1370,7 +1388,7 @@ __global__ void __launch_bounds__(kThreads, 1)
           if constexpr (MODE == kModeTopK)
             chunk_topk<RS>(vb, gsf + 32, fsf + 32, crow, colbase + 32, p.k, tv, ti, &tcnt, thr);
           if constexpr (MODE == kModeTopKShared)
-            chunk_topk_shared<RS>(vb, gsf + 32, fsf + 32, cc, colbase + 32, p.k, lv, tcnt, thr, sb);
+            chunk_topk_shared<RS, SMALL>(vb, gsf + 32, fsf + 32, cc, colbase + 32, p.k, lv, tcnt, thr, sb);
           if constexpr (MODE == kModeMu)
             chunk_mu<RS, mu_width(KB)>(vb, gsf + 32, fsf + 32, crow, colbase + 32, mu_lo, mu_hi, mu_s1, mu_s2, lane, mu_nrow,
                          mu_row, topk_list + ew * mu_stage_floats(KB), p);
@@ -1409,8 +1427,8 @@ __global__ void __launch_bounds__(kThreads, 1)
           if (j + 1 == merge_at) {
             merge_at += 1 + (merge_at - jb) / 4;
             if (!idle) {
-              thr = list_merge(lv, p.k, tcnt);
-              sb.publish(lv, p.k);
+              thr = list_merge<kSlotStride>(lv, p.k, tcnt);
+              sb.publish(lv, p.k, kSlotStride);
               tcnt = 0;
             }
           }
@@ -1434,7 +1452,7 @@ __global__ void __launch_bounds__(kThreads, 1)
         }
       }
       if constexpr (MODE == kModeTopKShared) {
-        if (!(SMALL && h == 1)) list_merge(lv, p.k, tcnt);
+        if (!(SMALL && h == 1)) list_merge<kSlotStride>(lv, p.k, tcnt);
       }
       // the two column halves of a row meet (double-buffered by own-tile
       // parity, handed over through bounded mbarrier waits)
@@ -1871,6 +1889,7 @@ cudaError_t launch_wide_pair(int kb, int fmt, bool split, const CUtensorMap* own
                              const CUtensorMap* fold, const FusedParams* p, int grid, cudaStream_t stream);
 cudaError_t launch_lists(int64_t kp, int fmt, const CUtensorMap& own, const CUtensorMap& partner,
                          const FusedParams& p, int grid, cudaStream_t stream, bool small);
+bool lists_want_small(int k, int64_t kp, int fmt);
 cudaError_t launch_mu(int64_t kp, int fmt, const CUtensorMap& own, const CUtensorMap& partner, const FusedParams& p,
                       int grid, cudaStream_t stream);
 

@@ -23,9 +23,15 @@ cudaError_t launch_wide_pair(int kb, int fmt, bool split, const CUtensorMap* own
   return launch_pair<kModeSweepWide>(kb, fmt, split, own, half, fold, p, grid, stream);
 }
 
+// Lists longer than kSharedTopK fit in shared memory only with 128-row tiles
+// (half of the threads have rows, so each has twice the slots).
+bool lists_want_small(int k, int64_t kp, int fmt) {
+  return k > kSharedTopK && k <= kSharedTopKSmall && k_blocks(kp, fmt) < 4;
+}
+
 cudaError_t launch_lists(int64_t kp, int fmt, const CUtensorMap& own, const CUtensorMap& partner,
                          const FusedParams& p, int grid, cudaStream_t stream, bool small) {
-  if (p.k <= kSharedTopK && k_blocks(kp, fmt) < 4)
+  if (p.k <= (small ? kSharedTopKSmall : kSharedTopK) && k_blocks(kp, fmt) < 4)
     return launch_any<kModeTopKShared>(kp, fmt, own, partner, p, grid, stream, small);
   return launch_any<kModeTopK>(kp, fmt, own, partner, p, grid, stream, small);
 }
