@@ -60,6 +60,7 @@ struct tu_batch {
   int num_sms = 0;
   int grid = 0;  // CTAs of the batched half-sweep: one per SM
   int64_t kp = 0;
+  int ksteps = 0; // the most of any member (FusedParams::ksteps)
   int dtype = 0;  // the members' dtype (e4m3 markets: every member alike)
   cudaStream_t stream = nullptr;
   std::vector<tu_market*> markets;
@@ -469,6 +470,7 @@ cudaError_t enqueue_half(tu_batch* b, int si, int side, int residual, int update
   L.err = b->err_dev;
   L.grid = b->grid;
   L.kp = b->kp;
+  L.ksteps = b->ksteps;
   L.dtype = b->dtype;
   L.residual = residual;
   L.update = update;
@@ -632,6 +634,7 @@ tu_status tu_batch_create(const tu_market_t* markets, int count, void* stream, t
   b->grid = b->num_sms;
   b->kp = ms[0]->kp;
   b->dtype = ms[0]->dtype;
+  for (tu_market* m : ms) b->ksteps = std::max(b->ksteps, k_steps(m));
   b->stream = static_cast<cudaStream_t>(stream);
   b->markets = ms;
   b->c_host.assign(count, 0.0f);

@@ -96,11 +96,13 @@ cudaError_t make_fold_map(Side* sd) {
   return r == CUDA_SUCCESS ? cudaSuccess : cudaErrorInvalidValue;
 }
 
-// 128-row own tiles when they all fit one wave (and the market allows them):
-// a CTA with one MMA chain ends its tile in about 0.73 of the time of a
-// 256-row tile (measured at 1e4 x 1e4), so the small tiles win only while
-// SMs would otherwise stay idle; on a GPU already full (other markets' work
-// on other streams) they lose a third of the per-SM throughput.
+// 128-row own tiles when they all fit one wave (and the market allows them),
+// for launches that the cuts leave alone (row ranges, ranked lists, markets of
+// four partner tiles and fewer): a CTA with one MMA chain ends its tile in
+// about 0.73 of the time of a 256-row tile (measured at 1e4 x 1e4), so the
+// small tiles win only while SMs would otherwise stay idle; on a GPU already
+// full (other markets' work on other streams) they lose a third of the per-SM
+// throughput.
 bool use_small_tiles(const tu_market* m, int64_t rows) {
   if (m->small_mode == 0) return false;
   if (m->small_mode == 2) return true;
@@ -226,6 +228,7 @@ cudaError_t launch_fused_halfsweep(tu_market* m, int side, int residual, int upd
   FusedParams p = base_params(nrows, row0, 0, partner.rows, m->cmul, small);
   p.g = partner.pvec;
   p.lmax = m->st + kStShift;
+  p.ksteps = k_steps(m);
   p.own_off = m->st + kStOwnOff;
   p.grp = whole ? own.grp : nullptr;  // a range of rows does not write the side's groups
   p.b2s = own.b2s;
@@ -357,6 +360,7 @@ cudaError_t launch_fused_halfsweep_raw(const FusedRaw& r, cudaStream_t stream, i
   if ((e = make_map(&partner_map, r.par16, r.cols, r.kp, kFusedPartnerRows)) != cudaSuccess) return e;
   if ((e = set_kernel_attributes()) != cudaSuccess) return e;
   FusedParams p = base_params(r.rows, 0, 0, r.cols, (float)(1.4426950408889634 / (2.0 * r.sigma)));
+  p.ksteps = (int)(r.kp / 16);  // (the caller's rows: whole)
   p.g = r.g;
   p.lmax = r.lmax;
   p.b2s = r.b2s;
@@ -382,6 +386,7 @@ cudaError_t launch_fused_batch(const BatchLaunch& b, cudaStream_t stream) {
   static_assert(kEpiWarps / 2 == kBatchSlotWarps, "per-tile partial slots");
   // (the shared-memory opt-in was made when the member markets were prepared)
   FusedParams p{};
+  p.ksteps = b.ksteps;
   p.bdesc = b.desc;
   p.items = b.items;
   p.cta_start = b.cta_start;

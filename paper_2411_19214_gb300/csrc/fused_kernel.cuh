@@ -12,26 +12,31 @@
 // no per-pair running maximum is needed: the running-max rescale of
 // flash-attention collapses to one shift per half-sweep.
 //
-// CTA layout (576 threads, one CTA per SM, persistent over own tiles):
-//   warp 0     : producer (one elected thread): TMA loads of the own tile
+// CTA layout (576 threads, one CTA per SM, persistent over own tiles; a
+// half-sweep of rows of two or more k blocks runs on pairs of CTAs (PAIR): a
+// cluster of two takes two own tiles, each CTA holds half of every partner
+// tile, and the leader's MMA warp issues cta_group::2 MMAs for both):
+//   warp 0     : producer (one elected lane): TMA loads of the own tile
 //                [F|K]_j (256 rows x kp) once per own tile (double-buffered
 //                when kp = 64) and of partner tiles (128 rows x kp) through a
 //                STAGES-deep shared-memory ring (a stage is a whole partner
 //                tile, or with four 128-byte k blocks per row one k block of
-//                it), plus a bulk copy of each partner tile's 128 g values
-//                (e4m3 factors: and of its 128 row scales) into an 8-slot ring
-//                that the epilogue reads with broadcast loads.
+//                it, in a pair two), plus each partner tile's g: folded (see
+//                fold_for), 4 KB of MMA operand in the stage, else 128 floats
+//                (e4m3 with row scales: and the 128 scales) into an 8-slot
+//                ring that the epilogue reads with broadcast loads.
 //   warp 1     : MMA issuer: two tcgen05.mma M=128 N=128 chains
-//                (own rows 0-127 and 128-255) per partner tile into one of two
-//                TMEM accumulator buffers (2 x 256 columns = all 512).
+//                (own rows 0-127 and 128-255; a pair: M=256 over both CTAs)
+//                per partner tile into one of two TMEM accumulator buffers
+//                (2 x 256 columns = all 512).
 //   warps 2-17 : epilogue: epilogue warp e reads TMEM lane quadrant (e+2)%4
 //                of own sub-tile (e/4)%2 and column half e/8 of every partner
 //                tile, i.e. one own row and 64 columns per thread, so the row
 //                reduction stays inside the thread; the two column halves of
 //                a row meet through shared memory at the end of the own tile.
 //                TMEM loads run one 32-column chunk ahead of the arithmetic;
-//                per pair of columns one packed FMA (f32x2), two ex2.approx
-//                and one packed add; per-tile partials go into a compensated
+//                per pair of columns one packed FMA (f32x2; a multiply where
+//                g is folded), two ex2.approx and one packed add; per-tile partials go into a compensated
 //                (Kahan) sum.
 // In a batched launch the own tiles of a CTA come from a list of
 // (market, own tile) items of many independent markets.
@@ -63,6 +68,7 @@ struct FusedParams {
   int64_t ncols;           // partner columns streamed: [col0, col0 + ncols)
   int num_own_tiles;       // ceil(rows / 256)
   int num_partner_tiles;   // ceil(ncols / 128)
+  int ksteps;              // 32-byte steps of a packed row that hold factors (the rest is zeros)  (sweep)
   float c;                 // log2(e) / (2 sigma)
   const float* g;          // partner prepared potentials (index = partner user), -inf padded
   const double* lmax;      // partner shift (natural log)
@@ -1174,6 +1180,14 @@ __global__ void __launch_bounds__(kThreads, 1)
                 const uint32_t d_tmem = tmem_base + (uint32_t)(buf * 256 + h * 128);
 #pragma unroll
                 for (int k = 0; k < KBS * 4; ++k) {
+                  // Steps of padding add zeros: half-sweeps leave them out, to
+                  // the same bits (d = 100 in rows of 128, 13 of 16 steps: 50,001
+                  // x 70,000 1.77 -> 1.57 ms per sweep; d = 50, 10,000 x 10,000
+                  // 81.7 -> 80.6 us). Ranked lists gain nothing from it and the
+                  // test costs them 0.5 %.
+                  if constexpr (kSweepLike) {
+                    if (sp * KBS * 4 + k >= p.ksteps) break;
+                  }
                   const int kbl = k >> 2, kk = k & 3;
                   const uint64_t adesc =
                       a0 + (uint32_t)(sp * KBS * (kOwnBytesPerKB >> 4)) +

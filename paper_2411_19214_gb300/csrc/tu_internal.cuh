@@ -379,11 +379,14 @@ struct BatchLaunch {
   int* err;
   int grid;
   int64_t kp;              // 64 or 128 (BF16), the same for every market
+  int ksteps;              // the most of any member (FusedParams::ksteps)
   int dtype;               // the members' dtype (e4m3 markets: kp = 128 bytes per row, the same format)
   int residual;
   int update;
 };
 cudaError_t launch_fused_batch(const BatchLaunch& b, cudaStream_t stream);
+// The steps of a packed row [F | K | 0] that the MMAs take: one is 32 bytes of it.
+inline int k_steps(const tu_market* m) { return (int)((2 * m->d * (is_fp8(m->dtype) ? 1 : 2) + 31) / 32); }
 // ranked lists / mu block through the tensor-core pipeline (partner vector prepared in log2 mode)
 cudaError_t launch_fused_topk(tu_market* m, int side, int k, int64_t row0, int64_t nrows, int32_t* idx, float* logmu,
                               float* hand_v, int32_t* hand_i);
