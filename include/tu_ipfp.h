@@ -314,15 +314,15 @@ tu_status tu_market_use_graphs(tu_market_t mkt, int enable);
 
 /* Launch shape of the fused half-sweep (no counterpart in the paper; results
  * are the same fixed point whatever the shape).
- * Own-tile height, mode = 0: 256-row own tiles; 1 (the default): 128-row
- * tiles when a market's 256-row tiles would leave SMs idle while its 128-row
- * tiles all fit one wave (twice the CTAs, each ending its tile sooner: an
- * isolated 1e4 x 1e4 sweep 0.171 -> 0.132 ms); 2: always 128-row tiles. A
- * 128-row tile delivers about two thirds of a 256-row tile's per-SM
- * throughput, so callers that keep the GPU full with many markets at once (a
- * serving loop) set 0. Results are bit-identical across modes (every row's
- * arithmetic is the same). Dense markets ignore it. TU_ERR_INVALID_ARG for
- * another mode. */
+ * Own-tile height, mode = 0: 256-row own tiles, one CTA each; 1 (the
+ * default): the partner tiles of own tiles that would fill their last wave
+ * badly are divided over all SMs (an isolated 1e4 x 1e4 sweep 0.123 -> 0.080
+ * ms), and launches that are not divided take 128-row tiles when a market's
+ * 256-row tiles would leave SMs idle while its 128-row tiles all fit one wave;
+ * 2: always 128-row tiles. Whole 256-row tiles use an SM best, so callers that
+ * keep the GPU full with many markets at once (a serving loop) set 0. Results
+ * are bit-identical across modes (every row's arithmetic is the same). Dense
+ * markets ignore it. TU_ERR_INVALID_ARG for another mode. */
 tu_status tu_market_set_small_tiles(tu_market_t mkt, int mode);
 
 /* Partner split, 1 <= split <= 8 (fused markets; TU_ERR_UNSUPPORTED on the
@@ -330,11 +330,12 @@ tu_status tu_market_set_small_tiles(tu_market_t mkt, int mode);
  * ranges handled by different CTAs, and the CTA that completes a tile's
  * block of rows sums the ranges' partial row sums in range order and updates
  * the rows, so a market with few waves of own tiles fills the GPU in finer
- * steps (1e5 users: 391 tiles of 256 rows are 2.6 waves on 148 SMs, in
- * thirds 7.9). The sums are the same terms in another order (results agree
- * to rounding, not bit for bit with split = 1). Allocates split x max(N, M)
- * x 16 bytes of partial sums on first use. Applies to whole-side sweeps of
- * markets within the single-shift range (see tu_market_create). */
+ * steps. (The default shape, split = 1, already divides tiles where that
+ * saves time: see tu_market_set_small_tiles.) The sums are the same terms in
+ * another order (results agree to rounding, not bit for bit with split = 1).
+ * Allocates split x max(N, M) x 16 bytes of partial sums on first use. Applies
+ * to whole-side sweeps of markets within the single-shift range (see
+ * tu_market_create). */
 tu_status tu_market_set_split(tu_market_t mkt, int split);
 
 /* Partner blocks, 1 <= blocks <= 8 (fused markets; TU_ERR_UNSUPPORTED on the
