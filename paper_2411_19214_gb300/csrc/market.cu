@@ -1387,10 +1387,13 @@ int64_t tu_market_footprint(int64_t N, int64_t M, int64_t d, int path) {
   if (path == TU_PATH_FUSED) {
     bytes += (N + M) * kp * 2 + (np > mp ? np : mp) * 4;  // factors, per-row shifts
     if (kp <= 2 * kKBlock) bytes += (np + mp) * 32;              // the extra MMA's g / c operand
-    bytes += 2 << 20;                                        // the cut sums' partials
+    // the cut sums' partials, on the part's 152 SMs
+    const int kb = (int)(kp / kKBlock);
+    const int64_t sx = cut_slots(cut_plan(N, M, kb, 152)), sy = cut_slots(cut_plan(M, N, kb, 152));
+    if (sx + sy > 0) bytes += (sx > sy ? sx : sy) * kFusedOwnRows * (16 + 8) + (np > mp ? np : mp) / 4 + 256;
   } else {
     bytes += (N + M) * kp * 4 + N * round_up(M, 4) * 4 + M * round_up(N, 4) * 4;
-    bytes += 8 << 20;  // column sums of the one-pass sweep
+    if (N >= 512 && M >= 512) bytes += 8 << 20;  // column sums of the one-pass sweep
   }
   return bytes;
 }
