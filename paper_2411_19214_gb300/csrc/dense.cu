@@ -352,7 +352,7 @@ __global__ void __launch_bounds__(kPassThreads) k_dense_rowpass(
 //                   its slot released.
 //   row warp        (the cluster's first CTA) the rows' stored potentials in
 //                   FP64, residual and groups, 32 rows at a time, off the path.
-// The pass takes 127 us at 20,000 x 10,000 (6.3 TB/s, 0.93 of the measured copy
+// The pass takes 122 us at 20,000 x 10,000 (6.5 TB/s, 0.96 of the measured copy
 // rate); a sweep 272 -> 151 us. Rows in clusters: 30,000 x 30,000 1,106 -> 755 us
 // per sweep, 3,000 x 40,000 208 -> 131. The shares and weights of a cluster travel
 // by asynchronous stores; with plain remote stores and releasing arrivals its
