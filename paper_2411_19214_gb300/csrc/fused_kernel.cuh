@@ -1096,11 +1096,27 @@ __global__ void __launch_bounds__(kThreads, 1)
           }
         }
       }
+      if constexpr (PAIR) {
+        // The first CTA's commits arrive on the barriers of both CTAs, and the
+        // cluster barrier at the end orders threads, not these asynchronous
+        // arrivals: each CTA stays until the last one on each of its barriers has
+        // been seen (those on tfull are the epilogue's), so that none lands in
+        // shared memory that another CTA has taken over. At most the ring's
+        // stages of MMAs are left here, while the epilogue still works.
+        for (int s = 0; s < STAGES && ok; ++s)
+          if (armed[s]) ok = mbar_wait(&empty[s], (armed[s] - 1u) & 1u, abort_flag);
+        for (int b = 0; b < ABUF && ok; ++b)
+          if (a_armed[b]) ok = mbar_wait(&a_empty[b], (a_armed[b] - 1u) & 1u, abort_flag);
+        if (ok) ok = mbar_wait(mma_done, 0, abort_flag);
+      }
       if (!ok) {
         if (!*abort_flag) raise_error(p.err, abort_flag, kErrTimeout);
+        // (the first CTA commits mma_done on every path, at the latest when its
+        // own waits have run out)
+        if constexpr (PAIR) mbar_wait_drain(mma_done, 0, 2 * kWaitLimitNs);
         // let the copies already issued land before the CTA's shared memory goes
         // away (a pair's second CTA cannot see the barriers they are counted on:
-        // it waits for longer than any copy takes)
+        // it waits for longer than any copy or arrival takes)
         if (PAIR && rank != 0) {
           const uint64_t t0 = global_timer_ns();
           while (global_timer_ns() - t0 < 10000000ull) {
