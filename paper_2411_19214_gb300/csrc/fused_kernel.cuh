@@ -174,11 +174,17 @@ constexpr int kTailBytes = 512 + 512 + 2 * kFusedOwnRows * 4;
 // 2.74 -> 2.60 ms (without pairs 2.73 -> 2.80: shared memory is short). With four
 // blocks the tensor pipe is the bound. e4m3: the fold MMA is a separate
 // kind::f16 MMA (BF16 ones x BF16 g / c) into the same FP32 accumulator. e4m3
-// rows with per-row scales cannot fold: the own row's scale multiplies phi, so
-// no per-column constant added to it gives g in every row.
+// rows with per-row scales do not fold: the accumulator holds phi over the own
+// row's scale, so a per-column constant is not g in every row. Wide half-sweeps
+// do not either: c phi and g may be hundreds and cancel, and g * (1 / c) through
+// the accumulator and back rounds three times at that size where a fused
+// multiply-add rounds once (rms error of log u at sigma = 0.01, d = 32, 6,001 x
+// 9,001: 4.6e-6 folded, 3.5e-6 not; 80,000 x 100,001, d = 64: 3.10 ms per sweep
+// folded, 3.45 not). In narrow markets the fold costs no accuracy (6,001 x 9,001,
+// d = 64, sigma = 0.5: 3.5e-8 folded, 7.2e-8 not).
 constexpr int kFoldBytes = kFusedPartnerRows * 32;
 constexpr bool fold_for(int KB, int MODE, bool BATCH, int fmt, bool nofold) {
-  return (MODE == kModeSweep || MODE == kModeSweepWide) && (fmt == kFmtBF16 || fmt == kFmtE4M3Side) && KB <= 2 && !nofold;
+  return MODE == kModeSweep && (fmt == kFmtBF16 || fmt == kFmtE4M3Side) && KB <= 2 && !nofold;
 }
 constexpr int stage_bytes(int KB, bool fold, bool pair = false) {
   return (kbs_for(KB, pair) * kPartnerBytesPerKB + (fold ? kFoldBytes : 0)) / (pair ? 2 : 1);
@@ -379,21 +385,12 @@ __device__ __forceinline__ float exp2_int(float d) {
 // sum over the earlier tiles) is multiplied by 2^(M - M'), a power of two,
 // so exactly; then acc += 2^(t - M). Every term is at most 1, and the row's
 // log-sum is log(sum) + M ln 2.
-template <bool RS, bool FOLD>
+template <bool RS>
 __device__ __forceinline__ void chunk_sum_wide(uint32_t (&v)[32], const float4* gs4, const float4* fs4, uint64_t cc,
                                                uint64_t (&acc)[4], float& M, float& sum, float& comp) {
   // the exponents replace the loaded values in place
-  if constexpr (FOLD) {
 #pragma unroll
-    for (int i = 0; i < 16; ++i) {
-      uint64_t t = ((uint64_t)v[2 * i + 1] << 32) | v[2 * i];
-      asm("mul.rn.f32x2 %0, %0, %1;" : "+l"(t) : "l"(cc));
-      v[2 * i] = (uint32_t)t;
-      v[2 * i + 1] = (uint32_t)(t >> 32);
-    }
-  }
-#pragma unroll
-  for (int i = 0; i < (FOLD ? 0 : 8); ++i) {
+  for (int i = 0; i < 8; ++i) {
     const float4 gg = gs4[i];
     float4 ff = make_float4(1.f, 1.f, 1.f, 1.f);
     if constexpr (RS) ff = fs4[i];
@@ -1390,9 +1387,9 @@ __global__ void __launch_bounds__(kThreads, 1)
           tmem_ld_issue(taddr, va);
           tmem_ld_wait(va);
           tmem_ld_issue(taddr + 32, vb);
-          if constexpr (FOLD && !WIDE) chunk_sum_fold(va, cc, acc);
+          if constexpr (FOLD) chunk_sum_fold(va, cc, acc);
           if constexpr (MODE == kModeSweep && !FOLD) chunk_sum<RS>(va, gs4, fs4, cc, acc);
-          if constexpr (MODE == kModeSweepWide) chunk_sum_wide<RS, FOLD>(va, gs4, fs4, cc, acc, wide_m, sum, comp);
+          if constexpr (MODE == kModeSweepWide) chunk_sum_wide<RS>(va, gs4, fs4, cc, acc, wide_m, sum, comp);
           if constexpr (MODE == kModeTopK) chunk_topk<RS>(va, gsf, fsf, crow, colbase, p.k, tv, ti, &tcnt, thr);
           if constexpr (MODE == kModeTopKShared)
             chunk_topk_shared<RS, SMALL>(va, gsf, fsf, cc, colbase, p.k, lv, tcnt, thr, sb);
@@ -1412,9 +1409,9 @@ __global__ void __launch_bounds__(kThreads, 1)
           }
         }
         if (!idle) {
-          if constexpr (FOLD && !WIDE) chunk_sum_fold(vb, cc, acc);
+          if constexpr (FOLD) chunk_sum_fold(vb, cc, acc);
           if constexpr (MODE == kModeSweep && !FOLD) chunk_sum<RS>(vb, gs4 + 8, fs4 + 8, cc, acc);
-          if constexpr (MODE == kModeSweepWide) chunk_sum_wide<RS, FOLD>(vb, gs4 + 8, fs4 + 8, cc, acc, wide_m, sum, comp);
+          if constexpr (MODE == kModeSweepWide) chunk_sum_wide<RS>(vb, gs4 + 8, fs4 + 8, cc, acc, wide_m, sum, comp);
           if constexpr (MODE == kModeTopK)
             chunk_topk<RS>(vb, gsf + 32, fsf + 32, crow, colbase + 32, p.k, tv, ti, &tcnt, thr);
           if constexpr (MODE == kModeTopKShared)

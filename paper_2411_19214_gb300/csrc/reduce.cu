@@ -506,7 +506,7 @@ cudaError_t launch_prep(tu_market* m, Side& partner, int fused_mode, int transla
   const int own = &partner == &m->Y ? 0 : 1;
   const int g = grid_for(partner.rows_pad, m->num_sms, 4);
   k_prep<<<g, kThreads, 0, m->stream>>>(partner.ell, partner.rows, partner.rows_pad, m->st, own, translate, fused_mode,
-                                        partner.pvec + offset, fused_mode ? reinterpret_cast<uint4*>(partner.fold) : nullptr,
+                                        partner.pvec + offset, fused_mode && !m->wide ? reinterpret_cast<uint4*>(partner.fold) : nullptr,
                                         1.0f / m->cmul);  // (the batched preparation rounds 1 / c alike)
   return cudaGetLastError();
 }
@@ -566,7 +566,7 @@ cudaError_t launch_between(tu_market* m, int nparts, int is_x, int residual, int
                           m->results, translate ? 2 : 1};
   k_between<<<1 + grid_for(own.rows_pad, m->num_sms, 4), kThreads, 0, m->stream>>>(
       a, own.ell, own.rows, own.rows_pad, fused_mode, own.pvec,
-      fused_mode ? reinterpret_cast<uint4*>(own.fold) : nullptr, 1.0f / m->cmul);
+      fused_mode && !m->wide ? reinterpret_cast<uint4*>(own.fold) : nullptr, 1.0f / m->cmul);
   return cudaGetLastError();
 }
 
