@@ -343,7 +343,7 @@ __global__ void __launch_bounds__(kPassThreads) k_dense_rowpass(
 //   producer warp   streams units of `rows` rows (one slice of a row in a
 //                   cluster) into a ring in shared memory with bulk copies.
 //   dot warps       every thread owns fixed columns, its part of v in registers;
-//                   a row's dot product is parked per warp.
+//                   a row's dot product (compensated) is parked per warp.
 //   update warp     (the cluster's first CTA) sums a unit's parked shares and
 //                   hands the rows' weights 2^(ell log2 e - R) to the sum warps
 //                   of the cluster, in FP32.
@@ -352,9 +352,12 @@ __global__ void __launch_bounds__(kPassThreads) k_dense_rowpass(
 //                   its slot released.
 //   row warp        (the cluster's first CTA) the rows' stored potentials in
 //                   FP64, residual and groups, 32 rows at a time, off the path.
-// The pass takes 122 us at 20,000 x 10,000 (6.5 TB/s, 0.96 of the measured copy
-// rate); a sweep 272 -> 151 us. Rows in clusters: 30,000 x 30,000 1,106 -> 755 us
-// per sweep, 3,000 x 40,000 208 -> 131. The shares and weights of a cluster travel
+// A sweep of 20,000 x 10,000 takes 174 us (two passes: 268); rows in clusters,
+// 30,000 x 30,000 808 us (1,101), 3,000 x 40,000 135 (206). With plain dot products
+// it was 149, 747 and 124 (the pass at 6.5 TB/s, 0.96 of the measured copy rate):
+// the compensation's three more operations per pair of terms are what bounds the
+// pass now. Eight dot warps, of 736 threads of 88 registers: five took 220 us at
+// 20,000 x 10,000, six 228, seven 211, ten 183. The shares and weights of a cluster travel
 // by asynchronous stores; with plain remote stores and releasing arrivals its
 // update warp took 1.5 us per row and the pass was slower than two.
 // A row passes through load, dot, update and sum one after another, about
@@ -373,7 +376,7 @@ __device__ __forceinline__ float exp2_whole(int d) {
 
 constexpr int kSweepWidth = 10240;  // columns of a slice, at most
 constexpr int kSweepSums = 12;      // sum warps (28 columns per thread, at most)
-constexpr int kSweepDots = 5;       // dot warps (64 columns per thread, at most)
+constexpr int kSweepDots = 8;       // dot warps (40 columns per thread, at most)
 constexpr int kSweepRows = 8;       // rows of a unit, at most
 constexpr int kSweepSlots = 24;     // ring slots, at most
 constexpr int kSweepCl = 8;         // cluster size, at most
@@ -411,12 +414,16 @@ __device__ __forceinline__ uint64_t mul2(uint64_t a, uint64_t b) {
   asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b));
   return d;
 }
+// s += n; what the addition rounds off stays in n
+__device__ __forceinline__ void carry2(uint64_t& s, uint64_t& n) {
+  const uint64_t t = add2(s, n);
+  n = sub2(n, sub2(t, s));
+  s = t;
+}
 // kahan_fma on pairs; n is the compensation with its sign turned
 __device__ __forceinline__ void kahan_fma2(uint64_t& s, uint64_t& n, uint64_t x, uint64_t w) {
-  const uint64_t y = fma2(x, w, n);
-  const uint64_t t = add2(s, y);
-  n = sub2(y, sub2(t, s));
-  s = t;
+  n = fma2(x, w, n);
+  carry2(s, n);
 }
 
 struct SweepSmem {
@@ -614,16 +621,20 @@ __global__ void __launch_bounds__(kSweepThreads, 1) k_dense_sweep(const SweepArg
       const int nb = (int)(a.rows - r0 < B ? a.rows - r0 : B);
       const Quad* r4 = reinterpret_cast<const Quad*>(ring + (size_t)t * slot_floats) + tid;
       for (int b = 0; b < nb; ++b, r4 += nq) {
-        uint64_t d0 = 0ull, d1 = 0ull;
+        // four compensated sums per thread, as in the row pass (carry2 outside the
+        // test: without a column it adds the compensation alone)
+        uint64_t d0 = 0ull, d1 = 0ull, n0 = 0ull, n1 = 0ull;
 #pragma unroll
         for (int j = 0; j < ND; ++j) {
           if (tid + j * kStep < nq) {
             const Quad x = r4[j * kStep];
-            d0 = fma2(x.x, w[j].x, d0);
-            d1 = fma2(x.y, w[j].y, d1);
+            n0 = fma2(x.x, w[j].x, n0);
+            n1 = fma2(x.y, w[j].y, n1);
           }
+          carry2(d0, n0);
+          carry2(d1, n1);
         }
-        d0 = add2(d0, d1);
+        d0 = add2(add2(d0, n0), add2(d1, n1));
         float r = low2(d0) + high2(d0);
         for (int o = 16; o > 0; o >>= 1) r += __shfl_xor_sync(0xffffffffu, r, o);
         if (lane == 0) {
@@ -842,19 +853,19 @@ typedef void (*SweepKernel)(SweepArgs);
 template <bool CLUSTER>
 SweepKernel sweep_kernel_for(int width) {
   const int na = (width / 4 + kSweepSums * 32 - 1) / (kSweepSums * 32);
-  if (na <= 1) return k_dense_sweep<1, 3, CLUSTER>;
-  if (na == 2) return k_dense_sweep<2, 5, CLUSTER>;
-  if (na == 3) return k_dense_sweep<3, 8, CLUSTER>;
-  if (na == 4) return k_dense_sweep<4, 10, CLUSTER>;
-  if (na == 5) return k_dense_sweep<5, 12, CLUSTER>;
-  if (na == 6) return k_dense_sweep<6, 15, CLUSTER>;
-  return k_dense_sweep<7, 16, CLUSTER>;
+  if (na <= 1) return k_dense_sweep<1, 2, CLUSTER>;
+  if (na == 2) return k_dense_sweep<2, 3, CLUSTER>;
+  if (na == 3) return k_dense_sweep<3, 5, CLUSTER>;
+  if (na == 4) return k_dense_sweep<4, 6, CLUSTER>;
+  if (na == 5) return k_dense_sweep<5, 8, CLUSTER>;
+  if (na == 6) return k_dense_sweep<6, 9, CLUSTER>;
+  return k_dense_sweep<7, 10, CLUSTER>;
 }
-// (a slice of up to na * 1,536 columns needs na * 2.4 quads per dot thread, the longest 16)
-static_assert(7 * kSweepSums * 128 >= kSweepWidth && 16 * kSweepDots * 128 >= kSweepWidth, "columns per thread");
-static_assert(kSweepDots * 3 >= kSweepSums && kSweepDots * 5 >= kSweepSums * 2 && kSweepDots * 8 >= kSweepSums * 3 &&
-                  kSweepDots * 10 >= kSweepSums * 4 && kSweepDots * 12 >= kSweepSums * 5 &&
-                  kSweepDots * 15 >= kSweepSums * 6,
+// (a slice of up to na * 1,536 columns needs na * 1.5 quads per dot thread, the longest 10)
+static_assert(7 * kSweepSums * 128 >= kSweepWidth && 10 * kSweepDots * 128 >= kSweepWidth, "columns per thread");
+static_assert(kSweepDots * 2 >= kSweepSums && kSweepDots * 3 >= kSweepSums * 2 && kSweepDots * 5 >= kSweepSums * 3 &&
+                  kSweepDots * 6 >= kSweepSums * 4 && kSweepDots * 8 >= kSweepSums * 5 &&
+                  kSweepDots * 9 >= kSweepSums * 6,
               "columns per thread");
 SweepKernel sweep_kernel(const DensePlan& p) {
   return p.cl > 1 ? sweep_kernel_for<true>(p.width) : sweep_kernel_for<false>(p.width);
