@@ -13,6 +13,8 @@
 // bytes of HBM instead of N * M * 4.
 #include "tu_internal.cuh"
 
+#include <type_traits>
+
 namespace tu {
 
 namespace {
@@ -352,11 +354,11 @@ __global__ void __launch_bounds__(kPassThreads) k_dense_rowpass(
 //                   its slot released.
 //   row warp        (the cluster's first CTA) the rows' stored potentials in
 //                   FP64, residual and groups, 32 rows at a time, off the path.
-// A sweep of 20,000 x 10,000 takes 174 us (two passes: 268); rows in clusters,
-// 30,000 x 30,000 808 us (1,101), 3,000 x 40,000 135 (206). With plain dot products
-// it was 149, 747 and 124 (the pass at 6.5 TB/s, 0.96 of the measured copy rate):
-// the compensation's three more operations per pair of terms are what bounds the
-// pass now. Eight dot warps, of 736 threads of 88 registers: five took 220 us at
+// A sweep of 20,000 x 10,000 takes 177 us (two passes: 268); rows in clusters,
+// 30,000 x 30,000 649 us (1,101), 3,000 x 40,000 143 (206). With plain dot products
+// and FP32 weights 20,000 x 10,000 took 149 (the pass at 6.5 TB/s, 0.96 of the
+// measured copy rate): the compensation's three more operations per pair of terms
+// are what bounds the pass now. Eight dot warps, of 736 threads with 80 registers: five took 220 us at
 // 20,000 x 10,000, six 228, seven 211, ten 183. The shares and weights of a cluster travel
 // by asynchronous stores; with plain remote stores and releasing arrivals its
 // update warp took 1.5 us per row and the pass was slower than two.
@@ -364,6 +366,12 @@ __global__ void __launch_bounds__(kPassThreads) k_dense_rowpass(
 // 5,000 cycles; with one slot of the ring per row in flight the SM still takes
 // one 40 KB row per 1,700 cycles, its share of HBM. (One set of warps doing
 // both products in turn was the bound: 165 us per 800 MB pass.)
+// A row's weight is that of its stored potential, rounded once: the FP32
+// logarithms are those of row_update, and what FP32 rounds off their sum is kept
+// (weight_pow2). The rms error of log v against float64 is then 0.93 of the two
+// passes' over 27 heights and widths (0.64 to 1.32: the FP32 logarithm of a sum
+// rounds by where in its binade the sum lies); with exp2f of an FP32 exponent
+// its mean was off by up to 3e-8, where the two passes' is by 1e-8.
 // R is an integer per cluster, raised when a row's exponent passes it by 40
 // (weights up to 2^40 against A-hat up to e^40 stay in the FP32 range); the
 // column sums so far are then rescaled by a power of two, exactly. At the end
@@ -372,6 +380,20 @@ __global__ void __launch_bounds__(kPassThreads) k_dense_rowpass(
 // 2^d for any integer d, exactly, flushed to 0 below FP32's normal range and to infinity above it
 __device__ __forceinline__ float exp2_whole(int d) {
   return d < -126 ? 0.0f : (d > 127 ? INFINITY : __int_as_float((127 + d) << 23));
+}
+
+// 2^(f + l), f in [-0.5, 0.5] and l a few units of f's last place, to half a
+// unit: the series of e^x - 1 at x = (f + l) ln 2, |x| <= 0.35, up to x^8 / 8!,
+// whose first term keeps its rounding.
+__device__ __forceinline__ float weight_pow2(float f, float l) {
+  const float kLn2 = 0.693147182464599609375f, kLn2Lo = -1.904654323e-9f;
+  const float x = f * kLn2;
+  const float xl = fmaf(f, kLn2, -x) + fmaf(f, kLn2Lo, l * kLn2);
+  // (in pairs of terms: the update warp's chain is what the clusters wait for)
+  const float x2 = x * x;
+  const float q6 = fmaf(x2, 1.0f / 40320.0f, fmaf(x, 1.0f / 5040.0f, 1.0f / 720.0f));
+  const float q0 = fmaf(x2, fmaf(x, 1.0f / 120.0f, 1.0f / 24.0f), fmaf(x, 1.0f / 6.0f, 0.5f));
+  return 1.0f + (x + fmaf(x2, fmaf(x2 * x2, q6, q0), xl));
 }
 
 constexpr int kSweepWidth = 10240;  // columns of a slice, at most
@@ -433,7 +455,8 @@ struct SweepSmem {
   float part[kSweepSlots][kSweepRows][kSweepDots];
   float weight[kSweepSlots][kSweepRows];
   float scale[kSweepSlots];
-  float4 row[2][32];            // a batch's rows: log2 constants of their updates
+  float4 row[2][32];            // a batch's rows: constants of their updates, see row warp
+  float4 frac[2][32];
   float2 sum[2][32];            // and their sums (hi, lo)
   uint64_t full[kSweepSlots];   // a unit has landed
   uint64_t empty[kSweepSlots];  // every sum warp is done with it
@@ -656,80 +679,118 @@ __global__ void __launch_bounds__(kSweepThreads, 1) k_dense_sweep(const SweepArg
   } else if (warp == kSweepUpdate) {
     // ---------------------------------------------------------- update warp
     if (rank == 0) {
+      // (A cluster's units are single rows, and this warp's chain of about 2,000
+      // cycles per turn is what it waits for: with slots to spare the half-warps
+      // take a unit each, 30,000 x 30,000 in 7 slots 891 -> 649 us per sweep. With
+      // 5 slots two units at a time leave too few loads in flight, 3,000 x 40,000
+      // 143 -> 167.)
       int R = 0, pb = 0;
       uint32_t dph = 0;
       bool ok = true;
-      for (int64_t k = 0; k < nu; ++k) {
-        const int64_t r0 = (cid + k * P) * B;
-        const int nb = (int)(a.rows - r0 < B ? a.rows - r0 : B);
-        const bool mine = lane < nb;
-        const int64_t batch = k * B / 32;
-        const int at = (int)(k * B % 32) + (mine ? lane : 0);  // this row in its batch
-        const int bb = (int)(batch & 1);
-        bool got = at - (mine ? lane : 0) != 0 || mbar_wait(&S.ahead[bb], (uint32_t)(batch >> 1) & 1u, abort_flag);
-        got = got && mbar_wait(&S.done[pb], dph, abort_flag);
-        if (!__all_sync(0xffffffffu, got)) {
-          ok = false;
-          break;
-        }
-        // the warps' shares of a row, added with their roundings kept
-        float hi = 0.0f, lo = 0.0f;
-        if constexpr (CLUSTER) {
-          const volatile float* p = S.part[pb][0];
-          for (int i = lane; i < kSweepDots * cl; i += 32) pair_add(hi, lo, p[i], 0.0f);
-          for (int o = 16; o > 0; o >>= 1)
-            pair_add(hi, lo, __shfl_xor_sync(0xffffffffu, hi, o), __shfl_xor_sync(0xffffffffu, lo, o));
-        } else {
-          const volatile float* p = S.part[pb][mine ? lane : 0];
+      auto update = [&](auto units) {
+        constexpr int U = decltype(units)::value, L = 32 / U;  // units at a time, lanes per unit
+        const int half = lane / L, hl = lane % L;
+        for (int64_t k = 0; k < nu; k += U) {
+          const bool here = k + half < nu;  // (this half-warp has a unit)
+          const int sl = pb + half < slots ? pb + half : pb + half - slots;
+          const uint32_t sph = pb + half < slots ? dph : dph ^ 1u;
+          const int64_t r0 = (cid + (k + half) * P) * B;
+          const int nb = !here ? 0 : (int)(a.rows - r0 < B ? a.rows - r0 : B);
+          const bool mine = hl < nb;
+          const int64_t batch = k * B / 32;
+          const int at = (int)(k * B % 32) + half + (mine ? hl : 0);  // this row in its batch
+          const int bb = (int)(batch & 1);
+          bool got = k * B % 32 != 0 || mbar_wait(&S.ahead[bb], (uint32_t)(batch >> 1) & 1u, abort_flag);
+          if (here) got = got && mbar_wait(&S.done[sl], sph, abort_flag);
+          if (!__all_sync(0xffffffffu, got)) {
+            ok = false;
+            break;
+          }
+          const float4 cst = S.row[bb][at], frc = S.frac[bb][at];
+          // the warps' shares of a row, added with their roundings kept
+          float hi = 0.0f, lo = 0.0f;
+          if constexpr (CLUSTER) {
+            const volatile float* p = S.part[sl][0];
+            for (int i = hl; i < kSweepDots * cl; i += L) pair_add(hi, lo, p[i], 0.0f);
+            for (int o = L / 2; o > 0; o >>= 1)
+              pair_add(hi, lo, __shfl_xor_sync(0xffffffffu, hi, o), __shfl_xor_sync(0xffffffffu, lo, o));
+          } else {
+            const volatile float* p = S.part[pb][mine ? lane : 0];
 #pragma unroll
-          for (int i = 0; i < kSweepDots; ++i) pair_add(hi, lo, p[i], 0.0f);
-        }
-        // The row's weight u 2^-R in FP32: log2 of the sum and of u are each an
-        // integer plus a fraction, so that no digits go to their size
-        // (row_update's closed form with z = log s - 1/2 log n in log2 units).
-        const volatile float4* cst = reinterpret_cast<const volatile float4*>(&S.row[bb][at]);
-        const int nc = __float_as_int(cst->x), nB = __float_as_int(cst->z);
-        const float fc = cst->y, fB = cst->w;
-        int ex;
-        const float m = frexpf(hi, &ex);
-        const float rel = __fdividef(lo, hi) * kLog2e;
-        const float lm = log2f(m) + rel;
-        const float z2 = (float)(nc + ex) + (fc + lm);
-        int n;
-        float f;
-        if (z2 > 0.0f) {
-          const float c = log1pf(sqrtf(1.0f + exp2f(-2.0f * z2)));
-          n = nB - nc - ex;
-          f = ((fB - fc) - lm) - c * kLog2e;
-        } else {
-          n = nB;
-          f = fB - asinhf(exp2f(z2)) * kLog2e;
-        }
-        const int top = __reduce_max_sync(0xffffffffu, mine ? n : -0x40000000);
-        float sc = 1.0f;
-        if (k == 0 || top > R + 40) {
-          if (k > 0) sc = exp2_whole(R - top);
-          R = top;
-        }
-        // (a sum that is not finite makes the weight so, or 0 for an infinite one)
-        const float u = exp2f(f) * exp2_whole(n - R);
-        if constexpr (CLUSTER) {
-          const float u0 = __shfl_sync(0xffffffffu, u, 0);
-          if (lane < cl)
-            cluster_store_async2(cluster_addr(&S.weight[pb][0], lane), u0, sc, cluster_addr(&S.ready[pb], lane));
-        } else {
-          if (mine) S.weight[pb][lane] = u;
-          if (lane == 0) S.scale[pb] = sc;
+            for (int i = 0; i < kSweepDots; ++i) pair_add(hi, lo, p[i], 0.0f);
+          }
+          // The row's weight u 2^-R in FP32 from row_update's closed form, z = log s -
+          // 1/2 log n and the logarithms with its values; log2 u is an integer plus a
+          // fraction in two floats, so that no digits go to its size.
+          // (log_row_sum_parts without its third part, which is 0)
+          int ex;
+          float rest;
+          const float total = two_sum(hi, lo, rest);
+          const float lm = __fadd_rn(logf(frexpf(total, &ex)), __fdividef(rest, total));
+          const float z = fmaf((float)(__float_as_int(cst.x) + ex), 0.69314718056f, cst.y) + lm;
+          int n;
+          float v, ve = 0.0f, f, l;  // the logarithm to take off (natural, two floats), and from what (log2)
+          if (z > 0.0f) {
+            v = two_sum(lm, log1pf(sqrtf(1.0f + expf(-2.0f * z))), ve);
+            n = __float_as_int(cst.z) - ex;
+            f = frc.x;
+            l = frc.y;
+          } else {
+            v = asinhf(expf(z));
+            n = __float_as_int(cst.w);
+            f = frc.z;
+            l = frc.w;
+          }
+          const float kLog2eLo = 1.925962989e-8f, pr = v * kLog2e;  // (kLog2e + kLog2eLo is log2 e)
+          float fe;
+          f = two_sum(f, -pr, fe);
+          l += fe - (fmaf(v, kLog2e, -pr) + fmaf(ve, kLog2e, v * kLog2eLo));
+          // (a sum that is not finite: 0 for an infinite one, else not a number)
+          const bool fin = v < INFINITY;
+          const float whole = fin ? rintf(f) : 0.0f;
+          n += (int)whole;
+          const float frac_u = fin ? weight_pow2(f - whole, l) : (v > 0.0f ? 0.0f : v);
+          // what the column sums so far take before each unit, and the units' scale
+          float sc = 1.0f;
+          int scale_here = R;
+          for (int h = 0; h < U && k + h < nu; ++h) {
+            const int top = CLUSTER ? __shfl_sync(0xffffffffu, n, h * L) : __reduce_max_sync(0xffffffffu, mine ? n : -0x40000000);
+            float s1 = 1.0f;
+            if (k + h == 0 || top > R + 40) {
+              if (k + h > 0) s1 = exp2_whole(R - top);
+              R = top;
+            }
+            if (half == h) {
+              sc = s1;
+              scale_here = R;
+            }
+          }
+          const float u = frac_u * exp2_whole(n - scale_here);
+          if constexpr (CLUSTER) {
+            const float u0 = __shfl_sync(0xffffffffu, u, half * L);
+            if (here && hl < cl)
+              cluster_store_async2(cluster_addr(&S.weight[sl][0], hl), u0, sc, cluster_addr(&S.ready[sl], hl));
+          } else {
+            if (mine) S.weight[pb][lane] = u;
+            if (lane == 0) S.scale[pb] = sc;
+            __syncwarp();
+            if (lane == 0) mbar_arrive(&S.ready[pb]);
+          }
+          if (mine) S.sum[bb][at] = make_float2(hi, lo);
           __syncwarp();
-          if (lane == 0) mbar_arrive(&S.ready[pb]);
+          if (lane == 0 && ((k + U) * B % 32 == 0 || k + U >= nu)) mbar_arrive(&S.summed[bb]);
+          pb += U;
+          if (pb >= slots) {
+            pb -= slots;
+            dph ^= 1u;
+          }
         }
-        if (mine) S.sum[bb][at] = make_float2(hi, lo);
-        __syncwarp();
-        if (lane == 0 && ((k + 1) * B % 32 == 0 || k == nu - 1)) mbar_arrive(&S.summed[bb]);
-        if (++pb == slots) {
-          pb = 0;
-          dph ^= 1u;
-        }
+      };
+      if constexpr (CLUSTER) {
+        if (slots >= 7) update(std::integral_constant<int, 2>());
+        else update(std::integral_constant<int, 1>());
+      } else {
+        update(std::integral_constant<int, 1>());
       }
       if (ok && lane == 0) a.scale[cid] = R;
       if (!ok && !*abort_flag) pass_abort(a.err, abort_flag);
@@ -753,10 +814,14 @@ __global__ void __launch_bounds__(kSweepThreads, 1) k_dense_sweep(const SweepArg
         const int64_t row = row_of(i);
         const double b = a.b2s != nullptr ? (double)a.b2s[row] : 0.0;
         const double hl = 0.5 * (double)logf((float)a.mass[row]);
+        // z is c2 plus the sum's logarithm; log u + b is d2 less that and log1p's
+        // (z > 0), or b2 less asinh's: in log2 units, as an integer and a fraction
         const double c2 = ((kLnHalf + b + shift) - hl) * 1.4426950408889634, b2 = (hl + b) * 1.4426950408889634;
-        const double cn = rint(c2), bn = rint(b2);
-        S.row[j & 1][lane] = make_float4(__int_as_float((int)cn), (float)(c2 - cn), __int_as_float((int)bn),
-                                         (float)(b2 - bn));
+        const double d2 = b2 - c2, cn = rint(c2), bn = rint(b2), dn = rint(d2);
+        const float df = (float)(d2 - dn), bf = (float)(b2 - bn);
+        S.row[j & 1][lane] = make_float4(__int_as_float((int)cn), (float)((c2 - cn) * 0.69314718055994530942),
+                                         __int_as_float((int)dn), __int_as_float((int)bn));
+        S.frac[j & 1][lane] = make_float4(df, (float)((d2 - dn) - (double)df), bf, (float)((b2 - bn) - (double)bf));
       }
       __syncwarp();
       if (lane == 0) mbar_arrive(&S.ahead[j & 1]);
