@@ -59,6 +59,7 @@ struct tu_batch {
   int device = 0;
   int num_sms = 0;
   int grid = 0;  // CTAs of the batched half-sweep: one per SM
+  int blocks = 1;  // blocks per market of the kernels over a market's users
   int64_t kp = 0;
   int ksteps = 0; // the most of any member (FusedParams::ksteps)
   int dtype = 0;  // the members' dtype (e4m3 markets: every member alike)
@@ -96,12 +97,26 @@ namespace {
 
 // A block has about kBlockRows users: with one block per market the largest
 // (50,000 users) kept a block busy for 50 to 220 us while the rest of the chip
-// was idle (flush 163 us, preparation 57, sum of squares 224; 56 markets).
+// was idle (flush 163 us, preparation 57, sum of squares 224; 56 markets). A
+// launch has the blocks of the batch's largest market for every market, at most
+// kMarketBlocks and kLaunchBlocks in all (blocks_per_market): those that a
+// smaller market does not need return at once, but starting them is not free
+// (32 blocks for each of 10,000 markets of 100 users: 1.66 ms per sweep, with
+// one 1.06; 4,000 such markets and one of 50,000 x 40,000: 1.50 and, with two,
+// 1.34).
 constexpr int kMarketBlocks = 32;
 constexpr int kBlockRows = 2048;
-__device__ __forceinline__ int market_blocks(int64_t rows) {
+constexpr int64_t kLaunchBlocks = 8192;
+__host__ __device__ __forceinline__ int market_blocks(int64_t rows, int most) {
+  if (most == 1) return 1;  // (without waiting for the market's rows)
   const int64_t n = (rows + kBlockRows - 1) / kBlockRows;
-  return n < 1 ? 1 : (n > kMarketBlocks ? kMarketBlocks : (int)n);
+  return n < 1 ? 1 : (n > most ? most : (int)n);
+}
+int blocks_per_market(const std::vector<tu_market*>& markets) {
+  int64_t rows = 1;
+  for (const tu_market* m : markets) rows = std::max(rows, std::max(m->X.rows_pad, m->Y.rows_pad));
+  const int64_t most = std::min<int64_t>(kMarketBlocks, kLaunchBlocks / (int64_t)markets.size());
+  return market_blocks(rows, (int)std::max<int64_t>(most, 1));
 }
 // Whether this block is the last of the market's `blocks` to get here (on every
 // thread); what the others wrote before is then visible. The counter is a
@@ -109,6 +124,7 @@ __device__ __forceinline__ int market_blocks(int64_t rows) {
 __device__ __forceinline__ bool last_block(double* st, int blocks) {
   __shared__ int last;
   __syncthreads();
+  if (blocks == 1) return true;
   if (threadIdx.x == 0) {
     __threadfence();
     last = atomicInc(reinterpret_cast<unsigned*>(st + kStCount), (unsigned)blocks - 1u) == (unsigned)blocks - 1u;
@@ -128,7 +144,7 @@ __global__ void __launch_bounds__(kPrepThreads) k_batch_prep(const BatchDesc* __
                                                             const int* __restrict__ n_list, int sweep) {
   if ((int)blockIdx.x >= *n_list) return;
   const BatchDesc& d = desc[list[blockIdx.x]];
-  const int blocks = market_blocks(d.partner_rows_pad);
+  const int blocks = market_blocks(d.partner_rows_pad, gridDim.y);
   if ((int)blockIdx.y >= blocks) return;
   const double top = d.st[kStLmax + (1 - d.own_side)];  // not written by prep_scalars
   if (blockIdx.y == 0 && threadIdx.x == 0) prep_scalars(d.st, d.own_side, sweep && d.translate);
@@ -213,7 +229,7 @@ __global__ void __launch_bounds__(kFinThreads) k_batch_reset(const BatchDesc* __
   __shared__ float redf[2 * kFinThreads / 32];
   const BatchDesc& x = desc_x[mk];
   const BatchDesc& y = desc_y[mk];
-  const int blocks = market_blocks(x.rows > y.rows ? x.rows : y.rows);
+  const int blocks = market_blocks(x.rows > y.rows ? x.rows : y.rows, gridDim.y);
   if ((int)blockIdx.y >= blocks) return;
   const int lane = threadIdx.x % 32;
   const int64_t warp = (int64_t)blockIdx.y * (kFinThreads / 32) + threadIdx.x / 32;
@@ -251,7 +267,7 @@ __global__ void __launch_bounds__(kFinThreads) k_batch_flush(const BatchDesc* __
   double* st = desc_x[mk].st;
   const double off[2] = {st[kStOff + 0], st[kStOff + 1]};
   const int64_t rx = desc_x[mk].rows, ry = desc_y[mk].rows;
-  const int blocks = market_blocks(rx > ry ? rx : ry);
+  const int blocks = market_blocks(rx > ry ? rx : ry, gridDim.y);
   if ((int)blockIdx.y >= blocks) return;
   for (int s = 0; s < 2; ++s) {
     if (off[s] == 0.0) continue;
@@ -279,7 +295,7 @@ __global__ void __launch_bounds__(kFinThreads) k_batch_sum_sq(const BatchDesc* _
   if ((int)blockIdx.x >= *n_list) return;
   const int mk = list[blockIdx.x];
   const BatchDesc& d = desc_y[mk];
-  const int blocks = market_blocks(d.rows);
+  const int blocks = market_blocks(d.rows, gridDim.y);
   if ((int)blockIdx.y >= blocks) return;
   __shared__ double red[kFinThreads / 32];
   double s = 0.0;
@@ -458,7 +474,7 @@ cudaError_t enqueue_half(tu_batch* b, int si, int side, int residual, int update
   const Schedule& S = b->sched[si];
   const int* n = S.dev;
   const int* list = S.dev + S.off_list;
-  k_batch_prep<<<dim3(b->count, kMarketBlocks), kPrepThreads, 0, b->stream>>>(b->desc_dev[side], list, n, update);
+  k_batch_prep<<<dim3(b->count, b->blocks), kPrepThreads, 0, b->stream>>>(b->desc_dev[side], list, n, update);
   cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess) return e;
   if ((e = profile_mark(b, true)) != cudaSuccess) return e;
@@ -490,7 +506,7 @@ cudaError_t enqueue_sweep(tu_batch* b) {
 // After a block of sweeps over schedule 0: pending offsets into the arrays.
 cudaError_t enqueue_flush(tu_batch* b) {
   const Schedule& S = b->sched[0];
-  k_batch_flush<<<dim3(b->count, kMarketBlocks), kFinThreads, 0, b->stream>>>(b->desc_dev[0], b->desc_dev[1], S.dev + S.off_list, S.dev);
+  k_batch_flush<<<dim3(b->count, b->blocks), kFinThreads, 0, b->stream>>>(b->desc_dev[0], b->desc_dev[1], S.dev + S.off_list, S.dev);
   return cudaGetLastError();
 }
 
@@ -637,6 +653,7 @@ tu_status tu_batch_create(const tu_market_t* markets, int count, void* stream, t
   for (tu_market* m : ms) b->ksteps = std::max(b->ksteps, k_steps(m));
   b->stream = static_cast<cudaStream_t>(stream);
   b->markets = ms;
+  b->blocks = blocks_per_market(ms);
   b->c_host.assign(count, 0.0f);
   if (cudaSetDevice(b->device) != cudaSuccess) return bail(TU_ERR_CUDA);
   // descriptors: side 0 updates X against Y, side 1 updates Y against X
@@ -776,7 +793,7 @@ tu_status tu_batch_solve(tu_batch_t b, double tol, int max_iter, int warm_start,
   for (int i = 0; i < count; ++i) all[i] = i;
   if (!warm_start) {
     TB_TRY(sched_set(b, b->sched[0], all));
-    k_batch_reset<<<dim3(count, kMarketBlocks), kFinThreads, 0, b->stream>>>(b->desc_dev[0], b->desc_dev[1],
+    k_batch_reset<<<dim3(count, b->blocks), kFinThreads, 0, b->stream>>>(b->desc_dev[0], b->desc_dev[1],
                                                                              b->sched[0].dev + 4, b->sched[0].dev);
     TB_CK(b, cudaGetLastError());
   }
@@ -879,7 +896,7 @@ tu_status tu_batch_solve(tu_batch_t b, double tol, int max_iter, int warm_start,
   TB_TRY(reset_omega(b));
   // match counts from the column equations: sum_xy mu_xy = sum m - sum v^2
   TB_TRY(sched_set(b, b->sched[1], all));
-  k_batch_sum_sq<<<dim3(count, kMarketBlocks), kFinThreads, 0, b->stream>>>(
+  k_batch_sum_sq<<<dim3(count, b->blocks), kFinThreads, 0, b->stream>>>(
       b->desc_dev[1], b->sched[1].dev + 4, b->sched[1].dev, b->sums, b->results);
   TB_CK(b, cudaGetLastError());
   TB_TRY(read_results(b));
