@@ -444,8 +444,8 @@ tu_status load_factors(tu_market* m, const void* F, const void* K, const void* G
   if (e == cudaSuccess) e = cudaStreamSynchronize(m->stream);
   if (e != cudaSuccess) return fail_cuda(m, e, "factor norms");
   const float* hn = read + kScratchNorms;
-  if (!std::isfinite(read[0]) || !std::isfinite(read[1]))
-    return fail(m, TU_ERR_NONFINITE, "popularity biases contain NaN or Inf");
+  if (!std::isfinite(read[0])) return fail(m, TU_ERR_NONFINITE, "bias_x contains NaN or Inf");
+  if (!std::isfinite(read[1])) return fail(m, TU_ERR_NONFINITE, "bias_y contains NaN or Inf");
   if (!std::isfinite(hn[0]) || !std::isfinite(hn[1]))
     return fail(m, TU_ERR_NONFINITE, "factor matrices contain NaN or Inf");
   const double bound = (double)hn[0] * (double)hn[1] / (2.0 * m->sigma);  // FP8: norms of the quantized rows
