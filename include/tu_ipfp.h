@@ -377,9 +377,11 @@ typedef struct {
 tu_status tu_market_autotune(tu_market_t mkt, int reps, tu_tune_info* info);
 
 /* The autotuner's cache as a JSON file (one entry per line; load merges the
- * file's entries, which replace cached ones with the same key). Save or load
- * of a path that cannot be opened, or load of a malformed file:
- * TU_ERR_INVALID_ARG (nothing is merged). */
+ * file's entries, which replace cached ones with the same key). New markets
+ * take an entry only if its "shapes" is this library's (2; none counts as 1):
+ * the tuner's choice holds against the default shape that it was timed
+ * against. Save or load of a path that cannot be opened, or load of a malformed
+ * file: TU_ERR_INVALID_ARG (nothing is merged). */
 tu_status tu_autotune_cache_save(const char* path);
 tu_status tu_autotune_cache_load(const char* path);
 void tu_autotune_cache_clear(void);

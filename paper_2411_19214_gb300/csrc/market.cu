@@ -1122,9 +1122,16 @@ struct TuneKey {
     return std::tie(nb, mb, kp, fmt, sms) < std::tie(o.nb, o.mb, o.kp, o.fmt, o.sms);
   }
 };
+// The set of launch shapes that an entry was timed against: raised when the
+// default shape changes. Entries of other sets (files without the field: 1,
+// before the default divided own tiles and ran on pairs of CTAs) stay in the
+// cache and in saved files, but no market takes them: they were faster than a
+// default that is gone (10,000 x 10,000, d = 50: 0.097 ms per sweep, now 0.078).
+constexpr int kTuneShapes = 2;
 struct TuneVal {
   int small_mode, split;
   double ms, ms_default;
+  int shapes;
 };
 std::mutex g_tune_mu;
 std::map<TuneKey, TuneVal> g_tune;
@@ -1141,7 +1148,7 @@ void apply_tuned(tu_market* m) {
   {
     std::lock_guard<std::mutex> lk(g_tune_mu);
     auto it = g_tune.find(tune_key(m));
-    if (it == g_tune.end()) return;
+    if (it == g_tune.end() || it->second.shapes != kTuneShapes) return;
     v = it->second;
   }
   if (set_shape_code(m, v.small_mode, v.split) != TU_OK) {
@@ -1252,7 +1259,7 @@ tu_status tu_market_autotune(tu_market_t m, int reps, tu_tune_info* info) {
   TU_TRY(clear_results(m));
   {
     std::lock_guard<std::mutex> lk(g_tune_mu);
-    g_tune[tune_key(m)] = TuneVal{cand[bi].first, cand[bi].second, best, ms_default};
+    g_tune[tune_key(m)] = TuneVal{cand[bi].first, cand[bi].second, best, ms_default, kTuneShapes};
   }
   if (info != nullptr) {
     info->small_tiles = cand[bi].first;
@@ -1275,9 +1282,9 @@ tu_status tu_autotune_cache_save(const char* path) {
     char line[320];
     snprintf(line, sizeof(line),
              "{\"n_bucket\": %d, \"m_bucket\": %d, \"kp\": %lld, \"dtype\": %d, \"sms\": %d, "
-             "\"small_tiles\": %d, \"split\": %d, \"ms\": %.6g, \"ms_default\": %.6g}%s\n",
+             "\"small_tiles\": %d, \"split\": %d, \"ms\": %.6g, \"ms_default\": %.6g, \"shapes\": %d}%s\n",
              kv.first.nb, kv.first.mb, (long long)kv.first.kp, kv.first.fmt, kv.first.sms, kv.second.small_mode,
-             kv.second.split, kv.second.ms, kv.second.ms_default, ++i < g_tune.size() ? "," : "");
+             kv.second.split, kv.second.ms, kv.second.ms_default, kv.second.shapes, ++i < g_tune.size() ? "," : "");
     f << line;
   }
   f << "]}\n";
@@ -1302,6 +1309,12 @@ tu_status tu_autotune_cache_load(const char* path) {
       return TU_ERR_INVALID_ARG;
     if (v.small_mode < 0 || v.small_mode > 2 || v.split == 0 || v.split < -kMaxSplit || v.split > kMaxSplit)
       return TU_ERR_INVALID_ARG;
+    const size_t at = line.find("\"shapes\":");
+    if (at == std::string::npos) {
+      v.shapes = 1;
+    } else if (sscanf(line.c_str() + at, "\"shapes\": %d", &v.shapes) != 1) {
+      return TU_ERR_INVALID_ARG;
+    }
     k.kp = kp;
     read[k] = v;
   }
