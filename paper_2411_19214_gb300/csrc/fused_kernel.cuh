@@ -165,14 +165,18 @@ constexpr int kbs_for(int KB, bool pair = false) { return KB == 4 ? (pair ? 2 : 
 //                [reduction: 512 B][row hand-over: 2 x 256 floats]
 constexpr int kTailBytes = 512 + 512 + 2 * kFusedOwnRows * 4;
 // folded g: the partner tile's K = 16 operand rides in its (last) stage, the
-// own side's constant operand (ones in columns 0-2) is one tile of its own.
+// own side's constant operand (ones in columns 0-3) is one tile of its own.
 // Taken for rows of one and two k blocks (d <= 64 in BF16, d <= 128 in e4m3 with
 // one scale per side), where the tensor pipe has room for one more MMA per
 // chain and the epilogue, which bounds these kernels, sheds its g loads.
 // One block: batched d = 32 half-sweep 5.44 -> 5.12 ms, a 1e5 d = 32 sweep
 // 3.54 -> 3.37 ms. Two blocks, on pairs of CTAs: a 100,003 x 79,999 d = 64 sweep
-// 2.74 -> 2.60 ms (without pairs 2.73 -> 2.80: shared memory is short). With four
-// blocks the tensor pipe is the bound. e4m3: the fold MMA is a separate
+// 2.74 -> 2.60 ms. Without pairs, where shared memory is short, two blocks lose a
+// little (own-tile mode 0, d = 64: 100,003 x 79,999 3.31 ms unfolded, 3.45 folded,
+// 20,000 x 15,001 0.249 and 0.254; a row range of 50,000 1.03 and 1.07; batches of
+// 56 markets 2.71 and 2.81, of 512 small ones 0.487 and 0.483) and fold all the
+// same: a market has the same bits in every launch shape. With four blocks the
+// tensor pipe is the bound. e4m3: the fold MMA is a separate
 // kind::f16 MMA (BF16 ones x BF16 g / c) into the same FP32 accumulator. e4m3
 // rows with per-row scales do not fold: the accumulator holds phi over the own
 // row's scale, so a per-column constant is not g in every row. Wide half-sweeps
@@ -180,8 +184,10 @@ constexpr int kTailBytes = 512 + 512 + 2 * kFusedOwnRows * 4;
 // the accumulator and back rounds three times at that size where a fused
 // multiply-add rounds once (rms error of log u at sigma = 0.01, d = 32, 6,001 x
 // 9,001: 4.6e-6 folded, 3.5e-6 not; 80,000 x 100,001, d = 64: 3.10 ms per sweep
-// folded, 3.45 not). In narrow markets the fold costs no accuracy (6,001 x 9,001,
-// d = 64, sigma = 0.5: 3.5e-8 folded, 7.2e-8 not).
+// folded, 3.45 not). In narrow markets the error is smaller folded for most sigma
+// (6,001 x 9,001, d = 64, rms of log u folded / not: 0.53 at sigma = 0.5 and 1, 0.9
+// at 0.35 and 0.7, 0.6 at 0.25, 1.0 at 0.1; below, where exponents reach tens, up
+// to 1.2 of 1e-7 to 3e-7).
 constexpr int kFoldBytes = kFusedPartnerRows * 32;
 constexpr bool fold_for(int KB, int MODE, bool BATCH, int fmt, bool nofold) {
   return MODE == kModeSweep && (fmt == kFmtBF16 || fmt == kFmtE4M3Side) && KB <= 2 && !nofold;
@@ -958,13 +964,13 @@ __global__ void __launch_bounds__(kThreads, 1)
     }
   }
   if constexpr (FOLD) {
-    // the own side's operand of the extra MMA: BF16 ones in columns 0-2 of
+    // the own side's operand of the extra MMA: BF16 ones in columns 0-3 of
     // every row (16-byte chunk q holds columns 0-7 when (q / 8) is even),
     // made visible to the tensor core's (async) proxy
     if (threadIdx.x < kFoldBytes / 16) {
       const bool cols0_7 = ((threadIdx.x / 8) % 2) == 0;
       reinterpret_cast<uint4*>(sOnes)[threadIdx.x] =
-          cols0_7 ? make_uint4(0x3F803F80u, 0x00003F80u, 0u, 0u) : make_uint4(0u, 0u, 0u, 0u);
+          cols0_7 ? make_uint4(0x3F803F80u, 0x3F803F80u, 0u, 0u) : make_uint4(0u, 0u, 0u, 0u);
     }
     asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
   }

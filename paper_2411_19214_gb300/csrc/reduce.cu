@@ -230,7 +230,7 @@ __global__ void k_row_norm_max(const float* __restrict__ f32, const __nv_bfloat1
 // the scalars it writes.
 __device__ __forceinline__ void prep_row(int64_t i, int64_t rows, const double* __restrict__ ell, double top,
                                         int fused_mode, float* __restrict__ out, uint4* __restrict__ fold,
-                                        float inv_c) {
+                                        float inv_c, float c) {
   float v;
   if (i < rows) {
     // the FP64 state is rounded once, to the FP32 vector the half-sweep streams
@@ -240,17 +240,17 @@ __device__ __forceinline__ void prep_row(int64_t i, int64_t rows, const double* 
     v = fused_mode ? -INFINITY : 0.0f;
   }
   out[i] = v;
-  if (fold != nullptr) write_fold_row(fold, i, v, inv_c);
+  if (fold != nullptr) write_fold_row(fold, i, v, inv_c, c);
 }
 
 __global__ void k_prep(const double* __restrict__ ell, int64_t rows, int64_t rows_pad, double* __restrict__ st,
                        int own, int translate, int fused_mode, float* __restrict__ out, uint4* __restrict__ fold,
-                       float inv_c) {
+                       float inv_c, float c) {
   const double top = st[kStLmax + (1 - own)];
   if (blockIdx.x == 0 && threadIdx.x == 0) prep_scalars(st, own, translate);
   for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < rows_pad;
        i += (int64_t)gridDim.x * blockDim.x) {
-    prep_row(i, rows, ell, top, fused_mode, out, fold, inv_c);
+    prep_row(i, rows, ell, top, fused_mode, out, fold, inv_c, c);
   }
 }
 
@@ -395,7 +395,7 @@ __global__ void __launch_bounds__(kThreads) k_finalize(const FinalizeArgs a) { f
 // and preparation one after the other took 12 us of a 10,000-user half-sweep.
 __global__ void __launch_bounds__(kThreads) k_between(const FinalizeArgs a, const double* __restrict__ ell,
                                                      int64_t rows, int64_t rows_pad, int fused_mode,
-                                                     float* __restrict__ out, uint4* __restrict__ fold, float inv_c) {
+                                                     float* __restrict__ out, uint4* __restrict__ fold, float inv_c, float c) {
   if (blockIdx.x == 0) {
     finalize_pass(a);
     return;
@@ -407,7 +407,7 @@ __global__ void __launch_bounds__(kThreads) k_between(const FinalizeArgs a, cons
   const double top = finite_or_zero((double)me);
   for (int64_t i = (blockIdx.x - 1) * (int64_t)kThreads + threadIdx.x; i < rows_pad;
        i += (int64_t)(gridDim.x - 1) * kThreads)
-    prep_row(i, rows, ell, top, fused_mode, out, fold, inv_c);
+    prep_row(i, rows, ell, top, fused_mode, out, fold, inv_c, c);
 }
 
 // sum_i exp(2 log u_i) in FP64 as per-block partials in the common format.
@@ -502,12 +502,16 @@ cudaError_t launch_pack_fp8_bytes(tu_market* m, Side& s, const uint8_t* A, const
   return cudaGetLastError();
 }
 
+// c for write_fold_row, in markets whose folded g makes good the rounding of 1 / c
+// (those that never run batched: the batched preparation has the three values)
+static float fold_c(const tu_market* m) { return m->dtype == TU_DTYPE_FP8E4M3_SIDE && m->kp == 256 ? m->cmul : 0.0f; }
+
 cudaError_t launch_prep(tu_market* m, Side& partner, int fused_mode, int translate, int offset) {
   const int own = &partner == &m->Y ? 0 : 1;
   const int g = grid_for(partner.rows_pad, m->num_sms, 4);
   k_prep<<<g, kThreads, 0, m->stream>>>(partner.ell, partner.rows, partner.rows_pad, m->st, own, translate, fused_mode,
                                         partner.pvec + offset, fused_mode && !m->wide ? reinterpret_cast<uint4*>(partner.fold) : nullptr,
-                                        1.0f / m->cmul);  // (the batched preparation rounds 1 / c alike)
+                                        1.0f / m->cmul, fold_c(m));  // (the batched preparation rounds 1 / c alike)
   return cudaGetLastError();
 }
 
@@ -566,7 +570,7 @@ cudaError_t launch_between(tu_market* m, int nparts, int is_x, int residual, int
                           m->results, translate ? 2 : 1};
   k_between<<<1 + grid_for(own.rows_pad, m->num_sms, 4), kThreads, 0, m->stream>>>(
       a, own.ell, own.rows, own.rows_pad, fused_mode, own.pvec,
-      fused_mode && !m->wide ? reinterpret_cast<uint4*>(own.fold) : nullptr, 1.0f / m->cmul);
+      fused_mode && !m->wide ? reinterpret_cast<uint4*>(own.fold) : nullptr, 1.0f / m->cmul, fold_c(m));
   return cudaGetLastError();
 }
 
