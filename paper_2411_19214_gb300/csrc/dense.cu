@@ -858,7 +858,16 @@ __global__ void __launch_bounds__(kSweepThreads, 1) k_dense_sweep(const SweepArg
     if (lane == 0) store_partials(a.partials + 4 * cid, acc);
   }
   // no CTA of a cluster leaves while another may still write to its shared memory
-  if constexpr (CLUSTER) cluster_sync();
+  // (the asynchronous stores of a pass that ends as it should have been counted by
+  // then; after an abort they get longer than any takes to land)
+  if constexpr (CLUSTER) {
+    cluster_sync();
+    if (*abort_flag) {
+      const uint64_t t0 = global_timer_ns();
+      while (global_timer_ns() - t0 < 10000000ull) {
+      }
+    }
+  }
 }
 
 // The Y update from the clusters' column sums: 32 columns per block, the
