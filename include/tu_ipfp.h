@@ -322,7 +322,9 @@ tu_status tu_market_use_graphs(tu_market_t mkt, int enable);
  * 2: always 128-row tiles. Whole 256-row tiles use an SM best, so callers that
  * keep the GPU full with many markets at once (a serving loop) set 0. Results
  * are bit-identical across modes (every row's arithmetic is the same). Dense
- * markets ignore it. TU_ERR_INVALID_ARG for another mode. */
+ * markets ignore it, and so do ranked lists of 15 to 32 entries of rows of up to
+ * 256 bytes, which run on 128-row tiles in every mode (their lists fit on chip
+ * there only). TU_ERR_INVALID_ARG for another mode. */
 tu_status tu_market_set_small_tiles(tu_market_t mkt, int mode);
 
 /* Partner split, 1 <= split <= 8 (fused markets; TU_ERR_UNSUPPORTED on the
@@ -565,7 +567,9 @@ tu_status tu_set_checked_mode(int enable);
  * violation (NUL-terminated, truncated to last_size) is written there. */
 int64_t tu_guard_violations(char* last, int64_t last_size);
 
-/* Free every resource of the market (safe on NULL). */
+/* Free every resource of the market (safe on NULL). When the last market of the
+ * process goes, up to 64 MB of device memory stay mapped in the library's pool
+ * for the next one; the rest goes back to the device. */
 void tu_market_destroy(tu_market_t mkt);
 
 /* Static description of a status code. */

@@ -90,8 +90,9 @@ struct Side {
   __nv_bfloat16* fac16 = nullptr;  // packed [F | K] (or [G | L]) rows x kp, bf16, zero padded
   uint8_t* fac8 = nullptr;         // FP8 markets: packed rows x kp e4m3 of [F | K] / fs (zero padded)
   float* fs = nullptr;             // FP8 markets: per-row scales, rows_pad (padding 1)
-  uint8_t* fold = nullptr;         // BF16 fused markets, kp <= 128: this side's g / c as the K = 16 operand of
-                                   // the partner tiles' extra MMA (rows_pad x 32 bytes, tcgen05 layout)
+  uint8_t* fold = nullptr;         // packed rows of one or two 128-byte blocks, BF16 or e4m3 with one scale per
+                                   // side: this side's g / c as the K = 16 operand of the partner tiles' extra
+                                   // MMA (rows_pad x 32 bytes, tcgen05 layout; unused while the market is wide)
   int fp8_exp = 0;                 // FP8 markets with one scale per side: its exponent (fs = 2^fp8_exp)
   float* fac32 = nullptr;          // packed rows x kp, fp32 (dense path), zero padded
   CUtensorMap tm_own;       // TMA map, box kKBlock x kFusedOwnRows
@@ -343,8 +344,8 @@ struct BatchDesc {
   double* ell;                 // own ell (out)
   const double* partner_ell;   // partner ell (read by the preparation kernel)
   float* g;                    // partner prepared vector (written by the preparation kernel)
-  uint8_t* gfold;              // BF16, kp = 64: the partner's g / c operand of the extra MMA (written by the
-                               // preparation kernel), else nullptr
+  uint8_t* gfold;              // the partner's g / c operand of the extra MMA (Side::fold, written by the
+                               // preparation kernel), or nullptr
   double* st;                  // the market's scalars (kSt*; shift and own offset of the pass)
   const float* fs_own;         // e4m3 markets: own per-row scales, else nullptr
   const float* fs_par;         // e4m3 markets: partner per-row scales, else nullptr
