@@ -727,7 +727,7 @@ __global__ void __launch_bounds__(kSweepThreads, 1) k_dense_sweep(const SweepArg
           float rest;
           const float total = two_sum(hi, lo, rest);
           const float lm = __fadd_rn(logf(frexpf(total, &ex)), __fdividef(rest, total));
-          const float z = fmaf((float)(__float_as_int(cst.x) + ex), 0.69314718056f, cst.y) + lm;
+          const float z = fmaf((float)(__float_as_int(cst.x) + ex), 0.69314718056f, cst.y + lm);
           int n;
           float v, ve = 0.0f, f, l;  // the logarithm to take off (natural, two floats), and from what (log2)
           if (z > 0.0f) {

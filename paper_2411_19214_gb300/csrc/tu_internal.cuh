@@ -499,12 +499,14 @@ __device__ __forceinline__ RowResult row_update(int ex, float lm, double shift, 
     o.r_abs = fabs(r);
     o.r_rel = fabs(r) / mass;
   } else if (residual == kResidualEstimate) {
-    const float e2 = expf((float)__dadd_rn(__dadd_rn(log_u_old, 0.69314718055994530942), ls) + lm);
+    const float e2 = expf((float)__dadd_rn(__dadd_rn(__dadd_rn(log_u_old, 0.69314718055994530942), ls), (double)lm));
     const double r = __dadd_rn(__dadd_rn((double)expf(2.0f * (float)log_u_old), -mass), (double)e2);
     o.r_abs = fabs(r);
     o.r_rel = (double)__fdiv_rn(fabsf((float)r), nf);
   }
-  const float z = (float)fma(-0.5, ln, ls) + lm;
+  // (rounded once: without lm the sum is the same for like rows, and so would be
+  // the error of rounding it first, up to 2e-8 of their log u)
+  const float z = (float)__dadd_rn(fma(-0.5, ln, ls), (double)lm);
   double lu;
   if (z > 0.0f) {
     const float c = log1pf(sqrtf(1.0f + expf(-2.0f * z)));
