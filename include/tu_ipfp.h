@@ -118,7 +118,7 @@ typedef struct {
  * half-sweep keeps every FP32 term in range; beyond ("wide" markets, strong
  * preferences or small sigma), the fused path keeps a running maximum of
  * every row's exponents and rescales the row's sum by an exact power of two
- * whenever it grows (one pass over the pairs, 1.2 to 1.3 times the time of
+ * whenever it grows (one pass over the pairs, 1.3 times the time of
  * a narrow half-sweep), and the dense path refuses the market
  * (TU_ERR_UNSUPPORTED: its materialised FP32 A-hat would overflow). In wide
  * markets the FP32 accumulation of phi carries an absolute error of about
